@@ -407,7 +407,8 @@ struct abs_ctx {
   cudaError_t launch_error = cudaSuccess;
   int next_cluster = 1;              // cluster width of the next launch (consumed by launch_on)
   int upd_blocks_per_sm = 8;         // resident blocks per SM of the Eq. 3 kernel
-  bool local_sgd = false;            // U > 1: one CTA per selected worker runs the worker's local steps
+  bool local_sgd = false;            // U > 1 on a single-layer model: one kernel runs the workers' local steps
+  local::Geo local_geo = {};         // ... with a cluster of local_geo.Q CTAs per worker (0: one CTA per worker)
   bool lsq_pipe = false;             // bf16 least squares through the bulk-copy pipeline kernel
   int lsq_stages = 0;
   bool lsq_v2 = false;               // least squares through the persistent 16-byte-load kernel
@@ -590,6 +591,13 @@ int setup_tc(abs_ctx* ctx) {
     if (!ok) return fail(ABS_ECUDA, "cuTensorMapEncodeTiled failed for layer %d", l);
   }
   return ABS_OK;
+}
+
+// the cluster form of the local-step kernel for C classes
+template <typename T>
+void (*local_cluster_fn(int C))(local::Args, local::Geo) {
+  return C <= 4 ? local::local_cluster_kernel<T, 4> : C <= 8 ? local::local_cluster_kernel<T, 8>
+         : C <= 12 ? local::local_cluster_kernel<T, 12> : local::local_cluster_kernel<T, 16>;
 }
 
 enum Phase : int { PH_GATHER = 0, PH_FORWARD = 1, PH_BACKWARD = 2 };
@@ -1080,10 +1088,18 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
   if (model->local_steps > 1 && !L.local_net) {
     const int C = model->kind == ABS_LSQ ? 1 : model->dims[1];
     const int n_par = model->kind == ABS_LSQ ? model->dims[0] : model->dims[0] * C + C;
-    const int sm = (int)local::smem_bytes(n_par, model->batch, C);
-    cudaError_t el = cudaFuncSetAttribute(local::local_sgd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (el == cudaSuccess) el = cudaFuncSetAttribute(local::local_sgd_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (el != cudaSuccess) return bail(cuda_fail(nullptr, el, "cudaFuncSetAttribute(local_sgd_kernel)"));
+    ctx->local_geo = local::cluster_plan(model->dims[0], C, model->batch, W, (int)L.esz);
+    cudaError_t el;
+    if (ctx->local_geo.Q > 0) {
+      const int sm = (int)local::cluster_smem(ctx->local_geo, (int)L.esz, model->batch, round_up(C, 4));
+      el = L.esz == 4 ? cudaFuncSetAttribute(local_cluster_fn<float>(C), cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
+                      : cudaFuncSetAttribute(local_cluster_fn<__nv_bfloat16>(C), cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    } else {
+      const int sm = (int)local::smem_bytes(n_par, model->batch, C);
+      el = L.esz == 4 ? cudaFuncSetAttribute(local::local_sgd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
+                      : cudaFuncSetAttribute(local::local_sgd_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    }
+    if (el != cudaSuccess) return bail(cuda_fail(nullptr, el, "cudaFuncSetAttribute(local-step kernel)"));
     ctx->local_sgd = true;
   }
   if (!ctx->local_sgd && model->kind == ABS_LSQ && model->dims[0] % 8 == 0 && model->dims[0] <= LSQ_MAX_D) {
@@ -1202,12 +1218,18 @@ int abs_enqueue_rounds(abs_ctx* ctx, int n) {
     q.in = ctx->m.dims[0]; q.C = q.lsq ? 1 : ctx->m.dims[1]; q.U = ctx->m.local_steps; q.lr = ctx->m.lr;
     const size_t sm = local::smem_bytes(q.lsq ? q.in : q.in * q.C + q.C, ctx->m.batch, q.C);
     const int nt = local::threads_for(q.lsq ? q.in : q.in * q.C + q.C);
+    const local::Geo geo = ctx->local_geo;
+    const size_t csm_local = geo.Q > 0 ? local::cluster_smem(geo, (int)ctx->L.esz, ctx->m.batch, round_up(q.C, 4)) : 0;
     for (int r = 0; r < n; ++r) {
       const int t = ctx->rounds_enqueued + r, par = t & 1;
       launch_ex(ctx, ABS_KC_CTL, ctl_kernel, dim3(1), dim3(ctl_threads), csm, ctx->ctl, 1, 1, t, 0, 0);
       q.ri = ctx->at<RoundInfo>(ctx->L.ri) + par;
       q.sel = ctx->ctl.sel[par]; q.sel_tau = ctx->ctl.sel_tau[par];
-      if (f32) launch_ex(ctx, ABS_KC_LSQ, local::local_sgd_kernel<float>, dim3(ctx->W), dim3(nt), sm, q);
+      if (geo.Q > 0) {
+        ctx->next_cluster = geo.Q;
+        launch_ex(ctx, ABS_KC_LSQ, f32 ? local_cluster_fn<float>(q.C) : local_cluster_fn<__nv_bfloat16>(q.C), dim3(ctx->W * geo.Q),
+                  dim3(local::CL_THREADS), csm_local, q, geo);
+      } else if (f32) launch_ex(ctx, ABS_KC_LSQ, local::local_sgd_kernel<float>, dim3(ctx->W), dim3(nt), sm, q);
       else launch_ex(ctx, ABS_KC_LSQ, local::local_sgd_kernel<__nv_bfloat16>, dim3(ctx->W), dim3(nt), sm, q);
       update(par);
     }

@@ -74,8 +74,9 @@ struct RoundInfo {
   int n_rows;       // padded gradient rows
   int K;            // K^t
   int t;            // round index
-  int diverged;     // set by the loss kernels of the round
+  int diverged;     // set by the loss kernels of the round; RI_TIMEOUT: a bounded wait of such a kernel expired
 };
+constexpr int RI_TIMEOUT = 2;
 
 // Pointers the control kernel works on (all device memory inside the workspace).
 struct CtlArgs {

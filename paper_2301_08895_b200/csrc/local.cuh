@@ -10,9 +10,12 @@
 // The chains of different workers are independent but each is strictly sequential, so the kernel
 // is latency-bound by design; a step is B short dot products and one rank-B update.
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 #include "ctl.cuh"
 #include "narrow.cuh"
+#include "lsqpipe.cuh"
 
 namespace absb {
 namespace local {
@@ -197,6 +200,447 @@ __global__ void __launch_bounds__(NT_MAX) local_sgd_kernel(Args a) {
     const float loss = __fdiv_rn(loss_sum, (float)U);
     a.loss[i] = loss;
     if (!isfinite(loss)) ri->diverged = 1;
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The same local steps with a CLUSTER of Q CTAs per selected worker.  The one-CTA kernel above uses K of
+// 148 SMs and walks every row twice through L2 with scalar loads; here CTA q of the cluster owns the features
+// [q F, (q + 1) F) of the worker's model, which stay in its shared memory for the whole job:
+//   - the slice of a step's B rows is copied once (asynchronously, one step ahead: a job's minibatches are known
+//     from the counter-based generator) and serves both the forward pass and the gradient,
+//   - the CTAs exchange their partial logits through distributed shared memory (one cluster barrier per step,
+//     then every CTA reads its peers' [B][C] blocks), and every CTA forms the soft-max, the deltas and the gradient
+//     of its own features,
+//   - a helper warp draws indices, issues the copies and finishes loss and bias, off the critical path.
+// A step is bound by its chain of phases (copy wait, partial dots, exchange, soft-max, gradient, reduction), each a
+// few hundred to a few thousand cycles of dependent shared-memory reads.
+struct Geo {
+  int Q;        // CTAs per worker (cluster width)
+  int F;        // features per CTA (a multiple of 8)
+  int pitch;    // elements between rows of the staged slices: an odd number of 16-byte groups, so that 16-byte
+                // reads of one column group by consecutive rows fall into different banks
+  int nbuf;     // row buffers (2: the next step's rows are copied during this one)
+  int PZ, PG;   // partial sums per row (forward) / per feature group (gradient) inside a CTA
+};
+
+constexpr int CL_NT = 224;               // compute threads
+constexpr int CL_THREADS = CL_NT + 32;   // and the helper warp (registers are handed out to four warps at a time)
+template <typename T> __host__ __device__ constexpr int group_elems() { return 16 / (int)sizeof(T); }
+
+inline size_t cluster_smem(const Geo& g, int esz, int B, int CP) {
+  const size_t zp = std::max((size_t)g.PZ * B * CP, (size_t)g.PG * g.F * CP);
+  return (size_t)g.nbuf * B * g.pitch * esz +
+         4 * ((size_t)(esz == 2 ? 3 : 2) * g.F * CP + zp + (size_t)3 * B * CP + (size_t)6 * round_up(B, 4) + 2 * 16) + 64;
+}
+
+// Cluster width and staging for a model of `in` features, C classes, W workers; Q = 0: the rows of a step do not
+// fit into a cluster's shared memory and the one-CTA kernel runs.
+// Q: as many CTAs as the chip holds twice over when every worker is selected, slices of at least 32 features.
+// Per launch on 784 -> 10 fp32, B = 64, U = 10: one-CTA kernel 366 us; clusters 74 us (8 workers), 85 us (16), 91 us
+// (32), 167 us (64); 512 instead of 224 compute threads lose the second CTA per SM (16 workers: 151 us).
+inline Geo cluster_plan(int in, int C, int B, int W, int esz) {
+  const int CP = round_up(C, 4), ge = 16 / esz;
+  auto geo = [&](int Q, int nbuf) {
+    Geo g;
+    g.Q = Q;
+    g.F = round_up((in + Q - 1) / Q, 8);
+    const int groups = g.F / ge;
+    g.pitch = (groups | 1) * ge;
+    g.nbuf = nbuf;
+    const int pairs = (B + 1) / 2;
+    g.PZ = std::max(1, std::min(std::min(CL_NT / std::max(1, pairs), 16), groups));
+    g.PG = std::max(1, std::min(std::min(CL_NT / groups, 8192 / (g.F * CP)), std::min(16, B / 4)));   // 32 KB of partial sums
+    return g;
+  };
+  int first = 8;
+  while (first > 1 && (W * first > 2 * 148 || in / first < 32)) first /= 2;
+  for (int nbuf = 2; nbuf >= 1; --nbuf)
+    for (int Q = first; Q <= 8; Q *= 2) {
+      const Geo g = geo(Q, nbuf);
+      if (cluster_smem(g, esz, B, CP) <= 220 * 1024) return g;
+    }
+  Geo none = geo(1, 1);
+  none.Q = 0;
+  return none;
+}
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+// x / n for x < 2^31 / n (items and rows of a step), by a multiplication: an integer division costs a few hundred
+// cycles of every phase otherwise
+struct FastDiv {
+  uint32_t m;
+  __device__ __forceinline__ explicit FastDiv(int n) : m(n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u) {}
+  __device__ __forceinline__ int div(int x) const { return m ? (int)__umulhi((uint32_t)x, m) : x; }
+};
+__device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;" ::"n"(CL_NT) : "memory"); }
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+// one 16-byte group of stored values as binary32
+__device__ __forceinline__ void load_group(const float* p, float (&v)[4]) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+__device__ __forceinline__ void load_group(const __nv_bfloat16* p, float (&v)[8]) { load8(p, v); }
+
+// CP: class count rounded up to a multiple of 4 (padded classes have zero weights and zero deltas)
+template <typename T, int CP>
+__global__ void __launch_bounds__(CL_THREADS, (group_elems<T>() * CP < 64) ? 2 : 1) local_cluster_kernel(Args a, Geo geo) {
+  grid_dependency_sync();
+  extern __shared__ __align__(16) unsigned char loc_raw[];
+  using lsqp::f32x2;
+  constexpr int NT = CL_NT, GE = group_elems<T>(), C4 = CP / 4;
+  DevState* st = a.st;
+  RoundInfo* ri = a.ri;
+  if (st->status != ST_OK) return;
+  const int Q = geo.Q, F = geo.F, pitch = geo.pitch, PZ = geo.PZ, PG = geo.PG;
+  const int i = (int)blockIdx.x / Q;
+  if (i >= ri->K) return;                            // same decision in every CTA of the cluster
+  const int rank = Q > 1 ? (int)tc::cluster_rank() : 0;
+  const int B = st->B, in = a.in, C = a.C, U = a.U, W = st->W;
+  const int n_w = in * C;
+  const int m0 = rank * F, nf = max(0, min(F, in - m0));     // this CTA's features
+  const int groups = F / GE, n_g = F * C4;           // 16-byte row groups; float4s of the slice's gradient
+  const int Br = round_up(B, 4);
+  T* xs = reinterpret_cast<T*>(loc_raw);                                     // [nbuf][B][pitch]
+  float* wl = reinterpret_cast<float*>(xs + (size_t)geo.nbuf * B * pitch);   // [F][CP] local model
+  float* wq = sizeof(T) == 2 ? wl + (size_t)F * CP : wl;                     // ... as the forward pass reads it (bf16 values)
+  float4* gs = reinterpret_cast<float4*>(wq + (size_t)F * CP);               // [GE * C4][groups] sum of the steps' gradient sums
+  float* zp = reinterpret_cast<float*>(gs + n_g);                            // partial logits / partial gradients
+  float* za = zp + max((size_t)PZ * B * CP, (size_t)PG * F * CP);            // [2][B][CP] this CTA's partial logits by step parity
+  float* dl = za + (size_t)2 * B * CP;                                       // [B][CP] deltas
+  float* rl = dl + (size_t)B * CP;                                           // [B] sample losses
+  float* bs = rl + Br;                                                       // [16] bias, [16] its gradient sum
+  int* sidx = reinterpret_cast<int*>(bs + 32);                               // [3][B] sample indices by step mod 3
+  uint32_t* ys = reinterpret_cast<uint32_t*>(sidx + 3 * Br);                 // [2][B] targets / labels by step parity
+  __shared__ uint64_t full[2];                       // rows of a buffer have landed
+  __shared__ int gave_up;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool helper = warp == NT / 32;
+  const int wn = a.sel[i], jb = a.job[wn];
+  const int slot = (ri->t - a.sel_tau[i]) % (st->S + 1);
+  const T* w0 = (const T*)a.ring + (size_t)slot * a.slot_stride;
+  const T* X = (const T*)a.X + m0;
+  const int nblk = (B + 3) >> 2;
+  const float step = __fdiv_rn(a.lr, (float)B);
+  i64 lo = 0;                                        // the worker's shard [lo, lo + len) (helper warp)
+  u64 len = 0;
+  uint32_t key0 = 0, key1 = 0;
+
+  // ---- what the helper warp does for the others
+  auto draw = [&](int u) {                           // sample indices of step u
+    int* dst = sidx + (u % 3) * Br;
+    for (int blk = lane; blk < nblk; blk += 32) {
+      uint32_t w4[4];
+      philox4x32_10((uint32_t)wn, (uint32_t)jb, 1u, (uint32_t)(u * nblk + blk), key0, key1, w4);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (blk * 4 + q < B) dst[blk * 4 + q] = (int)lo + (int)(((u64)w4[q] * len) >> 32);
+    }
+    __syncwarp();
+  };
+  // rows that start on 16-byte boundaries: the slice of a row is one bulk copy (F is a multiple of 8)
+  const bool bulk = ((size_t)in * sizeof(T)) % 16 == 0;
+  const bool vec4 = ((size_t)in * sizeof(T)) % 4 == 0;
+  auto fetch_rows = [&](int u) {                     // this CTA's slice of step u's rows
+    const int* idx = sidx + (u % 3) * Br;
+    const int buf = u % geo.nbuf;
+    T* dst = xs + (size_t)buf * B * pitch;
+    if (bulk) {
+      if (lane == 0) tc::mbar_expect_tx(&full[buf], (uint32_t)(B * nf * (int)sizeof(T)));
+      __syncwarp();
+      if (nf > 0)
+        for (int b = lane; b < B; b += 32)
+          lsqp::bulk_row(dst + (size_t)b * pitch, X + (size_t)idx[b] * in, (uint32_t)(nf * sizeof(T)), &full[buf]);
+    }
+    for (int b = lane; b < B; b += 32) cp_async4(ys + (u & 1) * Br + b, (const uint32_t*)a.y + idx[b]);
+  };
+  auto fetch_pieces = [&](int u) {                   // the same by every compute thread, for other row lengths
+    const int* idx = sidx + (u % 3) * Br;
+    T* dst = xs + (size_t)(u % geo.nbuf) * B * pitch;
+    if (vec4) {
+      constexpr int E4 = 4 / (int)sizeof(T);
+      const int per = nf / E4;                       // F and (here) `in` are even for 2-byte elements
+      for (int b = warp; b < B; b += NT / 32)
+        for (int v = lane; v < per; v += 32) cp_async4(dst + (size_t)b * pitch + v * E4, X + (size_t)idx[b] * in + v * E4);
+    } else {
+      for (int b = warp; b < B; b += NT / 32)
+        for (int v = lane; v < nf; v += 32) dst[(size_t)b * pitch + v] = X[(size_t)idx[b] * in + v];
+    }
+  };
+  auto fetch = [&](int u) {
+    if (helper) fetch_rows(u);
+    else if (!bulk) fetch_pieces(u);
+  };
+
+  if (tid == 0) {
+    tc::mbar_init(&full[0], 1);
+    tc::mbar_init(&full[1], 1);
+    gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (helper) {
+    const i64 M = st->n_samples;
+    lo = ((i64)wn * M) / W;
+    len = (u64)(((i64)(wn + 1) * M) / W - lo);
+    key0 = st->key0; key1 = st->key1;
+    draw(0);
+    if (U > 1) draw(1);
+  } else {
+    // columns behind the slice's features are read by the 16-byte groups but never copied: zero in every buffer
+    for (int r = warp; r < geo.nbuf * B; r += NT / 32)
+      for (int v = nf + lane; v < pitch; v += 32) stf(xs, (size_t)r * pitch + v, 0.f);
+  }
+  if (!helper) {
+#pragma unroll 8
+    for (int e = tid; e < F * CP; e += NT) {
+      const int m = e / CP, c = e - m * CP;
+      const float w = (m < nf && c < C) ? ldf(w0, (size_t)(m0 + m) * C + c) : 0.f;    // a stored model is already rounded
+      wl[e] = w;
+      wq[e] = w;
+    }
+    for (int e = tid; e < n_g; e += NT) gs[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < 16) {
+      bs[tid] = (!a.lsq && tid < C) ? ldf(w0, (size_t)n_w + tid) : 0.f;
+      bs[16 + tid] = 0.f;
+    }
+  }
+  __syncthreads();
+  fetch(0);
+  float loss_sum = 0.f;                              // helper warp
+  if (Q > 1) tc::cluster_sync_all();                 // peers have started: their shared memory may be read
+
+  // ---- logits, loss, deltas of a step (every thread): four lanes per row, four classes each
+  auto softmax = [&](int par) {
+    for (int b0 = 0; b0 < B; b0 += CL_THREADS / 4) {
+      const int b = b0 + (tid >> 2), l = tid & 3;
+      const bool have = b < B && l < C4;
+      float z[4] = {0.f, 0.f, 0.f, 0.f};
+      if (have) {
+        const uint32_t mine = tc::smem_u32(za + (size_t)(par * B + b) * CP + 4 * l);
+        float4 p[8];                                 // the cluster's partial logits of these classes
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          p[q] = q < Q ? ld_cluster4(Q > 1 ? tc::map_to_cta(mine, (uint32_t)q) : mine) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 s = p[0];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) s = add4(s, p[q]);
+        z[0] = s.x; z[1] = s.y; z[2] = s.z; z[3] = s.w;
+      }
+      float d[4] = {0.f, 0.f, 0.f, 0.f};
+      const uint32_t yb = b < B ? ys[par * Br + b] : 0u;
+      if (a.lsq) {
+        const float r = z[0] - __uint_as_float(yb);
+        if (have && l == 0) { d[0] = r; rl[b] = 0.5f * r * r; }
+      } else {
+        const int y = (int)yb;
+        float zy = 0.f, se = 0.f;
+        // padded classes: exp(-3e38 - max) = 0, and their delta is 0
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          z[k] = 4 * l + k < C ? z[k] : -3.0e38f;
+          zy = 4 * l + k == y ? z[k] : zy;
+        }
+        float zmax = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
+        zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 1));
+        zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 2));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) z[k] = expf(z[k] - zmax);
+        se = (z[0] + z[1]) + (z[2] + z[3]);
+        se += __shfl_xor_sync(0xffffffffu, se, 1);
+        se += __shfl_xor_sync(0xffffffffu, se, 2);
+        zy += __shfl_xor_sync(0xffffffffu, zy, 1);
+        zy += __shfl_xor_sync(0xffffffffu, zy, 2);
+        const float inv = 1.f / se;
+        // a delta is a stored quantity of the bf16 configurations: rounded like every other delta
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] = round_store(z[k] * inv - (4 * l + k == y ? 1.f : 0.f), (const T*)nullptr);
+        if (b < B && l == 0) rl[b] = logf(se) - (zy - zmax);
+      }
+      if (have) *reinterpret_cast<float4*>(dl + (size_t)b * CP + 4 * l) = make_float4(d[0], d[1], d[2], d[3]);
+    }
+  };
+
+  const int n_pairs = (B + 1) / 2;
+  const FastDiv by_pairs(n_pairs), by_groups(groups);
+  for (int u = 0; u < U; ++u) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // a wait that runs out ends the run (status below); the steps are finished on whatever is there, so that the
+    // cluster's barriers stay matched
+    if (bulk) tc::mbar_wait(&full[u % geo.nbuf], (uint32_t)(u / geo.nbuf) & 1u, &gave_up);
+    __syncthreads();                                 // rows of step u are here; the previous step is done with everything
+    // the helper warp adds nothing to the exchange: it arrives at once, so that nobody waits for its copies
+    if (helper && Q > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (geo.nbuf == 2 && u + 1 < U) fetch(u + 1);
+    const int par = u & 1;
+    if (helper) {
+      if (u + 2 < U) draw(u + 2);
+      if (Q > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      else asm volatile("bar.sync 2, %0;" ::"n"(CL_THREADS) : "memory");
+      softmax(par);
+      __syncthreads();                               // deltas are there
+      if (rank == 0) {                               // mean loss and bias step (fixed orders)
+        float part = 0.f;
+        for (int b = lane; b < B; b += 32) part += rl[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        loss_sum += __fdiv_rn(part, (float)B);
+        const int c = lane & 15;                     // two lanes per class, every second row each
+        float s = 0.f;
+        if (c < CP) {
+#pragma unroll 8
+          for (int b = lane >> 4; b < B; b += 2) s += dl[(size_t)b * CP + c];
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if (!a.lsq && lane < C) {
+          bs[16 + lane] += s;
+          bs[lane] = fmaf(-step, s, bs[lane]);
+        }
+      }
+      if (geo.nbuf == 1) {
+        __syncthreads();                             // the gradient has read the only row buffer
+        if (u + 1 < U) fetch(u + 1);
+      }
+      continue;
+    }
+    const T* xb = xs + (size_t)(u % geo.nbuf) * B * pitch;
+    // ---- partial logits of this slice: item = (row pair, every PZ-th column group)
+    for (int it = tid; it < n_pairs * PZ; it += NT) {
+      const int part = by_pairs.div(it), r0 = it - part * n_pairs, r1 = r0 + n_pairs;
+      const T* x0 = xb + r0 * pitch;
+      const T* x1 = xb + min(r1, B - 1) * pitch;
+      f32x2 z0[CP / 2], z1[CP / 2];
+#pragma unroll
+      for (int c = 0; c < CP / 2; ++c) z0[c] = z1[c] = 0ull;
+      for (int g = part; g < groups; g += PZ) {
+        float v0[GE], v1[GE];
+        load_group(x0 + g * GE, v0);
+        load_group(x1 + g * GE, v1);
+        const float* w = wq + g * (GE * CP);
+#pragma unroll
+        for (int j = 0; j < GE; ++j) {
+          const f32x2 p0 = lsqp::pack2(v0[j], v0[j]), p1 = lsqp::pack2(v1[j], v1[j]);
+#pragma unroll
+          for (int c = 0; c < C4; ++c) {
+            const ulonglong2 ww = *reinterpret_cast<const ulonglong2*>(w + j * CP + 4 * c);
+            lsqp::ffma2(z0[2 * c], p0, ww.x);
+            lsqp::ffma2(z0[2 * c + 1], p0, ww.y);
+            lsqp::ffma2(z1[2 * c], p1, ww.x);
+            lsqp::ffma2(z1[2 * c + 1], p1, ww.y);
+          }
+        }
+      }
+      float* o = zp + ((size_t)part * B + r0) * CP;
+#pragma unroll
+      for (int c = 0; c < C4; ++c) {
+        *reinterpret_cast<ulonglong2*>(o + 4 * c) = make_ulonglong2(z0[2 * c], z0[2 * c + 1]);
+        if (r1 < B) *reinterpret_cast<ulonglong2*>(o + (size_t)n_pairs * CP + 4 * c) = make_ulonglong2(z1[2 * c], z1[2 * c + 1]);
+      }
+    }
+    compute_sync();
+    for (int e = tid; e < B * C4; e += NT) {         // partial sums in order; the first CTA adds the bias
+      float4 z = reinterpret_cast<const float4*>(zp)[e];
+#pragma unroll 8
+      for (int p = 1; p < PZ; ++p) z = add4(z, reinterpret_cast<const float4*>(zp + (size_t)p * B * CP)[e]);
+      if (rank == 0) {
+        const float4 bq = reinterpret_cast<const float4*>(bs)[e % C4];
+        z = add4(z, make_float4(round_store(bq.x, (const T*)nullptr), round_store(bq.y, (const T*)nullptr),
+                                round_store(bq.z, (const T*)nullptr), round_store(bq.w, (const T*)nullptr)));
+      }
+      reinterpret_cast<float4*>(za + (size_t)par * B * CP)[e] = z;
+    }
+    if (Q > 1) tc::cluster_sync_all();
+    else asm volatile("bar.sync 2, %0;" ::"n"(CL_THREADS) : "memory");
+    softmax(par);
+    __syncthreads();
+    // ---- gradient of this slice: item = (column group, every PG-th row)
+    for (int it = tid; it < groups * PG; it += NT) {
+      const int part = by_groups.div(it), g = it - part * groups;
+      f32x2 acc[GE][CP / 2];
+#pragma unroll
+      for (int j = 0; j < GE; ++j)
+#pragma unroll
+        for (int c = 0; c < CP / 2; ++c) acc[j][c] = 0ull;
+#pragma unroll 2
+      for (int b = part; b < B; b += PG) {
+        float v[GE];
+        load_group(xb + b * pitch + g * GE, v);
+        f32x2 d2[CP / 2];
+#pragma unroll
+        for (int c = 0; c < C4; ++c) {
+          const ulonglong2 dd = *reinterpret_cast<const ulonglong2*>(dl + b * CP + 4 * c);
+          d2[2 * c] = dd.x;
+          d2[2 * c + 1] = dd.y;
+        }
+#pragma unroll
+        for (int j = 0; j < GE; ++j) {
+          const f32x2 p = lsqp::pack2(v[j], v[j]);
+#pragma unroll
+          for (int c = 0; c < CP / 2; ++c) lsqp::ffma2(acc[j][c], p, d2[c]);
+        }
+      }
+      ulonglong2* o = reinterpret_cast<ulonglong2*>(zp) + (size_t)part * n_g + g;
+#pragma unroll
+      for (int j = 0; j < GE; ++j)
+#pragma unroll
+        for (int c = 0; c < C4; ++c) o[(size_t)(j * C4 + c) * groups] = make_ulonglong2(acc[j][2 * c], acc[j][2 * c + 1]);
+    }
+    if (geo.nbuf == 1) {
+      __syncthreads();                               // the helper refills the only row buffer
+      if (!bulk && u + 1 < U) fetch(u + 1);
+    } else {
+      compute_sync();
+    }
+    // ---- the local step
+    for (int e = tid; e < n_g; e += NT) {
+      float4 s = reinterpret_cast<const float4*>(zp)[e];
+#pragma unroll 8
+      for (int p = 1; p < PG; ++p) s = add4(s, reinterpret_cast<const float4*>(zp)[(size_t)p * n_g + e]);
+      gs[e] = add4(gs[e], s);
+      const int jc = by_groups.div(e), g = e - jc * groups;
+      const int m = g * GE + jc / C4, c4 = jc % C4;
+      float4* w4 = reinterpret_cast<float4*>(wl + (size_t)m * CP) + c4;
+      float4 w = *w4;
+      w.x = fmaf(-step, s.x, w.x); w.y = fmaf(-step, s.y, w.y); w.z = fmaf(-step, s.z, w.z); w.w = fmaf(-step, s.w, w.w);
+      *w4 = w;
+      if (sizeof(T) == 2)
+        reinterpret_cast<float4*>(wq + (size_t)m * CP)[c4] =
+            make_float4(round_store(w.x, (const T*)nullptr), round_store(w.y, (const T*)nullptr),
+                        round_store(w.z, (const T*)nullptr), round_store(w.w, (const T*)nullptr));
+    }
+  }
+  if (Q > 1) tc::cluster_sync_all();                 // no peer still reads this CTA's partial logits
+  else __syncthreads();
+  float* out = a.G + (size_t)i * a.slot_stride;
+  const float sa = st->sa_penalty ? sa_weight(a.sel_tau[i]) : 1.f;   // staleness-aware step size: weight of the upload in Eq. 3
+  for (int e = tid; e < nf * C; e += CL_THREADS) {
+    const int m = e / C, c = e - m * C;
+    const float4 q = gs[(size_t)((m % GE) * C4 + c / 4) * groups + m / GE];
+    const int k = c & 3;
+    out[(size_t)m0 * C + e] = (k == 0 ? q.x : k == 1 ? q.y : k == 2 ? q.z : q.w) * sa;
+  }
+  if (rank == 0) {
+    if (!a.lsq && tid < C) out[(size_t)n_w + tid] = bs[16 + tid] * sa;
+    if (helper && lane == 0) {
+      const float loss = __fdiv_rn(loss_sum, (float)U);
+      a.loss[i] = loss;
+      if (!isfinite(loss)) ri->diverged = 1;
+    }
+  }
+  if (tid == 0 && gave_up) {
+    // let copies in flight land before the shared memory goes away
+    const unsigned long long t0 = tc::global_ns();
+    while (tc::global_ns() - t0 < 200000ull) {}
+    // not st->status: a cluster that starts later must find the same status in all of its CTAs
+    st->timeout_where = 300;
+    ri->diverged = RI_TIMEOUT;
   }
 }
 

@@ -193,6 +193,26 @@ def test_local_sgd_steps(kind, dims, dtype, W, B, U, forced):
     assert rows[-1]["loss_mean"] < rows[0]["loss_mean"]
 
 
+@pytest.mark.parametrize("kind,dims,dtype,W,B,U", [
+    (inputs.SOFTMAX, (784, 10), inputs.FP32, 5, 64, 4),         # eight CTAs per worker, bulk row copies
+    (inputs.SOFTMAX, (264, 16), inputs.BF16, 4, 33, 3),         # the last CTA of a cluster owns no feature; odd batch
+    (inputs.SOFTMAX, (262, 3), inputs.BF16, 6, 17, 2),          # rows that start on 4-byte boundaries only
+    (inputs.SOFTMAX, (259, 5), inputs.BF16, 4, 9, 3),           # ... on 2-byte boundaries
+    (inputs.SOFTMAX, (301, 2), inputs.FP32, 40, 70, 2),         # four CTAs per worker
+    (inputs.SOFTMAX, (96, 12), inputs.FP32, 160, 8, 2),         # one CTA per worker
+    (inputs.SOFTMAX, (400, 12), inputs.FP32, 5, 400, 3),        # a single row buffer
+    (inputs.SOFTMAX, (760, 16), inputs.FP32, 4, 512, 2),        # rows of a step too large for a cluster: one-CTA kernel
+    (inputs.LSQ, (12288, 1), inputs.FP32, 4, 4, 3),             # largest model of the path
+])
+def test_local_sgd_cluster_widths(kind, dims, dtype, W, B, U):
+    """Local steps of single-layer models: every cluster width, copy granularity and buffer count."""
+    cfg = _small_cfg(kind, dims, dtype, W, B, 3, 5, GAMMA3, lr=0.02 if dims[0] < 1000 else 1e-4)
+    X, y, w0 = _problem(cfg)
+    bf16 = dtype == inputs.BF16
+    compare_with_oracle(cfg, X, y, w0, 8, TOL_BF16 if bf16 else TOL_FP32, forced=True,
+                        loss_tol=5e-2 if bf16 else None, local_steps=U)
+
+
 @pytest.mark.parametrize("dims,W,B,U,K0,S", [
     ((64, 128, 10), 8, 16, 4, 3, 5),             # one tensor-core layer; a worker's rows are 16 of a 128-row tile
     ((72, 136, 256, 10), 12, 48, 3, 4, 6),       # two tensor-core layers, ragged widths
