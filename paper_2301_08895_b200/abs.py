@@ -301,17 +301,19 @@ class Context:
             pass
 
 
+def _raw_stream(torch, stream, X):
+    """cudaStream_t of `stream`, or of the current stream of X's device (without building a Stream object for it)."""
+    return stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(X.get_device())
+
+
 def lsq_gradient(X, y, w, idx, g_out, loss_out, scratch, stream=None):
     """abs_lsq_gradient on torch CUDA tensors: X [M, d] and w [d] float32 or bfloat16, y float32,
     idx int32 [n, B], g_out float32 [d], loss_out float32 [n], scratch float32 (>= n*d)."""
     import torch
     n, B = idx.shape
-    d = X.shape[1]
-    dtype = BF16_FP32MASTER if X.dtype == torch.bfloat16 else FP32
-    s = stream if stream is not None else torch.cuda.current_stream(X.device)
-    _check(lib().abs_lsq_gradient(X.data_ptr(), y.data_ptr(), w.data_ptr(), idx.data_ptr(), n, B, d,
-                                  dtype, scratch.data_ptr(), scratch.numel(), g_out.data_ptr(),
-                                  loss_out.data_ptr(), s.cuda_stream))
+    _check(lib().abs_lsq_gradient(X.data_ptr(), y.data_ptr(), w.data_ptr(), idx.data_ptr(), n, B, X.shape[1],
+                                  BF16_FP32MASTER if X.dtype == torch.bfloat16 else FP32, scratch.data_ptr(),
+                                  scratch.numel(), g_out.data_ptr(), loss_out.data_ptr(), _raw_stream(torch, stream, X)))
 
 
 def lsq_gradient_noalloc(X, y, w, idx, g_out, loss_out, stream=None):
@@ -320,12 +322,9 @@ def lsq_gradient_noalloc(X, y, w, idx, g_out, loss_out, stream=None):
     at most 1048576.  Calls sharing a device must not overlap on the GPU."""
     import torch
     n, B = idx.shape
-    d = X.shape[1]
-    dtype = BF16_FP32MASTER if X.dtype == torch.bfloat16 else FP32
-    s = stream if stream is not None else torch.cuda.current_stream(X.device)
-    _check(lib().abs_lsq_gradient_noalloc(X.data_ptr(), y.data_ptr(), w.data_ptr(), idx.data_ptr(),
-                                          n, B, d, dtype, g_out.data_ptr(), loss_out.data_ptr(),
-                                          s.cuda_stream))
+    _check(lib().abs_lsq_gradient_noalloc(X.data_ptr(), y.data_ptr(), w.data_ptr(), idx.data_ptr(), n, B, X.shape[1],
+                                          BF16_FP32MASTER if X.dtype == torch.bfloat16 else FP32, g_out.data_ptr(),
+                                          loss_out.data_ptr(), _raw_stream(torch, stream, X)))
 
 
 def trace_rows(tr):

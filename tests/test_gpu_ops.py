@@ -48,6 +48,19 @@ def test_lsq_gradient_matches_oracle(n, B, d, bf16):
     assert np.linalg.norm(g.cpu().numpy() - og) <= 1e-5 * max(np.linalg.norm(og), 1e-30)
 
 
+@pytest.mark.parametrize("n,B,d,bf16", [
+    (8, 32, 64, False), (9, 32, 64, False),          # one cluster (a single launch), two clusters
+    (1, 300, 100, False), (3, 47, 96, True),         # eight / two CTAs per worker, uneven row shares
+    (4, 9, 128, False), (4, 9, 132, False),          # 32 / 33 vectors per row
+    (4, 9, 1024, False), (4, 9, 1028, False),        # longest rows kept in registers, shortest of the two-pass kernel
+    (4, 9, 2048, True), (4, 9, 2056, True),
+    (2, 40, 255, True), (2, 40, 257, False),         # rows not on 16-byte boundaries
+    (2, 20, 8192, False), (3, 5, 8193, True),        # longest rows summed inside a cluster, shortest that are not
+])
+def test_lsq_gradient_kernel_edges(n, B, d, bf16):
+    test_lsq_gradient_matches_oracle(n, B, d, bf16)
+
+
 def test_lsq_gradient_rejects_bad_arguments():
     import torch
     X, y, w, idx, Xd, yd, wd, idxd = _case(4, 8, 16, 100, False, 1)
