@@ -19,6 +19,7 @@
 #include "localnet.cuh"
 #include "persist.cuh"
 #include "conv.cuh"
+#include "rownet.cuh"
 
 using namespace absb;
 
@@ -68,6 +69,8 @@ struct Layout {
   int fused_R = 0;                      // rows per block of the fused output-layer kernel (0: not used)
   int narrow_rpb = 64;                  // rows per block of the row-tiled output-layer kernels that are not fused
   bool out_mma = false;                 // output layer through the mma.sync kernel (bf16, 64 rows per CTA)
+  int row_R = 0;                        // whole network through rownet.cuh with this many rows per CTA (0: not used)
+  int step_Q = 1;                       // ... CTAs per tile of its gradient kernel
   size_t esz = 4;                       // bytes per stored element (4 or 2)
   size_t d = 0, d_pad = 0;
   size_t w_off[ABS_MAX_LAYERS] = {};    // element offset of W_l inside the padded vector
@@ -143,6 +146,8 @@ int check_model(const abs_model_desc* m, int W, int S) {
   return ABS_OK;
 }
 
+int step_tiles(int in, int out) { return ((in + 1 + rnet::GT - 1) / rnet::GT) * ((out + rnet::GT - 1) / rnet::GT); }
+
 void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   L->n_layers = m->n_layers;
   L->esz = m->dtype == ABS_FP32 ? 4 : 2;
@@ -186,7 +191,30 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       L->any_tc = true;
     } else L->path[l] = PATH_SIMT;
   }
-  L->RB = lsq ? m->batch : (L->any_tc ? 128 : 64);
+  // Networks without tensor-core layers and the fully connected part of the CNN: two kernels per round (rownet.cuh)
+  // if the rows' activations fit into shared memory.  Rows per CTA: bf16 one mma tile; fp32 4 while that leaves at most
+  // one CTA per SM (the chain of layers is what counts), 8 up to two waves, then 16 (fewer reads of the weights per row).
+  L->row_R = 0;
+  if (!lsq && m->local_steps <= 1 && (!L->any_tc || L->cnn)) {
+    const long long rows = (long long)W * m->batch;
+    rnet::RowsArgs ra;
+    ra.n_layers = m->n_layers;
+    for (int l = 0; l <= m->n_layers; ++l) ra.dims[l] = m->dims[l];
+    size_t smem = 0;
+    const int R0 = L->esz == 2 ? rnet::MMA_R : rows <= 148 * 4 ? 4 : rows <= 2 * 148 * 8 ? 8 : 16;
+    for (int R = R0; R >= (L->esz == 2 ? rnet::MMA_R : 4) && !L->row_R; R /= 2)
+      if (rnet::plan_rows(&ra, R, (int)L->esz, &smem)) L->row_R = R;
+    if (L->row_R) {
+      L->any_tc = false;
+      for (int l = 0; l < m->n_layers; ++l) if (L->path[l] == PATH_TC) L->path[l] = PATH_SIMT;
+      int tiles = 0;
+      for (int l = 0; l < m->n_layers; ++l) tiles += step_tiles(m->dims[l], m->dims[l + 1]);
+      // CTAs per tile: enough for two per SM, at least two pipeline steps of rows each
+      L->step_Q = 1;
+      while (L->step_Q < 8 && tiles * L->step_Q * 2 <= 2 * 148 && rows >= 4 * rnet::GK * L->step_Q) L->step_Q *= 2;
+    }
+  }
+  L->RB = lsq ? m->batch : L->row_R ? L->row_R : (L->any_tc ? 128 : 64);
   const int groups = (W < S + 1) ? W : S + 1;
   L->rows_cap = round_up(W * m->batch, L->RB) + groups * L->RB;
   L->local_net = !lsq && m->n_layers > 1 && m->local_steps > 1;
@@ -197,6 +225,8 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   L->n_tiles_cap = L->rows_cap / L->RB;
   if (lsq) {
     L->P = 0;
+  } else if (L->row_R) {
+    L->P = 1;
   } else if (L->any_tc) {
     // tile widths: widest tile that still gives every SM work; split count of the row reduction
     // sized so the largest weight gradient fills about two waves of 148 CTAs
@@ -311,7 +341,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       // the fused output-layer kernel keeps R input rows in shared memory
       const int inl = m->dims[m->n_layers - 1];
       L->fused_R = 0;
-      if (L->path[m->n_layers - 1] == PATH_NARROW && inl % 8 == 0)
+      if (L->path[m->n_layers - 1] == PATH_NARROW && inl % 8 == 0 && !L->row_R)
         for (int R : {32, 16, 8})     // (rows, transposed weights in fp32 or storage type, stored weights, deltas)
           if ((size_t)R * inl * L->esz + (size_t)C * (inl + 8) * 4 + (size_t)(inl + 1) * C * L->esz + 64 +
                   (size_t)R * 64 <= 100 * 1024) { L->fused_R = R; break; }
@@ -349,7 +379,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       // 1 / 2 / 4 / 8 rows per CTA give 1742 / 1617 / 1409 / 1222 rounds/s)
       L->cchunk = 1;
       while (L->cchunk < conv::MAX_CHUNK && (long long)W * m->batch / (2 * L->cchunk) >= 4 * 148) L->cchunk *= 2;
-      for (int b = 0; b < 2; ++b) L->cpart[b] = cv.take(4 * L->c_len[b] * (size_t)(L->rows_cap / L->cchunk));
+      for (int b = 0; b < 2; ++b) L->cpart[b] = cv.take(4 * L->c_len[b] * (size_t)((L->rows_cap + L->cchunk - 1) / L->cchunk));
     }
   }
   const size_t R = (size_t)m->max_rounds;
@@ -600,6 +630,13 @@ void (*local_cluster_fn(int C))(local::Args, local::Geo) {
          : C <= 12 ? local::local_cluster_kernel<T, 12> : local::local_cluster_kernel<T, 16>;
 }
 
+// the row kernel for R rows per CTA
+template <typename T>
+void (*rows_kernel_fn(int R))(rnet::RowsArgs) {
+  if (sizeof(T) == 2) return rnet::rows_mma_kernel;
+  return R == 4 ? rnet::rows_fma_kernel<4> : R == 8 ? rnet::rows_fma_kernel<8> : rnet::rows_fma_kernel<16>;
+}
+
 enum Phase : int { PH_GATHER = 0, PH_FORWARD = 1, PH_BACKWARD = 2 };
 
 // Kernels of one round, `par` = round parity (layout copy).  PH_GATHER: minibatch row copy (runs on
@@ -705,6 +742,26 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
                 st, ri, ctx->ctl.row_idx[par], (const __nv_bfloat16*)ctx->X, ctx->at<__nv_bfloat16>(par ? L.act0b : L.act[0]), m.dims[0]);
     return;
   }
+  if (L.row_R && phase == PH_FORWARD) {
+    rnet::RowsArgs a;
+    memset(&a, 0, sizeof a);
+    a.st = st; a.ri = ri; a.tile_slot = ctx->ctl.tile_slot[par]; a.row_idx = ctx->ctl.row_idx[par]; a.labels = (const int*)ctx->y;
+    a.ring = ctx->at<void>(L.ring); a.slot_stride = L.d_pad;
+    a.X = L.cnn ? ctx->at<void>(par ? L.act0b : L.act[0]) : ctx->X;
+    a.gather = L.cnn ? 0 : 1;
+    a.n_layers = nl; a.want_d0 = L.cnn ? 1 : 0; a.row_loss = ctx->ctl.row_loss;
+    for (int l = 0; l <= nl; ++l) {
+      a.dims[l] = m.dims[l];
+      if (l > 0 && l < nl) a.act[l] = ctx->at<void>(L.act[l]);
+      if (l > 0 || L.cnn) a.delta[l] = ctx->at<void>(L.delta[l]);
+      if (l < nl) a.w_off[l] = L.w_off[l];
+    }
+    size_t sm = 0;
+    rnet::plan_rows(&a, L.row_R, (int)L.esz, &sm);
+    launch_ex(ctx, ABS_KC_FWD, rows_kernel_fn<T>(L.row_R), dim3(L.rows_cap / L.row_R),
+              dim3(L.esz == 2 ? rnet::MMA_THREADS : rnet::THREADS), sm, a);
+    return;
+  }
   // ---- forward (Eq. 2 at the model version each worker holds)
   for (int l = 0; l < nl && phase == PH_FORWARD; ++l) {
     const bool last = l == nl - 1;
@@ -768,7 +825,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     }
   }
   // ---- backward: deltas, then the weight gradients summed over all selected workers (Eq. 3)
-  for (int l = nl - 1; l >= 0 && phase == PH_BACKWARD; --l) {
+  for (int l = nl - 1; l >= 0 && phase == PH_BACKWARD && !L.row_R; --l) {
     if (L.path[l] == PATH_TC) {
       tc::Params pd = tc_params(l, tc::DGRAD);
       pd.N_total = la[l].in; pd.K_total = la[l].out;
@@ -837,10 +894,11 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     if (b == 1)      // delta of the first block's pooled maps (one CTA per row)
       launch_ex(ctx, ABS_KC_CONV, conv::conv_block_dgrad_kernel<T>, dim3(L.rows_cap), dim3(conv::THREADS),
                 conv::dgrad_smem_bytes(c.Hi, c.Wi, c.Ci, c.k, c.Co), c);
-    launch_ex(ctx, ABS_KC_CONV, conv::conv_block_wgrad_kernel<T>, dim3(L.rows_cap / L.cchunk), dim3(conv::THREADS),
+    launch_ex(ctx, ABS_KC_CONV, conv::conv_block_wgrad_kernel<T>, dim3((L.rows_cap + L.cchunk - 1) / L.cchunk), dim3(conv::THREADS),
               conv::wgrad_smem_bytes(c.Hi, c.Wi, c.Ci, c.k, c.Co), c);
-    launch_ex(ctx, ABS_KC_CONV, chunk_reduce_kernel, dim3(((int)L.c_len[b] + 31) / 32), dim3(256), 0, st, ri, c.part, (int)L.c_len[b],
-              ctx->at<float>(L.G) + L.c_off[b], L.cchunk);
+    if (!L.row_R)      // (else grad_step_kernel adds the chunk sums up)
+      launch_ex(ctx, ABS_KC_CONV, chunk_reduce_kernel, dim3(((int)L.c_len[b] + 31) / 32), dim3(256), 0, st, ri, c.part, (int)L.c_len[b],
+                ctx->at<float>(L.G) + L.c_off[b], L.cchunk);
   }
 }
 
@@ -857,6 +915,33 @@ void enqueue_update(abs_ctx* ctx, int par) {
     q.loss = ctx->ctl.loss; q.groups = (ctx->m.batch + lsqp::GROUP - 1) / lsqp::GROUP;
     const int blocks = std::max((q.d + 31) / 32, (ctx->W + 31) / 32);
     launch_ex(ctx, ABS_KC_UPDATE, lsq_update_kernel<T>, dim3(blocks), dim3(256), 0, q);
+    return;
+  }
+  if (L.row_R) {
+    rnet::StepArgs q;
+    memset(&q, 0, sizeof q);
+    const int nl = ctx->m.n_layers;
+    q.st = ctx->at<DevState>(L.st); q.ri = ri; q.row_idx = ctx->ctl.row_idx[par];
+    q.X = L.cnn ? ctx->at<void>(par ? L.act0b : L.act[0]) : ctx->X;
+    q.gather = L.cnn ? 0 : 1;
+    q.master = ctx->at<float>(L.master); q.ring = ctx->at<void>(L.ring); q.d_pad = L.d_pad; q.lr = ctx->m.lr;
+    q.n_layers = nl; q.Q = L.step_Q;
+    for (int l = 0; l <= nl; ++l) {
+      q.dims[l] = ctx->m.dims[l];
+      if (l > 0 && l < nl) q.act[l] = ctx->at<void>(L.act[l]);
+      if (l > 0) q.delta[l] = ctx->at<void>(L.delta[l]);
+      if (l == nl) break;
+      q.w_off[l] = L.w_off[l];
+      q.first_tile[l + 1] = q.first_tile[l] + step_tiles(ctx->m.dims[l], ctx->m.dims[l + 1]);
+    }
+    int blocks = 0;
+    for (int b = 0; b < 2 && L.cnn; ++b) {
+      rnet::StepArgs::Region& G = q.region[q.n_regions++];
+      G.part = ctx->at<float>(L.cpart[b]); G.len = (int)L.c_len[b]; G.chunk_rows = L.cchunk; G.off = L.c_off[b]; G.first_block = blocks;
+      blocks += (G.len + 31) / 32;
+    }
+    ctx->next_cluster = q.Q;
+    launch_ex(ctx, ABS_KC_UPDATE, rnet::grad_step_kernel<T>, dim3(q.first_tile[nl] * q.Q + round_up(blocks, q.Q)), dim3(256), 0, q);
     return;
   }
   UpdateArgs u;
@@ -1084,6 +1169,11 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     if (ef == cudaSuccess)
       ef = cudaFuncSetAttribute(narrow_fused_cc_kernel<__nv_bfloat16, 10>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     if (ef != cudaSuccess) return bail(cuda_fail(nullptr, ef, "cudaFuncSetAttribute(narrow_fused_kernel)"));
+  }
+  if (L.row_R) {
+    const cudaError_t er = L.esz == 4 ? cudaFuncSetAttribute(rows_kernel_fn<float>(L.row_R), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024)
+                                      : cudaFuncSetAttribute(rows_kernel_fn<__nv_bfloat16>(L.row_R), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    if (er != cudaSuccess) return bail(cuda_fail(nullptr, er, "cudaFuncSetAttribute(row kernel)"));
   }
   if (model->local_steps > 1 && !L.local_net) {
     const int C = model->kind == ABS_LSQ ? 1 : model->dims[1];

@@ -1,0 +1,871 @@
+// Networks without tcgen05 layers (fp32 storage, or bf16 widths TMA cannot address) and the fully connected part of
+// the CNN, two kernels per round:
+//   rows_fma_kernel / rows_mma_kernel   CTA = R gradient rows of one model version: all layers forward (Eq. 2 at the
+//                     version the rows' workers hold), soft-max cross-entropy, all layers' deltas backward,
+//   grad_step_kernel  weight and bias gradients of all layers, each 32 x 32 block summed over all rows of the round
+//                     (Eq. 3), and the SGD step and ring write of that block in the same CTA.
+// One launch per layer and direction would be bound by launch gaps and by grids of a few CTAs: rounds of this model
+// class are a few hundred rows and 10^4 .. 10^6 parameters.
+// Measured per round (one launch per layer and direction -> this): 300-123-57-7 fp32, 13 workers x 37 rows: 114 -> 28 us
+// (11 -> 3 launches); 784-10 fp32, 16 x 64: 22 -> 19 us; the 400-120-84-10 part of the CNN, 640 rows: 13 -> 2 launches,
+// 21 us for the row kernel between two events (28 us with FP32 FMAs for the bf16 products).
+// Activations and deltas are rounded to the storage type where they are stored, sums are fp32 in a fixed order.
+#pragma once
+#include <algorithm>
+
+#include "common.cuh"
+#include "lsqpipe.cuh"
+#include "narrow.cuh"
+#include "outlayer.cuh"
+#include "tc.cuh"
+
+namespace absb {
+namespace rnet {
+
+using lsqp::f32x2;
+
+constexpr int NW = 8;                    // compute warps of the row kernels
+constexpr int NT = NW * 32;
+constexpr int THREADS = NT + 32;         // and the warp that fetches the weights
+constexpr int MAX_STAGES = 8;
+constexpr int MMA_R = 16;                // rows per CTA of the bf16 kernel (one mma row tile)
+constexpr int MMA_NW = 15;               // its compute warps: with the fetching warp 512 threads of up to 128 registers
+constexpr int MMA_THREADS = MMA_NW * 32 + 32;
+
+struct RowsArgs {
+  DevState* st;
+  RoundInfo* ri;
+  const int* tile_slot;                  // ring slot of every R rows (the row padding unit)
+  const int* row_idx;                    // sample index per gradient row, -1: padding
+  const int* labels;
+  const void* ring; size_t slot_stride;
+  const void* X; int gather;             // layer-0 input of row r: X[row_idx[r]] (gather) or X[r]
+  void* act[ABS_MAX_LAYERS + 1];         // [rows][dims[l]] stored ReLU outputs, l = 1 .. n_layers - 1
+  void* delta[ABS_MAX_LAYERS + 1];       // [rows][dims[l]] stored deltas, l = 1 .. n_layers; delta[0]: see want_d0
+  float* row_loss;                       // [rows]
+  size_t w_off[ABS_MAX_LAYERS];          // element offset of W[in][out]; the bias follows it as row `in`
+  int n_layers, dims[ABS_MAX_LAYERS + 1];
+  int want_d0;                           // also the delta of the layer-0 input (CNN features, masked by feature > 0)
+  // Weights in shared memory.  resident: every layer is copied once and stays (stage l = layer l, the backward pass
+  // reads it again); otherwise chunks of rpc[l] rows stream through `stages` stages, forward and again backward.
+  int resident, stages, stage_bytes;
+  int w_res[ABS_MAX_LAYERS];             // byte offset of layer l (resident)
+  int rpc[ABS_MAX_LAYERS];               // rows per chunk: a multiple of 16 (chunks start on 16 bytes), or all of them
+  int act_off[ABS_MAX_LAYERS];           // element offset (T) of layer l's input behind the weights
+  int out_off, red_off;                  // fma: logits [C] quads, partial sums (floats); mma: output delta (T), logits (bytes)
+};
+
+__host__ __device__ inline int mma_pitch(int n) { return round_up(n, 16) + 8; }   // bf16 row pitch, zero-padded to 16
+
+// Shared-memory plan for R rows per CTA; false: does not fit.
+inline bool plan_rows(RowsArgs* a, int R, int esz, size_t* smem) {
+  const bool mma = esz == 2;
+  int off = 0;
+  for (int l = 0; l < a->n_layers; ++l) {
+    if (a->dims[l + 1] > 1024) return false;           // columns all warps of a CTA can hold
+    a->act_off[l] = off;
+    off += mma ? R * mma_pitch(a->dims[l]) : (a->dims[l] + 1) * R;
+  }
+  a->out_off = off;
+  const int C = a->dims[a->n_layers];
+  size_t bytes;
+  if (mma) {
+    off += R * mma_pitch(C);
+    a->red_off = round_up(2 * off, 16);
+    bytes = (size_t)a->red_off + (size_t)4 * R * (C + 1);
+  } else {
+    off += C * R;
+    a->red_off = round_up(off, 4);
+    bytes = 4 * ((size_t)a->red_off + (size_t)NW * 128 * R);
+  }
+  bytes += 128;
+  size_t all = 0, stage = 0;
+  for (int l = 0; l < a->n_layers; ++l) {
+    a->w_res[l] = (int)std::min<size_t>(all, 1u << 30);
+    a->rpc[l] = a->dims[l] + 1;
+    all += round_up_sz((size_t)(a->dims[l] + 1) * a->dims[l + 1] * esz, 128);
+  }
+  a->resident = all + bytes <= 220 * 1024;
+  a->stages = a->n_layers;
+  a->stage_bytes = 0;
+  *smem = all + bytes;
+  if (a->resident) return true;
+  for (int l = 0; l < a->n_layers; ++l) {
+    const size_t row16 = (size_t)16 * a->dims[l + 1] * esz;
+    a->rpc[l] = 16 * (int)std::max<size_t>(1, 24576 / row16);
+    stage = std::max(stage, round_up_sz((size_t)a->rpc[l] * a->dims[l + 1] * esz, 128));
+  }
+  a->stage_bytes = (int)stage;
+  for (a->stages = MAX_STAGES; a->stages >= 2; --a->stages) {
+    *smem = (size_t)a->stages * stage + bytes;
+    if (*smem <= 220 * 1024) return true;
+  }
+  return false;
+}
+
+__device__ __forceinline__ void rows_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
+
+// The weights of the CTA's model version, in shared memory (see RowsArgs::resident).
+struct Weights {
+  const RowsArgs& a;
+  unsigned char* base;
+  uint64_t *full, *empty;
+  int* gave_up;
+  int stage = 0;
+  uint32_t phase = 0;
+  __device__ __forceinline__ Weights(const RowsArgs& a_, unsigned char* b, uint64_t* f, uint64_t* e, int* g)
+      : a(a_), base(b), full(f), empty(e), gave_up(g) {}
+  // one thread: all copies, in the order the consumers take them
+  template <typename T>
+  __device__ __forceinline__ void produce(const T* ring) {
+    const int L = a.n_layers, l_min = a.want_d0 ? 0 : 1;
+    bool ok = true;
+    for (int step = 0; step < (a.resident ? L : 2 * L - l_min) && ok; ++step) {
+      const int l = step < L ? step : 2 * L - 1 - step;
+      const int rows = a.dims[l] + 1, out = a.dims[l + 1], rpc = a.rpc[l];
+      const T* w = ring + a.w_off[l];
+      for (int k0 = 0; k0 < rows; k0 += rpc) {
+        if (!a.resident) ok = tc::mbar_wait(&empty[stage], phase ^ 1u, gave_up);
+        if (!ok) break;
+        // (the last piece of a layer may run up to 12 bytes into the padding behind it)
+        const uint32_t bytes = (uint32_t)round_up(min(rpc, rows - k0) * out * (int)sizeof(T), 16);
+        tc::mbar_expect_tx(&full[stage], bytes);
+        lsqp::bulk_row(base + (a.resident ? (size_t)a.w_res[l] : (size_t)stage * a.stage_bytes), w + (size_t)k0 * out, bytes, &full[stage]);
+        if (++stage == a.stages) { stage = 0; phase ^= 1u; }
+      }
+    }
+  }
+  // consumers: the next chunk (of layer l); a wait that runs out ends the run at the end of the kernel
+  __device__ __forceinline__ const void* take(int l) {
+    if (a.resident) {
+      tc::mbar_wait(&full[l], 0u, gave_up);
+      return base + a.w_res[l];
+    }
+    tc::mbar_wait(&full[stage], phase, gave_up);
+    return base + (size_t)stage * a.stage_bytes;
+  }
+  __device__ __forceinline__ void give(int lane) {
+    if (a.resident) return;
+    __syncwarp();
+    if (lane == 0) tc::mbar_arrive(&empty[stage]);
+    if (++stage == a.stages) { stage = 0; phase ^= 1u; }
+  }
+};
+
+__device__ __forceinline__ void weights_init(const RowsArgs& a, uint64_t* full, uint64_t* empty, int* gave_up, int n_warps) {
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < a.stages; ++s) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], n_warps); }
+    *gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void rows_end(const RowsArgs& a, const int* gave_up) {
+  __syncthreads();
+  if (threadIdx.x == 0 && *gave_up) {
+    // let copies in flight land before the shared memory goes away
+    const unsigned long long t0 = tc::global_ns();
+    while (tc::global_ns() - t0 < 200000ull) {}
+    a.st->timeout_where = 400;
+    a.ri->diverged = RI_TIMEOUT;
+  }
+}
+
+// Soft-max cross-entropy of one row by one warp: lane holds the logits of classes lane and lane + 32 (at most 64);
+// returns their deltas (0 for a padding row, label -1) and publishes the loss.
+template <typename T>
+__device__ __forceinline__ float2 row_softmax(const RowsArgs& a, float z0, float z1, int r, int yl, float sa, int lane) {
+  const int C = a.dims[a.n_layers];
+  z0 = lane < C ? z0 : -3.0e38f;
+  z1 = lane + 32 < C ? z1 : -3.0e38f;
+  float zmax = fmaxf(z0, z1);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+  const float e0 = expf(z0 - zmax), e1 = expf(z1 - zmax);
+  float se = e0 + e1, zy = (lane == yl ? z0 : 0.f) + (lane + 32 == yl ? z1 : 0.f);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    se += __shfl_xor_sync(0xffffffffu, se, o);
+    zy += __shfl_xor_sync(0xffffffffu, zy, o);
+  }
+  const float inv = 1.f / se;
+  if (lane == 0) {
+    const float loss = yl < 0 ? 0.f : logf(se) - (zy - zmax);
+    a.row_loss[r] = loss;
+    if (!isfinite(loss)) a.ri->diverged = 1;
+  }
+  // a delta is a stored quantity; sa: staleness-aware step size (weight of these rows in Eq. 3)
+  if (yl < 0) return make_float2(0.f, 0.f);
+  return make_float2(round_store((e0 * inv - (lane == yl ? 1.f : 0.f)) * sa, (const T*)nullptr),
+                     round_store((e1 * inv - (lane + 32 == yl ? 1.f : 0.f)) * sa, (const T*)nullptr));
+}
+
+// Sum over the lanes of 32 values per lane: afterwards lane l holds the sum of value l (31 exchanges; each halves the
+// values a lane still carries).
+__device__ __forceinline__ float lane_transpose_sum(float (&v)[32], int lane) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool hi = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < o) {
+        const float send = hi ? v[i] : v[i + o], keep = hi ? v[i + o] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+  }
+  return v[0];
+}
+
+// ---- fp32: rows kept as [R / 4][k][4], so that one 16-byte read serves four rows of an input (all lanes, forward) or of
+// 32 columns (backward).
+// Partial products of one chunk: lane owns columns n0 + CW j (j < CPT, CW lanes per group of columns), and takes every
+// KGS-th weight row.  Per row and warp: CPT 4-byte and R / 4 16-byte shared-memory reads (1 and 2 cycles) for CPT R / 2
+// packed FMAs (2 cycles on each of four schedulers): the reads bound it up to CPT = 2.
+template <int R, int CPT, int CW>
+__device__ __forceinline__ void fma_chunk(f32x2 (&z)[4][R / 2], const float* w, const float* x, int plane, int nk, int kg, int kgs,
+                                          int out, int n0) {
+  int col[CPT];
+#pragma unroll
+  for (int j = 0; j < CPT; ++j) col[j] = min(n0 + CW * j, out - 1);
+  const float* wp = w + kg * out;
+  const float* xp = x + kg * 4;
+  const int ws = kgs * out, xs = kgs * 4;
+  constexpr int UN = CPT == 4 ? 2 : 4;
+  int k = kg;
+  for (; k + (UN - 1) * kgs < nk; k += UN * kgs) {
+    float wv[UN][CPT];
+    ulonglong2 xv[UN][R / 4];
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+#pragma unroll
+      for (int j = 0; j < CPT; ++j) wv[u][j] = wp[u * ws + col[j]];
+#pragma unroll
+      for (int q = 0; q < R / 4; ++q) xv[u][q] = *reinterpret_cast<const ulonglong2*>(xp + u * xs + q * plane);
+    }
+#pragma unroll
+    for (int u = 0; u < UN; ++u)
+#pragma unroll
+      for (int j = 0; j < CPT; ++j) {
+        const f32x2 p = lsqp::pack2(wv[u][j], wv[u][j]);
+#pragma unroll
+        for (int q = 0; q < R / 4; ++q) {
+          lsqp::ffma2(z[j][2 * q], p, xv[u][q].x);
+          lsqp::ffma2(z[j][2 * q + 1], p, xv[u][q].y);
+        }
+      }
+    wp += UN * ws;
+    xp += UN * xs;
+  }
+  for (; k < nk; k += kgs) {
+#pragma unroll
+    for (int j = 0; j < CPT; ++j) {
+      const float wv = wp[col[j]];
+      const f32x2 p = lsqp::pack2(wv, wv);
+#pragma unroll
+      for (int q = 0; q < R / 4; ++q) {
+        const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(xp + q * plane);
+        lsqp::ffma2(z[j][2 * q], p, xv.x);
+        lsqp::ffma2(z[j][2 * q + 1], p, xv.y);
+      }
+    }
+    wp += ws;
+    xp += xs;
+  }
+}
+
+// Forward of one layer up to the partial sums red[KGS][NP][R] (NP = columns rounded up); returns KGS, NP.
+template <int R, int CPT, int CW>
+__device__ __forceinline__ int2 fma_layer(Weights& W, int l, const float* x, float* red, int warp, int lane) {
+  const int rows = W.a.dims[l] + 1, out = W.a.dims[l + 1], rpc = W.a.rpc[l];
+  constexpr int COLS = CPT * CW, SUB = 32 / CW;
+  const int ncw = (out + COLS - 1) / COLS, wk = NW / ncw;     // warps across the columns / across the weight rows
+  const int g = warp / ncw, cw = warp - g * ncw;
+  const int kg = g * SUB + lane / CW, kgs = wk * SUB, n0 = cw * COLS + lane % CW;
+  const int plane = rows * 4;
+  f32x2 z[4][R / 2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int q = 0; q < R / 2; ++q) z[j][q] = 0ull;
+  for (int k0 = 0; k0 < rows; k0 += rpc) {
+    const float* w = reinterpret_cast<const float*>(W.take(l));
+    if (g < wk) fma_chunk<R, CPT, CW>(z, w, x + k0 * 4, plane, min(rpc, rows - k0), kg, kgs, out, n0);
+    W.give(lane);
+  }
+  if (g < wk) {
+#pragma unroll
+    for (int j = 0; j < CPT; ++j) {
+      float* o = red + (size_t)(kg * ncw * COLS + n0 + CW * j) * R;
+#pragma unroll
+      for (int q = 0; q < R / 4; ++q) *reinterpret_cast<ulonglong2*>(o + 4 * q) = make_ulonglong2(z[j][2 * q], z[j][2 * q + 1]);
+    }
+  }
+  return make_int2(kgs, ncw * COLS);
+}
+
+template <int R>
+__global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_constant__ RowsArgs a) {
+  grid_dependency_sync();
+  extern __shared__ __align__(128) unsigned char rsm[];
+  __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES];
+  __shared__ int gave_up;
+  __shared__ int lab[R];                             // label of each row, -1: padding
+  DevState* st = a.st;
+  RoundInfo* ri = a.ri;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = (int)blockIdx.x * R;
+  // one wave of loads (the grid covers the row capacity, so every address exists)
+  const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[blockIdx.x];
+  const int my_idx = a.row_idx[r0 + lane % R];       // sample index of row lane % R
+  if (status != ST_OK || r0 >= n_rows) return;
+  const int L = a.n_layers;
+  const size_t w_bytes = a.resident ? (size_t)a.w_res[L - 1] + round_up((a.dims[L - 1] + 1) * a.dims[L] * 4, 128)
+                                    : (size_t)a.stages * a.stage_bytes;
+  float* fs = reinterpret_cast<float*>(rsm + w_bytes);
+  weights_init(a, full, empty, &gave_up, NW);
+  Weights W(a, rsm, full, empty, &gave_up);
+  constexpr int RQ = R / 4;
+
+  if (warp == NW) {
+    if (lane == 0) W.produce((const float*)a.ring + (size_t)slot * a.slot_stride);
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------------ input rows
+    {
+      const int in = a.dims[0];
+      float* x = fs + a.act_off[0];
+      const int rq = warp % RQ;                      // (RQ divides NW) four rows per warp
+      const float* src[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = r0 + rq * 4 + j;
+        const int s = __shfl_sync(0xffffffffu, my_idx, rq * 4 + j);
+        src[j] = (a.gather && s < 0) ? nullptr : (const float*)a.X + (size_t)(a.gather ? s : r) * in;
+      }
+#pragma unroll 2
+      for (int k = (warp / RQ) * 32 + lane; k < in; k += NW / RQ * 32) {
+        float4 v;
+        v.x = src[0] ? src[0][k] : 0.f;
+        v.y = src[1] ? src[1][k] : 0.f;
+        v.z = src[2] ? src[2][k] : 0.f;
+        v.w = src[3] ? src[3][k] : 0.f;
+        *reinterpret_cast<float4*>(x + (size_t)rq * (in + 1) * 4 + k * 4) = v;
+      }
+      if (tid < R) lab[tid] = my_idx < 0 ? -1 : a.labels[my_idx];
+      for (int e = tid; e < L * R; e += NT) {         // the input of the bias row
+        const int l = e / R, q = e % R / 4;
+        fs[a.act_off[l] + (q * (a.dims[l] + 1) + a.dims[l]) * 4 + (e & 3)] = 1.f;
+      }
+    }
+    rows_sync();
+    // ------------------------------------------------------------------ forward
+    float* red = fs + a.red_off;
+    for (int l = 0; l < L; ++l) {
+      const int out = a.dims[l + 1];
+      const bool last = l == L - 1;
+      const float* x = fs + a.act_off[l];
+      int2 kn;
+      if (out > 64) kn = fma_layer<R, 4, 32>(W, l, x, red, warp, lane);
+      else if (out > 32) kn = fma_layer<R, 2, 32>(W, l, x, red, warp, lane);
+      else if (out > 16) kn = fma_layer<R, 1, 32>(W, l, x, red, warp, lane);
+      else if (out > 8) kn = fma_layer<R, 1, 16>(W, l, x, red, warp, lane);
+      else kn = fma_layer<R, 1, 8>(W, l, x, red, warp, lane);
+      rows_sync();
+      float* y = fs + (last ? a.out_off : a.act_off[l + 1]);
+      const int y_plane = (last ? out : out + 1) * 4;
+      float* ga = last ? nullptr : (float*)a.act[l + 1];
+      for (int e = tid; e < out * RQ; e += NT) {      // partial sums in order, ReLU
+        const int n = e / RQ, q = e % RQ;
+        const float4* p = reinterpret_cast<const float4*>(red) + (size_t)n * RQ + q;
+        float4 s = p[0];
+#pragma unroll 4
+        for (int g = 1; g < kn.x; ++g) {
+          const float4 t = p[(size_t)g * kn.y * RQ];
+          s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+        }
+        if (!last) {
+          s.x = fmaxf(s.x, 0.f); s.y = fmaxf(s.y, 0.f); s.z = fmaxf(s.z, 0.f); s.w = fmaxf(s.w, 0.f);
+          const size_t o = (size_t)(r0 + 4 * q) * out + n;
+          ga[o] = s.x; ga[o + out] = s.y; ga[o + 2 * (size_t)out] = s.z; ga[o + 3 * (size_t)out] = s.w;
+        }
+        *reinterpret_cast<float4*>(y + (size_t)q * y_plane + n * 4) = s;
+      }
+      rows_sync();
+    }
+    // ------------------------------------------------------------------ loss and delta of the output layer: warp = row
+    {
+      const int C = a.dims[L];
+      float* z = fs + a.out_off;
+      for (int rr = warp; rr < R; rr += NW) {
+        float* zr = z + (rr / 4) * C * 4 + (rr & 3);
+        const float2 d = row_softmax<float>(a, lane < C ? zr[lane * 4] : 0.f, lane + 32 < C ? zr[(lane + 32) * 4] : 0.f, r0 + rr, lab[rr],
+                                            sa_slot_weight(st, ri->t, slot), lane);
+        float* gd = (float*)a.delta[L] + (size_t)(r0 + rr) * C;
+        if (lane < C) { zr[lane * 4] = d.x; gd[lane] = d.x; }
+        if (lane + 32 < C) { zr[(lane + 32) * 4] = d.y; gd[lane + 32] = d.y; }
+      }
+    }
+    rows_sync();
+    // ------------------------------------------------------------------ backward: the delta of layer l's input takes the
+    // place of that input (only its sign is still needed, by the lane that overwrites it)
+    for (int l = L - 1; l >= (a.want_d0 ? 0 : 1); --l) {
+      constexpr int MB = 32 / R;                     // weight rows per warp step
+      const int in = a.dims[l], out = a.dims[l + 1], rpc = a.rpc[l];
+      const float* dl = fs + (l == L - 1 ? a.out_off : a.act_off[l + 1]);
+      const int d_plane = (l == L - 1 ? out : out + 1) * 4;
+      float* h = fs + a.act_off[l];
+      float* gd = (float*)a.delta[l];
+      for (int k0 = 0; k0 < in + 1; k0 += rpc) {
+        const float* w = reinterpret_cast<const float*>(W.take(l));
+        const int nk = min(rpc, in - k0);
+        for (int mb = warp * MB; mb < nk; mb += NW * MB) {
+          f32x2 acc[MB][R / 2];
+#pragma unroll
+          for (int i = 0; i < MB; ++i)
+#pragma unroll
+            for (int j = 0; j < R / 2; ++j) acc[i][j] = 0ull;
+          const float* wr[MB];
+#pragma unroll
+          for (int i = 0; i < MB; ++i) wr[i] = w + min(mb + i, nk - 1) * out;
+#pragma unroll 2
+          for (int n = lane; n < out; n += 32) {
+            f32x2 d2[R / 2];
+#pragma unroll
+            for (int q = 0; q < RQ; ++q) {
+              const ulonglong2 dv = *reinterpret_cast<const ulonglong2*>(dl + q * d_plane + n * 4);
+              d2[2 * q] = dv.x;
+              d2[2 * q + 1] = dv.y;
+            }
+#pragma unroll
+            for (int i = 0; i < MB; ++i) {
+              const float wv = wr[i][n];
+              const f32x2 p = lsqp::pack2(wv, wv);
+#pragma unroll
+              for (int j = 0; j < R / 2; ++j) lsqp::ffma2(acc[i][j], p, d2[j]);
+            }
+          }
+          float v[32];
+#pragma unroll
+          for (int i = 0; i < MB; ++i)
+#pragma unroll
+            for (int j = 0; j < R / 2; ++j) lsqp::unpack2(acc[i][j], v[i * R + 2 * j], v[i * R + 2 * j + 1]);
+          const float s = lane_transpose_sum(v, lane);
+          const int mi = mb + lane / R, rr = lane % R;
+          if (mi < nk) {
+            float* hp = h + (size_t)(rr / 4) * (in + 1) * 4 + (size_t)(k0 + mi) * 4 + (rr & 3);
+            const float d = *hp > 0.f ? s : 0.f;
+            *hp = d;
+            gd[(size_t)(r0 + rr) * in + k0 + mi] = d;
+          }
+        }
+        W.give(lane);
+      }
+      rows_sync();
+    }
+  }
+  rows_end(a, &gave_up);
+}
+
+// ---- bf16: the same with the warp-level tensor-core instruction (mma m16n8k16, bf16 in, fp32 accumulate), 16 rows per
+// CTA kept as [row][k] (pitch: a multiple of 16 plus 8 elements, zero-padded), 8-column tiles dealt to the warps.  The
+// weight fragments are read element by element: the widths of this class rarely give 16-byte rows.  (tcgen05 tiles
+// would be 128 rows; a round has a few hundred rows in groups of any size.)
+__device__ __forceinline__ uint32_t pair16(const __nv_bfloat16* p, int stride) {          // p[0] | p[stride] << 16
+  const uint32_t lo = *reinterpret_cast<const unsigned short*>(p), hi = *reinterpret_cast<const unsigned short*>(p + stride);
+  return lo | (hi << 16);
+}
+
+// rows [R][pitch] of shared memory -> rows of n elements
+__device__ __forceinline__ void copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, int pitch, int n, int warp, int lane) {
+  for (int rr = warp; rr < MMA_R; rr += MMA_NW) {
+    if ((n & 7) == 0) {
+      for (int k = lane * 8; k < n; k += 256) *reinterpret_cast<uint4*>(dst + (size_t)rr * n + k) = *reinterpret_cast<const uint4*>(src + rr * pitch + k);
+    } else {
+      for (int k = lane; k < n; k += 32) dst[(size_t)rr * n + k] = src[rr * pitch + k];
+    }
+  }
+}
+
+static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const __grid_constant__ RowsArgs a) {
+  grid_dependency_sync();
+  extern __shared__ __align__(128) unsigned char rsm[];
+  __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES];
+  __shared__ int gave_up;
+  __shared__ int lab[MMA_R];                         // label of each row, -1: padding
+  typedef __nv_bfloat16 T;
+  constexpr int R = MMA_R, NWM = MMA_NW;
+  DevState* st = a.st;
+  RoundInfo* ri = a.ri;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = (int)blockIdx.x * R;
+  // one wave of loads (the grid covers the row capacity, so every address exists)
+  const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[blockIdx.x];
+  const int my_idx = a.row_idx[r0 + warp];           // warp w fetches row w
+  if (status != ST_OK || r0 >= n_rows) return;
+  const int g = lane >> 2, t = lane & 3;
+  const int L = a.n_layers;
+  const size_t w_bytes = a.resident ? (size_t)a.w_res[L - 1] + round_up((a.dims[L - 1] + 1) * a.dims[L] * 2, 128)
+                                    : (size_t)a.stages * a.stage_bytes;
+  T* ts = reinterpret_cast<T*>(rsm + w_bytes);
+  weights_init(a, full, empty, &gave_up, NWM);
+  Weights W(a, rsm, full, empty, &gave_up);
+  auto sync_compute = [] { asm volatile("bar.sync 1, %0;" ::"n"(NWM * 32) : "memory"); };
+  const T* w_ring = (const T*)a.ring + (size_t)slot * a.slot_stride;
+  if (a.resident && tid == NWM * 32) W.produce(w_ring);
+  __syncwarp();
+  {
+    // ---------------------------------------------------------------- input row of this warp; zero padding columns
+    const int in = a.dims[0];
+    const T* src = (a.gather && my_idx < 0) ? nullptr : (const T*)a.X + (size_t)(a.gather ? my_idx : r0 + warp) * in;
+    if (lane == 0) lab[warp] = my_idx < 0 ? -1 : a.labels[my_idx];
+    T* x = ts + a.act_off[0] + warp * mma_pitch(in);
+    if ((in & 7) == 0) {                              // rows on 16-byte boundaries
+#pragma unroll 4
+      for (int k = lane * 8; k < in; k += 256)
+        *reinterpret_cast<uint4*>(x + k) = src ? *reinterpret_cast<const uint4*>(src + k) : make_uint4(0u, 0u, 0u, 0u);
+    } else {
+#pragma unroll 8
+      for (int k = lane; k < in; k += 32) x[k] = src ? src[k] : (T)0.f;
+    }
+    for (int l = 0; l <= L; ++l) {
+      const int n = a.dims[l], p = mma_pitch(n);      // at most 8 + 15 padding columns
+      if (n + lane < p) ts[(l < L ? a.act_off[l] : a.out_off) + warp * p + n + lane] = (T)0.f;
+    }
+  }
+  __syncthreads();
+
+  if (warp == NWM) {
+    if (!a.resident && lane == 0) W.produce(w_ring);
+    __syncwarp();
+  } else {
+    const int sel_row = lane & 15, sel_col = (lane >> 4) * 8;         // ldmatrix addresses of an A tile
+    // ------------------------------------------------------------------ forward: warp takes column tiles warp, warp + 15, ...
+    float* logits = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(ts) + a.red_off);     // [R][C + 1]
+    for (int l = 0; l < L; ++l) {
+      const int in = a.dims[l], out = a.dims[l + 1], rpc = a.rpc[l], pitch = mma_pitch(in);
+      const bool last = l == L - 1;
+      const uint32_t a_base = outl::s_u32(ts + a.act_off[l] + sel_row * pitch + sel_col);
+      // streamed weights come once, so a warp finishes all its tiles chunk by chunk (1024 columns = 9 tiles per warp)
+      constexpr int TP = 3, PASSES = 3;
+      const int n_ct = (out + 7) >> 3;
+      float acc[PASSES * TP][4];
+#pragma unroll
+      for (int c = 0; c < PASSES * TP; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[c][i] = 0.f;
+      for (int k0 = 0; k0 < in + 1; k0 += rpc) {
+        const T* w = reinterpret_cast<const T*>(W.take(l));
+        const int nk = min(rpc, in - k0);             // weight rows of this chunk (the bias row apart)
+#pragma unroll
+        for (int pass = 0; pass < PASSES; ++pass) {
+          const int ct0 = warp + pass * TP * NWM;
+          if (ct0 >= n_ct) break;
+          const int n_here = min(TP, (n_ct - ct0 + NWM - 1) / NWM);
+          const T* wp[TP];                            // element (row 2t, column g) of each tile
+#pragma unroll
+          for (int c = 0; c < TP; ++c) wp[c] = w + 2 * t * out + min((ct0 + c * NWM) * 8 + g, out - 1);
+          const int step = 16 * out;
+          int k = 0;
+#pragma unroll 4
+          for (; k + 16 <= nk; k += 16) {
+            uint32_t af[4];
+            outl::ldsm4(a_base + (uint32_t)(k0 + k) * 2u, af);
+#pragma unroll
+            for (int c = 0; c < TP; ++c) {
+              if (c < n_here) outl::mma16816(acc[pass * TP + c], af, pair16(wp[c], out), pair16(wp[c] + 8 * out, out));
+              wp[c] += step;
+            }
+          }
+          if (k < nk) {
+            // rows behind the layer's last one meet zero activations: any finite weight will do
+            uint32_t af[4];
+            outl::ldsm4(a_base + (uint32_t)(k0 + k) * 2u, af);
+            const int lastr = nk - 1 - k;
+            const int ka = min(2 * t, lastr), kb = min(2 * t + 1, lastr), kc = min(2 * t + 8, lastr), kd = min(2 * t + 9, lastr);
+#pragma unroll
+            for (int c = 0; c < TP; ++c)
+              if (c < n_here) {
+                const T* q = wp[c] - 2 * t * out;
+                outl::mma16816(acc[pass * TP + c], af, pair16(q + ka * out, (kb - ka) * out), pair16(q + kc * out, (kd - kc) * out));
+              }
+          }
+        }
+        if (k0 + rpc >= in + 1) {                     // the last chunk ends with the bias row
+          const T* bias = w + (in - k0) * out;
+#pragma unroll
+          for (int c = 0; c < PASSES * TP; ++c) {
+            const int n = (warp + c * NWM) * 8 + 2 * t;
+            if (n < out) {
+              const float b0 = __bfloat162float(bias[n]), b1 = n + 1 < out ? __bfloat162float(bias[n + 1]) : 0.f;
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const float v0 = acc[c][2 * h] + b0, v1 = acc[c][2 * h + 1] + b1;
+                const int rr = g + 8 * h;
+                if (last) {
+                  logits[rr * (out + 1) + n] = v0;
+                  if (n + 1 < out) logits[rr * (out + 1) + n + 1] = v1;
+                } else {                              // (the column behind an odd last one is padding and stays zero)
+                  *reinterpret_cast<uint32_t*>(ts + a.act_off[l + 1] + rr * mma_pitch(out) + n) =
+                      outl::pack_bf16(fmaxf(v0, 0.f), n + 1 < out ? fmaxf(v1, 0.f) : 0.f);
+                }
+              }
+            }
+          }
+        }
+        W.give(lane);
+      }
+      sync_compute();
+      if (!last) copy_rows((T*)a.act[l + 1] + (size_t)r0 * out, ts + a.act_off[l + 1], mma_pitch(out), out, warp, lane);
+    }
+    // ------------------------------------------------------------------ loss and delta of the output layer
+    {
+      const int C = a.dims[L];
+      T* dl = ts + a.out_off;
+      const float sa = sa_slot_weight(st, ri->t, slot);
+      for (int rr = warp; rr < R; rr += NWM) {
+        const float* z = logits + rr * (C + 1);
+        const float2 d = row_softmax<T>(a, lane < C ? z[lane] : 0.f, lane + 32 < C ? z[lane + 32] : 0.f, r0 + rr, lab[rr], sa, lane);
+        T* gd = (T*)a.delta[L] + (size_t)(r0 + rr) * C;
+        if (lane < C) { dl[rr * mma_pitch(C) + lane] = __float2bfloat16_rn(d.x); gd[lane] = __float2bfloat16_rn(d.x); }
+        if (lane + 32 < C) { dl[rr * mma_pitch(C) + lane + 32] = __float2bfloat16_rn(d.y); gd[lane + 32] = __float2bfloat16_rn(d.y); }
+      }
+    }
+    sync_compute();
+    // ------------------------------------------------------------------ backward: tiles of 8 weight rows (= input columns)
+    for (int l = L - 1; l >= (a.want_d0 ? 0 : 1); --l) {
+      const int in = a.dims[l], out = a.dims[l + 1], rpc = a.rpc[l], pitch = mma_pitch(in);
+      const T* dl = ts + (l == L - 1 ? a.out_off : a.act_off[l + 1]);
+      const int dp = mma_pitch(out);
+      const uint32_t a_base = outl::s_u32(dl + sel_row * dp + sel_col);
+      T* h = ts + a.act_off[l];
+      const bool even = (out & 1) == 0;
+      for (int k0 = 0; k0 < in + 1; k0 += rpc) {
+        const T* w = reinterpret_cast<const T*>(W.take(l));
+        const int nk = min(rpc, in - k0);
+        constexpr int TP = 4;
+        for (int m0 = warp * 8; m0 < nk; m0 += NWM * 8 * TP) {
+          const int n_here = min(TP, (nk - m0 + NWM * 8 - 1) / (NWM * 8));
+          float acc[TP][4];
+          const T* wm[TP];                            // weight row g of each tile
+#pragma unroll
+          for (int c = 0; c < TP; ++c) {
+            wm[c] = w + min(m0 + c * NWM * 8 + g, nk - 1) * out;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[c][i] = 0.f;
+          }
+          int n = 0;
+          if (even) {                                 // pairs are 4-byte aligned
+#pragma unroll 4
+            for (; n + 16 <= out; n += 16) {
+              uint32_t af[4];
+              outl::ldsm4(a_base + (uint32_t)n * 2u, af);
+#pragma unroll
+              for (int c = 0; c < TP; ++c)
+                if (c < n_here)
+                  outl::mma16816(acc[c], af, *reinterpret_cast<const uint32_t*>(wm[c] + n + 2 * t), *reinterpret_cast<const uint32_t*>(wm[c] + n + 2 * t + 8));
+            }
+          } else {
+#pragma unroll 2
+            for (; n + 16 <= out; n += 16) {
+              uint32_t af[4];
+              outl::ldsm4(a_base + (uint32_t)n * 2u, af);
+#pragma unroll
+              for (int c = 0; c < TP; ++c)
+                if (c < n_here) outl::mma16816(acc[c], af, pair16(wm[c] + n + 2 * t, 1), pair16(wm[c] + n + 2 * t + 8, 1));
+            }
+          }
+          if (n < out) {                              // columns behind the last one meet zero deltas
+            uint32_t af[4];
+            outl::ldsm4(a_base + (uint32_t)n * 2u, af);
+            const int na = min(n + 2 * t, out - 1), nb = min(n + 2 * t + 1, out - 1), nc = min(n + 2 * t + 8, out - 1), nd = min(n + 2 * t + 9, out - 1);
+#pragma unroll
+            for (int c = 0; c < TP; ++c)
+              if (c < n_here) outl::mma16816(acc[c], af, pair16(wm[c] + na, nb - na), pair16(wm[c] + nc, nd - nc));
+          }
+#pragma unroll
+          for (int c = 0; c < TP; ++c) {
+            const int mi = m0 + c * NWM * 8 + 2 * t;
+            if (mi < nk) {                            // (the element behind an odd last one is padding and stays zero)
+#pragma unroll
+              for (int h2 = 0; h2 < 2; ++h2) {
+                uint32_t* hp = reinterpret_cast<uint32_t*>(h + (g + 8 * h2) * pitch + k0 + mi);
+                const float2 hv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(hp));
+                *hp = outl::pack_bf16(hv.x > 0.f ? acc[c][2 * h2] : 0.f, hv.y > 0.f ? acc[c][2 * h2 + 1] : 0.f);
+              }
+            }
+          }
+        }
+        W.give(lane);
+      }
+      sync_compute();
+      copy_rows((T*)a.delta[l] + (size_t)r0 * in, h, pitch, in, warp, lane);
+    }
+  }
+  rows_end(a, &gave_up);
+}
+
+// ---------------------------------------------------------------------------------------------
+constexpr int GT = 32;                   // features x outputs per tile of grad_step_kernel
+constexpr int GK = 64;                   // rows per pipeline step
+constexpr int GP = GT + 4;               // shared-memory pitch
+
+struct StepArgs {
+  const DevState* st;
+  const RoundInfo* ri;
+  const int* row_idx;
+  const void* X; int gather;
+  const void* act[ABS_MAX_LAYERS + 1];
+  const void* delta[ABS_MAX_LAYERS + 1];
+  float* master; void* ring; size_t d_pad;
+  float lr;
+  size_t w_off[ABS_MAX_LAYERS];
+  int n_layers, dims[ABS_MAX_LAYERS + 1];
+  int first_tile[ABS_MAX_LAYERS + 1];    // tiles of layer l: [first_tile[l], first_tile[l + 1])
+  int Q;                                 // CTAs (a cluster) per tile: they share the rows
+  // parts of the gradient left as per-chunk partial sums (the CNN's convolution blocks): blocks behind the tiles
+  struct Region { const float* part; int len, chunk_rows; size_t off; int first_block; } region[2];
+  int n_regions;
+};
+
+__device__ __forceinline__ float ld_cluster(const float* p, int rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(tc::map_to_cta(tc::smem_u32(p), (uint32_t)rank)) : "memory");
+  return v;
+}
+
+// Four groups of 64 threads take 16 rows of a 64-row step each (4 x 4 sums per thread: two 16-byte shared-memory reads
+// for eight packed FMAs), the next step's rows are loaded into registers meanwhile; groups, then cluster CTAs, are
+// added in order and the owner applies Eq. 3.
+template <typename T>
+__global__ void __launch_bounds__(256) grad_step_kernel(const __grid_constant__ StepArgs a) {
+  grid_dependency_sync();
+  __shared__ __align__(16) float As[2][GK][GP], Ds[2][GK][GP];
+  const DevState* st = a.st;
+  const RoundInfo* ri = a.ri;
+  const int status = st->status, diverged = ri->diverged, K = ri->K, n_rows = ri->n_rows, B = st->B, t = ri->t, S = st->S;
+  if (status != ST_OK || diverged) return;
+  const float step = __fdiv_rn(a.lr, (float)(K * B));
+  const int slot = (t + 1) % (S + 1);
+  T* dst = (T*)a.ring + (size_t)slot * a.d_pad;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n_tiles = a.first_tile[a.n_layers];
+  if ((int)blockIdx.x >= n_tiles * a.Q) {
+    // region block: 32 parameters x 8 lanes over the chunks, fixed order
+    float* red = &As[0][0][0];
+    const int rb = (int)blockIdx.x - n_tiles * a.Q;
+    const int q = (a.n_regions > 1 && rb >= a.region[1].first_block) ? 1 : 0;
+    const StepArgs::Region& G = a.region[q];
+    const int n_chunks = (n_rows + G.chunk_rows - 1) / G.chunk_rows;
+    const int j = (rb - G.first_block) * 32 + lane;
+    float acc = 0.f;
+    if (j < G.len) {
+#pragma unroll 8
+      for (int c = warp; c < n_chunks; c += 8) acc += G.part[(size_t)c * G.len + j];
+    }
+    red[warp * 33 + lane] = acc;
+    __syncthreads();
+    if (warp == 0 && j < G.len) {
+      float tot = 0.f;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) tot += red[c * 33 + lane];
+      const size_t e = G.off + (size_t)j;
+      const float m = fmaf(-step, tot, a.master[e]);
+      a.master[e] = m;
+      stf(dst, e, m);
+    }
+    return;
+  }
+  const int Q = a.Q, rank = (int)blockIdx.x % Q, tile = (int)blockIdx.x / Q;
+  int l = 0;
+  while (tile >= a.first_tile[l + 1]) ++l;
+  const int in = a.dims[l], out = a.dims[l + 1];
+  const int nct = (out + GT - 1) / GT, lt = tile - a.first_tile[l];
+  const int m0 = lt / nct * GT, n0 = (lt % nct) * GT;
+  const bool gather = l == 0 && a.gather;
+  const T* A = (const T*)(l == 0 ? a.X : a.act[l]);
+  const T* D = (const T*)a.delta[l + 1];
+  const int m = m0 + lane, n = n0 + lane;
+  const int n_steps = (n_rows + GK - 1) / GK;
+  // row 8 i + warp of a step is loaded by this warp; lane i < 8 holds its sample index
+  auto load_idx = [&](int s) -> int {
+    const int r = s * GK + 8 * lane + warp;
+    return (lane < 8 && r < n_rows && s < n_steps) ? (gather ? a.row_idx[r] : r) : -1;
+  };
+  float pa[8], pd[8];
+  auto load = [&](int s, int idx) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = s * GK + 8 * i + warp;
+      const int x = __shfl_sync(0xffffffffu, idx, i);
+      pa[i] = x < 0 ? 0.f : m < in ? ldf(A, (size_t)x * in + m) : m == in ? 1.f : 0.f;    // row `in`: the bias
+      pd[i] = (r < n_rows && n < out) ? ldf(D, (size_t)r * out + n) : 0.f;
+    }
+  };
+  f32x2 acc[4][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0ull;
+  const int kg = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
+  int idx = load_idx(rank);
+  if (rank < n_steps) load(rank, idx);
+  idx = load_idx(rank + Q);
+  int buf = 0;
+  for (int s = rank; s < n_steps; s += Q) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      As[buf][8 * i + warp][lane] = pa[i];
+      Ds[buf][8 * i + warp][lane] = pd[i];
+    }
+    __syncthreads();
+    if (s + Q < n_steps) {
+      load(s + Q, idx);
+      idx = load_idx(s + 2 * Q);
+    }
+#pragma unroll
+    for (int k = 0; k < GK / 4; ++k) {
+      const float4 av = *reinterpret_cast<const float4*>(&As[buf][kg * (GK / 4) + k][4 * ty]);
+      const ulonglong2 dv = *reinterpret_cast<const ulonglong2*>(&Ds[buf][kg * (GK / 4) + k][4 * tx]);
+      const f32x2 p[4] = {lsqp::pack2(av.x, av.x), lsqp::pack2(av.y, av.y), lsqp::pack2(av.z, av.z), lsqp::pack2(av.w, av.w)};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        lsqp::ffma2(acc[i][0], p[i], dv.x);
+        lsqp::ffma2(acc[i][1], p[i], dv.y);
+      }
+    }
+    buf ^= 1;
+  }
+  __syncthreads();
+  float* red = &As[0][0][0];                         // [4][GT][GT]
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<ulonglong2*>(red + (size_t)kg * GT * GT + (4 * ty + i) * GT + 4 * tx) = make_ulonglong2(acc[i][0], acc[i][1]);
+  __syncthreads();
+  float* sum = &Ds[0][0][0];                         // [GT][GT] this CTA's sum
+#pragma unroll
+  for (int e = tid; e < GT * GT; e += 256)
+    sum[e] = (red[e] + red[GT * GT + e]) + (red[2 * GT * GT + e] + red[3 * GT * GT + e]);
+  if (Q > 1) tc::cluster_sync_all();
+  else __syncthreads();
+  const int share = GT * GT / Q;
+  for (int e = rank * share + tid; e < (rank + 1) * share; e += 256) {
+    const int mm = m0 + e / GT, nn = n0 + e % GT;
+    if (mm > in || nn >= out) continue;
+    float g = 0.f;
+    if (Q > 1) {
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = q < Q ? ld_cluster(sum + e, q) : 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) g += v[q];
+    } else {
+      g = sum[e];
+    }
+    const size_t o = a.w_off[l] + (size_t)mm * out + nn;
+    const float w = fmaf(-step, g, a.master[o]);
+    a.master[o] = w;
+    stf(dst, o, w);
+  }
+  if (Q > 1) tc::cluster_sync_all();                 // nobody leaves while a peer reads its sum
+}
+
+}  // namespace rnet
+}  // namespace absb

@@ -243,6 +243,30 @@ def test_local_sgd_steps_multi_layer_network_fma_paths(dims, dtype, W, B, U, K0,
     assert rows[-1]["loss_mean"] < rows[0]["loss_mean"]
 
 
+@pytest.mark.parametrize("kind,dims,dtype,W,B,flags", [
+    (inputs.MLP, (37, 130, 64, 33), inputs.FP32, 6, 9, 0),       # 4 rows per CTA; four / two / two columns per lane
+    (inputs.MLP, (50, 24, 12, 6), inputs.FP32, 20, 40, 0),       # 8 rows; one column per lane of 32, 16 and 8 lanes
+    (inputs.MLP, (60, 20, 64), inputs.FP32, 24, 128, 0),         # 16 rows; the largest class count
+    (inputs.SOFTMAX, (33, 2), inputs.FP32, 64, 64, 0),
+    (inputs.MLP, (520, 310, 77, 10), inputs.FP32, 5, 30, 0),     # weights streamed through shared memory, 4 rows
+    (inputs.MLP, (300, 260, 10), inputs.FP32, 30, 90, 0),        # ... 16 rows
+    (inputs.MLP, (201, 133, 10), inputs.BF16, 7, 20, 0),         # bf16, weights resident, odd and even widths
+    (inputs.MLP, (128, 256, 48, 10), inputs.BF16, 7, 20, gpu.FLAG_NO_TENSOR_CORES),     # 16-byte rows
+    (inputs.MLP, (700, 301, 77, 10), inputs.BF16, 6, 17, 0),     # bf16, streamed
+    (inputs.MLP, (90, 1001, 10), inputs.BF16, 4, 12, 0),         # 126 column tiles
+])
+def test_row_kernels(kind, dims, dtype, W, B, flags):
+    """Networks through the row kernels: rows per CTA, columns per lane, resident and streamed weights.  Four rounds:
+    both sides agree to about 6e-8 (fp32) until a ReLU decision on a pre-activation within rounding of zero falls
+    differently in binary32 and binary64, which re-routes one delta (seen between rounds 4 and 8 of the 300-260-10
+    case: 1.2e-5 on the vector, the same with kernels that sum in another order)."""
+    cfg = _small_cfg(kind, dims, dtype, W, B, 3, 5, GAMMA3, lr=0.02)
+    X, y, w0 = _problem(cfg)
+    bf16 = dtype == inputs.BF16
+    compare_with_oracle(cfg, X, y, w0, 4, TOL_BF16 if bf16 else TOL_FP32, forced=True, loss_tol=5e-2 if bf16 else None,
+                        flags=flags)
+
+
 def test_lock_step_constant_times():
     cfg = _small_cfg(inputs.LSQ, (16, 1), inputs.FP32, 8, 4, 2, 3,
                      inputs.TimeSpec(inputs.T_CONST, shift=3.0))
