@@ -20,6 +20,7 @@
 #include "persist.cuh"
 #include "conv.cuh"
 #include "rownet.cuh"
+#include "convmma.cuh"
 
 using namespace absb;
 
@@ -86,6 +87,7 @@ struct Layout {
   size_t x_len = 0;                       // elements of one dataset row
   size_t pool1 = 0, dpool1 = 0, arg1 = 0, arg2 = 0, cpart[2] = {};  // pooled maps of block 1, their delta, pool positions, chunk sums
   int cchunk = 1;                         // gradient rows per CTA of the convolution weight-gradient kernel
+  bool conv_mma = false;                  // both blocks through convmma.cuh (bf16)
   size_t bits[ABS_MAX_LAYERS + 1];      // ReLU sign bits of act[l] (tensor-core layers)
   size_t act[ABS_MAX_LAYERS + 1], delta[ABS_MAX_LAYERS + 1];
   size_t tr_K, tr_R, tr_theta, tr_T, tr_loss, tr_comm, tr_sel_off, tr_rst_off;
@@ -144,6 +146,13 @@ int check_model(const abs_model_desc* m, int W, int S) {
   if (m->restart_rule == ABS_RESTART_EQ6 && S + 1 > ABS_MAX_BOUND)
     return fail(ABS_EINVAL, "staleness_bound %d: Eq. 6 as printed keeps one more version, at most %d", S, ABS_MAX_BOUND - 1);
   return ABS_OK;
+}
+
+void conv_blocks(const Layout& L, cmma::Block* b) {
+  for (int i = 0; i < 2; ++i) {
+    const int Ho = L.cHi[i] - L.ck + 1, Wo = L.cWi[i] - L.ck + 1;
+    b[i] = cmma::Block{L.cHi[i], L.cWi[i], L.cCi[i], Ho, Wo, Ho / 2, Wo / 2, L.cCo[i], L.c_off[i]};
+  }
 }
 
 int step_tiles(int in, int out) { return ((in + 1 + rnet::GT - 1) / rnet::GT) * ((out + rnet::GT - 1) / rnet::GT); }
@@ -379,6 +388,10 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       // 1 / 2 / 4 / 8 rows per CTA give 1742 / 1617 / 1409 / 1222 rounds/s)
       L->cchunk = 1;
       while (L->cchunk < conv::MAX_CHUNK && (long long)W * m->batch / (2 * L->cchunk) >= 4 * 148) L->cchunk *= 2;
+      cmma::Block cb[2];
+      conv_blocks(*L, cb);
+      L->conv_mma = L->esz == 2 && L->row_R > 0 && !(m->flags & ABS_FLAG_NO_TENSOR_CORES) && cmma::fits(L->ck, cb[0], cb[1]);
+      if (L->conv_mma) L->cchunk = cmma::FR;
       for (int b = 0; b < 2; ++b) L->cpart[b] = cv.take(4 * L->c_len[b] * (size_t)((L->rows_cap + L->cchunk - 1) / L->cchunk));
     }
   }
@@ -727,6 +740,31 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     a.rpb = L.narrow_rpb;
     return a;
   };
+  auto conv_mma_args = [&]() {
+    cmma::Args c;
+    memset(&c, 0, sizeof c);
+    c.st = st; c.ri = ri; c.tile_slot = ctx->ctl.tile_slot[par]; c.row_idx = ctx->ctl.row_idx[par];
+    c.ring = ctx->at<void>(L.ring); c.slot_stride = L.d_pad; c.k = L.ck;
+    conv_blocks(L, c.b);
+    c.X = (const __nv_bfloat16*)ctx->X;
+    c.pool1 = ctx->at<__nv_bfloat16>(L.pool1); c.arg1 = ctx->at<unsigned char>(L.arg1);
+    c.feat = ctx->at<__nv_bfloat16>(par ? L.act0b : L.act[0]); c.arg2 = ctx->at<unsigned char>(L.arg2);
+    c.dfeat = ctx->at<__nv_bfloat16>(L.delta[0]);
+    for (int b = 0; b < 2; ++b) c.part[b] = ctx->at<float>(L.cpart[b]);
+    return c;
+  };
+  if (L.conv_mma && phase == PH_GATHER) {
+    const cmma::Args c = conv_mma_args();
+    launch_ex(ctx, ABS_KC_CONV, cmma::conv_fwd_mma_kernel, dim3(L.rows_cap / cmma::FR), dim3(cmma::NT),
+              cmma::fwd_layout(c.k, c.b[0], c.b[1]).total, c);
+    return;
+  }
+  if (L.conv_mma && phase == PH_BACKWARD) {
+    const cmma::Args c = conv_mma_args();
+    launch_ex(ctx, ABS_KC_CONV, cmma::conv_bwd_mma_kernel, dim3(L.rows_cap / cmma::FR), dim3(cmma::NT),
+              cmma::bwd_layout(c.k, c.b[0], c.b[1]).total, c);
+    return;
+  }
   if (phase == PH_GATHER && L.cnn) {
     // Eq. 2 forward through the two convolution blocks: the features are the input rows of layer 0
     for (int b = 0; b < 2; ++b) {
@@ -1252,6 +1290,8 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_wgrad_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_dgrad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_dgrad_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    if (ec == cudaSuccess && L.conv_mma) ec = cudaFuncSetAttribute(cmma::conv_fwd_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);
+    if (ec == cudaSuccess && L.conv_mma) ec = cudaFuncSetAttribute(cmma::conv_bwd_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);
     if (ec != cudaSuccess) return bail(cuda_fail(nullptr, ec, "cudaFuncSetAttribute(conv_block kernels)"));
   }
   if (!(model->flags & ABS_FLAG_NO_OVERLAP) && L.any_tc && !L.local_net && !L.cnn) {
