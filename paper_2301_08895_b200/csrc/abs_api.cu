@@ -19,8 +19,8 @@
 #include "localnet.cuh"
 #include "persist.cuh"
 #include "conv.cuh"
-#include "rownet.cuh"
 #include "convmma.cuh"
+#include "rownet.cuh"
 
 using namespace absb;
 
@@ -88,6 +88,8 @@ struct Layout {
   size_t pool1 = 0, dpool1 = 0, arg1 = 0, arg2 = 0, cpart[2] = {};  // pooled maps of block 1, their delta, pool positions, chunk sums
   int cchunk = 1;                         // gradient rows per CTA of the convolution weight-gradient kernel
   bool conv_mma = false;                  // both blocks through convmma.cuh (bf16)
+  size_t conv_tab = 0;                    // ... its tables (cmma::fill_tables)
+  size_t frag = 0, frag_stride = 0;       // ... whose weights are kept as operand fragments per model version
   size_t bits[ABS_MAX_LAYERS + 1];      // ReLU sign bits of act[l] (tensor-core layers)
   size_t act[ABS_MAX_LAYERS + 1], delta[ABS_MAX_LAYERS + 1];
   size_t tr_K, tr_R, tr_theta, tr_T, tr_loss, tr_comm, tr_sel_off, tr_rst_off;
@@ -331,6 +333,15 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   L->master = cv.take(4 * L->d_pad);
   L->ring = cv.take(L->esz * L->d_pad * (S + 1));
   if (m->local_steps > 1) L->P = 0;      // Eq. 3 adds one upload per selected worker
+  if (L->cnn && L->row_R) {
+    cmma::Block cb[2];
+    conv_blocks(*L, cb);
+    L->conv_mma = L->esz == 2 && !(m->flags & ABS_FLAG_NO_TENSOR_CORES) && cmma::fits(L->ck, cb[0], cb[1]);
+    if (L->conv_mma) {
+      L->frag_stride = round_up_sz((size_t)cmma::frag_total(L->ck, cb[0], cb[1]), 64);
+      L->frag = cv.take(2 * L->frag_stride * (S + 1));
+    }
+  }
   L->G = cv.take(4 * L->d_pad * ((lsq || m->local_steps > 1) ? W : L->P));
   L->gring = L->ring;
   L->gslots = S + 1;
@@ -388,10 +399,12 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       // 1 / 2 / 4 / 8 rows per CTA give 1742 / 1617 / 1409 / 1222 rounds/s)
       L->cchunk = 1;
       while (L->cchunk < conv::MAX_CHUNK && (long long)W * m->batch / (2 * L->cchunk) >= 4 * 148) L->cchunk *= 2;
-      cmma::Block cb[2];
-      conv_blocks(*L, cb);
-      L->conv_mma = L->esz == 2 && L->row_R > 0 && !(m->flags & ABS_FLAG_NO_TENSOR_CORES) && cmma::fits(L->ck, cb[0], cb[1]);
       if (L->conv_mma) L->cchunk = cmma::FR;
+      if (L->conv_mma) {
+        cmma::Block cb[2];
+        conv_blocks(*L, cb);
+        L->conv_tab = cv.take(4 * (size_t)cmma::table_words(cmma::bwd_layout(L->ck, cb[0], cb[1])));
+      }
       for (int b = 0; b < 2; ++b) L->cpart[b] = cv.take(4 * L->c_len[b] * (size_t)((L->rows_cap + L->cchunk - 1) / L->cchunk));
     }
   }
@@ -643,6 +656,13 @@ void (*local_cluster_fn(int C))(local::Args, local::Geo) {
          : C <= 12 ? local::local_cluster_kernel<T, 12> : local::local_cluster_kernel<T, 16>;
 }
 
+cmma::FragMap frag_map(const abs_ctx* ctx) {
+  cmma::FragMap m;
+  m.frag = ctx->at<__nv_bfloat16>(ctx->L.frag); m.stride = ctx->L.frag_stride; m.k = ctx->L.ck;
+  conv_blocks(ctx->L, m.b);
+  return m;
+}
+
 // the row kernel for R rows per CTA
 template <typename T>
 void (*rows_kernel_fn(int R))(rnet::RowsArgs) {
@@ -751,18 +771,21 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     c.feat = ctx->at<__nv_bfloat16>(par ? L.act0b : L.act[0]); c.arg2 = ctx->at<unsigned char>(L.arg2);
     c.dfeat = ctx->at<__nv_bfloat16>(L.delta[0]);
     for (int b = 0; b < 2; ++b) c.part[b] = ctx->at<float>(L.cpart[b]);
+    c.frag = ctx->at<__nv_bfloat16>(L.frag); c.frag_stride = L.frag_stride;
+    c.taps = ctx->at<int>(L.conv_tab);
+    cmma::fill_shapes(&c);
     return c;
   };
   if (L.conv_mma && phase == PH_GATHER) {
     const cmma::Args c = conv_mma_args();
-    launch_ex(ctx, ABS_KC_CONV, cmma::conv_fwd_mma_kernel, dim3(L.rows_cap / cmma::FR), dim3(cmma::NT),
-              cmma::fwd_layout(c.k, c.b[0], c.b[1]).total, c);
+    launch_ex(ctx, ABS_KC_CONV, c.k == 5 ? cmma::conv_fwd_mma_kernel<5> : c.k == 3 ? cmma::conv_fwd_mma_kernel<3> : cmma::conv_fwd_mma_kernel<0>, dim3(L.rows_cap / cmma::FR), dim3(cmma::NT),
+              c.fl.total, c);
     return;
   }
   if (L.conv_mma && phase == PH_BACKWARD) {
     const cmma::Args c = conv_mma_args();
-    launch_ex(ctx, ABS_KC_CONV, cmma::conv_bwd_mma_kernel, dim3(L.rows_cap / cmma::FR), dim3(cmma::NT),
-              cmma::bwd_layout(c.k, c.b[0], c.b[1]).total, c);
+    launch_ex(ctx, ABS_KC_CONV, c.k == 5 ? cmma::conv_bwd_mma_kernel<5> : c.k == 3 ? cmma::conv_bwd_mma_kernel<3> : cmma::conv_bwd_mma_kernel<0>, dim3(L.rows_cap / cmma::FR), dim3(cmma::NT),
+              c.bl.total, c);
     return;
   }
   if (phase == PH_GATHER && L.cnn) {
@@ -978,6 +1001,7 @@ void enqueue_update(abs_ctx* ctx, int par) {
       G.part = ctx->at<float>(L.cpart[b]); G.len = (int)L.c_len[b]; G.chunk_rows = L.cchunk; G.off = L.c_off[b]; G.first_block = blocks;
       blocks += (G.len + 31) / 32;
     }
+    if (L.conv_mma) q.frag = frag_map(ctx);
     ctx->next_cluster = q.Q;
     launch_ex(ctx, ABS_KC_UPDATE, rnet::grad_step_kernel<T>, dim3(q.first_tile[nl] * q.Q + round_up(blocks, q.Q)), dim3(256), 0, q);
     return;
@@ -1290,8 +1314,9 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_wgrad_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_dgrad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_dgrad_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (ec == cudaSuccess && L.conv_mma) ec = cudaFuncSetAttribute(cmma::conv_fwd_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);
-    if (ec == cudaSuccess && L.conv_mma) ec = cudaFuncSetAttribute(cmma::conv_bwd_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);
+    for (auto fn : {cmma::conv_fwd_mma_kernel<0>, cmma::conv_fwd_mma_kernel<3>, cmma::conv_fwd_mma_kernel<5>, cmma::conv_bwd_mma_kernel<0>,
+                    cmma::conv_bwd_mma_kernel<3>, cmma::conv_bwd_mma_kernel<5>})
+      if (ec == cudaSuccess && L.conv_mma) ec = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);
     if (ec != cudaSuccess) return bail(cuda_fail(nullptr, ec, "cudaFuncSetAttribute(conv_block kernels)"));
   }
   if (!(model->flags & ABS_FLAG_NO_OVERLAP) && L.any_tc && !L.local_net && !L.cnn) {
@@ -1305,6 +1330,17 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
   if (model->dtype == ABS_FP32) ring_init_kernel<float><<<148, 256, 0, s>>>(ctx->at<float>(L.master), ctx->at<void>(L.ring), L.d_pad);
   else ring_init_kernel<__nv_bfloat16><<<148, 256, 0, s>>>(ctx->at<float>(L.master), ctx->at<void>(L.ring), L.d_pad);
   ctx->launches += 2;
+  if (L.conv_mma) {
+    cmma::Block cb[2];
+    conv_blocks(L, cb);
+    const cmma::BwdLayout bl = cmma::bwd_layout(L.ck, cb[0], cb[1]);
+    std::vector<int> tab(cmma::table_words(bl));
+    cmma::fill_tables(tab.data(), L.ck, cb[0], cb[1], bl);
+    e = cudaMemcpyAsync(ctx->at<int>(L.conv_tab), tab.data(), 4 * tab.size(), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return bail(cuda_fail(nullptr, e, "convolution tables"));
+    cmma::frag_init_kernel<<<16, 256, 0, s>>>(frag_map(ctx), ctx->at<float>(L.master));
+    ctx->launches += 1;
+  }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return bail(cuda_fail(nullptr, e, "set-up kernels"));

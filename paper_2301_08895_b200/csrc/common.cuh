@@ -108,6 +108,15 @@ __device__ __forceinline__ float ldf(const __nv_bfloat16* p, size_t i) { return 
 __device__ __forceinline__ void stf(float* p, size_t i, float v) { p[i] = v; }
 __device__ __forceinline__ void stf(__nv_bfloat16* p, size_t i, float v) { p[i] = __float2bfloat16_rn(v); }
 
+// x / n for x < 2^31 / n (items of a loop), by a multiplication: an integer division costs a few hundred
+// cycles otherwise
+struct FastDiv {
+  uint32_t m;
+  FastDiv() = default;
+  __host__ __device__ __forceinline__ explicit FastDiv(int n) : m(n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u) {}
+  __device__ __forceinline__ int div(int x) const { return m ? (int)__umulhi((uint32_t)x, m) : x; }
+};
+
 // First statement of every kernel of the round loop.  The kernels are launched with programmatic
 // stream serialization, so a kernel's CTAs may be resident before the kernel in front of it has
 // finished: wait until that kernel has completed (its writes are then visible), then allow the

@@ -273,13 +273,6 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
-// x / n for x < 2^31 / n (items and rows of a step), by a multiplication: an integer division costs a few hundred
-// cycles of every phase otherwise
-struct FastDiv {
-  uint32_t m;
-  __device__ __forceinline__ explicit FastDiv(int n) : m(n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u) {}
-  __device__ __forceinline__ int div(int x) const { return m ? (int)__umulhi((uint32_t)x, m) : x; }
-};
 __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;" ::"n"(CL_NT) : "memory"); }
 __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 

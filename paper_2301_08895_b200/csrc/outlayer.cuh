@@ -37,6 +37,17 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
                : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
+// d += a * b with the addition to d rounded to nearest: the instruction itself truncates where it adds to a large
+// accumulator, and stored (rounded) activations turn such errors into flipped ReLU / max-pool decisions.  It also leaves
+// consecutive products independent of one another.
+__device__ __forceinline__ void mma16816_rn(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  float p[4];
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+               : "=f"(p[0]), "=f"(p[1]), "=f"(p[2]), "=f"(p[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) d[i] += p[i];
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);

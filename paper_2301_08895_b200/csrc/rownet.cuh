@@ -14,6 +14,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "convmma.cuh"
 #include "lsqpipe.cuh"
 #include "narrow.cuh"
 #include "outlayer.cuh"
@@ -566,13 +567,30 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
           for (int c = 0; c < TP; ++c) wp[c] = w + 2 * t * out + min((ct0 + c * NWM) * 8 + g, out - 1);
           const int step = 16 * out;
           int k = 0;
-#pragma unroll 4
+          for (; k + 64 <= nk; k += 64) {             // four inner steps: their row operands first
+            uint32_t af[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) outl::ldsm4(a_base + (uint32_t)(k0 + k + 16 * u) * 2u, af[u]);
+#pragma unroll
+            for (int c = 0; c < TP; ++c)
+              if (c < n_here) {
+                uint32_t b[4][2];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  b[u][0] = pair16(wp[c] + u * step, out);
+                  b[u][1] = pair16(wp[c] + u * step + 8 * out, out);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) outl::mma16816_rn(acc[pass * TP + c], af[u], b[u][0], b[u][1]);
+                wp[c] += 4 * step;
+              }
+          }
           for (; k + 16 <= nk; k += 16) {
             uint32_t af[4];
             outl::ldsm4(a_base + (uint32_t)(k0 + k) * 2u, af);
 #pragma unroll
             for (int c = 0; c < TP; ++c) {
-              if (c < n_here) outl::mma16816(acc[pass * TP + c], af, pair16(wp[c], out), pair16(wp[c] + 8 * out, out));
+              if (c < n_here) outl::mma16816_rn(acc[pass * TP + c], af, pair16(wp[c], out), pair16(wp[c] + 8 * out, out));
               wp[c] += step;
             }
           }
@@ -586,7 +604,7 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
             for (int c = 0; c < TP; ++c)
               if (c < n_here) {
                 const T* q = wp[c] - 2 * t * out;
-                outl::mma16816(acc[pass * TP + c], af, pair16(q + ka * out, (kb - ka) * out), pair16(q + kc * out, (kd - kc) * out));
+                outl::mma16816_rn(acc[pass * TP + c], af, pair16(q + ka * out, (kb - ka) * out), pair16(q + kc * out, (kd - kc) * out));
               }
           }
         }
@@ -725,6 +743,7 @@ struct StepArgs {
   // parts of the gradient left as per-chunk partial sums (the CNN's convolution blocks): blocks behind the tiles
   struct Region { const float* part; int len, chunk_rows; size_t off; int first_block; } region[2];
   int n_regions;
+  cmma::FragMap frag;                    // region i = convolution block i: the weights also as operand fragments
 };
 
 __device__ __forceinline__ float ld_cluster(const float* p, int rank) {
@@ -772,6 +791,7 @@ __global__ void __launch_bounds__(256) grad_step_kernel(const __grid_constant__ 
       const float m = fmaf(-step, tot, a.master[e]);
       a.master[e] = m;
       stf(dst, e, m);
+      if (sizeof(T) == 2 && a.frag.frag != nullptr) cmma::frag_store(a.frag, slot, q, j, __float2bfloat16_rn(m));
     }
     return;
   }

@@ -52,6 +52,19 @@ def test_cnn_matches_oracle(conv, fc, dtype, W, B, rounds, tol):
     assert rows[-1]["loss_mean"] < rows[0]["loss_mean"]
 
 
+@pytest.mark.parametrize("conv,fc,W,B", [
+    ((16, 16, 1, 5, 5, 15), (20, 10), 7, 9),          # one input channel, odd channel counts, 2 x 2 final maps of one pixel
+    ((14, 18, 3, 3, 7, 9), (30, 21, 10), 6, 11),      # non-square, more than eight channels in the second block
+    ((15, 15, 3, 2, 4, 8), (16, 5), 5, 8),            # even kernel: odd image width, generic kernel size
+    ((24, 24, 3, 5, 8, 16), (40, 12, 10), 4, 33),     # most channels of the tensor-core path
+    ((16, 16, 4, 5, 6, 8), (12, 10), 4, 8),           # 100 taps: too many for it
+])
+def test_cnn_tensor_core_shapes(conv, fc, W, B):
+    cfg = _cnn_cfg(conv, fc, inputs.BF16, W, B, 3, 5, GAMMA3)
+    X, y, w0 = _problem(cfg)
+    compare_with_oracle(cfg, X, y, w0, 8, TOL_BF16, forced=True, loss_tol=5e-2)
+
+
 @pytest.mark.parametrize("conv,fc,W,B", [((14, 14, 2, 3, 3, 4), (7, 6, 5), 6, 10),
                                           ((32, 32, 3, 5, 6, 16), (120, 84, 10), 8, 32)])
 def test_cnn_gradient_of_one_round_block_by_block(conv, fc, W, B):
