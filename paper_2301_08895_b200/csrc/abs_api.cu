@@ -76,8 +76,8 @@ struct Layout {
   size_t d = 0, d_pad = 0;
   size_t w_off[ABS_MAX_LAYERS] = {};    // element offset of W_l inside the padded vector
   size_t w_src[ABS_MAX_LAYERS] = {};    // element offset of W_l inside the caller's vector
-  size_t st, ri, c, version, job, next_dur, dur_job, loss, row_loss;
-  size_t sel[2], sel_tau[2], sel_row0[2], row_idx[2], tile_slot[2];   // per-round layout, by round parity
+  size_t st, ri, c, version, job, next_dur, dur_job, shard, loss, row_loss;
+  size_t sel[2], sel_tau[2], sel_row0[2], row_idx[2], tile_slot[2], tile_real[2];   // per-round layout, by round parity
   size_t act0b;                         // second copy of the gathered input rows (odd rounds)
   size_t master, ring, G, logits, red, ones;
   // convolution blocks of ABS_CNN (two of them, in front of the affine layers)
@@ -321,12 +321,14 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   L->job = cv.take(4 * W);
   L->next_dur = cv.take(8 * W);
   L->dur_job = cv.take(4 * W);
+  L->shard = cv.take(8 * W);
   for (int q = 0; q < 2; ++q) {
     L->sel[q] = cv.take(4 * W);
     L->sel_tau[q] = cv.take(4 * W);
     L->sel_row0[q] = cv.take(4 * W);
     L->row_idx[q] = cv.take(4 * (size_t)L->rows_cap);
     L->tile_slot[q] = cv.take(4 * (size_t)L->n_tiles_cap);
+    L->tile_real[q] = cv.take(4 * (size_t)L->n_tiles_cap);
   }
   L->loss = cv.take(4 * W);
   L->row_loss = cv.take(4 * (size_t)L->rows_cap);
@@ -692,6 +694,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     if (ctx->lsq_pipe) {
       lsqp::Args q;
       q.st = st; q.ri = ri; q.sel = a.sel; q.job = a.job; q.sel_tau = a.sel_tau;
+      q.shard = ctx->ctl.shard; q.next_dur = ctx->ctl.next_dur; q.dur_job = ctx->ctl.dur_job;
       q.X = (const __nv_bfloat16*)ctx->X; q.y = a.y; q.ring = (const __nv_bfloat16*)a.ring; q.slot_stride = a.slot_stride;
       q.loss_part = ctx->at<float>(L.row_loss); q.G = a.G; q.d = a.d; q.stages = ctx->lsq_stages;
       q.groups = (m.batch + lsqp::GROUP - 1) / lsqp::GROUP;
@@ -798,7 +801,13 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     return;
   }
   if (phase == PH_GATHER) {
-    if (gathered)
+    if (gathered && !ctx->ctl.draw) {
+      DrawArgs q;
+      q.st = st; q.ri = ri; q.sel = ctx->ctl.sel[par]; q.sel_row0 = ctx->ctl.sel_row0[par]; q.job = ctx->ctl.job; q.shard = ctx->ctl.shard;
+      q.row_idx = ctx->ctl.row_idx[par]; q.by_B = FastDiv(m.batch); q.tile_real = ctx->ctl.tile_real[par]; q.RB = L.RB;
+      launch_on(ctx, ctx->overlap ? ctx->side : s, ABS_KC_GATHER, draw_gather_kernel, dim3(ctx->sm_count * 8), dim3(256), 0, q,
+                (const __nv_bfloat16*)ctx->X, ctx->at<__nv_bfloat16>(par ? L.act0b : L.act[0]), m.dims[0]);
+    } else if (gathered)
       launch_on(ctx, ctx->overlap ? ctx->side : s, ABS_KC_GATHER, gather_rows_kernel, dim3(ctx->sm_count * 8), dim3(256), 0,
                 st, ri, ctx->ctl.row_idx[par], (const __nv_bfloat16*)ctx->X, ctx->at<__nv_bfloat16>(par ? L.act0b : L.act[0]), m.dims[0]);
     return;
@@ -810,6 +819,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     a.ring = ctx->at<void>(L.ring); a.slot_stride = L.d_pad;
     a.X = L.cnn ? ctx->at<void>(par ? L.act0b : L.act[0]) : ctx->X;
     a.gather = L.cnn ? 0 : 1;
+    a.job = ctx->ctl.job; a.next_dur = ctx->ctl.next_dur; a.dur_job = ctx->ctl.dur_job; a.W = ctx->W;
     a.n_layers = nl; a.want_d0 = L.cnn ? 1 : 0; a.row_loss = ctx->ctl.row_loss;
     for (int l = 0; l <= nl; ++l) {
       a.dims[l] = m.dims[l];
@@ -1189,9 +1199,13 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
   for (int q = 0; q < 2; ++q) {
     c.sel[q] = ctx->at<int>(L.sel[q]); c.sel_tau[q] = ctx->at<int>(L.sel_tau[q]); c.sel_row0[q] = ctx->at<int>(L.sel_row0[q]);
     c.row_idx[q] = ctx->at<int>(L.row_idx[q]); c.tile_slot[q] = ctx->at<int>(L.tile_slot[q]);
+    c.tile_real[q] = ctx->at<int>(L.tile_real[q]);
   }
   c.loss = ctx->at<float>(L.loss);
   c.loss_part = nullptr; c.loss_groups = 0;
+  c.shard = ctx->at<int2>(L.shard);
+  c.by_blk = FastDiv((model->batch + 3) / 4);
+  c.draw = L.any_tc && !L.cnn && !L.local_net && L.path[0] == PATH_TC ? 0 : 1;      // drawn by draw_gather_kernel
   // with local steps a worker's loss is uploaded whole (no per-row losses, no row layout)
   c.row_loss = (model->kind == ABS_LSQ || model->local_steps > 1) ? nullptr : ctx->at<float>(L.row_loss);
   c.tr_K = ctx->at<int>(L.tr_K); c.tr_R = ctx->at<int>(L.tr_R); c.tr_theta = ctx->at<int>(L.tr_theta);
@@ -1448,17 +1462,19 @@ int abs_enqueue_rounds(abs_ctx* ctx, int n) {
     // launch: it starts once every block of the Eq. 3 kernel has passed its own wait, i.e. once the
     // gradient kernels of round t are complete), runs next to it, prepares the next job durations
     // itself and waits for the Eq. 3 kernel at its end.  The first control step of a call follows
-    // something else and waits at its start.
+    // something else and waits at its start.  (The gradient kernels that prepare the durations instead: row kernels and
+    // least-squares pipeline.)
+    const int look = ctx->L.row_R || ctx->lsq_pipe ? 0 : 1;
     for (int r = 0; r < n; ++r) {
       const int t = ctx->rounds_enqueued + r, par = t & 1;
       // the control kernel completes the previous round (if any) and selects this round's arrivals
-      launch_ex(ctx, ABS_KC_CTL, ctl_kernel, dim3(1), dim3(ctl_threads), csm, ctx->ctl, 1, 1, t, r > 0 ? 1 : 0, 1);
+      launch_ex(ctx, ABS_KC_CTL, ctl_kernel, dim3(1), dim3(ctl_threads), csm, ctx->ctl, 1, 1, t, r > 0 ? 1 : 0, look);
       gradient(par, PH_GATHER);
       gradient(par, PH_FORWARD);
       gradient(par, PH_BACKWARD);
       update(par);
     }
-    launch_ex(ctx, ABS_KC_CTL, ctl_kernel, dim3(1), dim3(ctl_threads), csm, ctx->ctl, 1, 0, ctx->rounds_enqueued + n, 1, 1);
+    launch_ex(ctx, ABS_KC_CTL, ctl_kernel, dim3(1), dim3(ctl_threads), csm, ctx->ctl, 1, 0, ctx->rounds_enqueued + n, 1, look);
   } else if (n > 0) {
     // Two streams.  Side stream per round t: control kernel (finish t-1, select t), row gather,
     // [event ctl], duration look-ahead.  Main stream: wait ctl, forward kernels, [event loss],

@@ -78,6 +78,15 @@ struct RoundInfo {
 };
 constexpr int RI_TIMEOUT = 2;
 
+// x / n for x < 2^31 / n (items of a loop), by a multiplication: an integer division costs a few hundred
+// cycles otherwise
+struct FastDiv {
+  uint32_t m;
+  FastDiv() = default;
+  __host__ __device__ __forceinline__ explicit FastDiv(int n) : m(n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u) {}
+  __device__ __forceinline__ int div(int x) const { return m ? (int)__umulhi((uint32_t)x, m) : x; }
+};
+
 // Pointers the control kernel works on (all device memory inside the workspace).
 struct CtlArgs {
   DevState* st;
@@ -93,8 +102,12 @@ struct CtlArgs {
   float* row_loss;     // [rows_cap] per-sample losses (network models), else null
   int* row_idx[2];     // [rows_cap] sample index of each gradient row, -1 for padding
   int* tile_slot[2];   // [rows_cap / RB] ring slot of each row tile
+  int* tile_real[2];   // [rows_cap / RB] rows of the tile that are not padding (they come first)
   u64* next_dur;       // [W] duration of the job each worker starts next, computed ahead of time
   int* dur_job;        // [W] job index next_dur[n] belongs to
+  int2* shard;         // [W] first sample and length of each worker's shard [n M / N, (n+1) M / N)
+  FastDiv by_blk;      // Philox blocks per minibatch, ceil(B / 4)
+  int draw;            // 1: the step draws the sample indices of the rows itself (0: the gather kernel does)
   const float* loss_part;  // least-squares pipeline: per (selected worker, row group) sums of 1/2 r^2, or null;
   int loss_groups;         // the upload's loss is their sum over the groups divided by B
   // trace
@@ -107,15 +120,6 @@ __device__ __forceinline__ float ldf(const float* p, size_t i) { return p[i]; }
 __device__ __forceinline__ float ldf(const __nv_bfloat16* p, size_t i) { return __bfloat162float(p[i]); }
 __device__ __forceinline__ void stf(float* p, size_t i, float v) { p[i] = v; }
 __device__ __forceinline__ void stf(__nv_bfloat16* p, size_t i, float v) { p[i] = __float2bfloat16_rn(v); }
-
-// x / n for x < 2^31 / n (items of a loop), by a multiplication: an integer division costs a few hundred
-// cycles otherwise
-struct FastDiv {
-  uint32_t m;
-  FastDiv() = default;
-  __host__ __device__ __forceinline__ explicit FastDiv(int n) : m(n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u) {}
-  __device__ __forceinline__ int div(int x) const { return m ? (int)__umulhi((uint32_t)x, m) : x; }
-};
 
 // First statement of every kernel of the round loop.  The kernels are launched with programmatic
 // stream serialization, so a kernel's CTAs may be resident before the kernel in front of it has

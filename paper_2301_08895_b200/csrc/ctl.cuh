@@ -88,11 +88,12 @@ __device__ __forceinline__ void refresh_next_durations(const DevState* st, const
 }
 
 // ---------------------------------------------------------------------------------------------
-// Sort of up to 1024 distinct 64-bit keys, one per thread, by ranking: inside a warp every key
-// counts the smaller keys of its warp (31 shuffles, no dependent chain); sorted runs are then
-// merged pairwise, each key finding its place in the sibling run by binary search.  All steps
-// are short and independent per thread, which matters because one CTA does this alone.
-// Returns the buffer (A or B) that holds the sorted keys.
+// Sort of up to 1024 distinct 64-bit keys, one per thread, by ranking: inside a warp every key counts the smaller keys
+// of its warp (31 shuffles, no dependent chain), which leaves sorted runs of 32.  Up to eight runs are merged at once:
+// a key's place is the number of smaller keys in every other run, found by binary searches that run side by side (256
+// keys: 1.5k cycles instead of 3.1k with pairwise merges); more runs are merged pairwise, where one search per key and
+// level is less shared-memory traffic.  Returns the buffer (A or B) that holds the sorted keys.
+template <int NT>
 __device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n_pow2) {
   const int tid = threadIdx.x, lane = tid & 31;
   const bool active = tid < n_pow2;            // whole warps: n_pow2 is a multiple of 32
@@ -103,6 +104,28 @@ __device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n_p
     A[(tid - lane) + rank] = key;
   }
   __syncthreads();
+  if (n_pow2 == 32) return A;
+  if (NT <= 512 && n_pow2 <= 256) {
+    if (active) {
+      const u64 k = A[tid];
+      const int own = tid >> 5, runs = n_pow2 >> 5;
+      int lo[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) lo[r] = 0;
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1)
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          if (r < runs) lo[r] += A[r * 32 + lo[r] + step - 1] < k ? step : 0;     // at most 31 of a run after the last step
+      int rank = 0;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < runs) rank += r == own ? lane : lo[r] + (A[r * 32 + lo[r]] < k ? 1 : 0);
+      B[rank] = k;
+    }
+    __syncthreads();
+    return B;
+  }
   u64* src = A;
   u64* dst = B;
   for (int L = 32; L < n_pow2; L <<= 1) {
@@ -125,10 +148,9 @@ __device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n_p
   return src;
 }
 
-__device__ __forceinline__ i64 floor_div(i64 a, i64 b) {  // b > 0
-  i64 q = a / b;
-  if ((a % b != 0) && (a < 0)) --q;
-  return q;
+__device__ __forceinline__ int floor_div(int a, int b) {  // b > 0
+  const int q = a / b;
+  return (a % b != 0 && a < 0) ? q - 1 : q;
 }
 
 struct CtlShared {
@@ -141,8 +163,7 @@ struct CtlShared {
   float lossv[1024];                   // mean minibatch loss of each selected worker
   int version[1024], job[1024];        // per-worker state after the round's bookkeeping
   int sel_n[1024];                     // worker id of each arrival, in arrival order
-  int shard_lo[1024];
-  unsigned shard_len[1024];
+  int2 shard[1024];                    // per worker: first sample and length of its shard
   float redf[32];
   int warp_tot[32];
   int scalar[8];
@@ -158,7 +179,7 @@ struct CtlShared {
 //              t_sel - 1 / t_sel picks the layout copy of the open / the new round)
 //   look_here: the workers that were renewed also get the duration of the job AFTER the one they
 //              start now prepared here, at the end of the step (see refresh_next_durations), for
-//              callers that have no other kernel between two control steps to do it
+//              callers whose gradient kernel does not do it (2000 cycles of binary64 series)
 //   late_status: when the step runs next to the Eq. 3 kernel of the round it finishes, a status it
 //              raises must not be seen by that kernel's blocks (they would skip a valid step):
 //              the status is left in *late_status (shared memory) for the caller to publish later
@@ -174,12 +195,19 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
   // ---- one wave of loads
   const int W = st->W, S = st->S, B = st->B, RB = st->RB, K0 = st->K0;
   const int po = (t_sel - 1) & 1, pn = t_sel & 1;     // layout copy of the open / of the new round
+  // (everything a later phase may need: all addresses exist whether or not a round is open)
+  int my_sel = 0, my_tau = 0, my_row0 = 0;
+  float my_loss = 0.f;
+  int2 my_shard = make_int2(0, 0);
+  if (tid < W) {
+    my_sel = a.sel[po][tid]; my_tau = a.sel_tau[po][tid]; my_row0 = a.sel_row0[po][tid];
+    my_shard = a.shard[tid];
+  }
   const int status0 = st->status, open0 = st->open, diverged0 = a.ri[po].diverged;
   const int k_mode = st->k_mode, bound_mode = st->bound_mode, max_rounds = st->max_rounds;
   const int bound_offset = st->bound_offset, Scap = st->theta_cap, literal = st->literal_eq6;
   const int no_restart = st->no_restart;
   const uint32_t key0 = st->key0, key1 = st->key1;
-  const i64 n_samples = st->n_samples;
   const u64 T_end0 = st->T_end;
   const float L0_prev = st->L0;
   const i64 sel_off = st->sel_total, rst_off = st->rst_total;
@@ -194,10 +222,7 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     my_c = a.c[tid]; my_version = a.version[tid]; my_job = a.job[tid];
     my_dur_job = a.dur_job[tid]; my_next_dur = a.next_dur[tid];
   }
-  int my_sel = 0, my_tau = 0, my_row0 = 0;
-  float my_loss = 0.f;
   if (fin && tid < K) {
-    my_sel = a.sel[po][tid]; my_tau = a.sel_tau[po][tid]; my_row0 = a.sel_row0[po][tid];
     if (!net && a.loss_part == nullptr) my_loss = a.loss[tid];
     if (!net && a.loss_part != nullptr) {
       // the least-squares pipeline leaves per-group sums; same order and rounding as its Eq. 3 kernel
@@ -225,7 +250,7 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
       float acc = 0.f;
       if (i < K) {
         const float* rl = a.row_loss + sh.row0[i];
-#pragma unroll 8
+#pragma unroll 16
         for (int b = sub; b < B; b += tpw) acc += rl[b];
       }
       for (int o = tpw >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -283,11 +308,8 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     // Eq. 4 with a = S - N/K0, in integers
     int theta = Scap;
     if (bound_mode == ABS_BOUND_ADAPTIVE) {
-      const i64 fl = floor_div((i64)W * (i64)(K0 - K_next), (i64)K_next * (i64)K0);
-      i64 th = (i64)Scap + fl;
-      if (th < 1) th = 1;
-      if (th > Scap) th = Scap;
-      theta = (int)th;
+      // (32-bit: at most 1024 workers)
+      theta = min(Scap, max(1, Scap + floor_div(W * (K0 - K_next), K_next * K0)));
     } else if (bound_mode == ABS_BOUND_OFFSET) {     // Eq. 4 with a given: floor(N/K + a) = floor(N/K) + a
       int th = W / K_next + bound_offset;
       if (th < 1) th = 1;
@@ -359,13 +381,14 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
   {
     sh.version[tid] = my_version;
     sh.job[tid] = my_job;
-    if (net) for (int i = tid; i < 32 * MAX_TAU; i += NT) (&sh.wcnt[0][0])[i] = 0;
+    sh.shard[tid] = my_shard;
+    if (net) for (int u = lane; u <= S; u += 32) sh.wcnt[warp][u] = 0;
     // arrivals: the K smallest (completion tick, worker id) keys; unused slots get distinct
     // keys above every real one
     int n_pow2 = 32;
     while (n_pow2 < W) n_pow2 <<= 1;
     const u64 key_in = (tid < W) ? ((my_c << 10) | (u64)tid) : (0xFFFFFFFFFFFFFC00ull | (u64)tid);
-    const u64* sorted = rank_merge_sort(key_in, sh.keysA, sh.keysB, n_pow2);
+    const u64* sorted = rank_merge_sort<NT>(key_in, sh.keysA, sh.keysB, n_pow2);
     const u64 T_end = sorted[K - 1] >> 10;
     int n = -1, tau = -1;
     if (tid < K) {
@@ -388,20 +411,25 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
       const int rank_in_warp = __popc(peers & ((1u << lane) - 1u));
       if (tau >= 0 && rank_in_warp == 0) sh.wcnt[warp][tau] = (unsigned short)__popc(peers);
       __syncthreads();
-      if (tid <= S) {
-        int c = 0;
-        for (int w = 0; w < 32; ++w) { const int x = sh.wcnt[w][tid]; sh.wcnt[w][tid] = (unsigned short)c; c += x; }
-        sh.cnt[tid] = c;
-      }
-      __syncthreads();
-      if (tid <= S) {
-        int r0 = 0, g = 0;
-        for (int q = 0; q < tid; ++q) { r0 += round_up(sh.cnt[q] * B, RB); g += sh.cnt[q] > 0; }
-        sh.grow0[tid] = r0;
-        if (tid == S) {
-          sh.scalar[0] = r0 + round_up(sh.cnt[S] * B, RB);
-          sh.scalar[1] = g + (sh.cnt[S] > 0);
+      if (warp == 0) {
+        // per staleness u: exclusive sums over the warps, then first rows by a scan over u (RB is a power of two)
+        int carry = 0, groups = 0;
+        for (int u0 = 0; u0 <= S; u0 += 32) {
+          const int u = u0 + lane;
+          int c = 0;
+          if (u <= S) {
+#pragma unroll
+            for (int w = 0; w < NT / 32; ++w) { const int x = sh.wcnt[w][u]; sh.wcnt[w][u] = (unsigned short)c; c += x; }
+          }
+          const int rows = (c * B + RB - 1) & ~(RB - 1);
+          int sum = rows;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, sum, o); if (lane >= o) sum += v; }
+          if (u <= S) { sh.cnt[u] = c; sh.grow0[u] = carry + sum - rows; }
+          carry += __shfl_sync(0xffffffffu, sum, 31);
+          groups += __popc(__ballot_sync(0xffffffffu, c > 0));
         }
+        if (lane == 0) { sh.scalar[0] = carry; sh.scalar[1] = groups; }
       }
       __syncthreads();
       if (tid < K) row0_me = sh.grow0[tau] + ((int)sh.wcnt[warp][tau] + rank_in_warp) * B;
@@ -416,16 +444,11 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
       sh.row0[tid] = row0;
       sh.sel_n[tid] = n;
       sh.flag[tid] = 0;
-      if (net) {
-        const i64 lo = ((i64)n * n_samples) / W, hi = ((i64)(n + 1) * n_samples) / W;
-        sh.shard_lo[tid] = (int)lo;
-        sh.shard_len[tid] = (unsigned)(hi - lo);
-      }
     }
     if (tid == 0) {
       st->T_end = T_end;
       st->n_rows = n_rows;
-      st->n_row_tiles = n_rows / RB;
+      st->n_row_tiles = net ? n_rows >> (__ffs(RB) - 1) : K;
       st->n_groups = n_groups;
       st->open = 1;
       RoundInfo info;
@@ -435,36 +458,37 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     }
     if (!net) return 0;           // least squares: no row tiles, minibatches drawn by its own kernel
     __syncthreads();
-    // ring slot of every row tile and padding rows
+    // ring slot of every row tile and padding rows, one warp per staleness group
     {
-      const int n_tiles = n_rows / RB;
-      for (int q = tid; q < n_tiles; q += NT) {
-        const int r = q * RB;
-        int g = 0;                                  // last non-empty group starting at or before r
-        for (int u = 0; u <= S; ++u) if (sh.cnt[u] > 0 && sh.grow0[u] <= r) g = u;
-        a.tile_slot[pn][q] = (t - g) % (S + 1);
-      }
-      for (int g = 0; g <= S; ++g) {
+      const int sh_rb = __ffs(RB) - 1, tm = t % (S + 1);
+      for (int g = warp; g <= S; g += NT / 32) {
         const int c = sh.cnt[g];
         if (c == 0) continue;
-        const int p0 = sh.grow0[g] + c * B, p1 = sh.grow0[g] + round_up(c * B, RB);
-        for (int r = p0 + tid; r < p1; r += NT) a.row_idx[pn][r] = -1;
+        const int r0 = sh.grow0[g], p0 = r0 + c * B, p1 = r0 + ((c * B + RB - 1) & ~(RB - 1));
+        const int slot = tm - g < 0 ? tm - g + S + 1 : tm - g;      // (t - g) mod (S + 1); g <= S
+        for (int q = (r0 >> sh_rb) + lane; q < (p1 >> sh_rb); q += 32) {
+          a.tile_slot[pn][q] = slot;
+          a.tile_real[pn][q] = min(RB, p0 - (q << sh_rb));
+        }
+        for (int r = p0 + lane; r < p1; r += 32) a.row_idx[pn][r] = -1;
       }
     }
+    if (!a.draw) return 0;
     // minibatch draws: sample b of job (n, j) = word b%4 of Philox block (n, j, 1, b/4),
     // mapped into the worker's shard [n M / N, (n+1) M / N)
     const int blocks_per = (B + 3) >> 2;
+#pragma unroll 2
     for (int item = tid; item < K * blocks_per; item += NT) {
-      const int i = item / blocks_per, blk = item - i * blocks_per;
+      const int i = a.by_blk.div(item), blk = item - i * blocks_per;
       const int wn = (int)(sorted[i] & 1023ull);
       uint32_t w4[4];
       philox4x32_10((uint32_t)wn, (uint32_t)sh.job[wn], 1u, (uint32_t)blk, key0, key1, w4);
-      const int lo = sh.shard_lo[i], row0 = sh.row0[i];
-      const u64 len = (u64)sh.shard_len[i];
+      const int2 shard = sh.shard[wn];
+      const int row0 = sh.row0[i];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int b = blk * 4 + q;
-        if (b < B) a.row_idx[pn][row0 + b] = lo + (int)(((u64)w4[q] * len) >> 32);
+        if (b < B) a.row_idx[pn][row0 + b] = shard.x + (int)__umulhi(w4[q], (unsigned)shard.y);
       }
     }
   }
@@ -521,6 +545,8 @@ __global__ void abs_init_state_kernel(CtlArgs a) {
   if (tid < st->W) {
     const u64 dt = job_ticks(st->dist, st->key0, st->key1, tid, 0);
     if (dt == 0ull) st->status = ST_RANGE;
+    const i64 M = st->n_samples, lo = ((i64)tid * M) / st->W, hi = ((i64)(tid + 1) * M) / st->W;
+    a.shard[tid] = make_int2((int)lo, (int)(hi - lo));
     a.c[tid] = dt;
     a.version[tid] = 0;
     a.job[tid] = 0;

@@ -36,6 +36,8 @@ struct Args {
   DevState* st;
   RoundInfo* ri;
   const int* sel; const int* job; const int* sel_tau;
+  const int2* shard;
+  u64* next_dur; int* dur_job;           // duration look-ahead (see refresh_next_durations)
   const __nv_bfloat16* X; const float* y;
   const __nv_bfloat16* ring; size_t slot_stride;
   float* loss_part;     // [K * groups] sum over the item's rows of 1/2 r_b^2
@@ -86,7 +88,7 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(Args a) {
   DevState* st = a.st;
   RoundInfo* ri = a.ri;
   if (st->status != ST_OK) return;
-  const int K = ri->K, B = st->B, d = a.d, W = st->W, S = st->S, t = ri->t;
+  const int K = ri->K, B = st->B, d = a.d, S = st->S, t = ri->t;
   const int groups = a.groups, n_items = K * groups;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nvec = d >> 3;
@@ -108,7 +110,6 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(Args a) {
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  const i64 M = st->n_samples;
   const uint32_t key0 = st->key0, key1 = st->key1;
   // items of this CTA: it = blockIdx.x + q * gridDim.x, q = 0 .. my_items - 1
   const int my_items = n_items > (int)blockIdx.x ? (n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
@@ -119,6 +120,13 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(Args a) {
   int stage = 0, buf = 0;
   uint32_t phase = 0;
   bool ok = true;
+  // the producer warp prepares job durations while the first stages are consumed: worker blockIdx.x + gridDim.x * lane
+  bool looked = warp != CONSUMERS / 32;
+  auto look = [&]() {
+    if (looked) return;
+    looked = true;
+    refresh_next_durations(st, a.job, a.next_dur, a.dur_job, (int)blockIdx.x + (int)gridDim.x * lane);
+  };
 
   for (int q0 = 0; q0 < my_items && ok; q0 += MAX_ITEMS) {
     const int nq = min(MAX_ITEMS, my_items - q0);
@@ -137,11 +145,11 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(Args a) {
       int idx = -1;
       float yv = 0.f;
       if (b < B) {
-        const i64 lo = ((i64)wn * M) / W, hi = ((i64)(wn + 1) * M) / W;
+        const int2 shard = a.shard[wn];
         uint32_t w4[4];
         philox4x32_10((uint32_t)wn, (uint32_t)a.job[wn], 1u, (uint32_t)(b >> 2), key0, key1, w4);
         const uint32_t wd = (b & 3) == 0 ? w4[0] : (b & 3) == 1 ? w4[1] : (b & 3) == 2 ? w4[2] : w4[3];
-        idx = (int)lo + (int)(((u64)wd * (u64)(hi - lo)) >> 32);
+        idx = shard.x + (int)__umulhi(wd, (unsigned)shard.y);
         yv = a.y[idx];
       }
       m_idx[e] = idx;
@@ -164,7 +172,9 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(Args a) {
         if (lane == GROUP)
           bulk_row(sb + (size_t)GROUP * row_bytes, a.ring + (size_t)m_slot[q] * a.slot_stride, row_bytes, &full[stage]);
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        if (q == STAGES - 1) look();
       }
+      if (ok) look();
     } else {
       // ------------------------------------------------------------------ consumers
       const int vec = tid;                           // the 16-byte column slice this thread owns
@@ -266,6 +276,7 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(Args a) {
     }
     ok = __syncthreads_and(ok ? 1 : 0) != 0;
   }
+  look();                                   // (a CTA without items)
   // the producer's copies have all been consumed (every full barrier was waited on), unless a wait
   // gave up: then let copies in flight land before the shared memory goes away
   if (!ok && tid == 0) {

@@ -11,32 +11,66 @@ namespace absb {
 constexpr int NARROW_MAX_C = 16;
 
 // act0[r][:] = X[row_idx[r]][:] (zeros for padding rows); bf16, `in` a multiple of 8.
+__device__ __forceinline__ void gather_row(__nv_bfloat16* act0, const __nv_bfloat16* X, int r, int s, int in, int lane) {
+  const int vec_per_row = in >> 3;
+  uint4* dst = reinterpret_cast<uint4*>(act0 + (size_t)r * in);
+  if (s < 0) {
+    for (int v = lane; v < vec_per_row; v += 32) dst[v] = make_uint4(0u, 0u, 0u, 0u);
+  } else {
+    // four 16-byte loads per lane in flight before the first store
+    const uint4* src = reinterpret_cast<const uint4*>(X + (size_t)s * in);
+    for (int v = lane; v < vec_per_row; v += 128) {
+      uint4 q[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (v + 32 * k < vec_per_row) q[k] = __ldg(src + v + 32 * k);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (v + 32 * k < vec_per_row) dst[v + 32 * k] = q[k];
+    }
+  }
+}
 __global__ void __launch_bounds__(256) gather_rows_kernel(const DevState* st, const RoundInfo* ri, const int* row_idx,
                                                           const __nv_bfloat16* X, __nv_bfloat16* act0, int in) {
   grid_dependency_sync();
   if (st->status != ST_OK) return;
   const int n_rows = ri->n_rows;
-  const int vec_per_row = in >> 3;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int r = blockIdx.x * 8 + warp; r < n_rows; r += gridDim.x * 8) {
-    const int s = row_idx[r];
-    uint4* dst = reinterpret_cast<uint4*>(act0 + (size_t)r * in);
-    if (s < 0) {
-      for (int v = lane; v < vec_per_row; v += 32) dst[v] = make_uint4(0u, 0u, 0u, 0u);
-    } else {
-      // four 16-byte loads per lane in flight before the first store
-      const uint4* src = reinterpret_cast<const uint4*>(X + (size_t)s * in);
-      for (int v = lane; v < vec_per_row; v += 128) {
-        uint4 q[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (v + 32 * k < vec_per_row) q[k] = __ldg(src + v + 32 * k);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (v + 32 * k < vec_per_row) dst[v + 32 * k] = q[k];
-      }
-    }
+  for (int r = blockIdx.x * 8 + warp; r < n_rows; r += gridDim.x * 8) gather_row(act0, X, r, row_idx[r], in, lane);
+}
+
+// The same for rounds of one local step, drawing the minibatches itself: sample b of job (n, j) = word b % 4 of Philox
+// block (n, j, 1, b / 4), mapped into the worker's shard.  A warp takes a (selected worker, row) pair, so the draws cost
+// a few hundred cycles here instead of a few thousand in the one-CTA control step in front (K = 128, B = 64: 7600).
+struct DrawArgs {
+  const DevState* st; const RoundInfo* ri;
+  const int* sel; const int* sel_row0; const int* job; const int2* shard;
+  int* row_idx;
+  const int* tile_real; int RB;
+  FastDiv by_B;
+};
+__global__ void __launch_bounds__(256) draw_gather_kernel(DrawArgs a, const __nv_bfloat16* X, __nv_bfloat16* act0, int in) {
+  grid_dependency_sync();
+  const int status = a.st->status, K = a.ri->K, B = a.st->B, n_rows = a.ri->n_rows;
+  const uint32_t key0 = a.st->key0, key1 = a.st->key1;
+  if (status != ST_OK) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w0 = blockIdx.x * 8 + warp, nw = gridDim.x * 8;
+  for (int it = w0; it < K * B; it += nw) {
+    const int i = a.by_B.div(it), b = it - i * B;
+    const int n = a.sel[i], r = a.sel_row0[i] + b;
+    const int2 shard = a.shard[n];
+    uint32_t w4[4];
+    philox4x32_10((uint32_t)n, (uint32_t)a.job[n], 1u, (uint32_t)(b >> 2), key0, key1, w4);
+    const uint32_t wd = (b & 3) == 0 ? w4[0] : (b & 3) == 1 ? w4[1] : (b & 3) == 2 ? w4[2] : w4[3];
+    const int s = shard.x + (int)__umulhi(wd, (unsigned)shard.y);
+    if (lane == 0) a.row_idx[r] = s;
+    gather_row(act0, X, r, s, in, lane);
   }
+  // padding rows (their sample index is already -1)
+  if (n_rows != K * B)
+    for (int r = w0; r < n_rows; r += nw)
+      if (r % a.RB >= a.tile_real[r / a.RB]) gather_row(act0, X, r, -1, in, lane);
 }
 
 struct NarrowArgs {

@@ -15,6 +15,7 @@
 
 #include "common.cuh"
 #include "convmma.cuh"
+#include "ctl.cuh"
 #include "lsqpipe.cuh"
 #include "narrow.cuh"
 #include "outlayer.cuh"
@@ -40,6 +41,7 @@ struct RowsArgs {
   const int* row_idx;                    // sample index per gradient row, -1: padding
   const int* labels;
   const void* ring; size_t slot_stride;
+  const int* job; u64* next_dur; int* dur_job; int W;    // duration look-ahead (see refresh_next_durations)
   const void* X; int gather;             // layer-0 input of row r: X[row_idx[r]] (gather) or X[r]
   void* act[ABS_MAX_LAYERS + 1];         // [rows][dims[l]] stored ReLU outputs, l = 1 .. n_layers - 1
   void* delta[ABS_MAX_LAYERS + 1];       // [rows][dims[l]] stored deltas, l = 1 .. n_layers; delta[0]: see want_d0
@@ -318,7 +320,13 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
   // one wave of loads (the grid covers the row capacity, so every address exists)
   const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[blockIdx.x];
   const int my_idx = a.row_idx[r0 + lane % R];       // sample index of row lane % R
-  if (status != ST_OK || r0 >= n_rows) return;
+  if (status != ST_OK) return;
+  // the fetching warps of the first CTAs also prepare job durations, off the critical path
+  const int look = (int)blockIdx.x * 32 < a.W ? (int)blockIdx.x * 32 + lane : a.W;
+  if (r0 >= n_rows) {
+    if (warp == NW) refresh_next_durations(st, a.job, a.next_dur, a.dur_job, look);
+    return;
+  }
   const int L = a.n_layers;
   const size_t w_bytes = a.resident ? (size_t)a.w_res[L - 1] + round_up((a.dims[L - 1] + 1) * a.dims[L] * 4, 128)
                                     : (size_t)a.stages * a.stage_bytes;
@@ -330,6 +338,7 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
   if (warp == NW) {
     if (lane == 0) W.produce((const float*)a.ring + (size_t)slot * a.slot_stride);
     __syncwarp();
+    refresh_next_durations(st, a.job, a.next_dur, a.dur_job, look);
   } else {
     // ------------------------------------------------------------------ input rows
     {
@@ -502,7 +511,12 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
   // one wave of loads (the grid covers the row capacity, so every address exists)
   const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[blockIdx.x];
   const int my_idx = a.row_idx[r0 + warp];           // warp w fetches row w
-  if (status != ST_OK || r0 >= n_rows) return;
+  if (status != ST_OK) return;
+  const int look = (int)blockIdx.x * 32 < a.W ? (int)blockIdx.x * 32 + lane : a.W;
+  if (r0 >= n_rows) {
+    if (warp == NWM) refresh_next_durations(st, a.job, a.next_dur, a.dur_job, look);
+    return;
+  }
   const int g = lane >> 2, t = lane & 3;
   const int L = a.n_layers;
   const size_t w_bytes = a.resident ? (size_t)a.w_res[L - 1] + round_up((a.dims[L - 1] + 1) * a.dims[L] * 2, 128)
@@ -538,6 +552,7 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
   if (warp == NWM) {
     if (!a.resident && lane == 0) W.produce(w_ring);
     __syncwarp();
+    refresh_next_durations(st, a.job, a.next_dur, a.dur_job, look);
   } else {
     const int sel_row = lane & 15, sel_col = (lane >> 4) * 8;         // ldmatrix addresses of an A tile
     // ------------------------------------------------------------------ forward: warp takes column tiles warp, warp + 15, ...
