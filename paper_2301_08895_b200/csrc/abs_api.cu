@@ -150,6 +150,67 @@ int check_model(const abs_model_desc* m, int W, int S) {
   return ABS_OK;
 }
 
+// Modelled time of a launch of `tiles` GEMM tiles of (128 cg) x bn with kb inner blocks of 64, in us: whole waves over the
+// SMs (or SM pairs).  Measured between two events (about 4 us more
+// than the kernel): 12 row tiles, 48 inner blocks, 1024 columns 36.5 / 27.0 / 37.5 us at 256 / 128 / 64; 16 blocks, 512
+// columns 25.1 / 14.9 / 16.9; 81 row tiles, 48 blocks, 1024 columns at 256: 49.6.
+double tc_launch_us(int bn, int cg, long tiles, double kb) {
+  const double fixed = bn == 256 ? 3.5 : bn == 128 ? 2.6 : 2.2;
+  const double per_kb = cg == 2 ? 0.5 : bn == 256 ? 0.34 : 0.25;
+  const long units = 148 / cg, waves = (tiles + units - 1) / units;
+  return (double)waves * (fixed + per_kb * kb);
+}
+
+// Tile widths of the tensor-core layers and the split count P of the row reduction, for rounds of `rows` gradient rows in
+// `row_tiles` tiles of 128: what the model above makes shortest, plus the partial sums the Eq. 3 step has to read.  At most
+// maxP splits, of at least 512 rows each (each is one more partial vector for the Eq. 3 step, and on small models a weight
+// gradient spread over more CTAs takes the SMs the side-stream kernels of the next round run on).
+void plan_tc(const abs_model_desc* m, long rows, long row_tiles, int maxP, Layout* L) {
+  auto pick = [L](int n, long other_tiles, double kb) {       // narrower tiles only where they are clearly faster
+    int best = n >= 256 && !L->local_net ? 256 : n >= 128 ? 128 : 64;      // (local steps: 256-wide tiles, whose epilogue
+    for (int bn : {128, 64})                                              // adds to the uploads, measured 15 % slower)
+      if (bn < best && tc_launch_us(bn, 1, other_tiles * ((n + bn - 1) / bn), kb) < 0.93 * tc_launch_us(best, 1, other_tiles * ((n + best - 1) / best), kb))
+        best = bn;
+    return best;
+  };
+  maxP = std::max(1, (int)std::min<long>(maxP, rows / (L->cnn ? 128 : 512)));
+  for (int l = 0; l < m->n_layers; ++l) {
+    if (L->path[l] != PATH_TC) continue;
+    const int in = m->dims[l], out = m->dims[l + 1];
+    L->bn_fwd[l] = pick(out, row_tiles, in / 64.0);
+    L->bn_dg[l] = pick(in, row_tiles, out / 64.0);
+    L->cg_wg[l] = 1;
+    L->pair_bwd[l] = false;
+    // a large weight gradient is bound by operand traffic into shared memory: CTA pairs halve the B operand each CTA has
+    // to stage (its tiles are features x outputs, so the row padding unit of the version groups is not involved)
+    if ((size_t)in * out >= ((size_t)1 << 21) && in >= 256 && out >= 256 && rows >= 4096) { L->cg_wg[l] = 2; L->bn_wg[l] = 256; }
+    // A short weight gradient (fewer tiles than SMs at the back-propagation's tile width) shares its launch with the layer's
+    // delta back-propagation: both have one or two tiles per CTA, so separate launches would pay the fixed costs twice.
+    else if (l > 0 && !L->local_net && !(m->flags & ABS_FLAG_NO_FUSED_BACKWARD) && out >= L->bn_dg[l]) {
+      const int bn = L->bn_dg[l];
+      if ((long)((in + 127) / 128 + 1) * ((out + bn - 1) / bn) * maxP < 148) { L->pair_bwd[l] = true; L->bn_wg[l] = bn; }
+    }
+  }
+  double best = 1e30;
+  int bestP = 1, bn_best[ABS_MAX_LAYERS] = {};
+  for (int P = 1; P <= maxP; ++P) {
+    double t = 4.0 * (double)L->d_pad * P / 6.5e6;
+    int bn_p[ABS_MAX_LAYERS] = {};
+    for (int l = 0; l < m->n_layers; ++l) {
+      if (L->path[l] != PATH_TC) continue;
+      const int in = m->dims[l], out = m->dims[l + 1], tm = 128 * L->cg_wg[l];
+      const long splits = L->local_net ? std::max<long>(1, row_tiles / (L->RBp / 128)) : P;    // local steps: one per worker
+      const long mt = ((in + tm - 1) / tm + (L->bias_colsum[l] ? 0 : 1)) * splits;
+      const double kb = (double)row_tiles * 2.0 / splits;
+      bn_p[l] = (L->cg_wg[l] == 2 || L->pair_bwd[l]) ? L->bn_wg[l] : pick(out, mt, kb);
+      t += tc_launch_us(bn_p[l], L->cg_wg[l], mt * ((out + bn_p[l] - 1) / bn_p[l]), kb);
+    }
+    if (t < best * 0.999) { best = t; bestP = P; memcpy(bn_best, bn_p, sizeof bn_p); }
+  }
+  for (int l = 0; l < m->n_layers; ++l) if (L->path[l] == PATH_TC) L->bn_wg[l] = bn_best[l];
+  L->P = bestP;
+}
+
 void conv_blocks(const Layout& L, cmma::Block* b) {
   for (int i = 0; i < 2; ++i) {
     const int Ho = L.cHi[i] - L.ck + 1, Wo = L.cWi[i] - L.ck + 1;
@@ -239,38 +300,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   } else if (L->row_R) {
     L->P = 1;
   } else if (L->any_tc) {
-    // tile widths: widest tile that still gives every SM work; split count of the row reduction
-    // sized so the largest weight gradient fills about two waves of 148 CTAs
-    const int row_tiles = L->rows_cap / 128;
-    auto pick = [](int n, int other_tiles) {
-      for (int bn : {256, 128}) if (n >= bn && other_tiles * ((n + bn - 1) / bn) >= 120) return bn;
-      return n >= 128 ? 128 : 64;
-    };
-    for (int l = 0; l < m->n_layers; ++l) {
-      if (L->path[l] != PATH_TC) continue;
-      const int in = m->dims[l], out = m->dims[l + 1];
-      L->bn_fwd[l] = pick(out, row_tiles);
-      L->bn_dg[l] = pick(in, row_tiles);
-      L->bn_wg[l] = pick(out, ((in + 127) / 128 + 1) * 3);
-      L->cg_fwd[l] = L->cg_dg[l] = L->cg_wg[l] = 1;
-      if ((size_t)in * out >= ((size_t)1 << 21) && in >= 256 && out >= 256 && W * m->batch >= 4096) {
-        // a large weight gradient is bound by operand traffic into shared memory: CTA pairs halve
-        // the B operand each CTA has to stage (its tiles are features x outputs, so the row padding
-        // unit of the version groups is not involved)
-        L->cg_wg[l] = 2; L->bn_wg[l] = 256;
-      }
-    }
-    // A short weight gradient (fewer tiles than SMs at the back-propagation's tile width) shares
-    // its launch with the layer's delta back-propagation: both have one or two tiles per CTA, so
-    // separate launches would pay the fixed costs of a launch twice.
-    for (int l = 1; l < m->n_layers; ++l) {
-      if (L->path[l] != PATH_TC || L->cg_dg[l] != 1 || L->cg_wg[l] != 1 || (m->flags & ABS_FLAG_NO_FUSED_BACKWARD)) continue;
-      if (L->local_net) continue;
-      const int in = m->dims[l], out = m->dims[l + 1], bn = L->bn_dg[l];
-      if (out < bn) continue;
-      const long wg_tiles_min = (long)((in + 127) / 128 + 1) * ((out + bn - 1) / bn);   // at P = 1
-      if (wg_tiles_min * 4 < 148) { L->pair_bwd[l] = true; L->bn_wg[l] = bn; }
-    }
+    for (int l = 0; l < m->n_layers; ++l) L->cg_fwd[l] = L->cg_dg[l] = L->cg_wg[l] = 1;
     // A layer whose output delta is produced by the tensor-core back-propagation of the layer above gets its bias
     // gradient from column sums taken in that kernel's epilogue; its weight gradient then needs no row tile of ones.
     // (for at most as many layers as the Eq. 3 kernel takes partial-sum regions besides the output layer's)
@@ -279,31 +309,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
                           n < UpdateArgs::MAX_REGIONS - 1;
       n += L->bias_colsum[l] ? 1 : 0;
     }
-    // split count P of the row reduction: the one that minimises the modelled time of all weight
-    // gradients (whole waves of 148 CTAs, one tile = 128 x BN x rows/P) plus the extra partial
-    // sums the Eq. 3 step then has to read
-    double best = 1e30;
-    int bestP = 1;
-    // splits of at least 512 rows, at most 4: each split is one more partial vector for the Eq. 3 step (7 splits cost
-    // it 12 us on configuration 4 and win the weight gradient nothing), and on small models a weight gradient spread
-    // over more CTAs takes the SMs the side-stream kernels of the next round run on (configuration 3: 8 splits make
-    // the kernel 4 us shorter and the round 5 us longer)
-    // (the CNN's affine layers see at most a few hundred rows per round and run on one stream: splits of 128 rows,
-    // so that its FP32 weight-gradient kernels, whose grid is tiles x splits, are more than a handful of CTAs)
-    const int maxP = std::max(1, std::min(4, W * m->batch / (L->cnn ? 128 : 512)));
-    for (int P = 1; P <= maxP; ++P) {
-      double t = 4.0 * (double)L->d_pad * P / 5e12;
-      for (int l = 0; l < m->n_layers; ++l) {
-        if (L->path[l] != PATH_TC) continue;
-        const int in = m->dims[l], out = m->dims[l + 1], bn = L->bn_wg[l];
-        const int cg = L->cg_wg[l], tm = 128 * cg, units = 148 / cg;
-        const long tiles = (long)((in + tm - 1) / tm + (L->bias_colsum[l] ? 0 : 1)) * ((out + bn - 1) / bn) * P;
-        const long waves = (tiles + units - 1) / units;
-        t += (double)waves * 2.0 * 128.0 * bn * ((double)L->rows_cap / P) / 9e12;
-      }
-      if (t < best * 0.999) { best = t; bestP = P; }
-    }
-    L->P = bestP;
+    plan_tc(m, (long)W * m->batch, L->rows_cap / 128, 4, L);
   } else {
     // split count of the row reduction in the weight-gradient kernels
     size_t tiles = 0;
@@ -754,6 +760,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
   auto narrow_args = [&](int l) {
     NarrowArgs a;
     a.st = st; a.ri = ri; a.tile_slot = ctx->ctl.tile_slot[par]; a.row_idx = ctx->ctl.row_idx[par]; a.labels = (const int*)ctx->y;
+    a.tile_shift = __builtin_ctz((unsigned)L.RB);     // (networks: a power of two)
     a.ring = ctx->at<void>(L.gring); a.slot_stride = L.d_pad; a.w_off = L.w_off[l];
     a.in = m.dims[l]; a.C = m.dims[l + 1];
     a.gather = la[l].gather; a.act_in = la[l].act_in;
@@ -1137,6 +1144,15 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
   make_layout(model, W, S_ring, &L);
   if (model->workspace_bytes < L.total)
     return fail(ABS_ENOSPACE, "workspace has %zu bytes, %zu needed", model->workspace_bytes, L.total);
+
+  if (L.any_tc && model->k_mode == ABS_K_FIXED && K0 < W) {
+    // K never changes: plan for the rows such a round has (its version groups add about half a tile each), within the
+    // buffers that are there
+    const long rows = (long)K0 * model->batch;
+    const int P = L.P;
+    plan_tc(model, rows, L.local_net ? (long)K0 * (L.RBp / 128) : (rows + 127) / 128 + std::min(K0, S_ring + 1) / 4, std::max(1, P), &L);
+    if (P == 0) L.P = 0;
+  }
 
   ctx = new (std::nothrow) abs_ctx();
   if (!ctx) return fail(ABS_EINVAL, "out of host memory");

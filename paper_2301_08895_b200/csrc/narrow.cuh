@@ -77,6 +77,7 @@ struct NarrowArgs {
   DevState* st;
   RoundInfo* ri;
   const int* tile_slot;
+  int tile_shift;          // log2 of the rows per tile_slot entry
   const int* row_idx;
   const int* labels;
   const void* ring; size_t slot_stride; size_t w_off;

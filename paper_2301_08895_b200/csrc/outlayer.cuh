@@ -66,9 +66,15 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
   extern __shared__ __align__(16) unsigned char osm_raw[];
   DevState* st = a.st;
   RoundInfo* ri = a.ri;
-  if (st->status != ST_OK) return;
   const int r0 = blockIdx.x * ROWS;
-  if (r0 >= ri->n_rows) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane >> 2, t = lane & 3;
+  // one wave of loads (the grid covers the row capacity, so every address exists); warp (mt, kh) finishes the soft-max of
+  // rows 16 mt + 8 kh + g
+  const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[r0 >> a.tile_shift];
+  const int my_row = 16 * (warp & 3) + 8 * (warp >> 2) + g;
+  const int my_idx = a.row_idx[r0 + my_row];
+  if (status != ST_OK || r0 >= n_rows) return;
   constexpr int IN = NT * 128;
   constexpr int HP = IN + 8;                    // row pitch of the input rows (elements): 16 bytes of padding
   const int C = a.C;
@@ -77,8 +83,6 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
   __nv_bfloat16* d3s = ws + (size_t)(IN + 8) * WP;                        // [ROWS][WP] deltas of this layer
   float* lp = reinterpret_cast<float*>(d3s + (size_t)ROWS * WP);          // [4][32][8] logit partial sums
   __nv_bfloat16* wraw = reinterpret_cast<__nv_bfloat16*>(lp + 4 * 32 * 8);  // [IN + 1][C] weights + bias as stored
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int g = lane >> 2, t = lane & 3;
 
   // ---- loads: the 64 input rows (asynchronous 16-byte copies), the weights of the rows' version
   const __nv_bfloat16* src = (const __nv_bfloat16*)a.act_in + (size_t)r0 * IN;
@@ -87,7 +91,7 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s_u32(hs + (size_t)rr * HP + v * 8)),
                  "l"(src + (size_t)rr * IN + v * 8) : "memory");
   }
-  const int slot = a.tile_slot[r0 / st->RB];
+  const int lab = my_idx < 0 ? -1 : a.labels[my_idx];
   const float sa = sa_slot_weight(st, ri->t, slot);     // staleness-aware step size: weight of these rows in Eq. 3
   const __nv_bfloat16* Wm = (const __nv_bfloat16*)a.ring + (size_t)slot * a.slot_stride + a.w_off;
   {
@@ -96,20 +100,17 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
     for (int i = tid; i < n16; i += THREADS)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s_u32(wraw + 8 * i)), "l"(Wm + 8 * i) : "memory");
   }
-  // labels of the two rows whose soft-max this thread takes part in (warps 0..3)
-  int lab[2] = {-1, -1};
-  if (warp < 4) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int s = a.row_idx[r0 + 16 * warp + g + 8 * h];
-      lab[h] = s < 0 ? -1 : a.labels[s];
-    }
-  }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  for (int i = tid; i < (IN + 1) * CP; i += THREADS) {      // class rows padded to 16 with zeros
-    const int k = i >> 4, c = i & 15;
-    ws[k * WP + c] = c < C ? wraw[k * C + c] : __float2bfloat16_rn(0.f);
+  for (int k = tid; k <= IN; k += THREADS) {                // class rows padded to 16 with zeros
+    const unsigned short* src_k = reinterpret_cast<const unsigned short*>(wraw) + k * C;
+    uint32_t v[CP / 2];
+#pragma unroll
+    for (int c = 0; c < CP; c += 2)
+      v[c / 2] = (c < C ? src_k[c] : 0u) | (c + 1 < C ? (uint32_t)src_k[c + 1] << 16 : 0u);
+    uint4* dst_k = reinterpret_cast<uint4*>(ws + k * WP);
+    dst_k[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    dst_k[1] = make_uint4(v[4], v[5], v[6], v[7]);
   }
   __syncthreads();
 
@@ -131,64 +132,56 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
       mma16816(acc[0], af, bf[0], bf[1]);
       mma16816(acc[1], af, bf[2], bf[3]);
     }
-    if (kh == 1) {
+    // the halves exchange partial sums: kh = 0 keeps row g of the tile, kh = 1 row g + 8; the sum is always formed as
+    // (first half + second half) + bias
+    {
+      float* to = lp + (mt * 32 + lane) * 8 + 4 * kh;
+      *reinterpret_cast<float4*>(to) = kh ? make_float4(acc[0][0], acc[0][1], acc[1][0], acc[1][1])
+                                          : make_float4(acc[0][2], acc[0][3], acc[1][2], acc[1][3]);
+    }
+    __syncthreads();
+    {
+      // thread: row g + 8 kh of the tile, classes 2t, 2t+1, 8+2t, 8+2t+1
+      const float4 o4 = *reinterpret_cast<const float4*>(lp + (mt * 32 + lane) * 8 + 4 * (1 - kh));
+      const float other[4] = {o4.x, o4.y, o4.z, o4.w};
+      float z[4];
+      int cls[4];
 #pragma unroll
       for (int n = 0; n < 2; ++n)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) lp[(mt * 32 + lane) * 8 + n * 4 + i] = acc[n][i];
-    }
-    __syncthreads();
-    if (kh == 0) {
-      // thread: rows g and g + 8 of the tile, classes 2t, 2t+1, 8+2t, 8+2t+1
-      bool bad = false;
-      uint32_t dpk[2][2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float z[4];
-        int cls[4];
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int c = 8 * n + 2 * t + j;
-            cls[2 * n + j] = c;
-            z[2 * n + j] = acc[n][2 * h + j] + lp[(mt * 32 + lane) * 8 + n * 4 + 2 * h + j] +
-                           __bfloat162float(ws[IN * WP + c]);
-          }
-        float zmax = -3.0e38f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) if (cls[i] < C) zmax = fmaxf(zmax, z[i]);
-        zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 1));
-        zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 2));
-        const int y = lab[h];
-        float se = 0.f, zy = 0.f, e[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          e[i] = cls[i] < C ? expf(z[i] - zmax) : 0.f;
-          se += e[i];
-          if (cls[i] == y) zy = z[i];
+        for (int j = 0; j < 2; ++j) {
+          const int c = 8 * n + 2 * t + j, e = 2 * n + j;
+          const float mine = kh ? acc[n][2 + j] : acc[n][j];
+          cls[e] = c;
+          z[e] = (kh ? other[e] + mine : mine + other[e]) + __bfloat162float(ws[IN * WP + c]);
+          z[e] = c < C ? z[e] : -3.0e38f;                   // padded classes: exp(-3e38 - max) = 0
         }
-        se += __shfl_xor_sync(0xffffffffu, se, 1);
-        se += __shfl_xor_sync(0xffffffffu, se, 2);
-        zy += __shfl_xor_sync(0xffffffffu, zy, 1);
-        zy += __shfl_xor_sync(0xffffffffu, zy, 2);
-        const float inv = 1.f / se;
-        float d[4];
+      float zmax = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
+      zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 1));
+      zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 2));
+      float se = 0.f, zy = 0.f, e[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          d[i] = (y >= 0 && cls[i] < C) ? (e[i] * inv - (cls[i] == y ? 1.f : 0.f)) * sa : 0.f;   // padding rows add nothing to Eq. 3
-        dpk[h][0] = pack_bf16(d[0], d[1]);
-        dpk[h][1] = pack_bf16(d[2], d[3]);
-        const int rr = 16 * mt + g + 8 * h;
-        *reinterpret_cast<uint32_t*>(d3s + rr * WP + 2 * t) = dpk[h][0];
-        *reinterpret_cast<uint32_t*>(d3s + rr * WP + 8 + 2 * t) = dpk[h][1];
-        if (t == 0) {
-          const float loss = y >= 0 ? logf(se) - (zy - zmax) : 0.f;
-          a.row_loss[r0 + rr] = loss;
-          bad |= !isfinite(loss);
-        }
+      for (int i = 0; i < 4; ++i) {
+        e[i] = expf(z[i] - zmax);
+        se += e[i];
+        zy = cls[i] == lab ? z[i] : zy;
       }
-      if (bad) ri->diverged = 1;
+      se += __shfl_xor_sync(0xffffffffu, se, 1);
+      se += __shfl_xor_sync(0xffffffffu, se, 2);
+      zy += __shfl_xor_sync(0xffffffffu, zy, 1);
+      zy += __shfl_xor_sync(0xffffffffu, zy, 2);
+      const float inv = 1.f / se;
+      float d[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        d[i] = (lab >= 0 && cls[i] < C) ? (e[i] * inv - (cls[i] == lab ? 1.f : 0.f)) * sa : 0.f;   // padding rows add nothing to Eq. 3
+      *reinterpret_cast<uint32_t*>(d3s + my_row * WP + 2 * t) = pack_bf16(d[0], d[1]);
+      *reinterpret_cast<uint32_t*>(d3s + my_row * WP + 8 + 2 * t) = pack_bf16(d[2], d[3]);
+      if (t == 0) {
+        const float loss = lab >= 0 ? logf(se) - (zy - zmax) : 0.f;
+        a.row_loss[r0 + my_row] = loss;
+        if (!isfinite(loss)) ri->diverged = 1;
+      }
     }
     __syncthreads();
   }
@@ -204,10 +197,17 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
         for (int i = 0; i < 4; ++i) acc[m][n][i] = 0.f;
     const uint32_t b_base = s_u32(d3s + (size_t)((lane & 7) + ((lane >> 3) & 1) * 8) * WP + (lane >> 4) * 8);
     const uint32_t a_base = s_u32(hs + (size_t)((lane & 7) + ((lane >> 4) & 1) * 8) * HP + ((lane >> 3) & 1) * 8);
+    // bias sums: a product with ones (every row of it is the column sum)
+    const uint32_t ones[4] = {0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u};
+    float bias_sum[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
     for (int ks = 0; ks < ROWS / 16; ++ks) {
       uint32_t bf[4];
       ldsm4t(b_base + ks * 16 * WP * 2, bf);
+      if (warp == 0) {
+        mma16816(bias_sum[0], ones, bf[0], bf[1]);
+        mma16816(bias_sum[1], ones, bf[2], bf[3]);
+      }
 #pragma unroll
       for (int m = 0; m < NT; ++m) {
         uint32_t af[4];
@@ -226,10 +226,12 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
           const int f = (warp + 8 * m) * 16 + g + 8 * (i >> 1), c = 8 * n + 2 * t + (i & 1);
           if (c < C) dst[(size_t)f * C + c] = acc[m][n][i];
         }
-    if (tid < C) {
-      float tot = 0.f;
-      for (int rr = 0; rr < ROWS; ++rr) tot += __bfloat162float(d3s[rr * WP + tid]);
-      dst[(size_t)IN * C + tid] = tot;
+    if (warp == 0 && g == 0) {
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (8 * n + 2 * t + j < C) dst[(size_t)IN * C + 8 * n + 2 * t + j] = bias_sum[n][j];
     }
   }
   if (!has_dgrad) return;
