@@ -97,6 +97,7 @@ struct Layout {
   size_t data_X, data_y;
   // U > 1 on a multi-layer network: the selected workers' own model copies and uploads
   bool local_net = false;
+  bool local_fused = false;             // ... all hidden layers on the tensor cores: steps taken by the weight-gradient kernel
   int RBp = 0;                          // rows reserved per worker in a local step's row layout
   size_t priv = 0, loss_acc = 0;          // the workers' copies (storage type); their uploads live in G
   size_t gring = 0;                     // the models the gradient kernels read: the ring, or the private copies
@@ -375,6 +376,8 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
                   (size_t)R * 64 <= 100 * 1024) { L->fused_R = R; break; }
       L->out_mma = L->fused_R && tc_ok && m->n_layers > 1 &&
                    (inl == 128 || inl == 256 || inl == 512 || inl == 1024);
+      L->local_fused = L->local_net && L->out_mma;
+      for (int l = 0; l + 1 < m->n_layers; ++l) L->local_fused = L->local_fused && L->path[l] == PATH_TC;
       // the non-fused output-layer kernels: fewer rows per block when a round has few rows, so that the grid is
       // more than a handful of blocks (each is a chain of dependent loads)
       L->narrow_rpb = 64;
@@ -478,6 +481,7 @@ struct abs_ctx {
   bool lsq_v2 = false;               // least squares through the persistent 16-byte-load kernel
   int lsq_grid = 0;                  // its grid = number of partial sums
   bool lsq_rounds = false;           // small least squares: all enqueued rounds in one persistent kernel
+  int local_u = 0;                   // local step being enqueued
   CtlArgs ctl;
   TcLayer tcl[ABS_MAX_LAYERS];
   CUtensorMap ones_map;
@@ -878,7 +882,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
           launch_ex(ctx, ABS_KC_OUTPUT, narrow_fused_kernel<T>, dim3(L.rows_cap / R), dim3(256), sm, a, part, R, has_dgrad);
         }
         // U = 1: the chunk partials are added up by extra blocks of the Eq. 3 kernel (one launch less)
-        if (L.local_net)
+        if (L.local_net && !L.local_fused)
           launch_ex(ctx, ABS_KC_OUTPUT, lnet::chunk_reduce_worker_kernel, dim3((len + 255) / 256, ctx->W), dim3(256), 0, st, ri, part, len,
                     dstw, L.d_pad, R, L.RBp);
       } else if (a.in % 8 == 0) {
@@ -918,6 +922,13 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
       p.M_total = la[l].in + 1; p.N_total = la[l].out;     // row `in` of the result is the bias gradient
       p.out_f32 = ctx->at<float>(L.G) + L.w_off[l];
       p.no_bias_tile = L.bias_colsum[l] ? 1 : 0;
+      if (L.local_fused) {
+        p.sel_tau = ctx->ctl.sel_tau[par];
+        p.start = ctx->at<__nv_bfloat16>(L.ring) + L.w_off[l];
+        p.copy = ctx->at<__nv_bfloat16>(L.priv) + L.w_off[l];
+        p.lstep = m.lr / (float)m.batch;
+        p.lfirst = ctx->local_u == 0; p.llast = ctx->local_u == m.local_steps - 1;
+      }
       const int bias_tiles = L.bias_colsum[l] ? 0 : 1;
       if (l > 0 && L.pair_bwd[l]) {
         // the layer's delta back-propagation shares the weight gradient's launch (same tile width)
@@ -1452,6 +1463,29 @@ int abs_enqueue_rounds(abs_ctx* ctx, int n) {
       q.ri = ctx->at<RoundInfo>(L.ri) + par;
       q.sel = ctx->ctl.sel[par]; q.sel_tau = ctx->ctl.sel_tau[par];
       q.row_idx = ctx->ctl.row_idx[par]; q.tile_slot = ctx->ctl.tile_slot[par];
+      if (L.local_fused) {
+        lnet::MidArgs mid;
+        memset(&mid, 0, sizeof mid);
+        const int last = ctx->m.n_layers - 1;
+        mid.part = ctx->at<float>(L.red); mid.len = (ctx->m.dims[last] + 1) * ctx->m.dims[last + 1]; mid.chunk_rows = outl::ROWS;
+        mid.w_off = L.w_off[last];
+        mid.X = (const __nv_bfloat16*)ctx->X; mid.act0 = ctx->at<__nv_bfloat16>(par ? L.act0b : L.act[0]); mid.in = ctx->m.dims[0];
+        mid.shard = ctx->ctl.shard; mid.by_RBp = FastDiv(L.RBp);
+        const int n_red = (mid.len + 255) / 256, n_copy = bx, rows_blocks = std::min(ctx->sm_count * 8, (ctx->W * L.RBp + 7) / 8);
+        mid.by_red = FastDiv(n_red); mid.by_copy = FastDiv(n_copy);
+        auto between = [&](int u) {
+          mid.u = u; mid.n_red = u >= 0 ? n_red : 0; mid.n_copy = u < 0 ? n_copy : 0;
+          launch_ex(ctx, ABS_KC_LSQ, lnet::mid_kernel, dim3(ctx->W * (mid.n_red + mid.n_copy) + (u < q.U - 1 ? rows_blocks : 0)), dim3(256), 0, q, mid);
+        };
+        between(-1);
+        for (ctx->local_u = 0; ctx->local_u < q.U; ++ctx->local_u) {
+          gradient(par, PH_FORWARD);
+          gradient(par, PH_BACKWARD);
+          between(ctx->local_u);
+        }
+        update(par);
+        continue;
+      }
       if (f32) launch_ex(ctx, ABS_KC_LSQ, lnet::local_begin_kernel<float>, dim3(bx, ctx->W), dim3(256), 0, q);
       else launch_ex(ctx, ABS_KC_LSQ, lnet::local_begin_kernel<__nv_bfloat16>, dim3(bx, ctx->W), dim3(256), 0, q);
       for (int u = 0; u < q.U; ++u) {

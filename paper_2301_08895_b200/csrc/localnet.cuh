@@ -16,6 +16,7 @@
 #pragma once
 #include "common.cuh"
 #include "ctl.cuh"
+#include "narrow.cuh"
 
 namespace absb {
 namespace lnet {
@@ -169,6 +170,108 @@ __global__ void __launch_bounds__(256) local_step_kernel(Args a, int u) {
         if (!isfinite(loss)) ri->diverged = 1;
       }
     }
+  }
+}
+
+// ---- Networks whose hidden layers run on the tensor cores: the weight-gradient kernel takes the local step in its
+// epilogue, and one kernel between two steps does the rest.  mid_kernel after step u (u = -1: start of the jobs):
+//   blocks [0, W n_red)            output layer: upload and copy of 256 parameters of one worker; the worker's first block
+//                                  also adds the step's mean loss (and writes the uploaded loss after the last step)
+//   the next W n_copy (u = -1)     copies = the model versions the workers hold
+//   the rest                       input rows of step u + 1: minibatch draws, row copy
+struct MidArgs {
+  int u, n_red, n_copy;
+  const float* part; int len, chunk_rows;     // output layer: per-chunk gradient sums [chunks][len]
+  size_t w_off;                               // its block inside the parameter vector
+  const __nv_bfloat16* X; __nv_bfloat16* act0; int in;
+  const int2* shard;
+  FastDiv by_red, by_copy, by_RBp;
+};
+static __global__ void __launch_bounds__(256) mid_kernel(Args a, MidArgs m) {
+  grid_dependency_sync();
+  __shared__ float red[8];
+  const DevState* st = a.st;
+  RoundInfo* ri = a.ri;
+  const int status = st->status, K = ri->K, t = ri->t, B = st->B, S = st->S, W = st->W, RB = st->RB;
+  const uint32_t key0 = st->key0, key1 = st->key1;
+  if (status != ST_OK) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  typedef __nv_bfloat16 T;
+  int blk = (int)blockIdx.x;
+  if (blk < W * m.n_red) {
+    const int i = m.by_red.div(blk), part = blk - i * m.n_red, j = part * 256 + tid;
+    if (i >= K) return;
+    const int last = m.u == a.U - 1;
+    if (j < m.len) {
+      const int per = a.RBp / m.chunk_rows;
+      const float* p = m.part + (size_t)i * per * m.len + j;
+      float tot = 0.f;
+      for (int q = 0; q < per; ++q) tot += p[(size_t)q * m.len];
+      const size_t o = (size_t)i * a.d_pad + m.w_off + j;
+      const float s = m.u == 0 ? tot : a.gsum[o] + tot;
+      a.gsum[o] = s;
+      if (!last) {
+        const int slot = (t - a.sel_tau[i]) % (S + 1);
+        const float w0 = __bfloat162float(((const T*)a.ring)[(size_t)slot * a.d_pad + m.w_off + j]);
+        ((T*)a.priv)[o] = __float2bfloat16_rn(fmaf(-__fdiv_rn(a.lr, (float)B), s, w0));
+      }
+    }
+    if (part == 0) {
+      float l = 0.f;
+      for (int b = tid; b < B; b += 256) l += a.row_loss[(size_t)i * a.RBp + b];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (lane == 0) red[warp] = l;
+      __syncthreads();
+      if (tid == 0) {
+        float tot = 0.f;
+        for (int q = 0; q < 8; ++q) tot += red[q];
+        const float acc = (m.u == 0 ? 0.f : a.loss_acc[i]) + __fdiv_rn(tot, (float)B);
+        a.loss_acc[i] = acc;
+        if (last) {
+          const float loss = __fdiv_rn(acc, (float)a.U);
+          a.loss[i] = loss;
+          if (!isfinite(loss)) ri->diverged = 1;
+        }
+      }
+    }
+    return;
+  }
+  blk -= W * m.n_red;
+  if (blk < W * m.n_copy) {
+    const int i = m.by_copy.div(blk), part = blk - i * m.n_copy;
+    if (blk == 0 && tid == 0) ri->n_rows = K * a.RBp;
+    if (i >= K) return;
+    if (part == 0)
+      for (int q = tid; q < a.RBp / RB; q += 256) a.tile_slot[i * (a.RBp / RB) + q] = i;
+    const int slot = (t - a.sel_tau[i]) % (S + 1);
+    const uint4* src = reinterpret_cast<const uint4*>((const T*)a.ring + (size_t)slot * a.d_pad);
+    uint4* dst = reinterpret_cast<uint4*>((T*)a.priv + (size_t)i * a.d_pad);
+    const size_t n16 = a.d_pad * sizeof(T) / 16;
+#pragma unroll 4
+    for (size_t v = (size_t)part * 256 + tid; v < n16; v += (size_t)m.n_copy * 256) dst[v] = src[v];
+    return;
+  }
+  blk -= W * m.n_copy;
+  const int n_blk = (int)gridDim.x - W * (m.n_red + m.n_copy);
+  const int nblk4 = (B + 3) >> 2;
+  for (int r = blk * 8 + warp; r < K * a.RBp; r += n_blk * 8) {
+    const int i = m.by_RBp.div(r), b = r - i * a.RBp;
+    if (b >= B) {                              // padding rows keep their place for the whole job
+      if (m.u < 0) {
+        if (lane == 0) a.row_idx[r] = -1;
+        gather_row(m.act0, m.X, r, -1, m.in, lane);
+      }
+      continue;
+    }
+    const int n = a.sel[i];
+    const int2 shard = m.shard[n];
+    uint32_t w4[4];
+    philox4x32_10((uint32_t)n, (uint32_t)a.job[n], 1u, (uint32_t)((m.u + 1) * nblk4 + (b >> 2)), key0, key1, w4);
+    const uint32_t wd = (b & 3) == 0 ? w4[0] : (b & 3) == 1 ? w4[1] : (b & 3) == 2 ? w4[2] : w4[3];
+    const int s = shard.x + (int)__umulhi(wd, (unsigned)shard.y);
+    if (lane == 0) a.row_idx[r] = s;
+    gather_row(m.act0, m.X, r, s, m.in, lane);
   }
 }
 

@@ -50,6 +50,13 @@ struct Params {
   float* colsum;                   // DGRAD: [rows / 32][N_total] column sums of the stored result over each group of 32
                                    // rows (they add up to the bias gradient of the layer below), or null
   int no_bias_tile;                // WGRAD: the bias gradient comes from such column sums: no extra row tile
+  // WGRAD with P = 0 and copy set: the epilogue also takes the local step (Eq. 2 unrolled): upload += tile, copy =
+  // starting version - lstep * upload.  split i = selected worker i; pointers at the layer's block.
+  const int* sel_tau;              // staleness of each selected worker (its starting version's ring slot)
+  const __nv_bfloat16* start;      // [S+1][slot_stride] model versions
+  __nv_bfloat16* copy;             // [W][slot_stride] the workers' copies
+  float lstep;                     // eta / B
+  int lfirst, llast;               // first step: the upload starts from zero; last step: the copies are not needed any more
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -541,6 +548,93 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             mw[i] = bits;
           }
         }
+      }
+      if (mode == WGRAD && p.copy != nullptr) {
+        // One local step of worker c.split.  With bulk reductions into the uploads and a kernel of its own that refreshes
+        // the copies, the uploads went through L2 twice more (784-256, 32 workers: 20.6 + 8 + 14 us per step, 27 now; a round of ten steps 513 -> 490 us).
+        // Eight lanes take a row of a 32-column box, so that global accesses are whole 128-byte rows; a box is done in
+        // two halves of 16 rows, and the uploads and starting weights of the next half are fetched during this one (those
+        // of the first half before the accumulator is ready).
+        const int in_rows = p.M_total - 1;
+        const int quad = lane & 7, rg = lane >> 3;
+        const int m0 = (c.bias_tile ? in_rows + rank * BM : c.a_row) + q * 32;       // first gradient row of this warp
+        const int m_end = c.bias_tile ? in_rows + 1 : in_rows;
+        const int n_half = works ? 2 * min(HALF_COLS / 32, max(0, (p.N_total - c.b_col - half * HALF_COLS + 31) / 32)) : 0;
+        const bool any = m0 < m_end;                 // uniform in the warp
+        const int slot = any && !p.llast ? (ri->t - p.sel_tau[c.split]) % (st->S + 1) : 0;
+        const int nq = c.b_col + half * HALF_COLS + 4 * quad;
+        float* up = p.out_f32 + (size_t)c.split * p.slot_stride + nq;
+        const __nv_bfloat16* w0 = p.start + (size_t)slot * p.slot_stride + nq;
+        __nv_bfloat16* cp = p.copy + (size_t)c.split * p.slot_stride + nq;
+        float4 g[4];
+        uint2 ws[4];
+        auto fetch = [&](int h, float4 (&gg)[4], uint2 (&ww)[4]) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int m = m0 + 16 * (h & 1) + 4 * k + rg, dn = 32 * (h >> 1);
+            const bool ok = any && h < n_half && nq + dn < p.N_total && m < m_end;
+            gg[k] = (ok && !p.lfirst) ? *reinterpret_cast<const float4*>(up + (size_t)m * p.N_total + dn) : make_float4(0.f, 0.f, 0.f, 0.f);
+            ww[k] = (ok && !p.llast) ? *reinterpret_cast<const uint2*>(w0 + (size_t)m * p.N_total + dn) : make_uint2(0u, 0u);
+          }
+        };
+        fetch(0, g, ws);
+        if (have) {
+          if (!mbar_wait(&acc_full[acc], acc_phase, abort)) break;
+          tc_fence_after();
+        }
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
+#pragma unroll 1
+        for (int h = 0; h < n_half && any; ++h) {
+          float4 gn[4];
+          uint2 wn[4];
+          fetch(h + 1, gn, wn);
+          if ((h & 1) == 0) {
+            uint32_t v[32];
+            if (have) tmem_ld32(t_row + (uint32_t)(half * HALF_COLS + 16 * h), v);
+            else {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) v[i] = 0u;
+            }
+            __syncwarp();                            // the box has been read
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<uint4*>(my_row + ((j ^ sw) << 4)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            __syncwarp();
+          }
+          const int dn = 32 * (h >> 1);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int rr = 16 * (h & 1) + 4 * k + rg, m = m0 + rr;
+            const float4 d = *reinterpret_cast<const float4*>(my_box + rr * 128 + ((quad ^ (rr & 7)) << 4));
+            if (nq + dn < p.N_total && m < m_end) {
+              const float4 s = make_float4(g[k].x + d.x, g[k].y + d.y, g[k].z + d.z, g[k].w + d.w);
+              *reinterpret_cast<float4*>(up + (size_t)m * p.N_total + dn) = s;
+              if (!p.llast) {
+                const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ws[k].x));
+                const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ws[k].y));
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(fmaf(-p.lstep, s.x, f0.x), fmaf(-p.lstep, s.y, f0.y));
+                const __nv_bfloat162 hi = __floats2bfloat162_rn(fmaf(-p.lstep, s.z, f1.x), fmaf(-p.lstep, s.w, f1.y));
+                uint2 pk;
+                pk.x = *reinterpret_cast<const unsigned*>(&lo);
+                pk.y = *reinterpret_cast<const unsigned*>(&hi);
+                *reinterpret_cast<uint2*>(cp + (size_t)m * p.N_total + dn) = pk;
+              }
+            }
+            g[k] = gn[k];
+            ws[k] = wn[k];
+          }
+        }
+        if (have) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {                       // the accumulator barrier lives in the leader CTA
+            if (CG == 2) mbar_arrive_cluster(acc_empty0_addr + 8u * (uint32_t)acc);
+            else mbar_arrive(&acc_empty[acc]);
+          }
+          acc ^= 1;
+          if (acc == 0) acc_phase ^= 1u;
+        }
+        continue;
       }
       if (have) {
         if (!mbar_wait(&acc_full[acc], acc_phase, abort)) break;

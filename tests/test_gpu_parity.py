@@ -227,6 +227,19 @@ def test_local_sgd_steps_multi_layer_network(dims, W, B, U, K0, S):
     assert rows[-1]["loss_mean"] < rows[0]["loss_mean"]
 
 
+@pytest.mark.parametrize("dims,W,B,U", [
+    ((128, 64, 10), 3, 5, 2),                    # bias row alone in a second row tile; half a box row of minibatch rows
+    ((264, 104, 72, 10), 6, 33, 3),              # 8 weight rows and 8 columns left over; last box a quarter full
+    ((104, 200, 64, 16), 40, 140, 2),            # more worker tiles than the chip runs at once, 16 classes
+    ((20, 128, 64, 10), 5, 12, 3),               # first layer on the FP32-FMA kernels: step in a kernel of its own
+])
+def test_local_sgd_step_in_weight_gradient(dims, W, B, U):
+    """The local step taken by the weight-gradient kernel: row and column remainders of its 32 x 32 boxes."""
+    cfg = _small_cfg(inputs.MLP, dims, inputs.BF16, W, B, 3, 5, GAMMA3, lr=0.05)
+    X, y, w0 = _problem(cfg)
+    compare_with_oracle(cfg, X, y, w0, 8, TOL_BF16, forced=True, loss_tol=5e-2, local_steps=U)
+
+
 @pytest.mark.parametrize("dims,dtype,W,B,U,K0,S,forced", [
     ((20, 32, 10), inputs.FP32, 8, 16, 4, 3, 5, False),          # FP32-FMA hidden layer, fused output layer; free running
     ((33, 50, 17, 5), inputs.FP32, 9, 70, 3, 2, 4, True),        # odd widths (plain output-layer kernels), two row tiles per worker
