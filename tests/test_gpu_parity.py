@@ -338,6 +338,22 @@ def test_rounds_in_several_calls_equal_one_call():
     ctx.close()
 
 
+@pytest.mark.parametrize("max_rounds", [60, 2000, 6000])      # trace storage: 10 KB in all; 80 KB without the arrivals; 240 KB without
+def test_trace_windows(max_rounds):
+    """A window of the trace equals that part of the whole one, however many copies it takes."""
+    cfg = _small_cfg(inputs.LSQ, (32, 1), inputs.FP32, 8, 4, 2, 5, GAMMA3)
+    X, y, w0 = _problem(cfg)
+    from helpers import to_device
+    Xd, yd = to_device(cfg, X, y)
+    ctx = gpu.context_from_config(cfg, Xd, yd, w0, max_rounds=max_rounds)
+    ctx.run_rounds(40)
+    whole = gpu.trace_rows(ctx.get_trace())
+    assert len(whole) == 40 and sum(len(r["sel"]) for r in whole) > 40
+    for first, n in ((0, 40), (0, 1), (7, 20), (39, 1), (40, 0)):
+        assert gpu.trace_rows(ctx.get_trace(first, n)) == whole[first:first + n]
+    ctx.close()
+
+
 def test_host_dataset_entry_gives_same_result():
     cfg = inputs.config(1)
     X, y, w0 = _problem(cfg)
