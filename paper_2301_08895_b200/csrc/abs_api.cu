@@ -283,9 +283,10 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       for (int l = 0; l < m->n_layers; ++l) if (L->path[l] == PATH_TC) L->path[l] = PATH_SIMT;
       int tiles = 0;
       for (int l = 0; l < m->n_layers; ++l) tiles += step_tiles(m->dims[l], m->dims[l + 1]);
-      // CTAs per tile: enough for two per SM, at least two pipeline steps of rows each
+      // CTAs per tile: up to two per SM, at least one pipeline step of rows each (50 tiles, 8 steps: 18.9 us a round with
+      // two steps each, 21.7 with four; 67 tiles, 12 steps: 89.6 with three, 94.5 with one and a half)
       L->step_Q = 1;
-      while (L->step_Q < 8 && tiles * L->step_Q * 2 <= 2 * 148 && rows >= 4 * rnet::GK * L->step_Q) L->step_Q *= 2;
+      while (L->step_Q < 8 && tiles * L->step_Q * 2 <= 2 * 148 && rows >= 2 * rnet::GK * L->step_Q) L->step_Q *= 2;
     }
   }
   L->RB = lsq ? m->batch : L->row_R ? L->row_R : (L->any_tc ? 128 : 64);
@@ -1015,13 +1016,15 @@ void enqueue_update(abs_ctx* ctx, int par) {
     q.X = L.cnn ? ctx->at<void>(par ? L.act0b : L.act[0]) : ctx->X;
     q.gather = L.cnn ? 0 : 1;
     q.master = ctx->at<float>(L.master); q.ring = ctx->at<void>(L.ring); q.d_pad = L.d_pad; q.lr = ctx->m.lr;
-    q.n_layers = nl; q.Q = L.step_Q;
+    q.n_layers = nl; q.Q = L.step_Q; q.rows_cap = L.rows_cap;
+    while ((1 << q.q_shift) < q.Q) ++q.q_shift;
     for (int l = 0; l <= nl; ++l) {
       q.dims[l] = ctx->m.dims[l];
       if (l > 0 && l < nl) q.act[l] = ctx->at<void>(L.act[l]);
       if (l > 0) q.delta[l] = ctx->at<void>(L.delta[l]);
       if (l == nl) break;
       q.w_off[l] = L.w_off[l];
+      q.nct[l] = FastDiv((ctx->m.dims[l + 1] + rnet::GT - 1) / rnet::GT);
       q.first_tile[l + 1] = q.first_tile[l] + step_tiles(ctx->m.dims[l], ctx->m.dims[l + 1]);
     }
     int blocks = 0;
@@ -1032,7 +1035,7 @@ void enqueue_update(abs_ctx* ctx, int par) {
     }
     if (L.conv_mma) q.frag = frag_map(ctx);
     ctx->next_cluster = q.Q;
-    launch_ex(ctx, ABS_KC_UPDATE, rnet::grad_step_kernel<T>, dim3(q.first_tile[nl] * q.Q + round_up(blocks, q.Q)), dim3(256), 0, q);
+    launch_ex(ctx, ABS_KC_UPDATE, rnet::grad_step_kernel<T, sizeof(T) == 4 ? 2 : 1>, dim3(q.first_tile[nl] * q.Q + round_up(blocks, q.Q)), dim3(256), 0, q);
     return;
   }
   UpdateArgs u;

@@ -6,8 +6,8 @@
 //                     (Eq. 3), and the SGD step and ring write of that block in the same CTA.
 // One launch per layer and direction would be bound by launch gaps and by grids of a few CTAs: rounds of this model
 // class are a few hundred rows and 10^4 .. 10^6 parameters.
-// Measured per round (one launch per layer and direction -> this): 300-123-57-7 fp32, 13 workers x 37 rows: 114 -> 28 us
-// (11 -> 3 launches); 784-10 fp32, 16 x 64: 22 -> 19 us; the 400-120-84-10 part of the CNN, 640 rows: 13 -> 2 launches,
+// Measured per round (one launch per layer and direction -> this): 300-123-57-7 fp32, 13 workers x 37 rows: 114 -> 18 us
+// (11 -> 3 launches); 784-10 fp32, 16 x 64: 22 -> 14 us; the 400-120-84-10 part of the CNN, 640 rows: 13 -> 2 launches,
 // 21 us for the row kernel between two events (28 us with FP32 FMAs for the bf16 products).
 // Activations and deltas are rounded to the storage type where they are stored, sums are fp32 in a fixed order.
 #pragma once
@@ -52,6 +52,7 @@ struct RowsArgs {
   // Weights in shared memory.  resident: every layer is copied once and stays (stage l = layer l, the backward pass
   // reads it again); otherwise chunks of rpc[l] rows stream through `stages` stages, forward and again backward.
   int resident, stages, stage_bytes;
+  int w_bytes;                           // ... all of them
   int w_res[ABS_MAX_LAYERS];             // byte offset of layer l (resident)
   int rpc[ABS_MAX_LAYERS];               // rows per chunk: a multiple of 16 (chunks start on 16 bytes), or all of them
   int act_off[ABS_MAX_LAYERS];           // element offset (T) of layer l's input behind the weights
@@ -92,6 +93,7 @@ inline bool plan_rows(RowsArgs* a, int R, int esz, size_t* smem) {
   a->stages = a->n_layers;
   a->stage_bytes = 0;
   *smem = all + bytes;
+  a->w_bytes = (int)std::min<size_t>(all, 1u << 30);
   if (a->resident) return true;
   for (int l = 0; l < a->n_layers; ++l) {
     const size_t row16 = (size_t)16 * a->dims[l + 1] * esz;
@@ -101,6 +103,7 @@ inline bool plan_rows(RowsArgs* a, int R, int esz, size_t* smem) {
   a->stage_bytes = (int)stage;
   for (a->stages = MAX_STAGES; a->stages >= 2; --a->stages) {
     *smem = (size_t)a->stages * stage + bytes;
+    a->w_bytes = a->stages * (int)stage;
     if (*smem <= 220 * 1024) return true;
   }
   return false;
@@ -308,11 +311,12 @@ __device__ __forceinline__ int2 fma_layer(Weights& W, int l, const float* x, flo
 
 template <int R>
 __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_constant__ RowsArgs a) {
-  grid_dependency_sync();
   extern __shared__ __align__(128) unsigned char rsm[];
   __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES];
   __shared__ int gave_up;
   __shared__ int lab[R];                             // label of each row, -1: padding
+  weights_init(a, full, empty, &gave_up, NW);        // before the wait: touches nothing of the kernels in front
+  grid_dependency_sync();
   DevState* st = a.st;
   RoundInfo* ri = a.ri;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -328,10 +332,7 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
     return;
   }
   const int L = a.n_layers;
-  const size_t w_bytes = a.resident ? (size_t)a.w_res[L - 1] + round_up((a.dims[L - 1] + 1) * a.dims[L] * 4, 128)
-                                    : (size_t)a.stages * a.stage_bytes;
-  float* fs = reinterpret_cast<float*>(rsm + w_bytes);
-  weights_init(a, full, empty, &gave_up, NW);
+  float* fs = reinterpret_cast<float*>(rsm + a.w_bytes);
   Weights W(a, rsm, full, empty, &gave_up);
   constexpr int RQ = R / 4;
 
@@ -344,6 +345,7 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
     {
       const int in = a.dims[0];
       float* x = fs + a.act_off[0];
+      const int label = (tid < R && my_idx >= 0) ? a.labels[my_idx] : -1;
       const int rq = warp % RQ;                      // (RQ divides NW) four rows per warp
       const float* src[4];
 #pragma unroll
@@ -352,16 +354,21 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
         const int s = __shfl_sync(0xffffffffu, my_idx, rq * 4 + j);
         src[j] = (a.gather && s < 0) ? nullptr : (const float*)a.X + (size_t)(a.gather ? s : r) * in;
       }
-#pragma unroll 2
-      for (int k = (warp / RQ) * 32 + lane; k < in; k += NW / RQ * 32) {
-        float4 v;
-        v.x = src[0] ? src[0][k] : 0.f;
-        v.y = src[1] ? src[1][k] : 0.f;
-        v.z = src[2] ? src[2][k] : 0.f;
-        v.w = src[3] ? src[3][k] : 0.f;
-        *reinterpret_cast<float4*>(x + (size_t)rq * (in + 1) * 4 + k * 4) = v;
+      // all loads of up to 32 / R x 256 features in flight at once: the rows come from all over the dataset (784
+      // features, 8 rows: 6000 cycles with two iterations in flight)
+      constexpr int KB = 8, KSTEP = NW / RQ * 32;
+      for (int kb = (warp / RQ) * 32 + lane; kb < in; kb += KB * KSTEP) {
+        float v[KB][4];
+#pragma unroll
+        for (int u = 0; u < KB; ++u)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[u][j] = (src[j] && kb + u * KSTEP < in) ? src[j][kb + u * KSTEP] : 0.f;
+#pragma unroll
+        for (int u = 0; u < KB; ++u)
+          if (kb + u * KSTEP < in)
+            *reinterpret_cast<float4*>(x + (size_t)rq * (in + 1) * 4 + (kb + u * KSTEP) * 4) = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
       }
-      if (tid < R) lab[tid] = my_idx < 0 ? -1 : a.labels[my_idx];
+      if (tid < R) lab[tid] = label;
       for (int e = tid; e < L * R; e += NT) {         // the input of the bias row
         const int l = e / R, q = e % R / 4;
         fs[a.act_off[l] + (q * (a.dims[l] + 1) + a.dims[l]) * 4 + (e & 3)] = 1.f;
@@ -497,13 +504,14 @@ __device__ __forceinline__ void copy_rows(__nv_bfloat16* dst, const __nv_bfloat1
 }
 
 static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const __grid_constant__ RowsArgs a) {
-  grid_dependency_sync();
   extern __shared__ __align__(128) unsigned char rsm[];
   __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES];
   __shared__ int gave_up;
   __shared__ int lab[MMA_R];                         // label of each row, -1: padding
   typedef __nv_bfloat16 T;
   constexpr int R = MMA_R, NWM = MMA_NW;
+  weights_init(a, full, empty, &gave_up, NWM);       // before the wait: touches nothing of the kernels in front
+  grid_dependency_sync();
   DevState* st = a.st;
   RoundInfo* ri = a.ri;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -519,10 +527,7 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
   }
   const int g = lane >> 2, t = lane & 3;
   const int L = a.n_layers;
-  const size_t w_bytes = a.resident ? (size_t)a.w_res[L - 1] + round_up((a.dims[L - 1] + 1) * a.dims[L] * 2, 128)
-                                    : (size_t)a.stages * a.stage_bytes;
-  T* ts = reinterpret_cast<T*>(rsm + w_bytes);
-  weights_init(a, full, empty, &gave_up, NWM);
+  T* ts = reinterpret_cast<T*>(rsm + a.w_bytes);
   Weights W(a, rsm, full, empty, &gave_up);
   auto sync_compute = [] { asm volatile("bar.sync 1, %0;" ::"n"(NWM * 32) : "memory"); };
   const T* w_ring = (const T*)a.ring + (size_t)slot * a.slot_stride;
@@ -532,7 +537,7 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
     // ---------------------------------------------------------------- input row of this warp; zero padding columns
     const int in = a.dims[0];
     const T* src = (a.gather && my_idx < 0) ? nullptr : (const T*)a.X + (size_t)(a.gather ? my_idx : r0 + warp) * in;
-    if (lane == 0) lab[warp] = my_idx < 0 ? -1 : a.labels[my_idx];
+    const int label = (lane == 0 && my_idx >= 0) ? a.labels[my_idx] : -1;
     T* x = ts + a.act_off[0] + warp * mma_pitch(in);
     if ((in & 7) == 0) {                              // rows on 16-byte boundaries
 #pragma unroll 4
@@ -542,6 +547,7 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
 #pragma unroll 8
       for (int k = lane; k < in; k += 32) x[k] = src ? src[k] : (T)0.f;
     }
+    if (lane == 0) lab[warp] = label;
     for (int l = 0; l <= L; ++l) {
       const int n = a.dims[l], p = mma_pitch(n);      // at most 8 + 15 padding columns
       if (n + lane < p) ts[(l < L ? a.act_off[l] : a.out_off) + warp * p + n + lane] = (T)0.f;
@@ -754,35 +760,55 @@ struct StepArgs {
   size_t w_off[ABS_MAX_LAYERS];
   int n_layers, dims[ABS_MAX_LAYERS + 1];
   int first_tile[ABS_MAX_LAYERS + 1];    // tiles of layer l: [first_tile[l], first_tile[l + 1])
-  int Q;                                 // CTAs (a cluster) per tile: they share the rows
+  FastDiv nct[ABS_MAX_LAYERS];           // column tiles of layer l
+  int Q, q_shift;                        // CTAs (a cluster, 2^q_shift) per tile: they share the rows
+  int rows_cap;                          // rows the buffers hold
   // parts of the gradient left as per-chunk partial sums (the CNN's convolution blocks): blocks behind the tiles
   struct Region { const float* part; int len, chunk_rows; size_t off; int first_block; } region[2];
   int n_regions;
   cmma::FragMap frag;                    // region i = convolution block i: the weights also as operand fragments
 };
 
-__device__ __forceinline__ float ld_cluster(const float* p, int rank) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(tc::map_to_cta(tc::smem_u32(p), (uint32_t)rank)) : "memory");
-  return v;
-}
+__device__ __forceinline__ float as_float(float v) { return v; }
+__device__ __forceinline__ float as_float(__nv_bfloat16 v) { return __bfloat162float(v); }
 
 // Four groups of 64 threads take 16 rows of a 64-row step each (4 x 4 sums per thread: two 16-byte shared-memory reads
-// for eight packed FMAs), the next step's rows are loaded into registers meanwhile; groups, then cluster CTAs, are
-// added in order and the owner applies Eq. 3.
-template <typename T>
-__global__ void __launch_bounds__(256) grad_step_kernel(const __grid_constant__ StepArgs a) {
-  grid_dependency_sync();
+// for eight packed FMAs); two steps' rows are in registers on the way.  Groups are added in order, each CTA of a cluster
+// hands its sums to the owner of their share, which adds them in order and applies Eq. 3.
+// Bound by the chain of dependent latencies (indices, rows, exchange), so: the tile is found before the wait for the
+// kernels in front, indices come with the round's sizes in one wave of loads, the weights a CTA updates are fetched
+// before its sums exist.  784 x 10 fp32, 1024 rows: 6.4 -> 4 us
+// with the row kernel's loads done likewise (19.3 -> 14.4 us a round); 300-123-57-7, 481 rows: 27.7 -> 18.3 us a round.
+template <typename T, int DEPTH>
+__global__ void __launch_bounds__(256, DEPTH == 2 ? 2 : 3) grad_step_kernel(const __grid_constant__ StepArgs a) {
   __shared__ __align__(16) float As[2][GK][GP], Ds[2][GK][GP];
+  __shared__ float box[GT * GT];                     // sums of this CTA's share: [CTA of the cluster][share]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n_tiles = a.first_tile[a.n_layers];
+  const int Q = a.Q, rank = (int)blockIdx.x & (Q - 1), tile = min((int)blockIdx.x >> a.q_shift, n_tiles - 1);
+  int l = 0;
+  while (tile >= a.first_tile[l + 1]) ++l;
+  const int in = a.dims[l], out = a.dims[l + 1], lt = tile - a.first_tile[l];
+  const int tm = a.nct[l].div(lt);
+  const int m0 = tm * GT, n0 = (lt - tm * ((out + GT - 1) / GT)) * GT;
+  const bool gather = l == 0 && a.gather;
+  const T* A = (const T*)(l == 0 ? a.X : a.act[l]);
+  const T* D = (const T*)a.delta[l + 1];
+  const int m = m0 + lane, n = n0 + lane;
+  grid_dependency_sync();
   const DevState* st = a.st;
   const RoundInfo* ri = a.ri;
+  // row 8 i + warp of a step is loaded by this warp; lane i < 8 holds its sample index
+  auto load_idx = [&](int s) -> int {
+    const int r = s * GK + 8 * lane + warp;
+    return (lane < 8 && r < a.rows_cap) ? (gather ? a.row_idx[r] : r) : -1;
+  };
+  int ia = load_idx(rank), ib = DEPTH == 2 ? load_idx(rank + Q) : -1;
   const int status = st->status, diverged = ri->diverged, K = ri->K, n_rows = ri->n_rows, B = st->B, t = ri->t, S = st->S;
   if (status != ST_OK || diverged) return;
   const float step = __fdiv_rn(a.lr, (float)(K * B));
   const int slot = (t + 1) % (S + 1);
   T* dst = (T*)a.ring + (size_t)slot * a.d_pad;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_tiles = a.first_tile[a.n_layers];
   if ((int)blockIdx.x >= n_tiles * a.Q) {
     // region block: 32 parameters x 8 lanes over the chunks, fixed order
     float* red = &As[0][0][0];
@@ -810,50 +836,53 @@ __global__ void __launch_bounds__(256) grad_step_kernel(const __grid_constant__ 
     }
     return;
   }
-  const int Q = a.Q, rank = (int)blockIdx.x % Q, tile = (int)blockIdx.x / Q;
-  int l = 0;
-  while (tile >= a.first_tile[l + 1]) ++l;
-  const int in = a.dims[l], out = a.dims[l + 1];
-  const int nct = (out + GT - 1) / GT, lt = tile - a.first_tile[l];
-  const int m0 = lt / nct * GT, n0 = (lt % nct) * GT;
-  const bool gather = l == 0 && a.gather;
-  const T* A = (const T*)(l == 0 ? a.X : a.act[l]);
-  const T* D = (const T*)a.delta[l + 1];
-  const int m = m0 + lane, n = n0 + lane;
   const int n_steps = (n_rows + GK - 1) / GK;
-  // row 8 i + warp of a step is loaded by this warp; lane i < 8 holds its sample index
-  auto load_idx = [&](int s) -> int {
-    const int r = s * GK + 8 * lane + warp;
-    return (lane < 8 && r < n_rows && s < n_steps) ? (gather ? a.row_idx[r] : r) : -1;
-  };
-  float pa[8], pd[8];
-  auto load = [&](int s, int idx) {
+  // Loads are unconditional (clamped addresses, selected when stored): a load and its conversion under a condition wait
+  // for each other.  The mask has the rows that count; indices behind the round's rows are leftovers.
+  struct Rows { T a[8], d[8]; unsigned ok; };
+  const T zero = T(0.f), one = T(1.f);
+  const T* Am = A + min(m, in - 1);
+  const T* Dn = D + min(n, out - 1);
+  auto load = [&](int s, int idx, Rows& p) {
+    const int r0 = s * GK + warp;
+    p.ok = __ballot_sync(0xffffffffu, idx >= 0 && r0 + 8 * lane < n_rows);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int r = s * GK + 8 * i + warp;
-      const int x = __shfl_sync(0xffffffffu, idx, i);
-      pa[i] = x < 0 ? 0.f : m < in ? ldf(A, (size_t)x * in + m) : m == in ? 1.f : 0.f;    // row `in`: the bias
-      pd[i] = (r < n_rows && n < out) ? ldf(D, (size_t)r * out + n) : 0.f;
+      p.a[i] = Am[(size_t)max(__shfl_sync(0xffffffffu, idx, i), 0) * in];
+      p.d[i] = Dn[(size_t)min(r0 + 8 * i, a.rows_cap - 1) * out];
     }
   };
+  Rows p0, p1;
+  load(rank, ia, p0);
+  if (DEPTH == 2) load(rank + Q, ib, p1);
+  ia = load_idx(rank + DEPTH * Q);
+  if (DEPTH == 2) ib = load_idx(rank + 3 * Q);
+  // this CTA's share of the tile: elements e_0 + tid + 256 i
+  const int share = (GT * GT) >> a.q_shift;
+  float w[4];
+  size_t o[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = rank * share + tid + 256 * i, mm = m0 + e / GT, nn = n0 + e % GT;
+    const bool mine = tid + 256 * i < share && mm <= in && nn < out;
+    o[i] = mine ? a.w_off[l] + (size_t)mm * out + nn : (size_t)-1;
+    w[i] = mine ? a.master[o[i]] : 0.f;
+  }
   f32x2 acc[4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0ull;
   const int kg = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
-  int idx = load_idx(rank);
-  if (rank < n_steps) load(rank, idx);
-  idx = load_idx(rank + Q);
-  int buf = 0;
-  for (int s = rank; s < n_steps; s += Q) {
+  auto one_step = [&](int s, int buf, int& idx, Rows& p) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      As[buf][8 * i + warp][lane] = pa[i];
-      Ds[buf][8 * i + warp][lane] = pd[i];
+      const bool ok = (p.ok >> i & 1u) != 0;
+      As[buf][8 * i + warp][lane] = as_float(m < in ? (ok ? p.a[i] : zero) : m == in ? one : zero);       // row `in`: the bias
+      Ds[buf][8 * i + warp][lane] = as_float(ok && n < out ? p.d[i] : zero);
     }
     __syncthreads();
-    if (s + Q < n_steps) {
-      load(s + Q, idx);
-      idx = load_idx(s + 2 * Q);
+    if (s + DEPTH * Q < n_steps) {
+      load(s + DEPTH * Q, idx, p);
+      idx = load_idx(s + 2 * DEPTH * Q);
     }
 #pragma unroll
     for (int k = 0; k < GK / 4; ++k) {
@@ -866,40 +895,44 @@ __global__ void __launch_bounds__(256) grad_step_kernel(const __grid_constant__ 
         lsqp::ffma2(acc[i][1], p[i], dv.y);
       }
     }
-    buf ^= 1;
+  };
+#pragma unroll 1
+  for (int s = rank; s < n_steps; s += 2 * Q) {
+    one_step(s, 0, ia, p0);
+    if (s + Q < n_steps) one_step(s + Q, 1, DEPTH == 2 ? ib : ia, DEPTH == 2 ? p1 : p0);
   }
+  if (Q > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");       // (peers have started: see below)
   __syncthreads();
   float* red = &As[0][0][0];                         // [4][GT][GT]
 #pragma unroll
   for (int i = 0; i < 4; ++i)
     *reinterpret_cast<ulonglong2*>(red + (size_t)kg * GT * GT + (4 * ty + i) * GT + 4 * tx) = make_ulonglong2(acc[i][0], acc[i][1]);
   __syncthreads();
-  float* sum = &Ds[0][0][0];                         // [GT][GT] this CTA's sum
+  if (Q > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 #pragma unroll
-  for (int e = tid; e < GT * GT; e += 256)
-    sum[e] = (red[e] + red[GT * GT + e]) + (red[2 * GT * GT + e] + red[3 * GT * GT + e]);
-  if (Q > 1) tc::cluster_sync_all();
-  else __syncthreads();
-  const int share = GT * GT / Q;
-  for (int e = rank * share + tid; e < (rank + 1) * share; e += 256) {
-    const int mm = m0 + e / GT, nn = n0 + e % GT;
-    if (mm > in || nn >= out) continue;
-    float g = 0.f;
+  for (int i = 0; i < 4; ++i) {
+    const int e = tid + 256 * i;
+    const float v = (red[e] + red[GT * GT + e]) + (red[2 * GT * GT + e] + red[3 * GT * GT + e]);
     if (Q > 1) {
-      float v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = q < Q ? ld_cluster(sum + e, q) : 0.f;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) g += v[q];
+      const int owner = e >> (10 - a.q_shift);       // (GT x GT = 2^10)
+      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(tc::map_to_cta(tc::smem_u32(box + rank * share + (e & (share - 1))), (uint32_t)owner)), "f"(v) : "memory");
     } else {
-      g = sum[e];
+      box[e] = v;                                    // read back by the same thread
     }
-    const size_t o = a.w_off[l] + (size_t)mm * out + nn;
-    const float w = fmaf(-step, g, a.master[o]);
-    a.master[o] = w;
-    stf(dst, o, w);
   }
-  if (Q > 1) tc::cluster_sync_all();                 // nobody leaves while a peer reads its sum
+  if (Q > 1) tc::cluster_sync_all();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (o[i] == (size_t)-1) continue;
+    float g = box[tid + 256 * i];
+    if (Q > 1)
+#pragma unroll
+      for (int q = 1; q < 8; ++q)
+        if (q < Q) g += box[q * share + tid + 256 * i];
+    const float m_new = fmaf(-step, g, w[i]);
+    a.master[o[i]] = m_new;
+    stf(dst, o[i], m_new);
+  }
 }
 
 }  // namespace rnet
