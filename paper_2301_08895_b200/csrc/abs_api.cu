@@ -72,6 +72,7 @@ struct Layout {
   int narrow_rpb = 64;                  // rows per block of the row-tiled output-layer kernels that are not fused
   bool out_mma = false;                 // output layer through the mma.sync kernel (bf16, 64 rows per CTA)
   int row_R = 0;                        // whole network through rownet.cuh with this many rows per CTA (0: not used)
+  bool row_resident = false;            // ... whose weights stay in shared memory
   int step_Q = 1;                       // ... CTAs per tile of its gradient kernel
   size_t esz = 4;                       // bytes per stored element (4 or 2)
   size_t d = 0, d_pad = 0;
@@ -266,7 +267,9 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
     } else L->path[l] = PATH_SIMT;
   }
   // Networks without tensor-core layers and the fully connected part of the CNN: two kernels per round (rownet.cuh)
-  // if the rows' activations fit into shared memory.  Rows per CTA: bf16 one mma tile; fp32 4 while that leaves at most
+  // if the rows' activations fit into shared memory.  Rows per CTA: bf16 8 (one column tile of the
+  // matrix instruction) while that leaves one CTA per SM, else 16 (300-100-10: 512 rows 15.2 / 16.3 us a round, 1024 rows
+  // 22.2 / 22.9; 201-133-10, 4096 rows: 69.6 / 60.7); fp32 4 while that leaves at most
   // one CTA per SM (the chain of layers is what counts), 8 up to two waves, then 16 (fewer reads of the weights per row).
   L->row_R = 0;
   if (!lsq && m->local_steps <= 1 && (!L->any_tc || L->cnn)) {
@@ -275,10 +278,11 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
     ra.n_layers = m->n_layers;
     for (int l = 0; l <= m->n_layers; ++l) ra.dims[l] = m->dims[l];
     size_t smem = 0;
-    const int R0 = L->esz == 2 ? rnet::MMA_R : rows <= 148 * 4 ? 4 : rows <= 2 * 148 * 8 ? 8 : 16;
-    for (int R = R0; R >= (L->esz == 2 ? rnet::MMA_R : 4) && !L->row_R; R /= 2)
+    const int R0 = L->esz == 2 ? (rows <= 148 * 8 ? 8 : 16) : rows <= 148 * 4 ? 4 : rows <= 2 * 148 * 8 ? 8 : 16;
+    for (int R = R0; R >= (L->esz == 2 ? 8 : 4) && !L->row_R; R /= 2)
       if (rnet::plan_rows(&ra, R, (int)L->esz, &smem)) L->row_R = R;
     if (L->row_R) {
+      L->row_resident = ra.resident != 0;
       L->any_tc = false;
       for (int l = 0; l < m->n_layers; ++l) if (L->path[l] == PATH_TC) L->path[l] = PATH_SIMT;
       int tiles = 0;
@@ -677,10 +681,11 @@ cmma::FragMap frag_map(const abs_ctx* ctx) {
   return m;
 }
 
-// the row kernel for R rows per CTA
+// the row kernel for R rows per CTA; fp32: any weights
 template <typename T>
-void (*rows_kernel_fn(int R))(rnet::RowsArgs) {
-  if (sizeof(T) == 2) return rnet::rows_mma_kernel;
+void (*rows_kernel_fn(int R, bool resident))(rnet::RowsArgs) {
+  if (sizeof(T) == 2) return R == 8 ? (resident ? rnet::rows_mma_kernel<8, true> : rnet::rows_mma_kernel<8, false>)
+                                      : (resident ? rnet::rows_mma_kernel<16, true> : rnet::rows_mma_kernel<16, false>);
   return R == 4 ? rnet::rows_fma_kernel<4> : R == 8 ? rnet::rows_fma_kernel<8> : rnet::rows_fma_kernel<16>;
 }
 
@@ -842,7 +847,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     }
     size_t sm = 0;
     rnet::plan_rows(&a, L.row_R, (int)L.esz, &sm);
-    launch_ex(ctx, ABS_KC_FWD, rows_kernel_fn<T>(L.row_R), dim3(L.rows_cap / L.row_R),
+    launch_ex(ctx, ABS_KC_FWD, rows_kernel_fn<T>(L.row_R, a.resident != 0), dim3(L.rows_cap / L.row_R),
               dim3(L.esz == 2 ? rnet::MMA_THREADS : rnet::THREADS), sm, a);
     return;
   }
@@ -1278,8 +1283,8 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     if (ef != cudaSuccess) return bail(cuda_fail(nullptr, ef, "cudaFuncSetAttribute(narrow_fused_kernel)"));
   }
   if (L.row_R) {
-    const cudaError_t er = L.esz == 4 ? cudaFuncSetAttribute(rows_kernel_fn<float>(L.row_R), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024)
-                                      : cudaFuncSetAttribute(rows_kernel_fn<__nv_bfloat16>(L.row_R), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    const cudaError_t er = L.esz == 4 ? cudaFuncSetAttribute(rows_kernel_fn<float>(L.row_R, L.row_resident), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024)
+                                      : cudaFuncSetAttribute(rows_kernel_fn<__nv_bfloat16>(L.row_R, L.row_resident), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     if (er != cudaSuccess) return bail(cuda_fail(nullptr, er, "cudaFuncSetAttribute(row kernel)"));
   }
   if (model->local_steps > 1 && !L.local_net) {

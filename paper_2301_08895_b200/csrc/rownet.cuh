@@ -8,7 +8,7 @@
 // class are a few hundred rows and 10^4 .. 10^6 parameters.
 // Measured per round (one launch per layer and direction -> this): 300-123-57-7 fp32, 13 workers x 37 rows: 114 -> 18 us
 // (11 -> 3 launches); 784-10 fp32, 16 x 64: 22 -> 14 us; the 400-120-84-10 part of the CNN, 640 rows: 13 -> 2 launches,
-// 21 us for the row kernel between two events (28 us with FP32 FMAs for the bf16 products).
+// 17 us for the row kernel between two events (28 us with FP32 FMAs for the bf16 products).
 // Activations and deltas are rounded to the storage type where they are stored, sums are fp32 in a fixed order.
 #pragma once
 #include <algorithm>
@@ -30,7 +30,6 @@ constexpr int NW = 8;                    // compute warps of the row kernels
 constexpr int NT = NW * 32;
 constexpr int THREADS = NT + 32;         // and the warp that fetches the weights
 constexpr int MAX_STAGES = 8;
-constexpr int MMA_R = 16;                // rows per CTA of the bf16 kernel (one mma row tile)
 constexpr int MMA_NW = 15;               // its compute warps: with the fetching warp 512 threads of up to 128 registers
 constexpr int MMA_THREADS = MMA_NW * 32 + 32;
 
@@ -341,11 +340,11 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
     __syncwarp();
     refresh_next_durations(st, a.job, a.next_dur, a.dur_job, look);
   } else {
+    const int label = (tid < R && my_idx >= 0) ? a.labels[my_idx] : -1;       // stored when first needed
     // ------------------------------------------------------------------ input rows
     {
       const int in = a.dims[0];
       float* x = fs + a.act_off[0];
-      const int label = (tid < R && my_idx >= 0) ? a.labels[my_idx] : -1;
       const int rq = warp % RQ;                      // (RQ divides NW) four rows per warp
       const float* src[4];
 #pragma unroll
@@ -368,7 +367,6 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
           if (kb + u * KSTEP < in)
             *reinterpret_cast<float4*>(x + (size_t)rq * (in + 1) * 4 + (kb + u * KSTEP) * 4) = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
       }
-      if (tid < R) lab[tid] = label;
       for (int e = tid; e < L * R; e += NT) {         // the input of the bias row
         const int l = e / R, q = e % R / 4;
         fs[a.act_off[l] + (q * (a.dims[l] + 1) + a.dims[l]) * 4 + (e & 3)] = 1.f;
@@ -407,6 +405,7 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
         }
         *reinterpret_cast<float4*>(y + (size_t)q * y_plane + n * 4) = s;
       }
+      if (last && tid < R) lab[tid] = label;
       rows_sync();
     }
     // ------------------------------------------------------------------ loss and delta of the output layer: warp = row
@@ -483,42 +482,139 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
   rows_end(a, &gave_up);
 }
 
-// ---- bf16: the same with the warp-level tensor-core instruction (mma m16n8k16, bf16 in, fp32 accumulate), 16 rows per
-// CTA kept as [row][k] (pitch: a multiple of 16 plus 8 elements, zero-padded), 8-column tiles dealt to the warps.  The
-// weight fragments are read element by element: the widths of this class rarely give 16-byte rows.  (tcgen05 tiles
-// would be 128 rows; a round has a few hundred rows in groups of any size.)
+// ---- bf16: the same with the warp-level tensor-core instruction (mma m16n8k16, bf16 in, fp32 accumulate): the weights
+// are the row operand (16 columns of a layer, backward 16 of its inputs), the CTA's gradient rows the column operand, 8
+// or 16 kept as [row][k] (pitch: a multiple of 16 plus 8 elements, zero-padded).  Row i of an operand tile is column 2i of the
+// layer, row i + 8 column 2i + 1, so that even widths are read as 4-byte pairs and results stored as pairs; the widths of
+// this class rarely give the 16-byte rows of ldmatrix.  (tcgen05 tiles would be 128 rows; a round has a few hundred rows
+// in groups of any size.)  Bound by shared-memory reads of the weights and the latency of the layers' chain.
+// 400-120-84-10, 640 rows: 16.8 us with the rows as row operand and unrolled tiles, 12.7 us now (between launches).
 __device__ __forceinline__ uint32_t pair16(const __nv_bfloat16* p, int stride) {          // p[0] | p[stride] << 16
   const uint32_t lo = *reinterpret_cast<const unsigned short*>(p), hi = *reinterpret_cast<const unsigned short*>(p + stride);
   return lo | (hi << 16);
 }
-
-// rows [R][pitch] of shared memory -> rows of n elements
-__device__ __forceinline__ void copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, int pitch, int n, int warp, int lane) {
-  for (int rr = warp; rr < MMA_R; rr += MMA_NW) {
-    if ((n & 7) == 0) {
-      for (int k = lane * 8; k < n; k += 256) *reinterpret_cast<uint4*>(dst + (size_t)rr * n + k) = *reinterpret_cast<const uint4*>(src + rr * pitch + k);
-    } else {
-      for (int k = lane; k < n; k += 32) dst[(size_t)rr * n + k] = src[rr * pitch + k];
+// elements c and c + 1 of a row of n, clamped to the row (what lies behind it meets zeros)
+template <bool EVEN>
+__device__ __forceinline__ uint32_t pair_at(const __nv_bfloat16* row, int c, int n) {
+  if (EVEN) return *reinterpret_cast<const uint32_t*>(row + min(c, n - 2));
+  const int c0 = min(c, n - 1);
+  return pair16(row + c0, min(c + 1, n - 1) - c0);
+}
+// One tile of 16 layer columns over rows [0, nk) of a chunk (n: this lane's two columns): the operands of the next 32 rows
+// are read while these are multiplied.  Rows behind the last one meet zero activations.  RT: column tiles of 8 gradient
+// rows, `xt` bytes apart.  UN: unrolled, for weights that come in many chunks; code that runs once or twice per CTA is
+// bound by fetching its instructions and kept short instead (400-120-84-10, 640 rows: 16.7 us unrolled, 12.7 us).
+template <bool EVEN, int RT, bool UN>
+__device__ __forceinline__ void forward_tile(float (&acc)[RT][4], const __nv_bfloat16* w, uint32_t x, uint32_t xt, int n, int nk, int out, int t) {
+  uint32_t b[RT][4], p[8];
+  auto load = [&](int k) {
+#pragma unroll
+    for (int r = 0; r < RT; ++r) outl::ldsm4(x + r * xt + (uint32_t)k * 2u, b[r]);       // (columns behind the padding are not used)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = pair_at<EVEN>(w + min(k + 2 * t + (i >> 1) * 8 + (i & 1), nk - 1) * out, n, out);
+  };
+  auto multiply = [&](bool both) {
+    uint32_t af[2][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) af[u][i] = __byte_perm(p[4 * u + (i & 2)], p[4 * u + (i & 2) + 1], (i & 1) ? 0x7632 : 0x5410);
+#pragma unroll
+    for (int r = 0; r < RT; ++r) outl::mma16816_rn(acc[r], af[0], b[r][0], b[r][1]);
+    if (both)
+#pragma unroll
+      for (int r = 0; r < RT; ++r) outl::mma16816_rn(acc[r], af[1], b[r][2], b[r][3]);
+  };
+  int k = 0;
+  if (UN) {
+    const __nv_bfloat16* q = w + 2 * t * out;
+#pragma unroll 2
+    for (; k + 32 <= nk; k += 32) {
+#pragma unroll
+      for (int r = 0; r < RT; ++r) outl::ldsm4(x + r * xt + (uint32_t)k * 2u, b[r]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) p[i] = pair_at<EVEN>(q + ((i >> 1) * 8 + (i & 1)) * out, n, out);
+      multiply(true);
+      q += 32 * out;
     }
+    if (k < nk) {
+      load(k);
+      multiply(k + 16 < nk);
+    }
+    return;
+  }
+  load(0);
+#pragma unroll 1
+  for (; k < nk; k += 32) {
+    uint32_t af[2][4], c[RT][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) af[u][i] = __byte_perm(p[4 * u + (i & 2)], p[4 * u + (i & 2) + 1], (i & 1) ? 0x7632 : 0x5410);
+#pragma unroll
+    for (int r = 0; r < RT; ++r)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) c[r][i] = b[r][i];
+    if (k + 32 < nk) load(k + 32);
+#pragma unroll
+    for (int r = 0; r < RT; ++r) outl::mma16816_rn(acc[r], af[0], c[r][0], c[r][1]);
+    if (k + 16 < nk)
+#pragma unroll
+      for (int r = 0; r < RT; ++r) outl::mma16816_rn(acc[r], af[1], c[r][2], c[r][3]);
+  }
+}
+// the same backward: 16 weight rows, of which wa, wb are this lane's, over the layer's columns
+template <bool EVEN, int RT, bool UN>
+__device__ __forceinline__ void backward_tile(float (&acc)[RT][4], const __nv_bfloat16* wa, const __nv_bfloat16* wb, uint32_t d, uint32_t dt, int out, int t) {
+#pragma unroll UN ? 2 : 1
+  for (int n = 0; n < out; n += 32) {
+    uint32_t b[RT][4], p[8];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) outl::ldsm4(d + r * dt + (uint32_t)n * 2u, b[r]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = pair_at<EVEN>((i & 1) ? wb : wa, n + 2 * t + (i >> 1) * 8, out);
+    const uint32_t a0[4] = {p[0], p[1], p[2], p[3]}, a1[4] = {p[4], p[5], p[6], p[7]};
+#pragma unroll
+    for (int r = 0; r < RT; ++r) outl::mma16816(acc[r], a0, b[r][0], b[r][1]);
+    if (n + 16 < out)
+#pragma unroll
+      for (int r = 0; r < RT; ++r) outl::mma16816(acc[r], a1, b[r][2], b[r][3]);
   }
 }
 
-static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const __grid_constant__ RowsArgs a) {
+// rows [R][pitch] of shared memory -> rows of n elements: R = 8 two warps per row (one for the last), 16 one (two for the last)
+template <int R>
+__device__ __forceinline__ void copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, int pitch, int n, int warp, int lane) {
+  if (R == 16 && warp == 0) copy_rows<1>(dst + 15 * (size_t)n, src + 15 * pitch, pitch, n, 0, lane);      // (15 warps)
+  const int rr = warp % R, at = warp / R, of = R == 8 && rr + R < MMA_NW ? 2 : 1;
+  if ((n & 7) == 0) {
+#pragma unroll 1
+    for (int k = (at * 32 + lane) * 8; k < n; k += of * 256)
+      *reinterpret_cast<uint4*>(dst + (size_t)rr * n + k) = *reinterpret_cast<const uint4*>(src + rr * pitch + k);
+  } else {
+#pragma unroll 1
+    for (int k = at * 32 + lane; k < n; k += of * 32) dst[(size_t)rr * n + k] = src[rr * pitch + k];
+  }
+}
+
+template <int R, bool RESIDENT>
+__global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const __grid_constant__ RowsArgs a) {
   extern __shared__ __align__(128) unsigned char rsm[];
   __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES];
   __shared__ int gave_up;
-  __shared__ int lab[MMA_R];                         // label of each row, -1: padding
+  __shared__ int lab[R];                             // label of each row, -1: padding
   typedef __nv_bfloat16 T;
-  constexpr int R = MMA_R, NWM = MMA_NW;
+  constexpr int RT = R / 8, WPR = 16 / R, NWM = MMA_NW;
   weights_init(a, full, empty, &gave_up, NWM);       // before the wait: touches nothing of the kernels in front
   grid_dependency_sync();
   DevState* st = a.st;
   RoundInfo* ri = a.ri;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = (int)blockIdx.x * R;
+  const int my_row = warp / WPR;                     // two warps (of 16) or one fetch a row
   // one wave of loads (the grid covers the row capacity, so every address exists)
   const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[blockIdx.x];
-  const int my_idx = a.row_idx[r0 + warp];           // warp w fetches row w
+  const int my_idx = a.row_idx[r0 + my_row], lab_idx = tid < R ? a.row_idx[r0 + tid] : -1;
   if (status != ST_OK) return;
   const int look = (int)blockIdx.x * 32 < a.W ? (int)blockIdx.x * 32 + lane : a.W;
   if (r0 >= n_rows) {
@@ -531,213 +627,142 @@ static __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const _
   Weights W(a, rsm, full, empty, &gave_up);
   auto sync_compute = [] { asm volatile("bar.sync 1, %0;" ::"n"(NWM * 32) : "memory"); };
   const T* w_ring = (const T*)a.ring + (size_t)slot * a.slot_stride;
-  if (a.resident && tid == NWM * 32) W.produce(w_ring);
+  if (RESIDENT && tid == NWM * 32) W.produce(w_ring);
   __syncwarp();
+  const int label = lab_idx >= 0 ? a.labels[lab_idx] : -1;       // stored when first needed
   {
-    // ---------------------------------------------------------------- input row of this warp; zero padding columns
-    const int in = a.dims[0];
-    const T* src = (a.gather && my_idx < 0) ? nullptr : (const T*)a.X + (size_t)(a.gather ? my_idx : r0 + warp) * in;
-    const int label = (lane == 0 && my_idx >= 0) ? a.labels[my_idx] : -1;
-    T* x = ts + a.act_off[0] + warp * mma_pitch(in);
+    // ---------------------------------------------------------------- input row (part) of this warp; zero padding columns
+    const int in = a.dims[0], part = warp % WPR;
+    const T* src = (a.gather && my_idx < 0) ? nullptr : (const T*)a.X + (size_t)(a.gather ? my_idx : r0 + my_row) * in;
+    T* x = ts + a.act_off[0] + my_row * mma_pitch(in);
     if ((in & 7) == 0) {                              // rows on 16-byte boundaries
 #pragma unroll 4
-      for (int k = lane * 8; k < in; k += 256)
+      for (int k = (part * 32 + lane) * 8; k < in; k += 256 * WPR)
         *reinterpret_cast<uint4*>(x + k) = src ? *reinterpret_cast<const uint4*>(src + k) : make_uint4(0u, 0u, 0u, 0u);
     } else {
 #pragma unroll 8
-      for (int k = lane; k < in; k += 32) x[k] = src ? src[k] : (T)0.f;
+      for (int k = part * 32 + lane; k < in; k += 32 * WPR) x[k] = src ? src[k] : (T)0.f;
     }
-    if (lane == 0) lab[warp] = label;
-    for (int l = 0; l <= L; ++l) {
-      const int n = a.dims[l], p = mma_pitch(n);      // at most 8 + 15 padding columns
-      if (n + lane < p) ts[(l < L ? a.act_off[l] : a.out_off) + warp * p + n + lane] = (T)0.f;
+    if (part == 0) {
+#pragma unroll 1
+      for (int l = 0; l <= L; ++l) {
+        const int n = a.dims[l], p = mma_pitch(n);    // at most 8 + 15 padding columns
+        if (n + lane < p) ts[(l < L ? a.act_off[l] : a.out_off) + my_row * p + n + lane] = (T)0.f;
+      }
     }
   }
   __syncthreads();
 
   if (warp == NWM) {
-    if (!a.resident && lane == 0) W.produce(w_ring);
+    if (!RESIDENT && lane == 0) W.produce(w_ring);
     __syncwarp();
     refresh_next_durations(st, a.job, a.next_dur, a.dur_job, look);
   } else {
-    const int sel_row = lane & 15, sel_col = (lane >> 4) * 8;         // ldmatrix addresses of an A tile
+    const int sel = (lane & 7), sel_col = (lane >> 3) * 8;            // ldmatrix addresses: two inner steps of 16 at once
     // ------------------------------------------------------------------ forward: warp takes column tiles warp, warp + 15, ...
     float* logits = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(ts) + a.red_off);     // [R][C + 1]
     for (int l = 0; l < L; ++l) {
       const int in = a.dims[l], out = a.dims[l + 1], rpc = a.rpc[l], pitch = mma_pitch(in);
-      const bool last = l == L - 1;
-      const uint32_t a_base = outl::s_u32(ts + a.act_off[l] + sel_row * pitch + sel_col);
-      // streamed weights come once, so a warp finishes all its tiles chunk by chunk (1024 columns = 9 tiles per warp)
-      constexpr int TP = 3, PASSES = 3;
-      const int n_ct = (out + 7) >> 3;
-      float acc[PASSES * TP][4];
+      const bool last = l == L - 1, even = (out & 1) == 0;
+      const uint32_t x_base = outl::s_u32(ts + a.act_off[l] + sel * pitch + sel_col);
+      const int n_ct = (out + 15) >> 4;
+      auto tile = [&](float (&acc)[RT][4], const T* w, int ct, int k0, int nk) {
+        if (even) forward_tile<true, RT, !RESIDENT>(acc, w, x_base + 2u * (uint32_t)k0, 16u * pitch, ct * 16 + 2 * g, nk, out, t);
+        else forward_tile<false, RT, !RESIDENT>(acc, w, x_base + 2u * (uint32_t)k0, 16u * pitch, ct * 16 + 2 * g, nk, out, t);
+      };
+      auto finish = [&](const float (&acc)[RT][4], const T* bias, int ct) {
+        const int n = ct * 16 + 2 * g;
+        if (n >= out) return;
+        const bool two = n + 1 < out;
+        const float b0 = __bfloat162float(bias[n]), b1 = two ? __bfloat162float(bias[n + 1]) : 0.f;
 #pragma unroll
-      for (int c = 0; c < PASSES * TP; ++c)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[c][i] = 0.f;
-      for (int k0 = 0; k0 < in + 1; k0 += rpc) {
+        for (int h = 0; h < 2 * RT; ++h) {            // gradient row 2t + h % 2 of column tile h / 2
+          const float v0 = acc[h >> 1][h & 1] + b0, v1 = acc[h >> 1][2 + (h & 1)] + b1;
+          const int rr = 8 * (h >> 1) + 2 * t + (h & 1);
+          if (last) {
+            logits[rr * (out + 1) + n] = v0;
+            if (two) logits[rr * (out + 1) + n + 1] = v1;
+          } else {                                    // (the column behind an odd last one is padding and stays zero)
+            *reinterpret_cast<uint32_t*>(ts + a.act_off[l + 1] + rr * mma_pitch(out) + n) =
+                outl::pack_bf16(fmaxf(v0, 0.f), two ? fmaxf(v1, 0.f) : 0.f);
+          }
+        }
+      };
+      if (RESIDENT) {
         const T* w = reinterpret_cast<const T*>(W.take(l));
-        const int nk = min(rpc, in - k0);             // weight rows of this chunk (the bias row apart)
+#pragma unroll 1
+        for (int ct = warp; ct < n_ct; ct += NWM) {
+          float acc[RT][4] = {};
+          tile(acc, w, ct, 0, in);
+          finish(acc, w + in * out, ct);
+        }
+      } else {
+        // streamed weights come once, so a warp takes all its tiles along, chunk by chunk (1024 columns: 5 tiles per warp)
+        constexpr int TP = 5;
+        float acc[TP][RT][4] = {};
+#pragma unroll 1
+        for (int k0 = 0; k0 < in + 1; k0 += rpc) {
+          const T* w = reinterpret_cast<const T*>(W.take(l));
+          const int nk = min(rpc, in - k0);           // weight rows of this chunk (the bias row apart)
 #pragma unroll
-        for (int pass = 0; pass < PASSES; ++pass) {
-          const int ct0 = warp + pass * TP * NWM;
-          if (ct0 >= n_ct) break;
-          const int n_here = min(TP, (n_ct - ct0 + NWM - 1) / NWM);
-          const T* wp[TP];                            // element (row 2t, column g) of each tile
-#pragma unroll
-          for (int c = 0; c < TP; ++c) wp[c] = w + 2 * t * out + min((ct0 + c * NWM) * 8 + g, out - 1);
-          const int step = 16 * out;
-          int k = 0;
-          for (; k + 64 <= nk; k += 64) {             // four inner steps: their row operands first
-            uint32_t af[4][4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) outl::ldsm4(a_base + (uint32_t)(k0 + k + 16 * u) * 2u, af[u]);
+          for (int c = 0; c < TP; ++c)
+            if (nk > 0 && warp + c * NWM < n_ct) tile(acc[c], w, warp + c * NWM, k0, nk);
+          if (k0 + rpc >= in + 1) {                   // the last chunk ends with the bias row
 #pragma unroll
             for (int c = 0; c < TP; ++c)
-              if (c < n_here) {
-                uint32_t b[4][2];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  b[u][0] = pair16(wp[c] + u * step, out);
-                  b[u][1] = pair16(wp[c] + u * step + 8 * out, out);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) outl::mma16816_rn(acc[pass * TP + c], af[u], b[u][0], b[u][1]);
-                wp[c] += 4 * step;
-              }
+              if (warp + c * NWM < n_ct) finish(acc[c], w + nk * out, warp + c * NWM);
           }
-          for (; k + 16 <= nk; k += 16) {
-            uint32_t af[4];
-            outl::ldsm4(a_base + (uint32_t)(k0 + k) * 2u, af);
-#pragma unroll
-            for (int c = 0; c < TP; ++c) {
-              if (c < n_here) outl::mma16816_rn(acc[pass * TP + c], af, pair16(wp[c], out), pair16(wp[c] + 8 * out, out));
-              wp[c] += step;
-            }
-          }
-          if (k < nk) {
-            // rows behind the layer's last one meet zero activations: any finite weight will do
-            uint32_t af[4];
-            outl::ldsm4(a_base + (uint32_t)(k0 + k) * 2u, af);
-            const int lastr = nk - 1 - k;
-            const int ka = min(2 * t, lastr), kb = min(2 * t + 1, lastr), kc = min(2 * t + 8, lastr), kd = min(2 * t + 9, lastr);
-#pragma unroll
-            for (int c = 0; c < TP; ++c)
-              if (c < n_here) {
-                const T* q = wp[c] - 2 * t * out;
-                outl::mma16816_rn(acc[pass * TP + c], af, pair16(q + ka * out, (kb - ka) * out), pair16(q + kc * out, (kd - kc) * out));
-              }
-          }
+          W.give(lane);
         }
-        if (k0 + rpc >= in + 1) {                     // the last chunk ends with the bias row
-          const T* bias = w + (in - k0) * out;
-#pragma unroll
-          for (int c = 0; c < PASSES * TP; ++c) {
-            const int n = (warp + c * NWM) * 8 + 2 * t;
-            if (n < out) {
-              const float b0 = __bfloat162float(bias[n]), b1 = n + 1 < out ? __bfloat162float(bias[n + 1]) : 0.f;
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const float v0 = acc[c][2 * h] + b0, v1 = acc[c][2 * h + 1] + b1;
-                const int rr = g + 8 * h;
-                if (last) {
-                  logits[rr * (out + 1) + n] = v0;
-                  if (n + 1 < out) logits[rr * (out + 1) + n + 1] = v1;
-                } else {                              // (the column behind an odd last one is padding and stays zero)
-                  *reinterpret_cast<uint32_t*>(ts + a.act_off[l + 1] + rr * mma_pitch(out) + n) =
-                      outl::pack_bf16(fmaxf(v0, 0.f), n + 1 < out ? fmaxf(v1, 0.f) : 0.f);
-                }
-              }
-            }
-          }
-        }
-        W.give(lane);
       }
+      if (last && tid < R) lab[tid] = label;
       sync_compute();
-      if (!last) copy_rows((T*)a.act[l + 1] + (size_t)r0 * out, ts + a.act_off[l + 1], mma_pitch(out), out, warp, lane);
+      if (!last) copy_rows<R>((T*)a.act[l + 1] + (size_t)r0 * out, ts + a.act_off[l + 1], mma_pitch(out), out, warp, lane);
     }
     // ------------------------------------------------------------------ loss and delta of the output layer
     {
       const int C = a.dims[L];
       T* dl = ts + a.out_off;
-      const float sa = sa_slot_weight(st, ri->t, slot);
       for (int rr = warp; rr < R; rr += NWM) {
         const float* z = logits + rr * (C + 1);
-        const float2 d = row_softmax<T>(a, lane < C ? z[lane] : 0.f, lane + 32 < C ? z[lane + 32] : 0.f, r0 + rr, lab[rr], sa, lane);
+        const float2 d = row_softmax<T>(a, lane < C ? z[lane] : 0.f, lane + 32 < C ? z[lane + 32] : 0.f, r0 + rr, lab[rr],
+                                        sa_slot_weight(st, ri->t, slot), lane);
         T* gd = (T*)a.delta[L] + (size_t)(r0 + rr) * C;
         if (lane < C) { dl[rr * mma_pitch(C) + lane] = __float2bfloat16_rn(d.x); gd[lane] = __float2bfloat16_rn(d.x); }
         if (lane + 32 < C) { dl[rr * mma_pitch(C) + lane + 32] = __float2bfloat16_rn(d.y); gd[lane + 32] = __float2bfloat16_rn(d.y); }
       }
     }
     sync_compute();
-    // ------------------------------------------------------------------ backward: tiles of 8 weight rows (= input columns)
+    // ------------------------------------------------------------------ backward: tiles of 16 weight rows (= input columns)
     for (int l = L - 1; l >= (a.want_d0 ? 0 : 1); --l) {
       const int in = a.dims[l], out = a.dims[l + 1], rpc = a.rpc[l], pitch = mma_pitch(in);
       const T* dl = ts + (l == L - 1 ? a.out_off : a.act_off[l + 1]);
-      const int dp = mma_pitch(out);
-      const uint32_t a_base = outl::s_u32(dl + sel_row * dp + sel_col);
+      const uint32_t d_base = outl::s_u32(dl + sel * mma_pitch(out) + sel_col);
       T* h = ts + a.act_off[l];
       const bool even = (out & 1) == 0;
       for (int k0 = 0; k0 < in + 1; k0 += rpc) {
         const T* w = reinterpret_cast<const T*>(W.take(l));
         const int nk = min(rpc, in - k0);
-        constexpr int TP = 4;
-        for (int m0 = warp * 8; m0 < nk; m0 += NWM * 8 * TP) {
-          const int n_here = min(TP, (nk - m0 + NWM * 8 - 1) / (NWM * 8));
-          float acc[TP][4];
-          const T* wm[TP];                            // weight row g of each tile
+#pragma unroll 1
+        for (int m0 = warp * 16; m0 < nk; m0 += NWM * 16) {
+          float acc[RT][4] = {};
+          const int mi = m0 + 2 * g;                  // this lane's weight rows: mi and mi + 1
+          const T *wa = w + min(mi, nk - 1) * out, *wb = w + min(mi + 1, nk - 1) * out;
+          if (even) backward_tile<true, RT, !RESIDENT>(acc, wa, wb, d_base, 16u * mma_pitch(out), out, t);
+          else backward_tile<false, RT, !RESIDENT>(acc, wa, wb, d_base, 16u * mma_pitch(out), out, t);
+          if (mi < nk) {                              // (the element behind an odd last one is padding and stays zero)
 #pragma unroll
-          for (int c = 0; c < TP; ++c) {
-            wm[c] = w + min(m0 + c * NWM * 8 + g, nk - 1) * out;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[c][i] = 0.f;
-          }
-          int n = 0;
-          if (even) {                                 // pairs are 4-byte aligned
-#pragma unroll 4
-            for (; n + 16 <= out; n += 16) {
-              uint32_t af[4];
-              outl::ldsm4(a_base + (uint32_t)n * 2u, af);
-#pragma unroll
-              for (int c = 0; c < TP; ++c)
-                if (c < n_here)
-                  outl::mma16816(acc[c], af, *reinterpret_cast<const uint32_t*>(wm[c] + n + 2 * t), *reinterpret_cast<const uint32_t*>(wm[c] + n + 2 * t + 8));
-            }
-          } else {
-#pragma unroll 2
-            for (; n + 16 <= out; n += 16) {
-              uint32_t af[4];
-              outl::ldsm4(a_base + (uint32_t)n * 2u, af);
-#pragma unroll
-              for (int c = 0; c < TP; ++c)
-                if (c < n_here) outl::mma16816(acc[c], af, pair16(wm[c] + n + 2 * t, 1), pair16(wm[c] + n + 2 * t + 8, 1));
-            }
-          }
-          if (n < out) {                              // columns behind the last one meet zero deltas
-            uint32_t af[4];
-            outl::ldsm4(a_base + (uint32_t)n * 2u, af);
-            const int na = min(n + 2 * t, out - 1), nb = min(n + 2 * t + 1, out - 1), nc = min(n + 2 * t + 8, out - 1), nd = min(n + 2 * t + 9, out - 1);
-#pragma unroll
-            for (int c = 0; c < TP; ++c)
-              if (c < n_here) outl::mma16816(acc[c], af, pair16(wm[c] + na, nb - na), pair16(wm[c] + nc, nd - nc));
-          }
-#pragma unroll
-          for (int c = 0; c < TP; ++c) {
-            const int mi = m0 + c * NWM * 8 + 2 * t;
-            if (mi < nk) {                            // (the element behind an odd last one is padding and stays zero)
-#pragma unroll
-              for (int h2 = 0; h2 < 2; ++h2) {
-                uint32_t* hp = reinterpret_cast<uint32_t*>(h + (g + 8 * h2) * pitch + k0 + mi);
-                const float2 hv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(hp));
-                *hp = outl::pack_bf16(hv.x > 0.f ? acc[c][2 * h2] : 0.f, hv.y > 0.f ? acc[c][2 * h2 + 1] : 0.f);
-              }
+            for (int q = 0; q < 2 * RT; ++q) {
+              uint32_t* hp = reinterpret_cast<uint32_t*>(h + (8 * (q >> 1) + 2 * t + (q & 1)) * pitch + k0 + mi);
+              const float2 hv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(hp));
+              *hp = outl::pack_bf16(hv.x > 0.f ? acc[q >> 1][q & 1] : 0.f, hv.y > 0.f ? acc[q >> 1][2 + (q & 1)] : 0.f);
             }
           }
         }
         W.give(lane);
       }
       sync_compute();
-      copy_rows((T*)a.delta[l] + (size_t)r0 * in, h, pitch, in, warp, lane);
+      copy_rows<R>((T*)a.delta[l] + (size_t)r0 * in, h, pitch, in, warp, lane);
     }
   }
   rows_end(a, &gave_up);

@@ -267,6 +267,9 @@ def test_local_sgd_steps_multi_layer_network_fma_paths(dims, dtype, W, B, U, K0,
     (inputs.MLP, (128, 256, 48, 10), inputs.BF16, 7, 20, gpu.FLAG_NO_TENSOR_CORES),     # 16-byte rows
     (inputs.MLP, (700, 301, 77, 10), inputs.BF16, 6, 17, 0),     # bf16, streamed
     (inputs.MLP, (90, 1001, 10), inputs.BF16, 4, 12, 0),         # 126 column tiles
+    (inputs.MLP, (50, 31, 18, 2), inputs.BF16, 40, 33, 0),       # bf16, 16 rows per CTA, resident; one class pair
+    (inputs.MLP, (700, 301, 77, 10), inputs.BF16, 40, 33, 0),    # ... streamed
+    (inputs.MLP, (17, 16, 33, 3), inputs.BF16, 5, 7, 0),         # bf16, inner sizes around one and two steps of 16
 ])
 def test_row_kernels(kind, dims, dtype, W, B, flags):
     """Networks through the row kernels: rows per CTA, columns per lane, resident and streamed weights.  Four rounds:
