@@ -772,6 +772,7 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const __grid_c
 constexpr int GT = 32;                   // features x outputs per tile of grad_step_kernel
 constexpr int GK = 64;                   // rows per pipeline step
 constexpr int GP = GT + 4;               // shared-memory pitch
+constexpr int MP = GT + 8;               // ... bf16 (five 16-byte units: ldmatrix reads without bank conflicts)
 
 struct StepArgs {
   const DevState* st;
@@ -794,19 +795,21 @@ struct StepArgs {
   cmma::FragMap frag;                    // region i = convolution block i: the weights also as operand fragments
 };
 
-__device__ __forceinline__ float as_float(float v) { return v; }
-__device__ __forceinline__ float as_float(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-// Four groups of 64 threads take 16 rows of a 64-row step each (4 x 4 sums per thread: two 16-byte shared-memory reads
-// for eight packed FMAs); two steps' rows are in registers on the way.  Groups are added in order, each CTA of a cluster
+// Four groups of 64 threads take 16 rows of a 64-row step each (fp32: 4 x 4 sums per thread, two 16-byte shared-memory
+// reads for eight packed FMAs, two steps' rows in registers on the way; bf16: matrix instructions with the products added
+// in fp32: the FMA form was bound by shared-memory reads; 201-133-10, 4096 rows: 60.7 -> 52.8 us a round, CNN 76.9 -> 75.5).  Groups are added in order, each CTA of a cluster
 // hands its sums to the owner of their share, which adds them in order and applies Eq. 3.
 // Bound by the chain of dependent latencies (indices, rows, exchange), so: the tile is found before the wait for the
 // kernels in front, indices come with the round's sizes in one wave of loads, the weights a CTA updates are fetched
 // before its sums exist.  784 x 10 fp32, 1024 rows: 6.4 -> 4 us
 // with the row kernel's loads done likewise (19.3 -> 14.4 us a round); 300-123-57-7, 481 rows: 27.7 -> 18.3 us a round.
 template <typename T, int DEPTH>
-__global__ void __launch_bounds__(256, DEPTH == 2 ? 2 : 3) grad_step_kernel(const __grid_constant__ StepArgs a) {
-  __shared__ __align__(16) float As[2][GK][GP], Ds[2][GK][GP];
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 3) grad_step_kernel(const __grid_constant__ StepArgs a) {
+  constexpr bool MMA = sizeof(T) == 2;
+  constexpr int P = MMA ? MP : GP;
+  __shared__ __align__(16) T tiles[4][GK][P];        // two stages of inputs, two of deltas
+  T (*As)[GK][P] = tiles, (*Ds)[GK][P] = tiles + 2;
+  float (*red)[GT * GT] = reinterpret_cast<float (*)[GT * GT]>(tiles);     // sums of the four groups, at the end
   __shared__ float box[GT * GT];                     // sums of this CTA's share: [CTA of the cluster][share]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_tiles = a.first_tile[a.n_layers];
@@ -836,7 +839,7 @@ __global__ void __launch_bounds__(256, DEPTH == 2 ? 2 : 3) grad_step_kernel(cons
   T* dst = (T*)a.ring + (size_t)slot * a.d_pad;
   if ((int)blockIdx.x >= n_tiles * a.Q) {
     // region block: 32 parameters x 8 lanes over the chunks, fixed order
-    float* red = &As[0][0][0];
+    float* part = &red[0][0];
     const int rb = (int)blockIdx.x - n_tiles * a.Q;
     const int q = (a.n_regions > 1 && rb >= a.region[1].first_block) ? 1 : 0;
     const StepArgs::Region& G = a.region[q];
@@ -847,12 +850,12 @@ __global__ void __launch_bounds__(256, DEPTH == 2 ? 2 : 3) grad_step_kernel(cons
 #pragma unroll 8
       for (int c = warp; c < n_chunks; c += 8) acc += G.part[(size_t)c * G.len + j];
     }
-    red[warp * 33 + lane] = acc;
+    part[warp * 33 + lane] = acc;
     __syncthreads();
     if (warp == 0 && j < G.len) {
       float tot = 0.f;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) tot += red[c * 33 + lane];
+      for (int c = 0; c < 8; ++c) tot += part[c * 33 + lane];
       const size_t e = G.off + (size_t)j;
       const float m = fmaf(-step, tot, a.master[e]);
       a.master[e] = m;
@@ -893,31 +896,42 @@ __global__ void __launch_bounds__(256, DEPTH == 2 ? 2 : 3) grad_step_kernel(cons
     o[i] = mine ? a.w_off[l] + (size_t)mm * out + nn : (size_t)-1;
     w[i] = mine ? a.master[o[i]] : 0.f;
   }
-  f32x2 acc[4][2];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0ull;
   const int kg = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
+  f32x2 acc[MMA ? 1 : 4][2] = {};                    // fp32: features 4 ty .., outputs 4 tx ..
+  float acm[MMA ? 4 : 1][4] = {};                    // bf16: features 16 (warp & 1) .., four 8-output tiles
   auto one_step = [&](int s, int buf, int& idx, Rows& p) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const bool ok = (p.ok >> i & 1u) != 0;
-      As[buf][8 * i + warp][lane] = as_float(m < in ? (ok ? p.a[i] : zero) : m == in ? one : zero);       // row `in`: the bias
-      Ds[buf][8 * i + warp][lane] = as_float(ok && n < out ? p.d[i] : zero);
+      As[buf][8 * i + warp][lane] = m < in ? (ok ? p.a[i] : zero) : m == in ? one : zero;       // row `in`: the bias
+      Ds[buf][8 * i + warp][lane] = ok && n < out ? p.d[i] : zero;
     }
     __syncthreads();
     if (s + DEPTH * Q < n_steps) {
       load(s + DEPTH * Q, idx, p);
       idx = load_idx(s + 2 * DEPTH * Q);
     }
+    if constexpr (MMA) {
+      uint32_t af[4], b[4];
+      const int k0 = kg * 16, x = lane & 7, h = lane >> 3;
+      outl::ldsm4t(outl::s_u32(&As[buf][k0 + (h >> 1) * 8 + x][(warp & 1) * 16 + (h & 1) * 8]), af);
 #pragma unroll
-    for (int k = 0; k < GK / 4; ++k) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[buf][kg * (GK / 4) + k][4 * ty]);
-      const ulonglong2 dv = *reinterpret_cast<const ulonglong2*>(&Ds[buf][kg * (GK / 4) + k][4 * tx]);
-      const f32x2 p[4] = {lsqp::pack2(av.x, av.x), lsqp::pack2(av.y, av.y), lsqp::pack2(av.z, av.z), lsqp::pack2(av.w, av.w)};
+      for (int q = 0; q < 2; ++q) {
+        outl::ldsm4t(outl::s_u32(&Ds[buf][k0 + (h & 1) * 8 + x][16 * q + (h >> 1) * 8]), b);
+        outl::mma16816_rn(acm[2 * q], af, b[0], b[1]);
+        outl::mma16816_rn(acm[2 * q + 1], af, b[2], b[3]);
+      }
+    } else {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        lsqp::ffma2(acc[i][0], p[i], dv.x);
-        lsqp::ffma2(acc[i][1], p[i], dv.y);
+      for (int k = 0; k < GK / 4; ++k) {
+        const float4 av = *reinterpret_cast<const float4*>(&As[buf][kg * (GK / 4) + k][4 * ty]);
+        const ulonglong2 dv = *reinterpret_cast<const ulonglong2*>(&Ds[buf][kg * (GK / 4) + k][4 * tx]);
+        const f32x2 p[4] = {lsqp::pack2(av.x, av.x), lsqp::pack2(av.y, av.y), lsqp::pack2(av.z, av.z), lsqp::pack2(av.w, av.w)};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          lsqp::ffma2(acc[i][0], p[i], dv.x);
+          lsqp::ffma2(acc[i][1], p[i], dv.y);
+        }
       }
     }
   };
@@ -928,16 +942,23 @@ __global__ void __launch_bounds__(256, DEPTH == 2 ? 2 : 3) grad_step_kernel(cons
   }
   if (Q > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");       // (peers have started: see below)
   __syncthreads();
-  float* red = &As[0][0][0];                         // [4][GT][GT]
+  if constexpr (MMA) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    *reinterpret_cast<ulonglong2*>(red + (size_t)kg * GT * GT + (4 * ty + i) * GT + 4 * tx) = make_ulonglong2(acc[i][0], acc[i][1]);
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        *reinterpret_cast<float2*>(&red[kg][(16 * (warp & 1) + (lane >> 2) + 8 * h) * GT + 8 * q + 2 * (lane & 3)]) = make_float2(acm[q][2 * h], acm[q][2 * h + 1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<ulonglong2*>(&red[kg][(4 * ty + i) * GT + 4 * tx]) = make_ulonglong2(acc[i][0], acc[i][1]);
+  }
   __syncthreads();
   if (Q > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int e = tid + 256 * i;
-    const float v = (red[e] + red[GT * GT + e]) + (red[2 * GT * GT + e] + red[3 * GT * GT + e]);
+    const float v = (red[0][e] + red[1][e]) + (red[2][e] + red[3][e]);
     if (Q > 1) {
       const int owner = e >> (10 - a.q_shift);       // (GT x GT = 2^10)
       asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(tc::map_to_cta(tc::smem_u32(box + rank * share + (e & (share - 1))), (uint32_t)owner)), "f"(v) : "memory");
