@@ -239,20 +239,26 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     const u64 T_end = T_end0;
     if (net) {
       // per-worker mean of the per-sample losses: TPW neighbouring threads share a worker, each
-      // adds every TPW-th row (independent loads), then the TPW partial sums are added by a
+      // adds every TPW-th row (eight loads at a time: with a runtime division and sixteen unrolled loads whose remainder ran
+      // this was 3800 cycles of 12000 for 16 workers x 64 rows, now 1700), then the TPW partial sums are added by a
       // fixed shuffle tree
       sh.row0[tid] = my_row0;
       __syncthreads();
-      int kp = 32;
-      while (kp < K) kp <<= 1;
-      const int tpw = min(32, NT / kp);
-      const int i = tid / tpw, sub = tid - i * tpw;
+      const int lg_k = max(5, 32 - __clz(K - 1)), lg_tpw = min(5, 31 - __clz(NT) - lg_k);      // (K >= 1; K = 1: clz(0) = 32)
+      const int tpw = 1 << lg_tpw, i = tid >> lg_tpw, sub = tid & (tpw - 1);
       float acc = 0.f;
       if (i < K) {
         const float* rl = a.row_loss + sh.row0[i];
-#pragma unroll 16
-        for (int b = sub; b < B; b += tpw) acc += rl[b];
+#pragma unroll 1
+        for (int b = sub; b < B; b += 8 * tpw) {
+          float x[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) x[u] = b + u * tpw < B ? rl[b + u * tpw] : 0.f;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) acc += x[u];
+        }
       }
+#pragma unroll 1
       for (int o = tpw >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       if (i < K && sub == 0) sh.lossv[i] = __fdiv_rn(acc, (float)B);
       __syncthreads();
