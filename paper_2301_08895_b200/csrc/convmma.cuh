@@ -16,7 +16,7 @@
 // beside the ring by the Eq. 3 kernel, so that a CTA copies them instead of gathering 2-byte elements.
 // FP32-FMA kernels with one CTA per row spent 315 us of a 640-row round of the 32 x 32 x 3 network here (5 % of the
 // FMA peak, bound by shared-memory reads per FMA).  These: 16 us forward, 37 us backward; bound by the shared-memory bytes
-// of the operand fragments (about 5000 cycles of reads per row backward) and the latency of their chains.
+// of the operand fragments (7000 shared-memory wavefronts per row backward) and the latency of their chains.
 #pragma once
 #include "common.cuh"
 #include "outlayer.cuh"
