@@ -599,6 +599,8 @@ __global__ void __launch_bounds__(NT, 3) conv_bwd_mma_kernel(const __grid_consta
       for (int i = 0; i < 2; ++i)
         if (8 * warp + 2 * t + i < y.Co) dst[K2 * y.Co + 8 * warp + 2 * t + i] = s2[i];
   }
+  // a CTA whose rows are all padding has not waited for its copies yet: they must not land on the sums below
+  fetch_wait();
   __syncthreads();
   constexpr int RW = (16 * MT1 + 1) * 8;              // floats per warp: [rows and bias][8 channels]
   float* red = reinterpret_cast<float*>(cs);

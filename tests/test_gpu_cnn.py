@@ -65,6 +65,29 @@ def test_cnn_tensor_core_shapes(conv, fc, W, B):
     compare_with_oracle(cfg, X, y, w0, 8, TOL_BF16, forced=True, loss_tol=5e-2)
 
 
+@pytest.mark.parametrize("conv,fc,W,B", [
+    ((16, 16, 1, 5, 6, 16), (20, 10), 3, 9),          # 27 rows of 32: two of the row pairs are padding
+    ((14, 14, 1, 3, 8, 16), (20, 10), 5, 33),         # 165 rows of 168: one pair
+    ((18, 18, 2, 3, 7, 9), (30, 21, 10), 6, 10),      # 60 rows of 64
+    ((20, 20, 1, 5, 6, 16), (12, 10), 5, 1),          # 5 rows of 8
+])
+def test_cnn_row_pairs_that_are_all_padding(conv, fc, W, B):
+    """Small images, whose copied operands lie where a CTA of the backward kernel forms its sums: a pair of padding rows
+    adds nothing to the first block's gradient, in every repetition."""
+    cfg = _cnn_cfg(conv, fc, inputs.BF16, W, B, W, 0, PARETO, lr=0.05)
+    X, y, w0 = _problem(cfg)
+    rows, orows, err, o = compare_with_oracle(cfg, X, y, w0, 2, TOL_BF16, forced=True, loss_tol=5e-2)
+    first = None
+    for _ in range(6):
+        _, params = gpu_run(cfg, X, y, w0, 2)
+        first = params if first is None else first
+        assert np.array_equal(params.view(np.uint32), first.view(np.uint32))
+    from helpers import layer_blocks
+    for name, sl in layer_blocks(cfg.kind, cfg.dims, cfg.conv)[:2]:
+        step, ref = first[sl].astype(np.float64) - w0[sl], o.w[sl] - w0[sl]
+        assert np.linalg.norm(step - ref) <= 0.1 * np.linalg.norm(ref), name
+
+
 @pytest.mark.parametrize("conv,fc,W,B", [((14, 14, 2, 3, 3, 4), (7, 6, 5), 6, 10),
                                           ((32, 32, 3, 5, 6, 16), (120, 84, 10), 8, 32)])
 def test_cnn_gradient_of_one_round_block_by_block(conv, fc, W, B):
