@@ -304,8 +304,8 @@ class Context:
 
 
 def _raw_stream(torch, stream, X):
-    """cudaStream_t of `stream`, or of the current stream of X's device (without building a Stream object for it)."""
-    return stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(X.get_device())
+    """cudaStream_t of `stream`, or of the current stream of X's device (which refuses an X that is not on a GPU)."""
+    return (stream if stream is not None else torch.cuda.current_stream(X.device)).cuda_stream
 
 
 def lsq_gradient(X, y, w, idx, g_out, loss_out, scratch, stream=None):

@@ -139,3 +139,26 @@ def test_null_context_calls():
     assert l.abs_save_state(None, None, 0, None) == gpu.EINVAL
     assert l.abs_restore_state(None, None, 0) == gpu.EINVAL
     assert l.abs_destroy(None) == gpu.OK
+
+
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_least_squares_operation_refuses_host_tensors(monkeypatch, noalloc):
+    """A host X has no stream: the call raises before any pointer reaches the library."""
+    import torch
+    reached = []
+
+    class Lib:
+        def __getattr__(self, name):
+            return lambda *args: reached.append(name) or 0
+    monkeypatch.setattr(gpu, "_lib", Lib())
+    monkeypatch.setattr(torch.cuda, "_lazy_init", lambda: None)      # (no device here)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 0, raising=False)
+    X, y, w = torch.zeros(8, 4), torch.zeros(8), torch.zeros(4)
+    idx = torch.zeros(2, 3, dtype=torch.int32)
+    g, loss, scratch = torch.zeros(4), torch.zeros(2), torch.zeros(8)
+    with pytest.raises(ValueError):
+        if noalloc:
+            gpu.lsq_gradient_noalloc(X, y, w, idx, g, loss)
+        else:
+            gpu.lsq_gradient(X, y, w, idx, g, loss, scratch)
+    assert reached == []
