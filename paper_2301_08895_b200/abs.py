@@ -237,11 +237,9 @@ class Context:
         a = dict(K=np.empty(n, np.int32), n_restart=np.empty(n, np.int32),
                  theta=np.empty(n, np.int32), T_end=np.empty(n, np.uint64),
                  loss_mean=np.empty(n, np.float32), comm=np.empty(n, np.uint64),
-                 sel_off=np.zeros(n + 1, np.int64), rst_off=np.zeros(n + 1, np.int64))
-        # one block for the per-arrival arrays: large blocks come on huge pages, and first touches of 4 KB pages cost more
-        # than the copy (500 rounds of 1024 workers: 3.0 ms as four arrays, 1.8 ms as one)
-        block = np.empty((4, n * W), np.int32)
-        a.update(sel_id=block[0], sel_tau=block[1], sel_loss=block[2].view(np.float32), rst_id=block[3])
+                 sel_off=np.zeros(n + 1, np.int64), rst_off=np.zeros(n + 1, np.int64),
+                 sel_id=np.empty(n * W, np.int32), sel_tau=np.empty(n * W, np.int32),
+                 sel_loss=np.empty(n * W, np.float32), rst_id=np.empty(n * W, np.int32))
         t = Trace()
         for k, v in a.items():
             setattr(t, k, v.ctypes.data)

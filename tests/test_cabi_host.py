@@ -162,3 +162,32 @@ def test_least_squares_operation_refuses_host_tensors(monkeypatch, noalloc):
         else:
             gpu.lsq_gradient(X, y, w, idx, g, loss, scratch)
     assert reached == []
+
+
+def test_trace_arrays_do_not_hold_each_other(monkeypatch):
+    """An array of the trace that is kept keeps its own storage alive and none of the others'."""
+    n, W = 6, 5
+
+    class Lib:
+        def abs_get_trace(self, ctx, first, rounds, ref):
+            t = ref._obj
+            C.cast(t.sel_off, C.POINTER(C.c_int64))[rounds] = 17
+            C.cast(t.rst_off, C.POINTER(C.c_int64))[rounds] = 3
+            return 0
+
+        def abs_destroy(self, ctx):
+            return 0
+    monkeypatch.setattr(gpu, "_lib", Lib())
+    ctx = gpu.Context.__new__(gpu.Context)
+    ctx.W, ctx._ctx = W, C.c_void_p(None)
+    tr = ctx.get_trace(0, n)
+    names = ("sel_id", "sel_tau", "sel_loss", "rst_id")
+    assert [len(tr[k]) for k in names] == [17, 17, 17, 3]
+    owners = []
+    for k in names:
+        a = tr[k]
+        while a.base is not None:
+            a = a.base
+        assert a.nbytes <= 4 * n * W, k
+        owners.append(id(a))
+    assert len(set(owners)) == 4
