@@ -86,7 +86,8 @@ extern "C" {
 #define ABS_T_GAMMA        4    /* shift + Gamma(shape, rate), integer shape in [1, 64]: the sum of `shape`
                                    exponential draws (the law the paper draws execution times from) */
 
-#define ABS_FLAG_NO_TENSOR_CORES 1  /* run the hidden-layer contractions on the FP32-FMA kernels */
+#define ABS_FLAG_NO_TENSOR_CORES 1  /* run the hidden-layer contractions (ABS_CNN: the convolutions too) on the
+                                       FP32-FMA kernels: no matrix instruction in any layer */
 #define ABS_FLAG_NO_OVERLAP      2  /* enqueue every kernel on the caller's stream (no side stream for the
                                        server-side kernels of the next round) */
 #define ABS_FLAG_NO_BULK_PIPELINE 32 /* bf16 least squares: per-warp 16-byte loads (rows read from HBM, then again

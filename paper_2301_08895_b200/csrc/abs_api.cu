@@ -272,7 +272,8 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   // 22.2 / 22.9; 201-133-10, 4096 rows: 69.6 / 60.7); fp32 4 while that leaves at most
   // one CTA per SM (the chain of layers is what counts), 8 up to two waves, then 16 (fewer reads of the weights per row).
   L->row_R = 0;
-  if (!lsq && m->local_steps <= 1 && (!L->any_tc || L->cnn)) {
+  // (their bf16 form is built on matrix instructions: not with ABS_FLAG_NO_TENSOR_CORES)
+  if (!lsq && m->local_steps <= 1 && (!L->any_tc || L->cnn) && (L->esz == 4 || tc_ok)) {
     const long long rows = (long long)W * m->batch;
     rnet::RowsArgs ra;
     ra.n_layers = m->n_layers;
@@ -351,7 +352,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   if (L->cnn && L->row_R) {
     cmma::Block cb[2];
     conv_blocks(*L, cb);
-    L->conv_mma = L->esz == 2 && !(m->flags & ABS_FLAG_NO_TENSOR_CORES) && cmma::fits(L->ck, cb[0], cb[1]);
+    L->conv_mma = L->esz == 2 && cmma::fits(L->ck, cb[0], cb[1]);
     if (L->conv_mma) {
       L->frag_stride = round_up_sz((size_t)cmma::frag_total(L->ck, cb[0], cb[1]), 64);
       L->frag = cv.take(2 * L->frag_stride * (S + 1));

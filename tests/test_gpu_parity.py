@@ -264,7 +264,8 @@ def test_local_sgd_steps_multi_layer_network_fma_paths(dims, dtype, W, B, U, K0,
     (inputs.MLP, (520, 310, 77, 10), inputs.FP32, 5, 30, 0),     # weights streamed through shared memory, 4 rows
     (inputs.MLP, (300, 260, 10), inputs.FP32, 30, 90, 0),        # ... 16 rows
     (inputs.MLP, (201, 133, 10), inputs.BF16, 7, 20, 0),         # bf16, weights resident, odd and even widths
-    (inputs.MLP, (128, 256, 48, 10), inputs.BF16, 7, 20, gpu.FLAG_NO_TENSOR_CORES),     # 16-byte rows
+    (inputs.MLP, (128, 256, 48, 10), inputs.BF16, 7, 20, gpu.FLAG_NO_TENSOR_CORES),     # (bf16 with the flag: FP32-FMA tiles)
+    (inputs.MLP, (128, 56, 48, 10), inputs.BF16, 7, 20, 0),      # bf16, rows on 16-byte boundaries, too narrow for the tiles
     (inputs.MLP, (700, 301, 77, 10), inputs.BF16, 6, 17, 0),     # bf16, streamed
     (inputs.MLP, (90, 1001, 10), inputs.BF16, 4, 12, 0),         # 126 column tiles
     (inputs.MLP, (50, 31, 18, 2), inputs.BF16, 40, 33, 0),       # bf16, 16 rows per CTA, resident; one class pair
@@ -439,6 +440,35 @@ def test_bf16_network_without_tensor_cores():
     assert ctx.plan()["path"] == [0, 0, 2]        # no layer on the tensor-core path
     ctx.close()
     compare_with_oracle(cfg, X, y, w0, 25, TOL_BF16, forced=True, loss_tol=5e-2, flags=gpu.FLAG_NO_TENSOR_CORES)
+
+
+@pytest.mark.parametrize("kind,dims,conv", [
+    (inputs.MLP, (201, 133, 10), None),
+    (inputs.MLP, (128, 256, 48, 10), None),
+    (inputs.CNN, (64, 24, 10), (14, 14, 3, 3, 4, 16)),
+])
+def test_no_tensor_cores_flag_runs_the_fma_kernels(kind, dims, conv):
+    """ABS_FLAG_NO_TENSOR_CORES on bf16 networks whose default path is the row kernels (matrix instructions): every hidden
+    layer has an FP32-FMA launch per direction, and the run agrees with the oracle."""
+    cfg = _small_cfg(kind, dims, inputs.BF16, 6, 20, 3, 5, PARETO, lr=0.01)
+    cfg.conv, cfg.w0 = conv, "he"
+    X, y, w0 = _problem(cfg)
+    Xd, yd = to_device(cfg, X, y)
+    per_round = {}
+    for flags in (0, gpu.FLAG_NO_TENSOR_CORES):
+        ctx = gpu.context_from_config(cfg, Xd, yd, w0, max_rounds=4, flags=flags)
+        ctx.profile_start(400)
+        ctx.run_rounds(4)
+        per_round[flags] = {k: v[0] // 4 for k, v in ctx.profile_read().items()}
+        ctx.close()
+    hidden = len(dims) - 2
+    flagged = per_round[gpu.FLAG_NO_TENSOR_CORES]
+    assert (flagged["fwd"], flagged["wgrad"], flagged["dgrad"]) == (hidden, hidden, hidden if conv else hidden - 1)
+    if conv:
+        assert flagged["conv"] == 7                     # forward and weight gradient of two blocks, one delta, two chunk sums
+    if dims[1] % 8:
+        assert per_round[0]["wgrad"] == 0               # (the default path of this network: the row kernels)
+    compare_with_oracle(cfg, X, y, w0, 12, TOL_BF16, forced=True, loss_tol=5e-2, flags=gpu.FLAG_NO_TENSOR_CORES)
 
 
 @pytest.mark.parametrize("d,W,B,K0,S", [(4096, 200, 32, 25, 32), (1000, 160, 19, 7, 6), (2056, 300, 8, 300, 0)])
