@@ -223,6 +223,33 @@ void conv_blocks(const Layout& L, cmma::Block* b) {
 
 int step_tiles(int in, int out) { return ((in + 1 + rnet::GT - 1) / rnet::GT) * ((out + rnet::GT - 1) / rnet::GT); }
 
+// Networks whose weights do not fit the row kernels' shared memory: every CTA then streams all of them for its few rows,
+// forward and (those a delta goes back through) backward, where the tile kernels read them once per 64 or 128 rows but
+// take a launch per layer and direction.  Where the tiles win (us a round with every worker selected, tiles / row kernels;
+// back-propagated weights in brackets):
+//   fp32, where only 4 rows fit and the CTAs are more than one wave: 1024-1024-512-10 [0.5 M]: 1024 rows 538 / 474, 2048
+//     869 / 932, 8192 2765 / 3392; 640 rows of 256-1024-1024-10 [1.1 M]: 428 / 477.  With 8 rows per CTA, or up to 592 rows,
+//     or most weights in the first layer the row kernels win or are even: 1024-768-768-10 8192 rows 2765 / 2515,
+//     1024-1024-640-10 256 rows 339 / 248, 2048-1024-10 8192 rows 3206 / 3019.
+//   bf16 widths TMA cannot address: one CTA's chain over the chunks counts when rows are few: 301-1001-1001-10 [1.0 M] 256
+//     rows 330 / 355, 640 rows 468 / 386; 785-513-511-10 [0.3 M] 256 rows 266 / 187.
+//   the CNN with tcgen05 layers instead: 400-768-768-10 [0.9 M] 256 rows 295 / 354, 2048 rows 813 / 573; 400-1024-768-10 [1.2 M]
+//     1024 rows 481 / 545, 2048 rows 820 / 701; 400-1024-1024-10 [1.5 M] 256 rows 309 / 519, 8192 rows 2829 / 3095;
+//     400-768-512-10 [0.7 M] 256 rows 289 / 302, 640 rows 343 / 326.
+// (Left where it is: fp32 layers of 513 to 640 columns keep five of a CTA's eight warps busy and cost 2 to 7 % from 4096 rows
+// on, the CNN's 400-640-384-10 1985 / 2127.)
+bool tiles_win(const abs_model_desc* m, const Layout& L, long long rows) {
+  size_t all = 0, back = 0;
+  for (int l = 0; l < m->n_layers; ++l) {
+    const size_t w = (size_t)m->dims[l] * m->dims[l + 1];
+    all += w;
+    if (l > 0 || L.cnn) back += w;
+  }
+  if (L.esz == 4) return L.row_R == 4 && rows > 4 * 148 && 4 * back > all;
+  if (L.any_tc) return back > 720000 && (rows < 2048 || back > 1250000);
+  return !L.cnn && back > 700000 && rows < 512;      // (the CNN's convolutions lose their matrix-instruction kernels with the row kernels)
+}
+
 void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   L->n_layers = m->n_layers;
   L->esz = m->dtype == ABS_FP32 ? 4 : 2;
@@ -282,6 +309,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
     const int R0 = L->esz == 2 ? (rows <= 148 * 8 ? 8 : 16) : rows <= 148 * 4 ? 4 : rows <= 2 * 148 * 8 ? 8 : 16;
     for (int R = R0; R >= (L->esz == 2 ? 8 : 4) && !L->row_R; R /= 2)
       if (rnet::plan_rows(&ra, R, (int)L->esz, &smem)) L->row_R = R;
+    if (L->row_R && !ra.resident && tiles_win(m, *L, rows)) L->row_R = 0;
     if (L->row_R) {
       L->row_resident = ra.resident != 0;
       L->any_tc = false;

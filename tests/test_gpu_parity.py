@@ -284,6 +284,31 @@ def test_row_kernels(kind, dims, dtype, W, B, flags):
                         flags=flags)
 
 
+@pytest.mark.parametrize("kind,dims,conv,dtype,W,B,tiles", [
+    (inputs.MLP, (256, 1024, 1024, 10), None, inputs.FP32, 19, 32, True),       # four rows per CTA fit: more than one wave
+    (inputs.MLP, (256, 1024, 1024, 10), None, inputs.FP32, 18, 32, False),      # ... one wave
+    (inputs.MLP, (301, 901, 901, 10), None, inputs.BF16, 8, 32, True),          # few rows, long streams
+    (inputs.MLP, (301, 901, 901, 10), None, inputs.BF16, 8, 64, False),
+    (inputs.CNN, (400, 1024, 1024, 10), (32, 32, 3, 5, 6, 16), inputs.BF16, 5, 16, True),     # tcgen05 affine layers, FMA convolutions
+    (inputs.CNN, (400, 768, 512, 10), (32, 32, 3, 5, 6, 16), inputs.BF16, 5, 16, False),
+])
+def test_streamed_weights_choose_between_row_and_tile_kernels(kind, dims, conv, dtype, W, B, tiles):
+    """Networks whose weights do not fit the row kernels' shared memory, on both sides of each line of the rule that
+    chooses their kernels: the kernels that run, and agreement with the oracle."""
+    cfg = _small_cfg(kind, dims, dtype, W, B, 3, 5, GAMMA3, lr=0.01)
+    cfg.conv, cfg.w0 = conv, "he"
+    X, y, w0 = _problem(cfg)
+    Xd, yd = to_device(cfg, X, y)
+    ctx = gpu.context_from_config(cfg, Xd, yd, w0, max_rounds=2)
+    ctx.profile_start(100)
+    ctx.run_rounds(2)
+    launches = {k: v[0] // 2 for k, v in ctx.profile_read().items()}
+    ctx.close()
+    assert (launches["wgrad"] > 0) == tiles and launches["fwd"] == (len(dims) - 2 if tiles else 1)
+    bf16 = dtype == inputs.BF16
+    compare_with_oracle(cfg, X, y, w0, 3, TOL_BF16 if bf16 else TOL_FP32, forced=True, loss_tol=5e-2 if bf16 else None)
+
+
 def test_lock_step_constant_times():
     cfg = _small_cfg(inputs.LSQ, (16, 1), inputs.FP32, 8, 4, 2, 3,
                      inputs.TimeSpec(inputs.T_CONST, shift=3.0))
