@@ -228,19 +228,28 @@ constexpr int CL_NT = 224;               // compute threads
 constexpr int CL_THREADS = CL_NT + 32;   // and the helper warp (registers are handed out to four warps at a time)
 template <typename T> __host__ __device__ constexpr int group_elems() { return 16 / (int)sizeof(T); }
 
+// CTAs of the cluster kernel per SM: by the registers of one group's sums (ge elements x CP classes)
+__host__ __device__ constexpr int cluster_ctas_per_sm(int ge, int CP) { return ge * CP < 64 ? 2 : 1; }
+
 inline size_t cluster_smem(const Geo& g, int esz, int B, int CP) {
   const size_t zp = std::max((size_t)g.PZ * B * CP, (size_t)g.PG * g.F * CP);
   return (size_t)g.nbuf * B * g.pitch * esz +
          4 * ((size_t)(esz == 2 ? 3 : 2) * g.F * CP + zp + (size_t)3 * B * CP + (size_t)6 * round_up(B, 4) + 2 * 16) + 64;
 }
 
-// Cluster width and staging for a model of `in` features, C classes, W workers; Q = 0: the rows of a step do not
-// fit into a cluster's shared memory and the one-CTA kernel runs.
-// Q: as many CTAs as the chip holds twice over when every worker is selected, slices of at least 32 features.
+// Cluster width and staging for a model of `in` features, C classes, when `n` workers run at once (K^0 where K is fixed,
+// else all W); Q = 0: the one-CTA kernel runs.
+// Q: as many CTAs as the chip holds when n workers are selected (two per SM, one where the registers of a group times
+// the classes allow no more), slices of at least 32 features.
 // Per launch on 784 -> 10 fp32, B = 64, U = 10: one-CTA kernel 366 us; clusters 74 us (8 workers), 85 us (16), 91 us
 // (32), 167 us (64); 512 instead of 224 compute threads lose the second CTA per SM (16 workers: 151 us).
-inline Geo cluster_plan(int in, int C, int B, int W, int esz) {
+// The one-CTA kernel stays where the rows of a step do not fit a cluster's shared memory, and for small models (its CTAs are
+// 256 threads there) on tiny batches once the clusters take more than one wave (us a round, one-CTA / cluster,
+// all workers selected, U = 10): 64 -> 10 bf16, 1024 workers, B = 4 178 / 288, B = 12 277 / 308, B = 16 306 / 313, 16
+// workers selected B = 4 the cluster by 1.4; 64 -> 1 fp32, 512 workers, B = 4 68 / 80, B = 8 81 / 84, B = 12 the cluster.
+inline Geo cluster_plan(int in, int C, int n_par, int B, int n, int esz) {
   const int CP = round_up(C, 4), ge = 16 / esz;
+  const int per_sm = cluster_ctas_per_sm(ge, CP);
   auto geo = [&](int Q, int nbuf) {
     Geo g;
     g.Q = Q;
@@ -254,14 +263,15 @@ inline Geo cluster_plan(int in, int C, int B, int W, int esz) {
     return g;
   };
   int first = 8;
-  while (first > 1 && (W * first > 2 * 148 || in / first < 32)) first /= 2;
+  while (first > 1 && (n * first > per_sm * 148 || in / first < 32)) first /= 2;
+  Geo none = geo(1, 1);
+  none.Q = 0;
+  if (n_par < 2048 && B <= (per_sm == 2 ? 8 : 12) && n * first > per_sm * 148) return none;
   for (int nbuf = 2; nbuf >= 1; --nbuf)
     for (int Q = first; Q <= 8; Q *= 2) {
       const Geo g = geo(Q, nbuf);
       if (cluster_smem(g, esz, B, CP) <= 220 * 1024) return g;
     }
-  Geo none = geo(1, 1);
-  none.Q = 0;
   return none;
 }
 
@@ -285,7 +295,7 @@ __device__ __forceinline__ void load_group(const __nv_bfloat16* p, float (&v)[8]
 
 // CP: class count rounded up to a multiple of 4 (padded classes have zero weights and zero deltas)
 template <typename T, int CP>
-__global__ void __launch_bounds__(CL_THREADS, (group_elems<T>() * CP < 64) ? 2 : 1) local_cluster_kernel(Args a, Geo geo) {
+__global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>(), CP)) local_cluster_kernel(Args a, Geo geo) {
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char loc_raw[];
   using lsqp::f32x2;
