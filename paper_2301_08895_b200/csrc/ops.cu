@@ -171,7 +171,9 @@ __global__ void __launch_bounds__(OP_NT) op_lsq_rows_kernel(OpArgs a) {
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-        const float res = dot - __shfl_sync(0xffffffffu, yv, t);       // row absent: 0 - 0
+        // (a row that is absent adds nothing, also where the weights are not finite and 0 w is a NaN)
+        const float target = __shfl_sync(0xffffffffu, yv, t);
+        const float res = __shfl_sync(0xffffffffu, s, t) >= 0 ? dot - target : 0.f;
         loss = fmaf(0.5f * res, res, loss);
 #pragma unroll
         for (int k = 0; k < NV; ++k) {

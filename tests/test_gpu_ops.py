@@ -61,6 +61,19 @@ def test_lsq_gradient_kernel_edges(n, B, d, bf16):
     test_lsq_gradient_matches_oracle(n, B, d, bf16)
 
 
+@pytest.mark.parametrize("n,B,d,bf16", [(8, 32, 64, False), (1, 5, 40, True), (3, 47, 1024, False), (2, 9, 4096, False)])
+def test_lsq_gradient_of_infinite_weights(n, B, d, bf16):
+    """An infinite weight and rows of positive features: every residual, loss and gradient element is +inf, and rows a
+    kernel pads its batch with bring no NaN into them."""
+    import torch
+    X, y, w, idx, Xd, yd, wd, idxd = _case(n, B, d, 500, bf16, 7)
+    Xd = Xd.abs() + 0.5
+    wd[d // 2] = float("inf")
+    g, loss = torch.zeros(d, device="cuda"), torch.zeros(n, device="cuda")
+    gpu.lsq_gradient(Xd, yd, wd, idxd, g, loss, torch.empty(n * d, device="cuda"))
+    assert torch.isposinf(loss).all() and torch.isposinf(g).all()
+
+
 def test_lsq_gradient_rejects_bad_arguments():
     import torch
     X, y, w, idx, Xd, yd, wd, idxd = _case(4, 8, 16, 100, False, 1)
