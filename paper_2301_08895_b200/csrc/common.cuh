@@ -116,6 +116,9 @@ struct CtlArgs {
   int* tr_sel_id; int* tr_sel_tau; float* tr_sel_loss; int* tr_rst_id;
 };
 
+// Logit of a class that does not exist: below every finite one, so that it is never the maximum of a soft-max.
+#define NO_CLASS (-__int_as_float(0x7f800000))
+
 __device__ __forceinline__ float ldf(const float* p, size_t i) { return p[i]; }
 __device__ __forceinline__ float ldf(const __nv_bfloat16* p, size_t i) { return __bfloat162float(p[i]); }
 __device__ __forceinline__ void stf(float* p, size_t i, float v) { p[i] = v; }

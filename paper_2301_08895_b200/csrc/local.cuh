@@ -445,10 +445,10 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
       } else {
         const int y = (int)yb;
         float zy = 0.f, se = 0.f;
-        // padded classes: exp(-3e38 - max) = 0, and their delta is 0
+        // padded classes: exp(NO_CLASS - max) = 0, and their delta is 0
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          z[k] = 4 * l + k < C ? z[k] : -3.0e38f;
+          z[k] = 4 * l + k < C ? z[k] : NO_CLASS;
           zy = 4 * l + k == y ? z[k] : zy;
         }
         float zmax = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
           const float mine = kh ? acc[n][2 + j] : acc[n][j];
           cls[e] = c;
           z[e] = (kh ? other[e] + mine : mine + other[e]) + __bfloat162float(ws[IN * WP + c]);
-          z[e] = c < C ? z[e] : -3.0e38f;                   // padded classes: exp(-3e38 - max) = 0
+          z[e] = c < C ? z[e] : NO_CLASS;                   // padded classes: exp(NO_CLASS - max) = 0
         }
       float zmax = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
       zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 1));

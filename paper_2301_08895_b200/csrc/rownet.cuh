@@ -181,8 +181,8 @@ __device__ __forceinline__ void rows_end(const RowsArgs& a, const int* gave_up) 
 template <typename T>
 __device__ __forceinline__ float2 row_softmax(const RowsArgs& a, float z0, float z1, int r, int yl, float sa, int lane) {
   const int C = a.dims[a.n_layers];
-  z0 = lane < C ? z0 : -3.0e38f;
-  z1 = lane + 32 < C ? z1 : -3.0e38f;
+  z0 = lane < C ? z0 : NO_CLASS;
+  z1 = lane + 32 < C ? z1 : NO_CLASS;
   float zmax = fmaxf(z0, z1);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));

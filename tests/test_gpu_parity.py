@@ -313,6 +313,24 @@ def test_streamed_weights_choose_between_row_and_tile_kernels(kind, dims, conv, 
     compare_with_oracle(cfg, X, y, w0, 3, TOL_BF16 if bf16 else TOL_FP32, forced=True, loss_tol=5e-2 if bf16 else None)
 
 
+@pytest.mark.parametrize("kind,dims,dtype,U", [
+    (inputs.SOFTMAX, (40, 6), inputs.FP32, 1),          # row kernel, fp32
+    (inputs.MLP, (20, 18, 10), inputs.BF16, 1),         # row kernel, bf16
+    (inputs.MLP, (64, 128, 10), inputs.BF16, 1),        # output layer on fragments
+    (inputs.SOFTMAX, (40, 6), inputs.FP32, 2),          # local steps, cluster kernel
+])
+def test_logits_at_the_lower_end_of_binary32(kind, dims, dtype, U):
+    """All output biases at -3.1e38: the logits are equal, so each loss is ln(classes); classes a kernel pads its rows with
+    are below any logit."""
+    cfg = _small_cfg(kind, dims, dtype, 4, 8, 2, 3, PARETO, lr=1e-3)
+    X, y, w0 = _problem(cfg)
+    w0[-dims[-1]:] = -3.1e38
+    rows, params = gpu_run(cfg, X, y, w0, 2, k_mode=gpu.K_FIXED, local_steps=U)
+    for r in rows:
+        assert np.allclose(r["sel_loss"], np.log(dims[-1]), rtol=1e-5)
+    assert np.isfinite(params).all()
+
+
 def test_lock_step_constant_times():
     cfg = _small_cfg(inputs.LSQ, (16, 1), inputs.FP32, 8, 4, 2, 3,
                      inputs.TimeSpec(inputs.T_CONST, shift=3.0))
