@@ -76,7 +76,10 @@ struct RoundInfo {
   int t;            // round index
   int diverged;     // set by the loss kernels of the round; RI_TIMEOUT: a bounded wait of such a kernel expired
 };
-constexpr int RI_TIMEOUT = 2;
+constexpr int RI_DIVERGED = 1, RI_TIMEOUT = 2;
+// For kernels in which both can happen: after a wait that ran out a CTA goes on with whatever is there, so that a
+// non-finite loss is likely as well; the caller is told about the wait.
+__device__ __forceinline__ void report(RoundInfo* ri, int what) { atomicMax(&ri->diverged, what); }
 
 // x / n for x < 2^31 / n (items of a loop), by a multiplication: an integer division costs a few hundred
 // cycles otherwise

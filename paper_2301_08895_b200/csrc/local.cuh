@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
     if (helper && lane == 0) {
       const float loss = __fdiv_rn(loss_sum, (float)U);
       a.loss[i] = loss;
-      if (!isfinite(loss)) ri->diverged = 1;
+      if (!isfinite(loss)) report(ri, RI_DIVERGED);
     }
   }
   if (tid == 0 && gave_up) {
@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
     while (tc::global_ns() - t0 < 200000ull) {}
     // not st->status: a cluster that starts later must find the same status in all of its CTAs
     st->timeout_where = 300;
-    ri->diverged = RI_TIMEOUT;
+    report(ri, RI_TIMEOUT);
   }
 }
 

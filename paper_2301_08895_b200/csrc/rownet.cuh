@@ -172,7 +172,7 @@ __device__ __forceinline__ void rows_end(const RowsArgs& a, const int* gave_up) 
     const unsigned long long t0 = tc::global_ns();
     while (tc::global_ns() - t0 < 200000ull) {}
     a.st->timeout_where = 400;
-    a.ri->diverged = RI_TIMEOUT;
+    report(a.ri, RI_TIMEOUT);
   }
 }
 
@@ -197,7 +197,7 @@ __device__ __forceinline__ float2 row_softmax(const RowsArgs& a, float z0, float
   if (lane == 0) {
     const float loss = yl < 0 ? 0.f : logf(se) - (zy - zmax);
     a.row_loss[r] = loss;
-    if (!isfinite(loss)) a.ri->diverged = 1;
+    if (!isfinite(loss)) report(a.ri, RI_DIVERGED);
   }
   // a delta is a stored quantity; sa: staleness-aware step size (weight of these rows in Eq. 3)
   if (yl < 0) return make_float2(0.f, 0.f);

@@ -191,3 +191,24 @@ def test_trace_arrays_do_not_hold_each_other(monkeypatch):
         assert a.nbytes <= 4 * n * W, k
         owners.append(id(a))
     assert len(set(owners)) == 4
+
+
+def test_a_timeout_is_not_overwritten_by_a_divergence():
+    """Kernels whose waits report through the round's status word (RI_TIMEOUT) must keep it when another CTA, or another
+    warp of the same one, reports a non-finite loss: every report of theirs takes the maximum, none is a plain store."""
+    csrc = os.path.join(ROOT, "paper_2301_08895_b200", "csrc")
+    checked = 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//.*", "", open(os.path.join(csrc, name)).read())
+        for kernel in re.split(r"__global__", text)[1:]:
+            body = kernel[:kernel.index("\n}\n")]
+            if "RI_TIMEOUT" in body or "row_softmax" in body or "rows_end" in body:
+                assert not re.search(r"->diverged\s*=[^=]", body), (name, kernel[:80])
+                checked += 1
+        for helper in re.findall(r"\n__device__[^{;]*\b(?:rows_end|row_softmax)\([^{;]*\{.*?\n\}\n", text, flags=re.S):
+            assert not re.search(r"->diverged\s*=[^=]", helper), name
+            checked += 1
+    assert checked >= 4
+    common = open(os.path.join(csrc, "common.cuh")).read()
+    assert re.search(r"void report\(RoundInfo\* ri, int what\) \{ atomicMax\(&ri->diverged, what\); \}", common)
+    assert re.search(r"RI_DIVERGED = 1, RI_TIMEOUT = 2", common)
