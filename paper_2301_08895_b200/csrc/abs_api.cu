@@ -1319,7 +1319,7 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
   if (model->local_steps > 1 && !L.local_net) {
     const int C = model->kind == ABS_LSQ ? 1 : model->dims[1];
     const int n_par = model->kind == ABS_LSQ ? model->dims[0] : model->dims[0] * C + C;
-    ctx->local_geo = local::cluster_plan(model->dims[0], C, n_par, model->batch, model->k_mode == ABS_K_FIXED ? K0 : W, (int)L.esz);
+    ctx->local_geo = local::cluster_plan(model->dims[0], C, n_par, model->batch, W, model->k_mode == ABS_K_FIXED ? K0 : W, (int)L.esz);
     cudaError_t el;
     if (ctx->local_geo.Q > 0) {
       const int sm = (int)local::cluster_smem(ctx->local_geo, (int)L.esz, model->batch, round_up(C, 4));

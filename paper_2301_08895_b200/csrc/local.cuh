@@ -237,19 +237,20 @@ inline size_t cluster_smem(const Geo& g, int esz, int B, int CP) {
          4 * ((size_t)(esz == 2 ? 3 : 2) * g.F * CP + zp + (size_t)3 * B * CP + (size_t)6 * round_up(B, 4) + 2 * 16) + 64;
 }
 
-// Cluster width and staging for a model of `in` features, C classes, when `n` workers run at once (K^0 where K is fixed,
-// else all W); Q = 0: the one-CTA kernel runs.
-// Q: as many CTAs as the chip holds when n workers are selected (two per SM, one where the registers of a group times
-// the classes allow no more), slices of at least 32 features.
+// Cluster width and staging for a model of `in` features, C classes, W workers of which n run at once (K^0 where K is
+// fixed, else all); Q = 0: the one-CTA kernel runs.
+// Q: as many CTAs as the chip holds twice over when every worker is selected, slices of at least 32 features.
 // Per launch on 784 -> 10 fp32, B = 64, U = 10: one-CTA kernel 366 us; clusters 74 us (8 workers), 85 us (16), 91 us
 // (32), 167 us (64); 512 instead of 224 compute threads lose the second CTA per SM (16 workers: 151 us).
-// The one-CTA kernel stays where the rows of a step do not fit a cluster's shared memory, and for small models (its CTAs are
-// 256 threads there) on tiny batches once the clusters take more than one wave (us a round, one-CTA / cluster,
-// all workers selected, U = 10): 64 -> 10 bf16, 1024 workers, B = 4 178 / 288, B = 12 277 / 308, B = 16 306 / 313, 16
-// workers selected B = 4 the cluster by 1.4; 64 -> 1 fp32, 512 workers, B = 4 68 / 80, B = 8 81 / 84, B = 12 the cluster.
-inline Geo cluster_plan(int in, int C, int n_par, int B, int n, int esz) {
+// The one-CTA kernel stays where the rows of a step do not fit a cluster's shared memory, and on batches of a few rows once
+// the clusters of n workers take more than one wave: for models below 2048 parameters (its CTAs are 256 threads there, and
+// several share an SM) and for large ones whose clusters of two take two partial waves.  us a round, one-CTA / cluster,
+// U = 10, all workers selected: 64 -> 10 bf16, 1024 workers, 4 rows 178 / 288, 8 rows 208 / 298, 12 rows 277 / 308; 200
+// workers, 8 rows 84 / 89, 12 rows 119 / 92; 64 -> 1 fp32, 512 workers, 4 rows 68 / 80, 8 rows 81 / 84, 12 rows the
+// cluster; 784 -> 10 bf16, 100 workers, 4 rows 123 / 156, 16 rows 168 / 166.
+inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) {
   const int CP = round_up(C, 4), ge = 16 / esz;
-  const int per_sm = cluster_ctas_per_sm(ge, CP);
+  const int wave = 148 * cluster_ctas_per_sm(ge, CP);
   auto geo = [&](int Q, int nbuf) {
     Geo g;
     g.Q = Q;
@@ -263,10 +264,11 @@ inline Geo cluster_plan(int in, int C, int n_par, int B, int n, int esz) {
     return g;
   };
   int first = 8;
-  while (first > 1 && (n * first > per_sm * 148 || in / first < 32)) first /= 2;
+  while (first > 1 && (W * first > 2 * 148 || in / first < 32)) first /= 2;
   Geo none = geo(1, 1);
   none.Q = 0;
-  if (n_par < 2048 && B <= (per_sm == 2 ? 8 : 12) && n * first > per_sm * 148) return none;
+  if (n_par < 2048 && (B <= 8 ? n * first > wave : B <= 12 && wave == 148 && n * first > 2 * wave)) return none;
+  if (n_par > 6000 && B <= 8 && first == 2 && n * first > wave) return none;
   for (int nbuf = 2; nbuf >= 1; --nbuf)
     for (int Q = first; Q <= 8; Q *= 2) {
       const Geo g = geo(Q, nbuf);

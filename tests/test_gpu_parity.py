@@ -203,8 +203,10 @@ def test_local_sgd_steps(kind, dims, dtype, W, B, U, forced):
     (inputs.SOFTMAX, (400, 12), inputs.FP32, 5, 400, 3),        # a single row buffer
     (inputs.SOFTMAX, (760, 16), inputs.FP32, 4, 512, 2),        # rows of a step too large for a cluster: one-CTA kernel
     (inputs.LSQ, (12288, 1), inputs.FP32, 4, 4, 3),             # largest model of the path
-    (inputs.SOFTMAX, (24, 5), inputs.BF16, 148, 12, 2),         # tiny steps: one wave of one-CTA clusters
-    (inputs.SOFTMAX, (24, 5), inputs.BF16, 149, 12, 2),         # ... more workers than that: one-CTA kernel
+    (inputs.SOFTMAX, (24, 5), inputs.BF16, 148, 8, 2),          # tiny steps: one wave of one-CTA clusters
+    (inputs.SOFTMAX, (24, 5), inputs.BF16, 149, 8, 2),          # ... more workers than that: one-CTA kernel
+    (inputs.SOFTMAX, (24, 5), inputs.BF16, 297, 12, 2),         # ... twice as many and twelve rows: one-CTA kernel
+    (inputs.SOFTMAX, (784, 10), inputs.BF16, 75, 8, 2),         # large model, two partial waves of clusters of two: one-CTA kernel
     (inputs.LSQ, (64, 1), inputs.FP32, 297, 9, 2),              # ... larger batch: cluster kernel
     (inputs.LSQ, (64, 1), inputs.FP32, 297, 8, 2),              # ... one-CTA kernel
 ])
