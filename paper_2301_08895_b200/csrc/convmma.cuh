@@ -516,15 +516,15 @@ __global__ void __launch_bounds__(NT, 3) conv_bwd_mma_kernel(const __grid_consta
           }
 #pragma unroll
           for (int dx = 0; dx < K; ++dx) {
-            if (dx & 1) outl::mma16816(d2, af[dx], b[dx].x, b[dx].y);
-            else outl::mma16816(d, af[dx], b[dx].x, b[dx].y);
+            if (dx & 1) outl::mma16816_rn(d2, af[dx], b[dx].x, b[dx].y);
+            else outl::mma16816_rn(d, af[dx], b[dx].x, b[dx].y);
           }
         } else {
           for (int dx = 0; dx < k; ++dx) {
             uint32_t af[4];
             outl::ldsm4(base - (uint32_t)((dy * f.zw + dx) * 48), af);
             const uint2 b = bd[(dy * k + dx) * 32 + lane];
-            outl::mma16816(d, af, b.x, b.y);
+            outl::mma16816_rn(d, af, b.x, b.y);
           }
         }
       }
@@ -560,12 +560,12 @@ __global__ void __launch_bounds__(NT, 3) conv_bwd_mma_kernel(const __grid_consta
       for (int m = 0; m < MT2; ++m)
         if (warp + NWARP * m < mt2) {
           const uint32_t af[4] = {lds(o2[m][0] + u), lds(o2[m][1] + u), lds(o2[m][0] + v), lds(o2[m][1] + v)};
-          outl::mma16816(c2[m][0], af, b[0][0], b[0][1]);
-          if (nc2 > 1) outl::mma16816(c2[m][1], af, b[1][0], b[1][1]);
+          outl::mma16816_rn(c2[m][0], af, b[0][0], b[0][1]);
+          if (nc2 > 1) outl::mma16816_rn(c2[m][1], af, b[1][0], b[1][1]);
         }
       if (warp < nc2) {
-        if (warp == 0) outl::mma16816(s2, ones, b[0][0], b[0][1]);
-        else outl::mma16816(s2, ones, b[1][0], b[1][1]);
+        if (warp == 0) outl::mma16816_rn(s2, ones, b[0][0], b[0][1]);
+        else outl::mma16816_rn(s2, ones, b[1][0], b[1][1]);
       }
     }
     __syncthreads();
@@ -577,9 +577,9 @@ __global__ void __launch_bounds__(NT, 3) conv_bwd_mma_kernel(const __grid_consta
       for (int m = 0; m < MT1; ++m)
         if (m < mt1) {
           const uint32_t af[4] = {lds(o1[m][0] + u), lds(o1[m][1] + u), lds(o1[m][0] + v), lds(o1[m][1] + v)};
-          outl::mma16816(c1[m], af, b0, b1);
+          outl::mma16816_rn(c1[m], af, b0, b1);
         }
-      outl::mma16816(s1, ones, b0, b1);
+      outl::mma16816_rn(s1, ones, b0, b1);
     }
   }
   // ---- this CTA's sums: [k k Ci][Co], then the bias

@@ -575,10 +575,10 @@ __device__ __forceinline__ void backward_tile(float (&acc)[RT][4], const __nv_bf
     for (int i = 0; i < 8; ++i) p[i] = pair_at<EVEN>((i & 1) ? wb : wa, n + 2 * t + (i >> 1) * 8, out);
     const uint32_t a0[4] = {p[0], p[1], p[2], p[3]}, a1[4] = {p[4], p[5], p[6], p[7]};
 #pragma unroll
-    for (int r = 0; r < RT; ++r) outl::mma16816(acc[r], a0, b[r][0], b[r][1]);
+    for (int r = 0; r < RT; ++r) outl::mma16816_rn(acc[r], a0, b[r][0], b[r][1]);
     if (n + 16 < out)
 #pragma unroll
-      for (int r = 0; r < RT; ++r) outl::mma16816(acc[r], a1, b[r][2], b[r][3]);
+      for (int r = 0; r < RT; ++r) outl::mma16816_rn(acc[r], a1, b[r][2], b[r][3]);
   }
 }
 
