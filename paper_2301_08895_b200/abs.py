@@ -306,10 +306,13 @@ def _raw_stream(torch, stream, X):
     raw-stream call saves building a Stream object (a call with 64 features: 7.4 us with it, 10.4 us without)."""
     if stream is not None:
         return stream.cuda_stream
-    if not X.is_cuda:
+    device = X.get_device()
+    if device < 0:
         raise ValueError("expected a tensor on a CUDA device, got one on %s" % X.device)
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    return raw(X.get_device()) if raw is not None else torch.cuda.current_stream(X.device).cuda_stream
+    try:
+        return torch._C._cuda_getCurrentRawStream(device)
+    except AttributeError:               # (not a public name of torch)
+        return torch.cuda.current_stream(X.device).cuda_stream
 
 
 def lsq_gradient(X, y, w, idx, g_out, loss_out, scratch, stream=None):
