@@ -235,7 +235,9 @@ int abs_get_trace(abs_ctx* ctx, int first_round, int n_rounds, abs_trace* out_ho
  * created with the same model kind and sizes, batch, step size, dtype, local steps, flags, W, K0,
  * staleness bound, modes, time distribution, seed and max_rounds (ABS_EINVAL otherwise, context
  * unchanged); the context then continues with
- * round `rounds completed in the image`, bit-identically to the context that saved it.  The
+ * round `rounds completed in the image`, bit-identically to the context that saved it (an image of
+ * an earlier build of the library is accepted too, whatever its workspace layout was; its run goes
+ * on with this build's kernels).  The
  * dataset, w0 and profiling state are not part of the image.  Host memory is the caller's. */
 int abs_state_bytes(abs_ctx* ctx, size_t* out);
 int abs_save_state(abs_ctx* ctx, void* dst_host, size_t cap, size_t* written);

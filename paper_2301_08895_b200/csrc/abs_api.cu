@@ -250,6 +250,49 @@ bool tiles_win(const abs_model_desc* m, const Layout& L, long long rows) {
   return !L.cnn && back > 700000 && rows < 512;      // (the CNN's convolutions lose their matrix-instruction kernels with the row kernels)
 }
 
+// Gradient rows the buffers hold when version groups are padded to L->RB rows.
+void row_capacity(const abs_model_desc* m, int W, int S, Layout* L) {
+  const int groups = (W < S + 1) ? W : S + 1;
+  L->rows_cap = round_up(W * m->batch, L->RB) + groups * L->RB;
+  if (L->local_net) {
+    L->RBp = round_up(m->batch, L->RB);
+    L->rows_cap = std::max(L->rows_cap, W * L->RBp);
+  }
+  L->n_tiles_cap = L->rows_cap / L->RB;
+}
+
+// First part of the workspace: what a run continues from, and the layouts of its rounds.  first_form: as it was before
+// the shards and the real rows of a tile were kept (see image_layout).
+void carve_state(Layout* L, Carver& cv, int W, int S, bool first_form = false) {
+  L->st = cv.take(sizeof(DevState));
+  L->ri = cv.take(2 * sizeof(RoundInfo));
+  L->c = cv.take(sizeof(u64) * W);
+  L->version = cv.take(4 * W);
+  L->job = cv.take(4 * W);
+  L->next_dur = cv.take(8 * W);
+  L->dur_job = cv.take(4 * W);
+  if (!first_form) L->shard = cv.take(8 * W);
+  for (int q = 0; q < 2; ++q) {
+    L->sel[q] = cv.take(4 * W);
+    L->sel_tau[q] = cv.take(4 * W);
+    L->sel_row0[q] = cv.take(4 * W);
+    L->row_idx[q] = cv.take(4 * (size_t)L->rows_cap);
+    L->tile_slot[q] = cv.take(4 * (size_t)L->n_tiles_cap);
+    if (!first_form) L->tile_real[q] = cv.take(4 * (size_t)L->n_tiles_cap);
+  }
+  L->loss = cv.take(4 * W);
+  L->row_loss = cv.take(4 * (size_t)L->rows_cap);
+  L->master = cv.take(4 * L->d_pad);
+  L->ring = cv.take(L->esz * L->d_pad * (S + 1));
+}
+
+// Elements of one model version's operand fragments (CNN).
+size_t frag_stride(const Layout& L) {
+  cmma::Block cb[2];
+  conv_blocks(L, cb);
+  return round_up_sz((size_t)cmma::frag_total(L.ck, cb[0], cb[1]), 64);
+}
+
 void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
   L->n_layers = m->n_layers;
   L->esz = m->dtype == ABS_FP32 ? 4 : 2;
@@ -323,14 +366,8 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
     }
   }
   L->RB = lsq ? m->batch : L->row_R ? L->row_R : (L->any_tc ? 128 : 64);
-  const int groups = (W < S + 1) ? W : S + 1;
-  L->rows_cap = round_up(W * m->batch, L->RB) + groups * L->RB;
   L->local_net = !lsq && m->n_layers > 1 && m->local_steps > 1;
-  if (L->local_net) {
-    L->RBp = round_up(m->batch, L->RB);
-    L->rows_cap = std::max(L->rows_cap, W * L->RBp);
-  }
-  L->n_tiles_cap = L->rows_cap / L->RB;
+  row_capacity(m, W, S, L);
   if (lsq) {
     L->P = 0;
   } else if (L->row_R) {
@@ -356,33 +393,14 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
     L->P = std::max(1, std::min(P, 16));
   }
   Carver cv;
-  L->st = cv.take(sizeof(DevState));
-  L->ri = cv.take(2 * sizeof(RoundInfo));
-  L->c = cv.take(sizeof(u64) * W);
-  L->version = cv.take(4 * W);
-  L->job = cv.take(4 * W);
-  L->next_dur = cv.take(8 * W);
-  L->dur_job = cv.take(4 * W);
-  L->shard = cv.take(8 * W);
-  for (int q = 0; q < 2; ++q) {
-    L->sel[q] = cv.take(4 * W);
-    L->sel_tau[q] = cv.take(4 * W);
-    L->sel_row0[q] = cv.take(4 * W);
-    L->row_idx[q] = cv.take(4 * (size_t)L->rows_cap);
-    L->tile_slot[q] = cv.take(4 * (size_t)L->n_tiles_cap);
-    L->tile_real[q] = cv.take(4 * (size_t)L->n_tiles_cap);
-  }
-  L->loss = cv.take(4 * W);
-  L->row_loss = cv.take(4 * (size_t)L->rows_cap);
-  L->master = cv.take(4 * L->d_pad);
-  L->ring = cv.take(L->esz * L->d_pad * (S + 1));
+  carve_state(L, cv, W, S);
   if (m->local_steps > 1) L->P = 0;      // Eq. 3 adds one upload per selected worker
   if (L->cnn && L->row_R) {
     cmma::Block cb[2];
     conv_blocks(*L, cb);
     L->conv_mma = L->esz == 2 && cmma::fits(L->ck, cb[0], cb[1]);
     if (L->conv_mma) {
-      L->frag_stride = round_up_sz((size_t)cmma::frag_total(L->ck, cb[0], cb[1]), 64);
+      L->frag_stride = frag_stride(*L);
       L->frag = cv.take(2 * L->frag_stride * (S + 1));
     }
   }
@@ -1417,7 +1435,7 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     cmma::fill_tables(tab.data(), L.ck, cb[0], cb[1], bl);
     e = cudaMemcpyAsync(ctx->at<int>(L.conv_tab), tab.data(), 4 * tab.size(), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return bail(cuda_fail(nullptr, e, "convolution tables"));
-    cmma::frag_init_kernel<<<16, 256, 0, s>>>(frag_map(ctx), ctx->at<float>(L.master));
+    cmma::frag_fill_kernel<<<16, 256, 0, s>>>(frag_map(ctx), ctx->at<__nv_bfloat16>(L.ring), L.d_pad);      // (slot 0)
     ctx->launches += 1;
   }
   e = cudaGetLastError();
@@ -1665,13 +1683,29 @@ void state_blocks(const Layout& L, size_t* b1_off, size_t* b1, size_t* b2_off, s
 }
 
 bool same_constants(const DevState& a, const DevState& b) {
-  return a.W == b.W && a.K0 == b.K0 && a.S == b.S && a.B == b.B && a.RB == b.RB && a.k_mode == b.k_mode &&
+  return a.W == b.W && a.K0 == b.K0 && a.S == b.S && a.B == b.B && a.k_mode == b.k_mode &&
          a.bound_mode == b.bound_mode && a.max_rounds == b.max_rounds && a.bound_offset == b.bound_offset &&
          a.theta_cap == b.theta_cap && a.literal_eq6 == b.literal_eq6 && a.no_restart == b.no_restart &&
          a.sa_penalty == b.sa_penalty && a.n_samples == b.n_samples &&
          a.key0 == b.key0 && a.key1 == b.key1 && a.dist.kind == b.dist.kind && a.dist.shift == b.dist.shift &&
          a.dist.rate == b.dist.rate && a.dist.scale == b.dist.scale && a.dist.slow_mod == b.dist.slow_mod &&
          a.dist.slow_rem == b.dist.slow_rem && a.dist.slow_factor == b.dist.slow_factor && a.dist.shape == b.dist.shape;
+}
+
+// Where an image keeps its pieces.  They lie as in the workspace of the build that saved it, which may have padded the
+// version groups to other rows, had no shards and real rows of tiles yet, or kept (no) operand fragments behind the ring.
+bool image_layout(const abs_ctx* ctx, const StateHeader& h, Layout* im) {
+  *im = ctx->L;
+  im->RB = h.st.RB;
+  if (im->RB < 1 || im->RB > 1024) return false;
+  row_capacity(&ctx->m, ctx->W, ctx->S, im);
+  const size_t frags = im->cnn && im->esz == 2 ? round_up_sz(2 * frag_stride(*im) * (ctx->S + 1), 256) : 0;
+  for (bool first_form : {false, true}) {
+    Carver cv;
+    carve_state(im, cv, ctx->W, ctx->S, first_form);
+    if (h.block1 == cv.off || (!first_form && h.block1 == cv.off + frags)) return true;
+  }
+  return false;
 }
 
 }  // namespace
@@ -1730,15 +1764,36 @@ int abs_restore_state(abs_ctx* ctx, const void* src, size_t bytes) {
   DevState cur;
   int rc = read_status(ctx, &cur);
   if (rc != ABS_OK) return rc;
-  if (h.d_pad != ctx->L.d_pad || h.esz != ctx->L.esz || h.block1 != b1 || h.block2 != b2 ||
-      h.max_rounds != (unsigned long long)ctx->m.max_rounds || !same_constants(h.st, cur))
+  const Layout& L = ctx->L;
+  Layout im;
+  if (h.d_pad != L.d_pad || h.esz != L.esz || h.block2 != b2 || h.max_rounds != (unsigned long long)ctx->m.max_rounds ||
+      !same_constants(h.st, cur) || !image_layout(ctx, h, &im))
     return fail(ABS_EINVAL, "the image was saved by a context with other sizes, modes, time distribution or seed");
-  if (bytes != sizeof h + b1 + b2) return fail(ABS_EINVAL, "image has %zu bytes, %zu expected", bytes, sizeof h + b1 + b2);
+  if (bytes != sizeof h + h.block1 + b2) return fail(ABS_EINVAL, "image has %zu bytes, %zu expected", bytes, (size_t)(sizeof h + h.block1 + b2));
   if (h.rounds_enqueued < 0 || h.rounds_enqueued > ctx->m.max_rounds || h.st.t != h.rounds_enqueued)
     return fail(ABS_EINVAL, "image is inconsistent (rounds %d, completed %d)", h.rounds_enqueued, h.st.t);
-  const char* p = (const char*)src;
-  CU(cudaMemcpyAsync(ctx->ws + o1, p + sizeof h, b1, cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaMemcpyAsync(ctx->ws + o2, p + sizeof h + b1, b2, cudaMemcpyHostToDevice, ctx->stream));
+  const char* p = (const char*)src + sizeof h;
+  if (h.block1 == b1 && im.RB == L.RB) {
+    CU(cudaMemcpyAsync(ctx->ws + o1, p, b1, cudaMemcpyHostToDevice, ctx->stream));
+  } else {
+    // another layout: piece by piece (a round's row layout is made by its control step); the fragments follow from the ring
+    DevState st;
+    memcpy(&st, p + im.st, sizeof st);
+    st.RB = L.RB;
+    CU(cudaMemcpyAsync(ctx->at<DevState>(L.st), &st, sizeof st, cudaMemcpyHostToDevice, ctx->stream));
+    const struct { size_t to, from, n; } parts[] = {
+        {L.ri, im.ri, 2 * sizeof(RoundInfo)}, {L.c, im.c, sizeof(u64) * ctx->W}, {L.version, im.version, (size_t)4 * ctx->W},
+        {L.job, im.job, (size_t)4 * ctx->W}, {L.next_dur, im.next_dur, (size_t)8 * ctx->W}, {L.dur_job, im.dur_job, (size_t)4 * ctx->W},
+        {L.master, im.master, 4 * L.d_pad}, {L.ring, im.ring, L.esz * L.d_pad * (ctx->S + 1)}};
+    for (const auto& q : parts)
+      CU(cudaMemcpyAsync(ctx->ws + q.to, p + q.from, q.n, cudaMemcpyHostToDevice, ctx->stream));
+    if (L.conv_mma) {
+      cmma::frag_fill_kernel<<<dim3(16, ctx->S + 1), 256, 0, ctx->stream>>>(frag_map(ctx), ctx->at<__nv_bfloat16>(L.ring), L.d_pad);
+      CU(cudaGetLastError());
+      ctx->launches += 1;
+    }
+  }
+  CU(cudaMemcpyAsync(ctx->ws + o2, p + h.block1, b2, cudaMemcpyHostToDevice, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
   ctx->rounds_enqueued = h.rounds_enqueued;
   return ABS_OK;

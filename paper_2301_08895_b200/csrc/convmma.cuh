@@ -79,12 +79,13 @@ __device__ __forceinline__ void frag_store(const FragMap& m, int slot, int i, in
   f[(i ? frag_fwd(m.k, m.b[0]) : 0) + frag_at((dy * ks + kk / 16) * nc + co / 8, kk % 16, co % 8)] = v;
   if (i == 1) f[frag_fwd(m.k, m.b[0]) + frag_fwd(m.k, b) + frag_at(tap, co, ci)] = v;
 }
-// fragments of the initial model (slot 0)
-static __global__ void frag_init_kernel(FragMap m, const float* master) {
+// fragments of the model versions in slots 0 .. gridDim.y - 1 of the ring
+static __global__ void frag_fill_kernel(FragMap m, const bf16* ring, size_t slot_stride) {
+  const int slot = blockIdx.y;
   for (int i = 0; i < 2; ++i) {
     const int len = m.k * m.k * m.b[i].Ci * m.b[i].Co;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < len; j += gridDim.x * blockDim.x)
-      frag_store(m, 0, i, j, __float2bfloat16_rn(master[m.b[i].w_off + j]));
+      frag_store(m, slot, i, j, ring[(size_t)slot * slot_stride + m.b[i].w_off + j]);
   }
 }
 
