@@ -98,6 +98,25 @@ def assert_params_close(cfg, params, ref, tol, path=None):
     return err
 
 
+def assert_movement_close(cfg, params, w0, ref, path, tol):
+    """Relative L2 of every layer block's difference within tol of the length of the path the block travelled (its norm, which
+    w0 dominates in short runs, does not enter), and the comparison can see a wrong tile: each 32 x 32 tile of every
+    affine layer's weights moved by more than that in the reference."""
+    ref, got, w0 = (np.asarray(v, np.float64) for v in (ref, params, w0))
+    for name, sl in layer_blocks(cfg.kind, cfg.dims, getattr(cfg, "conv", None)):
+        e = np.linalg.norm(got[sl] - ref[sl]) / path[name]
+        assert e <= tol, "movement of block %s differs: %.3g of the path > %.3g" % (name, e, tol)
+        moved = ref[sl] - w0[sl]
+        if name[0] == "W" and name[1:].isdigit():
+            n_in, n_out = cfg.dims[int(name[1:]) - 1:int(name[1:]) + 1]
+            a = moved.reshape(n_in, n_out)
+            tiles = [a[i:i + 32, j:j + 32] for i in range(0, n_in, 32) for j in range(0, n_out, 32)]
+        else:
+            tiles = [moved]
+        least = min(np.linalg.norm(t) for t in tiles) / path[name]
+        assert least > tol, "a tile of block %s moved by %.3g of the path only" % (name, least)
+
+
 def oracle_run_with_paths(cfg, o, rounds, forced_losses=None):
     """o.run(rounds), also returning per layer block the summed norm of the per-round updates."""
     blocks = layer_blocks(cfg.kind, cfg.dims, getattr(cfg, "conv", None))
@@ -129,6 +148,8 @@ def compare_with_oracle(cfg, X, y, w0, rounds, tol, forced=False, loss_tol=None,
     assert mm is None, "integer trace differs at round %s field %s: gpu %s oracle %s (oracle " \
         "decision margin %.3g)" % (mm + (o.min_margin,))
     err = assert_params_close(cfg, params, o.w, tol, path)
+    if "move_tol" in kw:
+        assert_movement_close(cfg, params, w0, o.w, path, kw["move_tol"])
     lt = loss_tol if loss_tol is not None else tol * 10
     for t, (a, b) in enumerate(zip(rows, orows)):
         la, lb = np.array(a["sel_loss"]), np.array(b["sel_loss"])

@@ -6,7 +6,7 @@ import pytest
 from helpers import compare_with_oracle, gpu_run, to_device
 from paper_2301_08895_b200 import abs as gpu
 from paper_2301_08895_b200 import inputs
-from test_gpu_parity import GAMMA3, PARETO, TOL_BF16, TOL_FP32, _problem
+from test_gpu_parity import GAMMA3, PARETO, TOL_BF16, TOL_FP32, TOL_MOVE_BF16, _problem
 
 pytestmark = pytest.mark.gpu
 
@@ -62,7 +62,7 @@ def test_cnn_matches_oracle(conv, fc, dtype, W, B, rounds, tol):
 def test_cnn_tensor_core_shapes(conv, fc, W, B):
     cfg = _cnn_cfg(conv, fc, inputs.BF16, W, B, 3, 5, GAMMA3)
     X, y, w0 = _problem(cfg)
-    compare_with_oracle(cfg, X, y, w0, 8, TOL_BF16, forced=True, loss_tol=5e-2)
+    compare_with_oracle(cfg, X, y, w0, 8, TOL_BF16, forced=True, loss_tol=5e-2, move_tol=TOL_MOVE_BF16)
 
 
 @pytest.mark.parametrize("conv,fc,W,B", [

@@ -49,8 +49,9 @@ def test_lsq_gradient_matches_oracle(n, B, d, bf16):
 
 
 @pytest.mark.parametrize("n,B,d,bf16", [
-    (8, 32, 64, False), (9, 32, 64, False),          # one cluster (a single launch), two clusters
-    (1, 300, 100, False), (3, 47, 96, True),         # eight / two CTAs per worker, uneven row shares
+    (8, 15, 64, False), (9, 15, 64, False),          # one CTA per worker: one cluster (a single launch), two clusters
+    (8, 32, 64, False), (9, 32, 64, False),          # four CTAs per worker: four clusters, five
+    (1, 300, 100, False), (3, 47, 96, True),         # eight CTAs per worker; four, uneven row shares
     (4, 9, 128, False), (4, 9, 132, False),          # 32 / 33 vectors per row
     (4, 9, 1024, False), (4, 9, 1028, False),        # longest rows kept in registers, shortest of the two-pass kernel
     (4, 9, 2048, True), (4, 9, 2056, True),

@@ -15,6 +15,11 @@ from paper_2301_08895_b200 import inputs
 pytestmark = pytest.mark.gpu
 
 TOL_FP32, TOL_BF16 = 1e-5, 2e-2
+# Difference of a block over the path it travelled, bf16 storage: both sides round the same quantities at the same points,
+# so they differ by stored values whose rounding or ReLU / pool decision falls differently in binary32 and binary64 (up to
+# 7e-4 of one round's step on the networks tested; a handful of rounds adds them up).  A weight tile that is not updated
+# is off by 0.024 or more.
+TOL_MOVE_BF16 = 1e-2
 
 
 def _problem(cfg):
@@ -286,8 +291,9 @@ def test_row_kernels(kind, dims, dtype, W, B, flags):
     cfg = _small_cfg(kind, dims, dtype, W, B, 3, 5, GAMMA3, lr=0.02)
     X, y, w0 = _problem(cfg)
     bf16 = dtype == inputs.BF16
+    kw = {"move_tol": TOL_MOVE_BF16} if bf16 else {}
     compare_with_oracle(cfg, X, y, w0, 4, TOL_BF16 if bf16 else TOL_FP32, forced=True, loss_tol=5e-2 if bf16 else None,
-                        flags=flags)
+                        flags=flags, **kw)
 
 
 @pytest.mark.parametrize("kind,dims,conv,dtype,W,B,tiles", [
