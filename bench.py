@@ -416,27 +416,24 @@ def main():
     out["kernel_ms_profiled_step"] = kernels
     tot_prof = sum(t for _, t in prof.values())
     if U > 1:
-        # local steps: every worker's chain of U steps is sequential, one CTA per worker
+        # local steps: every worker's chain of U steps is sequential
         n_l, t_l = prof["lsq"]
         if cfg.kind == inputs.MLP and len(cfg.dims) > 2:
-            # multi-layer network: the workers' copies live in HBM; after each step but the last the refresh
-            # kernel streams, per selected worker, the upload sum (4 B/parameter), the model version the
-            # worker started from and the new copy (storage type each)
+            # multi-layer network, all hidden layers on the tensor cores: the weight-gradient kernel adds its tile to the
+            # worker's upload (4 B read, but in the first step, and 4 B written per parameter) and writes the refreshed
+            # copy from the version the worker started from (storage type each, but after the last step)
             d_pad = plan.get("d_pad") or sum(cfg.dims[l] * cfg.dims[l + 1] + cfg.dims[l + 1] for l in range(len(cfg.dims) - 1))
             n_rounds_prof = max(1, prof["update"][0])             # rounds the recorded launches cover
-            n_upd = (U - 1) * n_rounds_prof
-            per_par = 4.0 + 2.0 * (2 if bf16 else 4)
-            bytes_l = per_par * d_pad * float(np.mean(ks[:n_rounds_prof]))   # per refresh launch: bytes x d x K^t
-            # the class also holds the begin and layout kernels (1 + U launches per round, small)
-            out["roofline"] = {"bound": "hbm", "kernel": "local_step_kernel (+ local_begin launches)",
-                               "launches": n_l, "avg_us": 1e3 * t_l / max(1, n_l),
-                               "achieved": bytes_l * n_upd / (t_l * 1e-3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                               "frac": bytes_l * n_upd / (t_l * 1e-3) / 1e9 / peaks["hbm_gbs"], "traffic": None,
-                               "peak_source": peaks["source"], "share_of_profiled_time": t_l / tot_prof,
-                               "note": "algorithmic bytes of the U - 1 copy refreshes per round only, over the time of the "
-                                       "whole class (begin and last-step launches included)"}
+            n_w, t_w = prof["wgrad"]
+            per_par = 4.0 * U + (4.0 + 2.0 * (2 if bf16 else 4)) * (U - 1)
+            ach = per_par * d_pad * float(np.sum(ks[:n_rounds_prof])) / (t_w * 1e-3) / 1e9
+            out["roofline"] = {"bound": "l2", "kernel": "tc_gemm_kernel (weight gradients with the local step in their epilogue)",
+                               "launches": n_w, "avg_us": 1e3 * t_w / max(1, n_w), "achieved": ach, "peak": peaks["hbm_gbs"],
+                               "unit": "GB/s", "frac": ach / peaks["hbm_gbs"], "traffic": None, "peak_source": peaks["source"],
+                               "share_of_profiled_time": t_w / tot_prof,
+                               "note": "algorithmic bytes of uploads and copies, which mostly stay in L2, against the HBM copy bandwidth"}
         else:
-            out["roofline"] = {"bound": "latency", "kernel": "local_sgd_kernel", "achieved": None, "peak": None,
+            out["roofline"] = {"bound": "latency", "kernel": "local_cluster_kernel", "achieved": None, "peak": None,
                                "unit": None, "frac": None, "traffic": None,
                                "avg_us": 1e3 * t_l / max(1, n_l), "share_of_profiled_time": t_l / tot_prof,
                                "note": "U sequential minibatch steps per job; see minibatch_gradients_per_sec"}
@@ -455,14 +452,18 @@ def main():
                            "traffic": None, "peak_source": peaks["source"],
                            "share_of_profiled_time": t_l / tot_prof}
     elif cfg.kind == inputs.CNN:
-        # FP32-FMA kernels: 148 SMs x 128 lanes x 2 flop per clock at the maximum SM clock
         n_c, t_c = prof["conv"]
-        peak = 148 * 128 * 2 * 1.965e9 / 1e12
         ach = wg_p * flops["conv"] / (t_c * 1e-3) / 1e12
-        out["roofline"] = {"bound": "alu", "kernel": "conv_block_fwd_kernel + conv_block_bwd_kernel (+ chunk sums)",
-                           "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
-                           "peak_source": "148 SMs x 128 FP32 lanes x 2 flop x 1.965 GHz",
-                           "share_of_profiled_time": t_c / tot_prof}
+        if bf16 and not (args.flags & 1):
+            # matrix instructions on maps in shared memory: bound by operand reads and the latency of their chains
+            peak, src = peaks.get("bf16_tflops_sustained") or peaks["bf16_tflops"], peaks["source"] + " (sustained bf16)"
+            bound, kernel = "latency", "conv_fwd_mma_kernel + conv_bwd_mma_kernel"
+        else:
+            # FP32-FMA kernels: 148 SMs x 128 lanes x 2 flop per clock at the maximum SM clock
+            peak, src = 148 * 128 * 2 * 1.965e9 / 1e12, "148 SMs x 128 FP32 lanes x 2 flop x 1.965 GHz"
+            bound, kernel = "alu", "conv_block_fwd_kernel + conv_block_dgrad_kernel + conv_block_wgrad_kernel"
+        out["roofline"] = {"bound": bound, "kernel": kernel, "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+                           "frac": ach / peak, "traffic": None, "peak_source": src, "share_of_profiled_time": t_c / tot_prof}
     elif prof["fwd"][0] and bf16:
         t_g = prof["fwd"][1] + prof["dgrad"][1] + prof["wgrad"][1]
         fl = wg_p * (flops["fwd"] + flops["dgrad"] + flops["wgrad"])
@@ -485,7 +486,12 @@ def main():
                            "frac": None, "traffic": None,
                            "note": "launch/dependency-latency bound configuration; see rounds_per_sec"}
     n_u, t_u = prof["update"]
-    if n_u:
+    if n_u and U == 1 and cfg.kind != inputs.LSQ and prof["wgrad"][0] == 0:
+        # two kernels a round: the Eq. 3 step shares a kernel with the weight gradients of all layers
+        out["roofline_update"] = {"bound": "latency", "kernel": "grad_step_kernel (weight gradients of all layers, Eq. 3 step)",
+                                  "launches": n_u, "avg_us": 1e3 * t_u / n_u, "achieved": None, "peak": None, "unit": None,
+                                  "frac": None, "traffic": None}
+    elif n_u:
         # Eq. 3 step: read fp32 master + P fp32 partial sums, write master + storage-type ring slot
         esz = 2 if bf16 else 4
         P = plan["partials"] if plan["partials"] > 0 else float(np.mean(ks[:n_u]))
@@ -493,7 +499,8 @@ def main():
         ach = bytes_launch / (t_u / n_u * 1e-3) / 1e9
         traffic_u = measured_traffic("update", args.config, not args.samples)
         sec_u = t_u / n_u * 1e-3
-        out["roofline_update"] = {"bound": "hbm", "kernel": "update_kernel", "launches": n_u,
+        out["roofline_update"] = {"bound": "hbm", "kernel": "lsq_update_kernel" if cfg.kind == inputs.LSQ and U == 1 else "update_kernel",
+                                  "launches": n_u,
                                   "avg_us": 1e3 * t_u / n_u, "partials": P,
                                   "bytes_per_launch": bytes_launch, "achieved": ach,
                                   "peak": peaks["hbm_gbs"], "unit": "GB/s",

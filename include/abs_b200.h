@@ -100,13 +100,18 @@ extern "C" {
 /* kernel classes reported by abs_profile_read */
 #define ABS_KC_CTL     0  /* arrival selection + Eq. 4-6 bookkeeping */
 #define ABS_KC_GATHER  1  /* minibatch row gather */
-#define ABS_KC_FWD     2  /* hidden-layer forward contraction (Eq. 2) */
+#define ABS_KC_FWD     2  /* hidden-layer forward contraction (Eq. 2); networks without tensor-core layers and the
+                             affine layers of ABS_CNN, where two kernels make a round: all layers forward, loss and
+                             all deltas backward */
 #define ABS_KC_DGRAD   3  /* hidden-layer delta back-propagation */
-#define ABS_KC_WGRAD   4  /* weight gradient summed over the selected workers (Eq. 3) */
+#define ABS_KC_WGRAD   4  /* weight gradient summed over the selected workers (Eq. 3); with local_steps > 1 and all
+                             hidden layers on the tensor cores also the local step of those layers */
 #define ABS_KC_OUTPUT  5  /* output layer: forward + loss, its back-propagation and gradient */
 #define ABS_KC_LSQ     6  /* least-squares residual + gradient; with local_steps > 1: the workers' local steps
-                             (single-layer models), or their set-up, row layouts and copy refreshes (networks) */
-#define ABS_KC_UPDATE  7  /* Eq. 3 step + ring write */
+                             (single-layer models), or their set-up, row layouts, output-layer steps and copy
+                             refreshes (networks) */
+#define ABS_KC_UPDATE  7  /* Eq. 3 step + ring write; where two kernels make a round (see ABS_KC_FWD) with the weight
+                             and bias gradients of all layers */
 #define ABS_KC_ROUNDS  8  /* whole rounds (control step + Eq. 2 + Eq. 3) of a small least-squares problem
                              in one persistent kernel; one launch per abs_enqueue_rounds call */
 #define ABS_KC_CONV    9  /* ABS_CNN: the convolution blocks, forward and backward */

@@ -160,7 +160,7 @@ int check_model(const abs_model_desc* m, int W, int S) {
 double tc_launch_us(int bn, int cg, long tiles, double kb) {
   const double fixed = bn == 256 ? 3.5 : bn == 128 ? 2.6 : 2.2;
   const double per_kb = cg == 2 ? 0.5 : bn == 256 ? 0.34 : 0.25;
-  const long units = 148 / cg, waves = (tiles + units - 1) / units;
+  const long units = PLAN_SMS / cg, waves = (tiles + units - 1) / units;
   return (double)waves * (fixed + per_kb * kb);
 }
 
@@ -191,7 +191,7 @@ void plan_tc(const abs_model_desc* m, long rows, long row_tiles, int maxP, Layou
     // delta back-propagation: both have one or two tiles per CTA, so separate launches would pay the fixed costs twice.
     else if (l > 0 && !L->local_net && !(m->flags & ABS_FLAG_NO_FUSED_BACKWARD) && out >= L->bn_dg[l]) {
       const int bn = L->bn_dg[l];
-      if ((long)((in + 127) / 128 + 1) * ((out + bn - 1) / bn) * maxP < 148) { L->pair_bwd[l] = true; L->bn_wg[l] = bn; }
+      if ((long)((in + 127) / 128 + 1) * ((out + bn - 1) / bn) * maxP < PLAN_SMS) { L->pair_bwd[l] = true; L->bn_wg[l] = bn; }
     }
   }
   double best = 1e30;
@@ -245,7 +245,7 @@ bool tiles_win(const abs_model_desc* m, const Layout& L, long long rows) {
     all += w;
     if (l > 0 || L.cnn) back += w;
   }
-  if (L.esz == 4) return L.row_R == 4 && rows > 4 * 148 && 4 * back > all;
+  if (L.esz == 4) return L.row_R == 4 && rows > 4 * PLAN_SMS && 4 * back > all;
   if (L.any_tc) return back > 720000 && (rows < 2048 || back > 1250000);
   return !L.cnn && back > 700000 && rows < 512;      // (the CNN's convolutions lose their matrix-instruction kernels with the row kernels)
 }
@@ -349,7 +349,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
     ra.n_layers = m->n_layers;
     for (int l = 0; l <= m->n_layers; ++l) ra.dims[l] = m->dims[l];
     size_t smem = 0;
-    const int R0 = L->esz == 2 ? (rows <= 148 * 8 ? 8 : 16) : rows <= 148 * 4 ? 4 : rows <= 2 * 148 * 8 ? 8 : 16;
+    const int R0 = L->esz == 2 ? (rows <= PLAN_SMS * 8 ? 8 : 16) : rows <= PLAN_SMS * 4 ? 4 : rows <= 2 * PLAN_SMS * 8 ? 8 : 16;
     for (int R = R0; R >= (L->esz == 2 ? 8 : 4) && !L->row_R; R /= 2)
       if (rnet::plan_rows(&ra, R, (int)L->esz, &smem)) L->row_R = R;
     if (L->row_R && !ra.resident && tiles_win(m, *L, rows)) L->row_R = 0;
@@ -362,7 +362,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       // CTAs per tile: up to two per SM, at least one pipeline step of rows each (50 tiles, 8 steps: 18.9 us a round with
       // two steps each, 21.7 with four; 67 tiles, 12 steps: 89.6 with three, 94.5 with one and a half)
       L->step_Q = 1;
-      while (L->step_Q < 8 && tiles * L->step_Q * 2 <= 2 * 148 && rows >= 2 * rnet::GK * L->step_Q) L->step_Q *= 2;
+      while (L->step_Q < 8 && tiles * L->step_Q * 2 <= 2 * PLAN_SMS && rows >= 2 * rnet::GK * L->step_Q) L->step_Q *= 2;
     }
   }
   L->RB = lsq ? m->batch : L->row_R ? L->row_R : (L->any_tc ? 128 : 64);
@@ -435,7 +435,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       // more than a handful of blocks (each is a chain of dependent loads)
       L->narrow_rpb = 64;
       if (!L->local_net)
-        while (L->narrow_rpb > 8 && (long long)W * m->batch / L->narrow_rpb < 2 * 148) L->narrow_rpb /= 2;
+        while (L->narrow_rpb > 8 && (long long)W * m->batch / L->narrow_rpb < 2 * PLAN_SMS) L->narrow_rpb /= 2;
       L->red = cv.take(4 * len * (size_t)(L->rows_cap / (L->fused_R ? L->fused_R : L->narrow_rpb)));
     }
     L->ones = L->any_tc ? cv.take(2 * 64 * (size_t)L->rows_cap) : 0;
@@ -462,7 +462,7 @@ void make_layout(const abs_model_desc* m, int W, int S, Layout* L) {
       // worker is selected (a CTA is 8 warps on a chain of shared-memory loads: measured on 640 rows per round,
       // 1 / 2 / 4 / 8 rows per CTA give 1742 / 1617 / 1409 / 1222 rounds/s)
       L->cchunk = 1;
-      while (L->cchunk < conv::MAX_CHUNK && (long long)W * m->batch / (2 * L->cchunk) >= 4 * 148) L->cchunk *= 2;
+      while (L->cchunk < conv::MAX_CHUNK && (long long)W * m->batch / (2 * L->cchunk) >= 4 * PLAN_SMS) L->cchunk *= 2;
       if (L->conv_mma) L->cchunk = cmma::FR;
       if (L->conv_mma) {
         cmma::Block cb[2];
@@ -511,7 +511,7 @@ struct abs_ctx {
   abs_model_desc m;
   Layout L;
   int W, K0, S;
-  int sm_count = 148;
+  int sm_count = PLAN_SMS;
   cudaStream_t stream;
   // The control kernel (and the row gather) of round t+1 only need the losses of round t, so they
   // run on a second stream next to the backward kernels of round t.

@@ -23,6 +23,9 @@ enum : int {
 };
 
 constexpr int MAX_W = ABS_MAX_WORKERS;
+// SMs of the GPU the plans are made for.  A plan must not depend on a device: abs_workspace_bytes needs none and has to agree
+// with abs_init.  (Grids of persistent kernels follow the device's count.)
+constexpr int PLAN_SMS = 148;
 constexpr int MAX_TAU = ABS_MAX_BOUND + 1;
 
 struct TimeDist {

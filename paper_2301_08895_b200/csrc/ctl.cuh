@@ -503,10 +503,11 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
 
 // pdl = 0: the step waits for the kernel in front of it before it starts.  pdl = 1: the kernel in
 // front is the Eq. 3 step of the round being finished, which this step does not depend on (it reads
-// the uploaded losses, which were complete before the Eq. 3 kernel passed its own wait, and it
-// prepares the job durations itself): the two run side by side, and this kernel waits for the
-// Eq. 3 kernel only at its end, so that whatever follows in the stream sees both complete.
-// look: see ctl_round (the Eq. 3 kernel then does not touch the prepared durations).
+// the uploaded losses, which were complete before the Eq. 3 kernel passed its own wait, and the job
+// durations, which it prepares itself (look, see ctl_round) or the round's gradient kernels have
+// prepared: row kernels and least-squares pipeline): the two run side by side, and this kernel waits
+// for the Eq. 3 kernel only at its end, so that whatever follows in the stream sees both complete.
+// The Eq. 3 kernel does not touch the prepared durations on these paths.
 __global__ void __launch_bounds__(1024, 1) abs_ctl_kernel(CtlArgs a, int do_finish, int do_select, int t_sel, int pdl, int look) {
   if (pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   else grid_dependency_sync();

@@ -1,5 +1,6 @@
-// Local SGD inside a job (Eq. 2 with U > 1): one CTA per selected worker runs the worker's U
-// minibatch steps one after the other on its own copy of the model, which starts at the version the
+// Local SGD inside a job (Eq. 2 with U > 1): a cluster of CTAs per selected worker (local_cluster_kernel), or one CTA
+// (local_sgd_kernel: steps whose rows do not fit a cluster, tiny steps of many workers; see cluster_plan), runs the worker's U
+// minibatch steps one after the other on the worker's own copy of the model, which starts at the version the
 // worker holds (its ring slot) and lives in shared memory as fp32 (bf16 configurations compute each
 // step with the bf16 rounding of that copy, as their tensor-core paths must).  Step u draws its minibatch from
 // Philox blocks (n, j, 1, u * ceil(B/4) + b/4).  The upload is the sum over the steps of the
@@ -7,8 +8,8 @@
 // minibatch losses (Algorithm 1, last worker line); Eq. 3 then reads the K uploads like the
 // partial sums of the U = 1 path.  Single-layer models only (least squares, soft-max regression
 // with at most 16 classes): their parameter vector fits in shared memory twice.
-// The chains of different workers are independent but each is strictly sequential, so the kernel
-// is latency-bound by design; a step is B short dot products and one rank-B update.
+// The chains of different workers are independent but each is strictly sequential, so the kernels
+// are latency-bound by design; a step is B short dot products and one rank-B update.
 #pragma once
 #include <algorithm>
 
@@ -250,7 +251,7 @@ inline size_t cluster_smem(const Geo& g, int esz, int B, int CP) {
 // cluster; 784 -> 10 bf16, 100 workers, 4 rows 123 / 156, 16 rows 168 / 166.
 inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) {
   const int CP = round_up(C, 4), ge = 16 / esz;
-  const int wave = 148 * cluster_ctas_per_sm(ge, CP);
+  const int wave = PLAN_SMS * cluster_ctas_per_sm(ge, CP);
   auto geo = [&](int Q, int nbuf) {
     Geo g;
     g.Q = Q;
@@ -264,10 +265,10 @@ inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) 
     return g;
   };
   int first = 8;
-  while (first > 1 && (W * first > 2 * 148 || in / first < 32)) first /= 2;
+  while (first > 1 && (W * first > 2 * PLAN_SMS || in / first < 32)) first /= 2;
   Geo none = geo(1, 1);
   none.Q = 0;
-  if (n_par < 2048 && (B <= 8 ? n * first > wave : B <= 12 && wave == 148 && n * first > 2 * wave)) return none;
+  if (n_par < 2048 && (B <= 8 ? n * first > wave : B <= 12 && wave == PLAN_SMS && n * first > 2 * wave)) return none;
   if (n_par > 6000 && B <= 8 && first == 2 && n * first > wave) return none;
   for (int nbuf = 2; nbuf >= 1; --nbuf)
     for (int Q = first; Q <= 8; Q *= 2) {

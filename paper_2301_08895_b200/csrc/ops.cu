@@ -350,7 +350,7 @@ int run(const void* X, const float* y, const void* w, const int* idx, int n, int
   const bool vec = (((uintptr_t)X | (uintptr_t)w | ((uintptr_t)d * esz)) & 15) == 0;    // rows on 16-byte boundaries
   OpArgs a = {X, y, w, idx, n, B, d, 1, scratch, loss_out, g_out, 0, d > OP_SMEM_D ? 1 : 0};
   // CTAs per worker: enough for two per SM, at least a row per warp
-  while (!a.direct && a.Q < CL && n * a.Q * 2 <= 2 * 148 && B >= 2 * a.Q * OP_NW) a.Q *= 2;
+  while (!a.direct && a.Q < CL && n * a.Q * 2 <= 2 * PLAN_SMS && B >= 2 * a.Q * OP_NW) a.Q *= 2;
   const int per = CL / a.Q, clusters = (n + per - 1) / per;
   a.single = !a.direct && clusters == 1 ? 1 : 0;
   size_t smem = 0;
