@@ -558,6 +558,18 @@ int cuda_fail(abs_ctx* ctx, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call);       \
   } while (0)
 
+// The dynamic shared memory a kernel may be launched with belongs to the kernel and not to a context: where it depends on
+// the model it is set to the most there is (227 KB less the kernel's own), so that a context that is created later does not
+// lower it under one that is still running.
+template <typename... KArgs>
+cudaError_t allow_smem(void (*kernel)(KArgs...), size_t need) {
+  cudaFuncAttributes fa;
+  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  const size_t most = 227 * 1024 - fa.sharedSizeBytes;
+  return need > most ? cudaErrorInvalidValue : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // One kernel launch on ctx->stream, counted and, while profiling, bracketed by events.  Launches
 // carry the programmatic-stream-serialization attribute: the next kernel's CTAs may be scheduled
 // while this one drains; every kernel of the round loop starts with griddepcontrol.wait, which
@@ -1312,11 +1324,11 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     if (eb != cudaSuccess) return bail(cuda_fail(nullptr, eb, "cudaFuncSetAttribute(abs_ctl_small_kernel)"));
   }
   if (L.out_mma) {
-    const int osm = (int)outl::smem_bytes(model->dims[model->n_layers - 1], model->dims[model->n_layers]);
-    cudaError_t eo = cudaFuncSetAttribute(outl::out_layer_mma_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, osm);
-    if (eo == cudaSuccess) eo = cudaFuncSetAttribute(outl::out_layer_mma_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, osm);
-    if (eo == cudaSuccess) eo = cudaFuncSetAttribute(outl::out_layer_mma_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, osm);
-    if (eo == cudaSuccess) eo = cudaFuncSetAttribute(outl::out_layer_mma_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, osm);
+    const size_t osm = outl::smem_bytes(model->dims[model->n_layers - 1], model->dims[model->n_layers]);
+    cudaError_t eo = allow_smem(outl::out_layer_mma_kernel<1>, osm);
+    if (eo == cudaSuccess) eo = allow_smem(outl::out_layer_mma_kernel<2>, osm);
+    if (eo == cudaSuccess) eo = allow_smem(outl::out_layer_mma_kernel<4>, osm);
+    if (eo == cudaSuccess) eo = allow_smem(outl::out_layer_mma_kernel<8>, osm);
     if (eo != cudaSuccess) return bail(cuda_fail(nullptr, eo, "cudaFuncSetAttribute(out_layer_mma_kernel)"));
   }
   if (L.fused_R) {
@@ -1340,13 +1352,13 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     ctx->local_geo = local::cluster_plan(model->dims[0], C, n_par, model->batch, W, model->k_mode == ABS_K_FIXED ? K0 : W, (int)L.esz);
     cudaError_t el;
     if (ctx->local_geo.Q > 0) {
-      const int sm = (int)local::cluster_smem(ctx->local_geo, (int)L.esz, model->batch, round_up(C, 4));
-      el = L.esz == 4 ? cudaFuncSetAttribute(local_cluster_fn<float>(C), cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                      : cudaFuncSetAttribute(local_cluster_fn<__nv_bfloat16>(C), cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+      const size_t sm = local::cluster_smem(ctx->local_geo, (int)L.esz, model->batch, round_up(C, 4));
+      el = L.esz == 4 ? allow_smem(local_cluster_fn<float>(C), sm)
+                      : allow_smem(local_cluster_fn<__nv_bfloat16>(C), sm);
     } else {
-      const int sm = (int)local::smem_bytes(n_par, model->batch, C);
-      el = L.esz == 4 ? cudaFuncSetAttribute(local::local_sgd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                      : cudaFuncSetAttribute(local::local_sgd_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+      const size_t sm = local::smem_bytes(n_par, model->batch, C);
+      el = L.esz == 4 ? allow_smem(local::local_sgd_kernel<float>, sm)
+                      : allow_smem(local::local_sgd_kernel<__nv_bfloat16>, sm);
     }
     if (el != cudaSuccess) return bail(cuda_fail(nullptr, el, "cudaFuncSetAttribute(local-step kernel)"));
     ctx->local_sgd = true;
@@ -1359,8 +1371,8 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
       int stages = lsqp::MAX_STAGES;
       while (stages >= 2 && lsqp::smem_bytes(model->dims[0], stages) > 227 * 1024) --stages;
       if (stages >= 2) {
-        const int sm = (int)lsqp::smem_bytes(model->dims[0], stages);
-        cudaError_t ep = cudaFuncSetAttribute(lsqp::lsq_pipe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        const size_t sm = lsqp::smem_bytes(model->dims[0], stages);
+        cudaError_t ep = allow_smem(lsqp::lsq_pipe_kernel, sm);
         if (ep != cudaSuccess) return bail(cuda_fail(nullptr, ep, "cudaFuncSetAttribute(lsq_pipe_kernel)"));
         ctx->lsq_pipe = true;
         ctx->lsq_stages = stages;
@@ -1372,9 +1384,9 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
       model->dims[0] <= LSQ_ROUNDS_MAX_D && W <= LSQ_ROUNDS_NTG && (size_t)W * model->batch <= LSQ_ROUNDS_MAX_ROWS &&
       (size_t)(S_ring + 1) * model->dims[0] * 4 <= 64 * 1024) {
     const size_t sm = lsq_rounds_smem(S_ring, model->dims[0]);
-    cudaError_t er = cudaFuncSetAttribute(abs_lsq_rounds_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t er = allow_smem(abs_lsq_rounds_kernel<float>, sm);
     if (er == cudaSuccess)
-      er = cudaFuncSetAttribute(abs_lsq_rounds_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      er = allow_smem(abs_lsq_rounds_kernel<__nv_bfloat16>, sm);
     if (er != cudaSuccess) return bail(cuda_fail(nullptr, er, "cudaFuncSetAttribute(abs_lsq_rounds_kernel)"));
     ctx->lsq_rounds = true;
   }
@@ -1405,12 +1417,12 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     for (int b = 0; b < 2; ++b)
       need = std::max(need, std::max(conv::fwd_smem_bytes(L.cHi[b], L.cWi[b], L.cCi[b], L.ck, L.cCo[b]),
                                      conv::bwd_smem_bytes(L.cHi[b], L.cWi[b], L.cCi[b], L.ck, L.cCo[b])));
-    cudaError_t ec = cudaFuncSetAttribute(conv::conv_block_fwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_fwd_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_wgrad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_wgrad_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_dgrad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (ec == cudaSuccess) ec = cudaFuncSetAttribute(conv::conv_block_dgrad_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    cudaError_t ec = allow_smem(conv::conv_block_fwd_kernel<float>, need);
+    if (ec == cudaSuccess) ec = allow_smem(conv::conv_block_fwd_kernel<__nv_bfloat16>, need);
+    if (ec == cudaSuccess) ec = allow_smem(conv::conv_block_wgrad_kernel<float>, need);
+    if (ec == cudaSuccess) ec = allow_smem(conv::conv_block_wgrad_kernel<__nv_bfloat16>, need);
+    if (ec == cudaSuccess) ec = allow_smem(conv::conv_block_dgrad_kernel<float>, need);
+    if (ec == cudaSuccess) ec = allow_smem(conv::conv_block_dgrad_kernel<__nv_bfloat16>, need);
     for (auto fn : {cmma::conv_fwd_mma_kernel<0>, cmma::conv_fwd_mma_kernel<3>, cmma::conv_fwd_mma_kernel<5>, cmma::conv_bwd_mma_kernel<0>,
                     cmma::conv_bwd_mma_kernel<3>, cmma::conv_bwd_mma_kernel<5>})
       if (ec == cudaSuccess && L.conv_mma) ec = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);

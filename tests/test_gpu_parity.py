@@ -413,6 +413,37 @@ def test_trace_windows(max_rounds):
     ctx.close()
 
 
+@pytest.mark.parametrize("kind,dtype,large,small,kw", [
+    (inputs.SOFTMAX, inputs.FP32, (784, 10), (24, 10), {"local_steps": 2}),          # local steps, cluster kernel
+    (inputs.LSQ, inputs.BF16, (4096, 1), (64, 1), {"flags": gpu.FLAG_NO_PERSISTENT}),  # bulk-copy pipeline
+    (inputs.LSQ, inputs.FP32, (256, 1), (16, 1), {}),                                # all rounds in one kernel
+    (inputs.MLP, inputs.BF16, (64, 128, 16), (64, 128, 3), {}),                      # output layer
+    (inputs.CNN, inputs.FP32, (32, 32, 3, 5, 6, 16), (14, 14, 1, 3, 4, 4), {}),      # FP32 convolutions
+])
+def test_a_later_smaller_context_leaves_an_earlier_one_running(kind, dtype, large, small, kw):
+    """Two contexts at once: the kernels' shared-memory limits of the first survive the set-up of the second."""
+    def problem(dims):
+        conv = None
+        if kind == inputs.CNN:
+            conv, (H, Wd, _, k, _, c2) = dims, dims
+            dims = ((((H - k + 1) // 2 - k + 1) // 2) * (((Wd - k + 1) // 2 - k + 1) // 2) * c2, 12, 5)
+        cfg = _small_cfg(kind, dims, dtype, 8, 16, 3, 5, GAMMA3, lr=1e-4)
+        cfg.conv, cfg.w0 = conv, cfg.w0 if conv is None else "he"
+        X, y, w0 = _problem(cfg)
+        Xd, yd = to_device(cfg, X, y)
+        return lambda: gpu.context_from_config(cfg, Xd, yd, w0, max_rounds=6, **kw)
+    make_large, make_small = problem(large), problem(small)
+    alone = make_large()
+    alone.run_rounds(6)
+    a = make_large()
+    b = make_small()
+    a.run_rounds(6)
+    b.run_rounds(6)
+    assert np.array_equal(a.get_params().view(np.uint32), alone.get_params().view(np.uint32))
+    for c in (alone, a, b):
+        c.close()
+
+
 def test_host_dataset_entry_gives_same_result():
     cfg = inputs.config(1)
     X, y, w0 = _problem(cfg)
