@@ -42,8 +42,9 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
 // consecutive products independent of one another.  Sums over many products use it (gradients, back-propagated deltas, bias
 // sums): the additions hide behind the operand reads (CNN 75.9 -> 75.7 us a round, 785-513-511-10 bf16 291 -> 296).  One
 // step of the 32 x 32 x 3 CNN against binary64 with the same storage rounding, mean of four inputs: 4.6e-4 on the first
-// convolution's weights (FP32 FMAs 6.8e-4), 7e-5 on the first affine layer's (2.7e-4): what flipped decisions leave; the
-// truncating form differs from this one by 3e-7 of the step.
+// convolution's weights (FP32 FMAs 6.8e-4), 7e-5 on the first affine layer's (2.7e-4): what flipped decisions leave.  Its
+// parameters after 200 rounds: 3.65e-4 from binary64 (FP32 FMAs 3.64e-4, truncating chains 4.77e-4; binary64 itself from
+// weights perturbed by 1e-7: 5.2e-4).
 __device__ __forceinline__ void mma16816_rn(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   float p[4];
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
