@@ -79,10 +79,11 @@ struct RoundInfo {
   int t;            // round index
   int diverged;     // set by the loss kernels of the round; RI_TIMEOUT: a bounded wait of such a kernel expired
 };
-constexpr int RI_DIVERGED = 1, RI_TIMEOUT = 2;
+constexpr int RI_DIVERGED = 1, RI_TIMEOUT = 0x100;
 // For kernels in which both can happen: after a wait that ran out a CTA goes on with whatever is there, so that a
-// non-finite loss is likely as well; the caller is told about the wait.
-__device__ __forceinline__ void report(RoundInfo* ri, int what) { atomicMax(&ri->diverged, what); }
+// non-finite loss is likely as well; the caller is told about the wait.  Each has a byte of its own in the word (an atomic
+// maximum made the row kernel of a 144 -> 10 fp32 round of 3596 rows 14.25 -> 14.55 us).
+__device__ __forceinline__ void report(RoundInfo* ri, int what) { reinterpret_cast<unsigned char*>(&ri->diverged)[what >> 8] = 1; }
 
 // x / n for x < 2^31 / n (items of a loop), by a multiplication: an integer division costs a few hundred
 // cycles otherwise

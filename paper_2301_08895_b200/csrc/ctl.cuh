@@ -266,7 +266,7 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     }
     const int bad = __syncthreads_or((tid < K) && !isfinite(my_loss)) || diverged0;
     if (bad) {
-      if (tid == 0) { raise(diverged0 == RI_TIMEOUT ? ST_TIMEOUT : ST_DIVERGED); st->open = 0; }
+      if (tid == 0) { raise(diverged0 & RI_TIMEOUT ? ST_TIMEOUT : ST_DIVERGED); st->open = 0; }
       return 1;
     }
     // loss estimate: adjacent-pair tree sum in binary32 over 1024 leaves, /K in binary32

@@ -195,7 +195,7 @@ def test_trace_arrays_do_not_hold_each_other(monkeypatch):
 
 def test_a_timeout_is_not_overwritten_by_a_divergence():
     """Kernels whose waits report through the round's status word (RI_TIMEOUT) must keep it when another CTA, or another
-    warp of the same one, reports a non-finite loss: every report of theirs takes the maximum, none is a plain store."""
+    warp of the same one, reports a non-finite loss: every report of theirs has a byte of its own, none stores the word."""
     csrc = os.path.join(ROOT, "paper_2301_08895_b200", "csrc")
     checked = 0
     for name in sorted(os.listdir(csrc)):
@@ -209,6 +209,8 @@ def test_a_timeout_is_not_overwritten_by_a_divergence():
             assert not re.search(r"->diverged\s*=[^=]", helper), name
             checked += 1
     assert checked >= 4
-    common = open(os.path.join(csrc, "common.cuh")).read()
-    assert re.search(r"void report\(RoundInfo\* ri, int what\) \{ atomicMax\(&ri->diverged, what\); \}", common)
-    assert re.search(r"RI_DIVERGED = 1, RI_TIMEOUT = 2", common)
+    read = lambda name: open(os.path.join(csrc, name)).read()
+    assert re.search(r"RI_DIVERGED = 1, RI_TIMEOUT = 0x100;", read("common.cuh"))          # bytes 0 and 1 of the word
+    assert re.search(r"void report\(RoundInfo\* ri, int what\) \{ reinterpret_cast<unsigned char\*>\(&ri->diverged\)\[what >> 8\] = 1; \}",
+                     read("common.cuh"))
+    assert re.search(r"diverged0 & RI_TIMEOUT \? ST_TIMEOUT : ST_DIVERGED", read("ctl.cuh"))
