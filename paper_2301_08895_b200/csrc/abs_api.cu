@@ -1485,7 +1485,7 @@ int abs_enqueue_rounds(abs_ctx* ctx, int n) {
     local::Args q;
     q.st = ctx->at<DevState>(ctx->L.st);
     q.sel = nullptr; q.sel_tau = nullptr; q.ri = nullptr;
-    q.job = ctx->ctl.job; q.X = ctx->X; q.y = ctx->y;
+    q.job = ctx->ctl.job; q.shard = ctx->ctl.shard; q.X = ctx->X; q.y = ctx->y;
     q.ring = ctx->at<void>(ctx->L.ring); q.slot_stride = ctx->L.d_pad;
     q.loss = ctx->ctl.loss; q.G = ctx->at<float>(ctx->L.G);
     q.lsq = ctx->m.kind == ABS_LSQ ? 1 : 0;
@@ -1502,7 +1502,7 @@ int abs_enqueue_rounds(abs_ctx* ctx, int n) {
       if (geo.Q > 0) {
         ctx->next_cluster = geo.Q;
         launch_ex(ctx, ABS_KC_LSQ, f32 ? local_cluster_fn<float>(q.C) : local_cluster_fn<__nv_bfloat16>(q.C), dim3(ctx->W * geo.Q),
-                  dim3(local::CL_THREADS), csm_local, q, geo);
+                  dim3(local::CL_NT), csm_local, q, geo);
       } else if (f32) launch_ex(ctx, ABS_KC_LSQ, local::local_sgd_kernel<float>, dim3(ctx->W), dim3(nt), sm, q);
       else launch_ex(ctx, ABS_KC_LSQ, local::local_sgd_kernel<__nv_bfloat16>, dim3(ctx->W), dim3(nt), sm, q);
       update(par);

@@ -31,6 +31,7 @@ struct Args {
   DevState* st;
   RoundInfo* ri;
   const int* sel; const int* job; const int* sel_tau;
+  const int2* shard;                  // [W] first sample and length of each worker's shard
   const void* X; const void* y;       // y: float targets (least squares) or int labels
   const void* ring; size_t slot_stride;
   float* loss;                        // [W] uploaded loss of each selected worker
@@ -207,26 +208,33 @@ __global__ void __launch_bounds__(NT_MAX) local_sgd_kernel(Args a) {
 // ---------------------------------------------------------------------------------------------
 // The same local steps with a CLUSTER of Q CTAs per selected worker.  The one-CTA kernel above uses K of
 // 148 SMs and walks every row twice through L2 with scalar loads; here CTA q of the cluster owns the features
-// [q F, (q + 1) F) of the worker's model, which stay in its shared memory for the whole job:
+// [q F, (q + 1) F) of the worker's model, which stay in its shared memory for the whole job, and the soft-max of the
+// rows [q RQ, (q + 1) RQ) of every step:
 //   - the slice of a step's B rows is copied once (asynchronously, one step ahead: a job's minibatches are known
 //     from the counter-based generator) and serves both the forward pass and the gradient,
-//   - the CTAs exchange their partial logits through distributed shared memory (one cluster barrier per step,
-//     then every CTA reads its peers' [B][C] blocks), and every CTA forms the soft-max, the deltas and the gradient
-//     of its own features,
-//   - a helper warp draws indices, issues the copies and finishes loss and bias, off the critical path.
-// A step is bound by its chain of phases (copy wait, partial dots, exchange, soft-max, gradient, reduction), each a
-// few hundred to a few thousand cycles of dependent shared-memory reads.
+//   - each CTA sends its partial logits of a row to the row's owner and the owner sends the row's deltas to every CTA,
+//     both as remote stores that complete on the receiver's mbarrier (st.async; launched as a cluster only, Q > 1): no
+//     cluster barrier inside a step,
+//   - the copies of the next rows and the draws of the step after that are issued while the exchange is on its way.
+// A step is bound by its chain of phases (partial dots, exchange, soft-max, exchange, gradient, reduction), each a few
+// hundred to 1500 cycles of dependent shared-memory reads.  With a cluster barrier and remote loads (2400 cycles: its release
+// waits for all stores), bulk copies of the row slices by one warp that also took part in the soft-max (64 copies: 6900
+// cycles) a step of 784 -> 10, 16 workers x 64 rows took 14000 cycles, now 9000 (a round of ten steps 91.7 -> 73.1 us; 20 to 64
+// workers 74 us and 143 us; 2 to 16 classes, 87 to 687 features 1.12 to 1.43 times as fast).
+// Both buffers of the exchange are used again in the next step.  A CTA sends step u + 1's logits after it has all deltas of
+// step u, so every owner has read its logits of step u; an owner sends step u + 1's deltas after every CTA has sent its
+// logits of step u + 1, that is after the gradient of step u.
 struct Geo {
   int Q;        // CTAs per worker (cluster width)
   int F;        // features per CTA (a multiple of 8)
+  int RQ;       // rows of a step per CTA (soft-max)
   int pitch;    // elements between rows of the staged slices: an odd number of 16-byte groups, so that 16-byte
                 // reads of one column group by consecutive rows fall into different banks
   int nbuf;     // row buffers (2: the next step's rows are copied during this one)
   int PZ, PG;   // partial sums per row (forward) / per feature group (gradient) inside a CTA
 };
 
-constexpr int CL_NT = 224;               // compute threads
-constexpr int CL_THREADS = CL_NT + 32;   // and the helper warp (registers are handed out to four warps at a time)
+constexpr int CL_NT = 256;
 template <typename T> __host__ __device__ constexpr int group_elems() { return 16 / (int)sizeof(T); }
 
 // CTAs of the cluster kernel per SM: by the registers of one group's sums (ge elements x CP classes)
@@ -235,20 +243,19 @@ __host__ __device__ constexpr int cluster_ctas_per_sm(int ge, int CP) { return g
 inline size_t cluster_smem(const Geo& g, int esz, int B, int CP) {
   const size_t zp = std::max((size_t)g.PZ * B * CP, (size_t)g.PG * g.F * CP);
   return (size_t)g.nbuf * B * g.pitch * esz +
-         4 * ((size_t)(esz == 2 ? 3 : 2) * g.F * CP + zp + (size_t)3 * B * CP + (size_t)6 * round_up(B, 4) + 2 * 16) + 64;
+         4 * ((size_t)(esz == 2 ? 3 : 2) * g.F * CP + zp + ((size_t)g.Q * g.RQ + B) * CP + (size_t)4 * round_up(B, 4) + 2 * round_up(g.RQ, 4) + 2 * 16) + 64;
 }
 
 // Cluster width and staging for a model of `in` features, C classes, W workers of which n run at once (K^0 where K is
 // fixed, else all); Q = 0: the one-CTA kernel runs.
 // Q: as many CTAs as the chip holds twice over when every worker is selected, slices of at least 32 features.
-// Per launch on 784 -> 10 fp32, B = 64, U = 10: one-CTA kernel 366 us; clusters 74 us (8 workers), 85 us (16), 91 us
-// (32), 167 us (64); 512 instead of 224 compute threads lose the second CTA per SM (16 workers: 151 us).
 // The one-CTA kernel stays where the rows of a step do not fit a cluster's shared memory, and on batches of a few rows once
 // the clusters of n workers take more than one wave: for models below 2048 parameters (its CTAs are 256 threads there, and
 // several share an SM) and for large ones whose clusters of two take two partial waves.  us a round, one-CTA / cluster,
-// U = 10, all workers selected: 64 -> 10 bf16, 1024 workers, 4 rows 178 / 288, 8 rows 208 / 298, 12 rows 277 / 308; 200
-// workers, 8 rows 84 / 89, 12 rows 119 / 92; 64 -> 1 fp32, 512 workers, 4 rows 68 / 80, 8 rows 81 / 84, 12 rows the
-// cluster; 784 -> 10 bf16, 100 workers, 4 rows 123 / 156, 16 rows 168 / 166.
+// U = 10, all workers selected: 64 -> 10 bf16, 1024 workers, 4 rows 176 / 282, 8 rows 204 / 292, 12 rows 274 / 293; 200
+// workers, 8 rows 84 / 85, 12 rows 117 / 86; 64 -> 1 fp32, 512 workers, 4 rows 64 / 78, 8 rows 76 / 82, 12 rows 91 / 84;
+// 784 -> 10 bf16, 100 workers, 4 rows 117 / 147, 8 rows 129 / 143, 16 rows 165 / 159; 784 -> 10 fp32, 145 workers, 64 rows
+// 363 / 343.
 inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) {
   const int CP = round_up(C, 4), ge = 16 / esz;
   const int wave = PLAN_SMS * cluster_ctas_per_sm(ge, CP);
@@ -256,12 +263,15 @@ inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) 
     Geo g;
     g.Q = Q;
     g.F = round_up((in + Q - 1) / Q, 8);
+    g.RQ = (B + Q - 1) / Q;
     const int groups = g.F / ge;
     g.pitch = (groups | 1) * ge;
     g.nbuf = nbuf;
     const int pairs = (B + 1) / 2;
     g.PZ = std::max(1, std::min(std::min(CL_NT / std::max(1, pairs), 16), groups));
-    g.PG = std::max(1, std::min(std::min(CL_NT / groups, 8192 / (g.F * CP)), std::min(16, B / 4)));   // 32 KB of partial sums
+    // (32 KB of partial gradients: two CTAs have to fit an SM, since the chip has no room for 16 clusters of eight with an SM
+    // per CTA: with 48 KB the 16 workers above took two waves, 103 instead of 65 us)
+    g.PG = std::max(1, std::min(std::min(CL_NT / groups, 8192 / (g.F * CP)), std::min(16, B / 4)));
     return g;
   };
   int first = 8;
@@ -281,12 +291,35 @@ inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-  return v;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;" ::"n"(CL_NT) : "memory"); }
+// stores to shared memory of a CTA of the cluster, counted on that CTA's mbarrier (addresses: mapa)
+__device__ __forceinline__ void st_async4(uint32_t addr, float4 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async1(uint32_t addr, float v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
+}
+// the bytes other CTAs stored have arrived (acquire at cluster scope); bounded like tc::mbar_wait
+__device__ __forceinline__ uint32_t test_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(tc::smem_u32(bar)), "r"(parity) : "memory");
+  return ok;
+}
+__device__ __noinline__ void wait_cluster_slow(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+  const unsigned long long t0 = tc::global_ns();
+  for (uint32_t i = 1; i < (1u << 28); ++i) {
+    if (test_cluster(bar, parity)) return;
+    if ((i & 63u) == 0u && (*gave_up || tc::global_ns() - t0 > tc::WAIT_LIMIT_NS)) break;
+  }
+  *gave_up = 1;
+}
+__device__ __forceinline__ void wait_cluster(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+  if (!test_cluster(bar, parity)) wait_cluster_slow(bar, parity, gave_up);
+}
 __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
 // one 16-byte group of stored values as binary32
@@ -298,7 +331,7 @@ __device__ __forceinline__ void load_group(const __nv_bfloat16* p, float (&v)[8]
 
 // CP: class count rounded up to a multiple of 4 (padded classes have zero weights and zero deltas)
 template <typename T, int CP>
-__global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>(), CP)) local_cluster_kernel(Args a, Geo geo) {
+__global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), CP)) local_cluster_kernel(Args a, Geo geo) {
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char loc_raw[];
   using lsqp::f32x2;
@@ -306,145 +339,138 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
   DevState* st = a.st;
   RoundInfo* ri = a.ri;
   if (st->status != ST_OK) return;
-  const int Q = geo.Q, F = geo.F, pitch = geo.pitch, PZ = geo.PZ, PG = geo.PG;
+  const int Q = geo.Q, F = geo.F, RQ = geo.RQ, pitch = geo.pitch, PZ = geo.PZ, PG = geo.PG;
   const int i = (int)blockIdx.x / Q;
   if (i >= ri->K) return;                            // same decision in every CTA of the cluster
   const int rank = Q > 1 ? (int)tc::cluster_rank() : 0;
-  const int B = st->B, in = a.in, C = a.C, U = a.U, W = st->W;
+  const int B = st->B, in = a.in, C = a.C, U = a.U;
   const int n_w = in * C;
   const int m0 = rank * F, nf = max(0, min(F, in - m0));     // this CTA's features
+  const int b_own = rank * RQ, n_own = max(0, min(RQ, B - b_own));      // rows whose soft-max it forms
   const int groups = F / GE, n_g = F * C4;           // 16-byte row groups; float4s of the slice's gradient
-  const int Br = round_up(B, 4);
+  const int Br = round_up(B, 4), Rr = round_up(RQ, 4);
   T* xs = reinterpret_cast<T*>(loc_raw);                                     // [nbuf][B][pitch]
   float* wl = reinterpret_cast<float*>(xs + (size_t)geo.nbuf * B * pitch);   // [F][CP] local model
   float* wq = sizeof(T) == 2 ? wl + (size_t)F * CP : wl;                     // ... as the forward pass reads it (bf16 values)
   float4* gs = reinterpret_cast<float4*>(wq + (size_t)F * CP);               // [GE * C4][groups] sum of the steps' gradient sums
   float* zp = reinterpret_cast<float*>(gs + n_g);                            // partial logits / partial gradients
-  float* za = zp + max((size_t)PZ * B * CP, (size_t)PG * F * CP);            // [2][B][CP] this CTA's partial logits by step parity
-  float* dl = za + (size_t)2 * B * CP;                                       // [B][CP] deltas
-  float* rl = dl + (size_t)B * CP;                                           // [B] sample losses
+  float* zin = zp + max((size_t)PZ * B * CP, (size_t)PG * F * CP);           // [Q][RQ][CP] the CTAs' partial logits of this CTA's rows
+  float* dl = zin + (size_t)Q * RQ * CP;                                     // [B][CP] deltas, from the rows' owners
+  float* rl = dl + (size_t)B * CP;                                           // [B] sample losses (first CTA)
   float* bs = rl + Br;                                                       // [16] bias, [16] its gradient sum
   int* sidx = reinterpret_cast<int*>(bs + 32);                               // [3][B] sample indices by step mod 3
-  uint32_t* ys = reinterpret_cast<uint32_t*>(sidx + 3 * Br);                 // [2][B] targets / labels by step parity
-  __shared__ uint64_t full[2];                       // rows of a buffer have landed
+  uint32_t* ys = reinterpret_cast<uint32_t*>(sidx + 3 * Br);                 // [2][RQ] targets / labels by step parity
+  __shared__ uint64_t bar_z, bar_d;                  // logits / deltas of the step have arrived
   __shared__ int gave_up;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool helper = warp == NT / 32;
+  const bool last_warp = warp == NT / 32 - 1;
   const int wn = a.sel[i], jb = a.job[wn];
+  const int2 shard = a.shard[wn];
   const int slot = (ri->t - a.sel_tau[i]) % (st->S + 1);
   const T* w0 = (const T*)a.ring + (size_t)slot * a.slot_stride;
   const T* X = (const T*)a.X + m0;
   const int nblk = (B + 3) >> 2;
   const float step = __fdiv_rn(a.lr, (float)B);
-  i64 lo = 0;                                        // the worker's shard [lo, lo + len) (helper warp)
-  u64 len = 0;
-  uint32_t key0 = 0, key1 = 0;
+  const uint32_t key0 = st->key0, key1 = st->key1;
 
-  // ---- what the helper warp does for the others
-  auto draw = [&](int u) {                           // sample indices of step u
+  auto draw = [&](int u) {                           // sample indices of step u (last warp)
     int* dst = sidx + (u % 3) * Br;
     for (int blk = lane; blk < nblk; blk += 32) {
       uint32_t w4[4];
       philox4x32_10((uint32_t)wn, (uint32_t)jb, 1u, (uint32_t)(u * nblk + blk), key0, key1, w4);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (blk * 4 + q < B) dst[blk * 4 + q] = (int)lo + (int)(((u64)w4[q] * len) >> 32);
+        if (blk * 4 + q < B) dst[blk * 4 + q] = shard.x + (int)__umulhi(w4[q], (uint32_t)shard.y);
     }
-    __syncwarp();
   };
-  // rows that start on 16-byte boundaries: the slice of a row is one bulk copy (F is a multiple of 8)
-  const bool bulk = ((size_t)in * sizeof(T)) % 16 == 0;
-  const bool vec4 = ((size_t)in * sizeof(T)) % 4 == 0;
-  auto fetch_rows = [&](int u) {                     // this CTA's slice of step u's rows
-    const int* idx = sidx + (u % 3) * Br;
-    const int buf = u % geo.nbuf;
-    T* dst = xs + (size_t)buf * B * pitch;
-    if (bulk) {
-      if (lane == 0) tc::mbar_expect_tx(&full[buf], (uint32_t)(B * nf * (int)sizeof(T)));
-      __syncwarp();
-      if (nf > 0)
-        for (int b = lane; b < B; b += 32)
-          lsqp::bulk_row(dst + (size_t)b * pitch, X + (size_t)idx[b] * in, (uint32_t)(nf * sizeof(T)), &full[buf]);
-    }
-    for (int b = lane; b < B; b += 32) cp_async4(ys + (u & 1) * Br + b, (const uint32_t*)a.y + idx[b]);
-  };
-  auto fetch_pieces = [&](int u) {                   // the same by every compute thread, for other row lengths
+  // this CTA's slice of step u's rows, in the widest pieces the rows' starts allow (F is a multiple of 8), and the labels of
+  // its own rows
+  const int row_bytes_mod = (int)(((size_t)in * sizeof(T)) % 16);
+  const int per = row_bytes_mod == 0 ? nf / GE : row_bytes_mod % 4 == 0 ? nf * (int)sizeof(T) / 4 : nf;
+  const FastDiv by_per(max(per, 1));
+  auto fetch = [&](int u) {
     const int* idx = sidx + (u % 3) * Br;
     T* dst = xs + (size_t)(u % geo.nbuf) * B * pitch;
-    if (vec4) {
-      constexpr int E4 = 4 / (int)sizeof(T);
-      const int per = nf / E4;                       // F and (here) `in` are even for 2-byte elements
-      for (int b = warp; b < B; b += NT / 32)
-        for (int v = lane; v < per; v += 32) cp_async4(dst + (size_t)b * pitch + v * E4, X + (size_t)idx[b] * in + v * E4);
+    if (row_bytes_mod == 0) {
+#pragma unroll 2
+      for (int e = tid; e < B * per; e += NT) {
+        const int b = by_per.div(e), v = (e - b * per) * GE;
+        cp_async16(dst + b * pitch + v, X + (size_t)idx[b] * in + v);
+      }
+    } else if (row_bytes_mod % 4 == 0) {
+      constexpr int E4 = 4 / (int)sizeof(T);         // (F and here `in` are even for 2-byte elements)
+#pragma unroll 2
+      for (int e = tid; e < B * per; e += NT) {
+        const int b = by_per.div(e), v = (e - b * per) * E4;
+        cp_async4(dst + b * pitch + v, X + (size_t)idx[b] * in + v);
+      }
     } else {
-      for (int b = warp; b < B; b += NT / 32)
-        for (int v = lane; v < nf; v += 32) dst[(size_t)b * pitch + v] = X[(size_t)idx[b] * in + v];
+      for (int e = tid; e < B * per; e += NT) {
+        const int b = by_per.div(e), v = e - b * per;
+        dst[b * pitch + v] = X[(size_t)idx[b] * in + v];
+      }
     }
-  };
-  auto fetch = [&](int u) {
-    if (helper) fetch_rows(u);
-    else if (!bulk) fetch_pieces(u);
+    for (int b = tid; b < n_own; b += NT) cp_async4(ys + (u & 1) * Rr + b, (const uint32_t*)a.y + idx[b_own + b]);
   };
 
   if (tid == 0) {
-    tc::mbar_init(&full[0], 1);
-    tc::mbar_init(&full[1], 1);
+    tc::mbar_init(&bar_z, 1);
+    tc::mbar_init(&bar_d, 1);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (helper) {
-    const i64 M = st->n_samples;
-    lo = ((i64)wn * M) / W;
-    len = (u64)(((i64)(wn + 1) * M) / W - lo);
-    key0 = st->key0; key1 = st->key1;
+  if (last_warp) {
     draw(0);
     if (U > 1) draw(1);
-  } else {
-    // columns behind the slice's features are read by the 16-byte groups but never copied: zero in every buffer
-    for (int r = warp; r < geo.nbuf * B; r += NT / 32)
-      for (int v = nf + lane; v < pitch; v += 32) stf(xs, (size_t)r * pitch + v, 0.f);
   }
-  if (!helper) {
-#pragma unroll 8
-    for (int e = tid; e < F * CP; e += NT) {
-      const int m = e / CP, c = e - m * CP;
-      const float w = (m < nf && c < C) ? ldf(w0, (size_t)(m0 + m) * C + c) : 0.f;    // a stored model is already rounded
-      wl[e] = w;
-      wq[e] = w;
-    }
-    for (int e = tid; e < n_g; e += NT) gs[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid < 16) {
-      bs[tid] = (!a.lsq && tid < C) ? ldf(w0, (size_t)n_w + tid) : 0.f;
-      bs[16 + tid] = 0.f;
-    }
+  // columns behind the slice's features are read by the 16-byte groups but never copied: zero in every buffer
+  for (int r = warp; r < geo.nbuf * B; r += NT / 32)
+    for (int v = nf + lane; v < pitch; v += 32) stf(xs, (size_t)r * pitch + v, 0.f);
+#pragma unroll 4
+  for (int e = tid; e < F * CP; e += NT) {
+    const int m = e / CP, c = e - m * CP;
+    const float w = (m < nf && c < C) ? ldf(w0, (size_t)(m0 + m) * C + c) : 0.f;    // a stored model is already rounded
+    wl[e] = w;
+    wq[e] = w;
+  }
+  for (int e = tid; e < n_g; e += NT) gs[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (tid < 16) {
+    bs[tid] = (!a.lsq && tid < C) ? ldf(w0, (size_t)n_w + tid) : 0.f;
+    bs[16 + tid] = 0.f;
   }
   __syncthreads();
   fetch(0);
-  float loss_sum = 0.f;                              // helper warp
-  if (Q > 1) tc::cluster_sync_all();                 // peers have started: their shared memory may be read
+  float loss_sum = 0.f;                              // last warp of the first CTA
+  if (Q > 1) tc::cluster_sync_all();                 // peers have started: their barriers and shared memory exist
 
-  // ---- logits, loss, deltas of a step (every thread): four lanes per row, four classes each
-  auto softmax = [&](int par) {
-    for (int b0 = 0; b0 < B; b0 += CL_THREADS / 4) {
-      const int b = b0 + (tid >> 2), l = tid & 3;
-      const bool have = b < B && l < C4;
+  const uint32_t bar_z_a = tc::smem_u32(&bar_z), bar_d_a = tc::smem_u32(&bar_d);
+  const uint32_t zin_a = tc::smem_u32(zin + (size_t)rank * RQ * CP), dl_a = tc::smem_u32(dl);
+  // ---- logits, loss, deltas of this CTA's rows: four lanes per row, four classes each
+  auto softmax = [&](int par, uint32_t parity) {
+    if (warp * 8 >= n_own) return;
+    if (Q > 1) wait_cluster(&bar_z, parity, &gave_up);
+#pragma unroll 1
+    for (int b0 = 0; b0 + warp * 8 < n_own; b0 += NT / 4) {
+      const int b = b0 + (tid >> 2), l = tid & 3;    // row b_own + b
+      const bool have = b < n_own && l < C4;
       float z[4] = {0.f, 0.f, 0.f, 0.f};
       if (have) {
-        const uint32_t mine = tc::smem_u32(za + (size_t)(par * B + b) * CP + 4 * l);
+        const float* mine = zin + (size_t)b * CP + 4 * l;
         float4 p[8];                                 // the cluster's partial logits of these classes
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          p[q] = q < Q ? ld_cluster4(Q > 1 ? tc::map_to_cta(mine, (uint32_t)q) : mine) : make_float4(0.f, 0.f, 0.f, 0.f);
+          p[q] = q < Q ? *reinterpret_cast<const float4*>(mine + (size_t)q * RQ * CP) : make_float4(0.f, 0.f, 0.f, 0.f);
         float4 s = p[0];
 #pragma unroll
         for (int q = 1; q < 8; ++q) s = add4(s, p[q]);
         z[0] = s.x; z[1] = s.y; z[2] = s.z; z[3] = s.w;
       }
-      float d[4] = {0.f, 0.f, 0.f, 0.f};
-      const uint32_t yb = b < B ? ys[par * Br + b] : 0u;
+      float d[4] = {0.f, 0.f, 0.f, 0.f}, loss;
+      const uint32_t yb = b < n_own ? ys[par * Rr + b] : 0u;
       if (a.lsq) {
         const float r = z[0] - __uint_as_float(yb);
-        if (have && l == 0) { d[0] = r; rl[b] = 0.5f * r * r; }
+        loss = 0.5f * r * r;
+        if (l == 0) d[0] = r;
       } else {
         const int y = (int)yb;
         float zy = 0.f, se = 0.f;
@@ -468,54 +494,34 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
         // a delta is a stored quantity of the bf16 configurations: rounded like every other delta
 #pragma unroll
         for (int k = 0; k < 4; ++k) d[k] = round_store(z[k] * inv - (4 * l + k == y ? 1.f : 0.f), (const T*)nullptr);
-        if (b < B && l == 0) rl[b] = logf(se) - (zy - zmax);
+        loss = logf(se) - (zy - zmax);
       }
-      if (have) *reinterpret_cast<float4*>(dl + (size_t)b * CP + 4 * l) = make_float4(d[0], d[1], d[2], d[3]);
+      if (have) {
+        const uint32_t off = (uint32_t)(((b_own + b) * CP + 4 * l) * 4);
+        const float4 dv = make_float4(d[0], d[1], d[2], d[3]);
+        if (Q > 1) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (q < Q) st_async4(tc::map_to_cta(dl_a + off, (uint32_t)q), dv, tc::map_to_cta(bar_d_a, (uint32_t)q));
+          if (l == 0) st_async1(tc::map_to_cta(tc::smem_u32(rl + b_own + b), 0u), loss, tc::map_to_cta(bar_d_a, 0u));
+        } else {
+          *reinterpret_cast<float4*>(dl + (size_t)b * CP + 4 * l) = dv;
+          if (l == 0) rl[b] = loss;
+        }
+      }
     }
   };
 
   const int n_pairs = (B + 1) / 2;
-  const FastDiv by_pairs(n_pairs), by_groups(groups);
+  const FastDiv by_pairs(n_pairs), by_groups(groups), by_rq(RQ);
   for (int u = 0; u < U; ++u) {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    // a wait that runs out ends the run (status below); the steps are finished on whatever is there, so that the
-    // cluster's barriers stay matched
-    if (bulk) tc::mbar_wait(&full[u % geo.nbuf], (uint32_t)(u / geo.nbuf) & 1u, &gave_up);
-    __syncthreads();                                 // rows of step u are here; the previous step is done with everything
-    // the helper warp adds nothing to the exchange: it arrives at once, so that nobody waits for its copies
-    if (helper && Q > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    if (geo.nbuf == 2 && u + 1 < U) fetch(u + 1);
-    const int par = u & 1;
-    if (helper) {
-      if (u + 2 < U) draw(u + 2);
-      if (Q > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-      else asm volatile("bar.sync 2, %0;" ::"n"(CL_THREADS) : "memory");
-      softmax(par);
-      __syncthreads();                               // deltas are there
-      if (rank == 0) {                               // mean loss and bias step (fixed orders)
-        float part = 0.f;
-        for (int b = lane; b < B; b += 32) part += rl[b];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        loss_sum += __fdiv_rn(part, (float)B);
-        const int c = lane & 15;                     // two lanes per class, every second row each
-        float s = 0.f;
-        if (c < CP) {
-#pragma unroll 8
-          for (int b = lane >> 4; b < B; b += 2) s += dl[(size_t)b * CP + c];
-        }
-        s += __shfl_xor_sync(0xffffffffu, s, 16);
-        if (!a.lsq && lane < C) {
-          bs[16 + lane] += s;
-          bs[lane] = fmaf(-step, s, bs[lane]);
-        }
-      }
-      if (geo.nbuf == 1) {
-        __syncthreads();                             // the gradient has read the only row buffer
-        if (u + 1 < U) fetch(u + 1);
-      }
-      continue;
+    const uint32_t parity = (uint32_t)u & 1u;
+    if (Q > 1 && tid == 0) {                         // what this step's exchange brings
+      tc::mbar_expect_tx(&bar_z, (uint32_t)(Q * n_own * CP * 4));
+      tc::mbar_expect_tx(&bar_d, (uint32_t)(B * CP * 4 + (rank == 0 ? B * 4 : 0)));
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();                                 // rows of step u are here; the previous step is done with everything
     const T* xb = xs + (size_t)(u % geo.nbuf) * B * pitch;
     // ---- partial logits of this slice: item = (row pair, every PZ-th column group)
     for (int it = tid; it < n_pairs * PZ; it += NT) {
@@ -550,22 +556,33 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
         if (r1 < B) *reinterpret_cast<ulonglong2*>(o + (size_t)n_pairs * CP + 4 * c) = make_ulonglong2(z1[2 * c], z1[2 * c + 1]);
       }
     }
-    compute_sync();
+    __syncthreads();
     for (int e = tid; e < B * C4; e += NT) {         // partial sums in order; the first CTA adds the bias
       float4 z = reinterpret_cast<const float4*>(zp)[e];
 #pragma unroll 8
       for (int p = 1; p < PZ; ++p) z = add4(z, reinterpret_cast<const float4*>(zp + (size_t)p * B * CP)[e]);
+      const int b = e / C4;
       if (rank == 0) {
-        const float4 bq = reinterpret_cast<const float4*>(bs)[e % C4];
+        const float4 bq = reinterpret_cast<const float4*>(bs)[e - b * C4];
         z = add4(z, make_float4(round_store(bq.x, (const T*)nullptr), round_store(bq.y, (const T*)nullptr),
                                 round_store(bq.z, (const T*)nullptr), round_store(bq.w, (const T*)nullptr)));
       }
-      reinterpret_cast<float4*>(za + (size_t)par * B * CP)[e] = z;
+      if (Q == 1) {
+        reinterpret_cast<float4*>(zin)[e] = z;
+        continue;
+      }
+      const int owner = by_rq.div(b);                // element e of the step is element e - owner RQ C4 of its owner's
+      st_async4(tc::map_to_cta(zin_a + (uint32_t)(e - owner * RQ * C4) * 16u, (uint32_t)owner), z, tc::map_to_cta(bar_z_a, (uint32_t)owner));
     }
-    if (Q > 1) tc::cluster_sync_all();
-    else asm volatile("bar.sync 2, %0;" ::"n"(CL_THREADS) : "memory");
-    softmax(par);
-    __syncthreads();
+    // the next rows are fetched while the exchange is on its way (behind the soft-max by the warps that form it)
+    if (Q == 1) __syncthreads();
+    const bool early = warp * 8 < n_own, ahead = geo.nbuf == 2 && u + 1 < U;
+    if (ahead && !early) fetch(u + 1);
+    softmax(u & 1, parity);
+    if (ahead && early) fetch(u + 1);
+    if (last_warp && u + 2 < U) draw(u + 2);
+    if (Q > 1) wait_cluster(&bar_d, parity, &gave_up);
+    else __syncthreads();
     // ---- gradient of this slice: item = (column group, every PG-th row)
     for (int it = tid; it < groups * PG; it += NT) {
       const int part = by_groups.div(it), g = it - part * groups;
@@ -598,12 +615,26 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
 #pragma unroll
         for (int c = 0; c < C4; ++c) o[(size_t)(j * C4 + c) * groups] = make_ulonglong2(acc[j][2 * c], acc[j][2 * c + 1]);
     }
-    if (geo.nbuf == 1) {
-      __syncthreads();                               // the helper refills the only row buffer
-      if (!bulk && u + 1 < U) fetch(u + 1);
-    } else {
-      compute_sync();
+    if (last_warp && rank == 0) {                    // mean loss and bias step (fixed orders)
+      float part = 0.f;
+      for (int b = lane; b < B; b += 32) part += rl[b];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      loss_sum += __fdiv_rn(part, (float)B);
+      const int c = lane & 15;                       // two lanes per class, every second row each
+      float s = 0.f;
+      if (c < CP) {
+#pragma unroll 8
+        for (int b = lane >> 4; b < B; b += 2) s += dl[(size_t)b * CP + c];
+      }
+      s += __shfl_xor_sync(0xffffffffu, s, 16);
+      if (!a.lsq && lane < C) {
+        bs[16 + lane] += s;
+        bs[lane] = fmaf(-step, s, bs[lane]);
+      }
     }
+    __syncthreads();
+    if (geo.nbuf == 1 && u + 1 < U) fetch(u + 1);    // the gradient has read the only row buffer
     // ---- the local step
     for (int e = tid; e < n_g; e += NT) {
       float4 s = reinterpret_cast<const float4*>(zp)[e];
@@ -622,11 +653,11 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
                         round_store(w.z, (const T*)nullptr), round_store(w.w, (const T*)nullptr));
     }
   }
-  if (Q > 1) tc::cluster_sync_all();                 // no peer still reads this CTA's partial logits
+  if (Q > 1) tc::cluster_sync_all();                 // (a wait that ran out: no peer stores to a CTA that has left)
   else __syncthreads();
   float* out = a.G + (size_t)i * a.slot_stride;
   const float sa = st->sa_penalty ? sa_weight(a.sel_tau[i]) : 1.f;   // staleness-aware step size: weight of the upload in Eq. 3
-  for (int e = tid; e < nf * C; e += CL_THREADS) {
+  for (int e = tid; e < nf * C; e += NT) {
     const int m = e / C, c = e - m * C;
     const float4 q = gs[(size_t)((m % GE) * C4 + c / 4) * groups + m / GE];
     const int k = c & 3;
@@ -634,16 +665,13 @@ __global__ void __launch_bounds__(CL_THREADS, cluster_ctas_per_sm(group_elems<T>
   }
   if (rank == 0) {
     if (!a.lsq && tid < C) out[(size_t)n_w + tid] = bs[16 + tid] * sa;
-    if (helper && lane == 0) {
+    if (last_warp && lane == 0) {
       const float loss = __fdiv_rn(loss_sum, (float)U);
       a.loss[i] = loss;
       if (!isfinite(loss)) report(ri, RI_DIVERGED);
     }
   }
   if (tid == 0 && gave_up) {
-    // let copies in flight land before the shared memory goes away
-    const unsigned long long t0 = tc::global_ns();
-    while (tc::global_ns() - t0 < 200000ull) {}
     // not st->status: a cluster that starts later must find the same status in all of its CTAs
     st->timeout_where = 300;
     report(ri, RI_TIMEOUT);
