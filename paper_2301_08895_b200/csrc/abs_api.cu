@@ -1287,6 +1287,11 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
   if (e != cudaSuccess) return bail(cuda_fail(nullptr, e, "state copy"));
 
   CtlArgs& c = ctx->ctl;
+  c.k.W = W; c.k.K0 = K0; c.k.S = S_ring; c.k.B = model->batch;
+  for (c.k.rb_shift = 0; (1 << c.k.rb_shift) < L.RB; ++c.k.rb_shift) {}      // (networks: a power of two)
+  c.k.k_mode = h.k_mode; c.k.bound_mode = h.bound_mode; c.k.max_rounds = h.max_rounds; c.k.bound_offset = h.bound_offset;
+  c.k.theta_cap = h.theta_cap; c.k.literal_eq6 = h.literal_eq6; c.k.no_restart = h.no_restart; c.k.key0 = h.key0; c.k.key1 = h.key1;
+  c.rows_cap = L.rows_cap;
   c.st = ctx->at<DevState>(L.st);
   c.c = ctx->at<u64>(L.c); c.version = ctx->at<int>(L.version); c.job = ctx->at<int>(L.job);
   c.next_dur = ctx->at<u64>(L.next_dur); c.dur_job = ctx->at<int>(L.dur_job);

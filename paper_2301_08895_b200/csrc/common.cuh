@@ -65,7 +65,7 @@ struct DevState {
   u64 T_end;                      // end tick of the open round
   int n_rows;                     // padded gradient rows of the open round
   int n_row_tiles;                // n_rows / RB
-  int n_groups;
+  int last_id;                    // worker of the open round's last arrival
   i64 sel_total, rst_total;       // flat trace fill
   u64 comm;                       // communication-round counter (Sec. V-B)
   int timeout_where;
@@ -94,8 +94,16 @@ struct FastDiv {
   __device__ __forceinline__ int div(int x) const { return m ? (int)__umulhi((uint32_t)x, m) : x; }
 };
 
-// Pointers the control kernel works on (all device memory inside the workspace).
+// Constants of the run as the control step takes them (DevState's, which other kernels read).
+struct CtlConst {
+  int W, K0, S, B, rb_shift;      // RB = 1 << rb_shift (networks)
+  int k_mode, bound_mode, max_rounds, bound_offset, theta_cap, literal_eq6, no_restart;
+  uint32_t key0, key1;
+};
+
+// What the control kernel works on (pointers: all device memory inside the workspace).
 struct CtlArgs {
+  CtlConst k;
   DevState* st;
   RoundInfo* ri;       // [2] by round parity
   u64* c;              // [W] completion tick of each worker's job in flight
@@ -107,6 +115,7 @@ struct CtlArgs {
   int* sel_row0[2];    // [W] first gradient row of each selected worker
   float* loss;         // [W] mean minibatch loss of each selected worker
   float* row_loss;     // [rows_cap] per-sample losses (network models), else null
+  int rows_cap;
   int* row_idx[2];     // [rows_cap] sample index of each gradient row, -1 for padding
   int* tile_slot[2];   // [rows_cap / RB] ring slot of each row tile
   int* tile_real[2];   // [rows_cap / RB] rows of the tile that are not padding (they come first)

@@ -154,27 +154,36 @@ __device__ __forceinline__ int floor_div(int a, int b) {  // b > 0
 }
 
 struct CtlShared {
-  u64 keysA[1024], keysB[1024];
+  u64 keysA[1024], keysB[1024];        // (row losses of the open round before the sort)
   unsigned short wcnt[32][MAX_TAU];   // per-warp count of selected workers per staleness
   int cnt[MAX_TAU];                    // selected workers per staleness
   int grow0[MAX_TAU];                  // first row of each staleness group
-  unsigned char flag[1024];            // selected marker per worker id
   int row0[1024];                      // first gradient row of each selected worker
   float lossv[1024];                   // mean minibatch loss of each selected worker
   int version[1024], job[1024];        // per-worker state after the round's bookkeeping
   int sel_n[1024];                     // worker id of each arrival, in arrival order
   int2 shard[1024];                    // per worker: first sample and length of its shard
   float redf[32];
+  int bad[32];
   int warp_tot[32];
   int scalar[8];
 };
+
+// A duration that was not prepared ahead of time (rare: kept out of the step's straight-line code)
+static __device__ __noinline__ u64 job_ticks_call(const DevState* st, uint32_t key0, uint32_t key1, int n, int j) {
+  return job_ticks(st->dist, key0, key1, n, j);
+}
 
 // Completes the open round (Eq. 5, Eq. 4, Eq. 6, trace row), then selects the arrivals of the
 // next round and lays out its gradient rows.
 //   do_finish: complete the open round if there is one
 //   do_select: open the next round
-// A dependent global-memory access costs this lone CTA close to a microsecond, so everything it
-// needs is loaded up front in one wave and later phases work from registers and shared memory.
+// A lone CTA is bound by its chain of dependent phases: a global-memory access costs close to a microsecond, a block-wide
+// barrier with what leads to it a few hundred cycles, and straight-line code that runs once a launch about ten cycles an
+// instruction.  So everything a later phase needs is loaded up front in one wave (the run's constants come with the
+// launch), sums over the arrivals and the rules that follow from them are formed by every warp itself instead of by one for
+// all, rules that rarely change anything (Eq. 5 raising K, Eq. 4 after it) have a short test in front, and a worker's rank
+// is counted.  OLDNEW
 //   t_sel:     index of the round that follows the open one (the host counts rounds; parity of
 //              t_sel - 1 / t_sel picks the layout copy of the open / the new round)
 //   look_here: the workers that were renewed also get the duration of the job AFTER the one they
@@ -186,74 +195,80 @@ struct CtlShared {
 template <int NT>
 __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do_finish, int do_select, int t_sel,
                                          int look_here = 0, int* late_status = nullptr) {
+  constexpr int NWP = NT / 32;
+  constexpr int ROWS = NT >= 1024 ? 4 : 8;            // row losses a thread fetches ahead of time
   DevState* st = a.st;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   auto raise = [&](int code) {
     if (late_status != nullptr) *late_status = code;
     else st->status = code;
   };
-  // ---- one wave of loads
-  const int W = st->W, S = st->S, B = st->B, RB = st->RB, K0 = st->K0;
+  // ---- one wave of loads (everything a later phase may need: all addresses exist whether or not a round is open)
+  const CtlConst& k = a.k;
+  const int W = k.W, S = k.S, B = k.B;
   const int po = (t_sel - 1) & 1, pn = t_sel & 1;     // layout copy of the open / of the new round
-  // (everything a later phase may need: all addresses exist whether or not a round is open)
-  int my_sel = 0, my_tau = 0, my_row0 = 0;
+  const bool net = a.row_loss != nullptr;
+  const bool ahead = net && do_finish && a.rows_cap <= ROWS * NT;      // all row losses fit
+  int my_sel = 0, my_tau = 0, my_row0 = 0, my_version = 0, my_job = 0, my_dur_job = -1;
   float my_loss = 0.f;
   int2 my_shard = make_int2(0, 0);
+  u64 my_c = 0, my_next_dur = 0;
+  float rl[ROWS];
+  if (ahead) {
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) rl[u] = tid + u * NT < a.rows_cap ? a.row_loss[tid + u * NT] : 0.f;
+  }
   if (tid < W) {
+    my_c = a.c[tid]; my_version = a.version[tid]; my_job = a.job[tid];
+    my_dur_job = a.dur_job[tid]; my_next_dur = a.next_dur[tid];
     my_sel = a.sel[po][tid]; my_tau = a.sel_tau[po][tid]; my_row0 = a.sel_row0[po][tid];
-    my_shard = a.shard[tid];
+    if (a.draw) my_shard = a.shard[tid];
+    if (do_finish && !net && a.loss_part == nullptr) my_loss = a.loss[tid];
   }
   const int status0 = st->status, open0 = st->open, diverged0 = a.ri[po].diverged;
-  const int k_mode = st->k_mode, bound_mode = st->bound_mode, max_rounds = st->max_rounds;
-  const int bound_offset = st->bound_offset, Scap = st->theta_cap, literal = st->literal_eq6;
-  const int no_restart = st->no_restart;
-  const uint32_t key0 = st->key0, key1 = st->key1;
   const u64 T_end0 = st->T_end;
   const float L0_prev = st->L0;
   const i64 sel_off = st->sel_total, rst_off = st->rst_total;
   const u64 comm0 = st->comm;
+  const int last_id = st->last_id, theta0 = st->theta;
   int t = st->t, K = st->K;
-  const bool net = a.row_loss != nullptr;
-  const bool fin = do_finish && open0;
-  u64 my_c = 0;
-  int my_version = 0, my_job = 0, my_dur_job = -1;
-  u64 my_next_dur = 0;
-  if (tid < W) {
-    my_c = a.c[tid]; my_version = a.version[tid]; my_job = a.job[tid];
-    my_dur_job = a.dur_job[tid]; my_next_dur = a.next_dur[tid];
-  }
-  if (fin && tid < K) {
-    if (!net && a.loss_part == nullptr) my_loss = a.loss[tid];
-    if (!net && a.loss_part != nullptr) {
-      // the least-squares pipeline leaves per-group sums; same order and rounding as its Eq. 3 kernel
-      float s = 0.f;
-      for (int g = 0; g < a.loss_groups; ++g) s += a.loss_part[(size_t)tid * a.loss_groups + g];
-      my_loss = __fdiv_rn(s, (float)B);
-    }
+  if (do_finish && !net && a.loss_part != nullptr && tid < W) {
+    // the least-squares pipeline leaves per-group sums; same order and rounding as its Eq. 3 kernel
+    const float* p = a.loss_part + (size_t)tid * a.loss_groups;
+    float s = 0.f;
+#pragma unroll 4
+    for (int g = 0; g < a.loss_groups; ++g) s += p[g];
+    my_loss = __fdiv_rn(s, (float)B);
   }
   if (status0 != ST_OK) return 1;
+  const bool fin = do_finish && open0;
 
-  int renewed = 0;          // this thread's worker started a new job in the finish step
+  int restart = 0, renewed = 0;                       // this thread's worker started a new job in the finish step
+  int K_next = K, theta = theta0;
+  float Lt = 0.f, L0 = 0.f;
   // ------------------------------------------------------------------ finish round t
   if (fin) {
-    const u64 T_end = T_end0;
     if (net) {
       // per-worker mean of the per-sample losses: TPW neighbouring threads share a worker, each
-      // adds every TPW-th row (eight loads at a time: with a runtime division and sixteen unrolled loads whose remainder ran
-      // this was 3800 cycles of 12000 for 16 workers x 64 rows, now 1700), then the TPW partial sums are added by a
+      // adds every TPW-th row (eight at a time), then the TPW partial sums are added by a
       // fixed shuffle tree
+      float* rls = reinterpret_cast<float*>(sh.keysA);
       sh.row0[tid] = my_row0;
+      if (ahead) {
+#pragma unroll
+        for (int u = 0; u < ROWS; ++u) rls[tid + u * NT] = rl[u];
+      }
       __syncthreads();
       const int lg_k = max(5, 32 - __clz(K - 1)), lg_tpw = min(5, 31 - __clz(NT) - lg_k);      // (K >= 1; K = 1: clz(0) = 32)
       const int tpw = 1 << lg_tpw, i = tid >> lg_tpw, sub = tid & (tpw - 1);
       float acc = 0.f;
       if (i < K) {
-        const float* rl = a.row_loss + sh.row0[i];
+        const float* src = (ahead ? rls : a.row_loss) + sh.row0[i];
 #pragma unroll 1
         for (int b = sub; b < B; b += 8 * tpw) {
           float x[8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) x[u] = b + u * tpw < B ? rl[b + u * tpw] : 0.f;
+          for (int u = 0; u < 8; ++u) x[u] = b + u * tpw < B ? src[b + u * tpw] : 0.f;
 #pragma unroll
           for (int u = 0; u < 8; ++u) acc += x[u];
         }
@@ -261,101 +276,114 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
 #pragma unroll 1
       for (int o = tpw >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       if (i < K && sub == 0) sh.lossv[i] = __fdiv_rn(acc, (float)B);
-      __syncthreads();
-      if (tid < K) my_loss = sh.lossv[tid];
+    } else if (tid < K) {
+      sh.lossv[tid] = my_loss;
     }
-    const int bad = __syncthreads_or((tid < K) && !isfinite(my_loss)) || diverged0;
-    if (bad) {
+    __syncthreads();
+    // loss estimate: adjacent-pair tree sum in binary32 over 1024 leaves (missing ones are zero), /K in binary32
+    auto tree = [&](float v) {
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) v = __fadd_rn(v, __shfl_down_sync(0xffffffffu, v, o));
+      return v;
+    };
+    float v = 0.f;
+    int bad = 0;
+    if (tid < K) my_loss = sh.lossv[tid];
+    if (K <= 32) {
+      if (lane < K) v = sh.lossv[lane];
+      bad = __any_sync(0xffffffffu, !isfinite(v));
+      v = tree(v);
+    } else {
+      if (tid < K) v = my_loss;
+      bad = __any_sync(0xffffffffu, !isfinite(v));
+      v = tree(v);
+      if (lane == 0) { sh.redf[warp] = v; sh.bad[warp] = bad; }
+      __syncthreads();
+      v = lane < NWP ? sh.redf[lane] : 0.f;
+      bad = __any_sync(0xffffffffu, lane < NWP && sh.bad[lane]);
+      v = tree(v);
+    }
+    v = __shfl_sync(0xffffffffu, v, 0);
+    if (bad || diverged0) {
       if (tid == 0) { raise(diverged0 & RI_TIMEOUT ? ST_TIMEOUT : ST_DIVERGED); st->open = 0; }
       return 1;
     }
-    // loss estimate: adjacent-pair tree sum in binary32 over 1024 leaves, /K in binary32
-    float v = (tid < K) ? my_loss : 0.f;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) v = __fadd_rn(v, __shfl_down_sync(0xffffffffu, v, o));
-    if (lane == 0) sh.redf[warp] = v;
-    sh.flag[tid] = 0;
-    __syncthreads();
-    if (warp == 0) {
-      float x = (lane < NT / 32) ? sh.redf[lane] : 0.f;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) x = __fadd_rn(x, __shfl_down_sync(0xffffffffu, x, o));
-      if (lane == 0) {
-        const float Lt0 = __fdiv_rn(x, (float)K);
-        const float L00 = (t == 0) ? Lt0 : L0_prev;
-        // Eq. 5 as an exact integer rule: largest k with k^2 Lt <= K0^2 L0 (binary64 products of a
-        // 20-bit integer and a binary32 value are exact).  A binary32 estimate of K0 sqrt(L0/Lt)
-        // is corrected with the exact test, so only a handful of double operations are issued.
-        int kr = 0;
-        if (k_mode == ABS_K_ADAPTIVE) {
-          if (Lt0 <= 0.f) {
-            kr = W;
-          } else {
-            const double rhs = __dmul_rn((double)(K0 * K0), (double)L00);
-            const double lt = (double)Lt0;
-            const float est = (float)K0 * sqrtf(L00 / Lt0);
-            int k = (est >= (float)W) ? W : ((est >= 1.f) ? (int)est : 1);
-            while (k < W && __dmul_rn((double)((k + 1) * (k + 1)), lt) <= rhs) ++k;
-            while (k >= 1 && !(__dmul_rn((double)(k * k), lt) <= rhs)) --k;
-            kr = k;
-          }
-        }
-        sh.redf[0] = Lt0;
-        sh.redf[1] = L00;
-        sh.scalar[2] = kr;
+    Lt = __fdiv_rn(v, (float)K);
+    L0 = (t == 0) ? Lt : L0_prev;
+    // Eq. 5 as an exact integer rule: the largest k with k^2 Lt <= K0^2 L0, if above K (binary64 products of a 20-bit
+    // integer and a binary32 value are exact).  K + 1 is tested first; only when it passes, a binary32 estimate of
+    // K0 sqrt(L0/Lt) is corrected with the exact test.
+    if (k.k_mode == ABS_K_ADAPTIVE && K < W) {
+      const double rhs = __dmul_rn((double)(k.K0 * k.K0), (double)L0), lt = (double)Lt;
+      auto holds = [&](int n) { return __dmul_rn((double)(n * n), lt) <= rhs; };
+      if (Lt <= 0.f) {
+        K_next = W;
+      } else if (holds(K + 1)) {
+        const float est = (float)k.K0 * sqrtf(L0 / Lt);
+        int n = (est >= (float)W) ? W : max(K + 1, (est >= 1.f) ? (int)est : 1);
+        while (n < W && holds(n + 1)) ++n;
+        while (!holds(n)) --n;                        // (ends at K + 1 at the latest)
+        K_next = n;
       }
     }
-    if (tid < K) sh.flag[my_sel] = 1;
-    __syncthreads();
-    const float Lt = sh.redf[0];
-    const float L0 = sh.redf[1];
-    int K_next = K;
-    if (k_mode == ABS_K_ADAPTIVE) K_next = min(W, max(K, sh.scalar[2]));
-    // Eq. 4 with a = S - N/K0, in integers
-    int theta = Scap;
-    if (bound_mode == ABS_BOUND_ADAPTIVE) {
-      // (32-bit: at most 1024 workers)
-      theta = min(Scap, max(1, Scap + floor_div(W * (K0 - K_next), K_next * K0)));
-    } else if (bound_mode == ABS_BOUND_OFFSET) {     // Eq. 4 with a given: floor(N/K + a) = floor(N/K) + a
-      int th = W / K_next + bound_offset;
-      if (th < 1) th = 1;
-      if (th > Scap) th = Scap;
-      theta = th;
+    // Eq. 4 with a = S - N/K0, in integers: a function of K, so the last round's threshold stands while K does
+    if (K_next != K || t == 0) {
+      theta = k.theta_cap;
+      if (k.bound_mode == ABS_BOUND_ADAPTIVE) {
+        // (32-bit: at most 1024 workers)
+        theta = min(theta, max(1, theta + floor_div(W * (k.K0 - K_next), K_next * k.K0)));
+      } else if (k.bound_mode == ABS_BOUND_OFFSET) {     // Eq. 4 with a given: floor(N/K + a) = floor(N/K) + a
+        theta = min(theta, max(1, W / K_next + k.bound_offset));
+      }
     }
-    // Eq. 6 in Algorithm 1's order: arrivals and over-stale workers get w^{t+1}
-    int restart = 0, renew = 0;
-    if (tid < W) {
-      const int sel_me = sh.flag[tid];
-      restart = (!sel_me) && !no_restart && ((t + 1 - literal - my_version) > theta);
-      renew = sel_me || restart;
-    }
+    // Eq. 6 in Algorithm 1's order: arrivals and over-stale workers get w^{t+1}.  The arrivals are the workers up to the last
+    // one's (completion tick, id).
     int range_err = 0;
-    if (renew) {
-      const int j = my_job + 1;
-      const u64 dt = (my_dur_job == j) ? my_next_dur : job_ticks(st->dist, key0, key1, tid, j);
-      const u64 cn = T_end + dt;
-      if (dt == 0ull || cn >= (1ull << 53)) range_err = 1;
-      my_job = j; my_version = t + 1; my_c = cn;
-      renewed = 1;
-      a.job[tid] = j;
-      a.version[tid] = t + 1;
-      a.c[tid] = cn;
+    if (tid < W) {
+      const bool sel_me = ((my_c << 10) | (u64)tid) <= ((T_end0 << 10) | (u64)last_id);
+      restart = !sel_me && !k.no_restart && (t + 1 - k.literal_eq6 - my_version) > theta;
+      if (sel_me || restart) {
+        const int j = my_job + 1;
+        const u64 dt = (my_dur_job == j) ? my_next_dur : job_ticks_call(st, k.key0, k.key1, tid, j);
+        const u64 cn = T_end0 + dt;
+        if (dt == 0ull || cn >= (1ull << 53)) range_err = 1;
+        my_job = j; my_version = t + 1; my_c = cn;
+        renewed = 1;
+        a.job[tid] = j;
+        a.version[tid] = t + 1;
+        a.c[tid] = cn;
+      }
     }
-    // ascending list of restarted ids
-    const unsigned rb = __ballot_sync(0xffffffffu, restart);
-    if (lane == 0) sh.warp_tot[warp] = __popc(rb);
-    range_err = __syncthreads_or(range_err);
-    int base = 0, R = 0;
-    for (int w = 0; w < NT / 32; ++w) { const int c = sh.warp_tot[w]; if (w < warp) base += c; R += c; }
-    if (restart) a.tr_rst_id[rst_off + base + __popc(rb & ((1u << lane) - 1u))] = tid;
+    // (for the ascending list of restarted ids)
+    const unsigned rb = __ballot_sync(0xffffffffu, restart), eb = __ballot_sync(0xffffffffu, range_err);
+    if (lane == 0) sh.warp_tot[warp] = __popc(rb) | (eb != 0u ? 1 << 16 : 0);
+  }
+  if (do_select) {
+    // unused slots get distinct keys above every real one
+    sh.keysA[tid] = (tid < W) ? ((my_c << 10) | (u64)tid) : (0xFFFFFFFFFFFFFC00ull | (u64)tid);
+    sh.version[tid] = my_version;
+    sh.job[tid] = my_job;
+    sh.shard[tid] = my_shard;
+    if (net) for (int u = lane; u <= S; u += 32) sh.wcnt[warp][u] = 0;
+  }
+  __syncthreads();
+  if (fin) {
+    const int x = lane < NWP ? sh.warp_tot[lane] : 0;
+    const int R = __reduce_add_sync(0xffffffffu, x & 0xffff);
+    const bool range_err = __any_sync(0xffffffffu, x >> 16);
+    if (R > 0) {                                      // ascending list of restarted ids
+      const unsigned rb = __ballot_sync(0xffffffffu, restart);
+      const int base = __reduce_add_sync(0xffffffffu, lane < warp ? x & 0xffff : 0);
+      if (restart) a.tr_rst_id[rst_off + base + __popc(rb & ((1u << lane) - 1u))] = tid;
+    }
     if (tid < K) {
       a.tr_sel_id[sel_off + tid] = my_sel;
       a.tr_sel_tau[sel_off + tid] = my_tau;
       a.tr_sel_loss[sel_off + tid] = my_loss;
     }
-    const u64 comm = comm0 + (u64)(K + R);
     if (tid == 0) {
-      a.tr_K[t] = K; a.tr_R[t] = R; a.tr_theta[t] = theta; a.tr_T[t] = T_end;
+      const u64 comm = comm0 + (u64)(K + R);
+      a.tr_K[t] = K; a.tr_R[t] = R; a.tr_theta[t] = theta; a.tr_T[t] = T_end0;
       a.tr_loss[t] = Lt; a.tr_comm[t] = comm;
       a.tr_sel_off[t] = sel_off; a.tr_rst_off[t] = rst_off;
       a.tr_sel_off[t + 1] = sel_off + K; a.tr_rst_off[t + 1] = rst_off + R;
@@ -366,12 +394,11 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     if (range_err) return 1;
     t = t + 1;
     K = K_next;
-    __syncthreads();
   }
 
   // duration of the job after the one just started, for the next control step to look up
   if (look_here && renewed) {
-    a.next_dur[tid] = job_ticks(st->dist, key0, key1, tid, my_job + 1);
+    a.next_dur[tid] = job_ticks_call(st, k.key0, k.key1, tid, my_job + 1);
     a.dur_job[tid] = my_job + 1;
   }
   // ------------------------------------------------------------------ select round t
@@ -380,122 +407,139 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     if (tid == 0) raise(ST_INTERNAL);
     return 1;
   }
-  if (t >= max_rounds) {
+  if (t >= k.max_rounds) {
     if (tid == 0) raise(ST_NOSPACE);
     return 1;
   }
-  {
-    sh.version[tid] = my_version;
-    sh.job[tid] = my_job;
-    sh.shard[tid] = my_shard;
-    if (net) for (int u = lane; u <= S; u += 32) sh.wcnt[warp][u] = 0;
-    // arrivals: the K smallest (completion tick, worker id) keys; unused slots get distinct
-    // keys above every real one
+  // arrivals: the K smallest (completion tick, worker id) keys
+  const u64* sorted = sh.keysA;
+  const bool count = NT < 1024 && W <= 128;
+  if (count) {
+    // the rank of a key is the number of smaller ones: 8, 4 or 2 lanes share a key and take every 8th, 4th, 2nd other (64
+    // keys: RANK64)
+    const int lg_p = W <= 32 ? 3 : W <= 64 ? 2 : 1, per = 256 >> (2 * lg_p);
+    const int n = tid >> lg_p, part = tid & ((1 << lg_p) - 1);
+    if (tid < 256) {
+      const u64 mine = sh.keysA[n];
+      int rank = 0;
+      const u64* p = sh.keysA + part;
+#pragma unroll 4
+      for (int q = 0; q < per; ++q) rank += p[q << lg_p] < mine ? 1 : 0;
+#pragma unroll 1
+      for (int o = (1 << lg_p) >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+      if (part == 0 && rank < K) sh.sel_n[rank] = n;     // (n < W: the keys of unused slots rank behind)
+    }
+    __syncthreads();
+  } else {
     int n_pow2 = 32;
     while (n_pow2 < W) n_pow2 <<= 1;
-    const u64 key_in = (tid < W) ? ((my_c << 10) | (u64)tid) : (0xFFFFFFFFFFFFFC00ull | (u64)tid);
-    const u64* sorted = rank_merge_sort<NT>(key_in, sh.keysA, sh.keysB, n_pow2);
-    const u64 T_end = sorted[K - 1] >> 10;
-    int n = -1, tau = -1;
-    if (tid < K) {
-      n = (int)(sorted[tid] & 1023ull);
-      tau = t - sh.version[n];
-    }
-    const int tau_bad = __syncthreads_or(tid < K && (tau < 0 || tau > S));
-    if (tau_bad) {
-      // with forced restarts this cannot happen (consumed staleness <= threshold <= S); without
-      // them the arrival's model version may have left the ring: the run ends here, before any
-      // kernel reads the slot that was overwritten
-      if (tid == 0) raise(no_restart ? ST_STALE : ST_INTERNAL);
-      return 1;
-    }
+    sorted = rank_merge_sort<NT>(sh.keysA[tid], sh.keysA, sh.keysB, n_pow2);
+  }
+  int n = -1, tau = -1;
+  u64 T_end = 0ull;
+  if (tid < K) {
+    n = count ? sh.sel_n[tid] : (int)(sorted[tid] & 1023ull);
+    tau = t - sh.version[n];
+  }
+  int last = 0;
+  if (tid == 0) {
+    last = count ? sh.sel_n[K - 1] : (int)(sorted[K - 1] & 1023ull);
+    T_end = sorted[count ? last : K - 1] >> 10;
+  }
+  int rank_in_warp = 0;
+  if (net) {
     // network models: group the arrivals by staleness (all members of a group read the same
     // ring slot); inside a group keep arrival order.  Least squares needs no row layout.
-    int row0_me = tid * B;
-    if (net) {
-      const unsigned peers = __match_any_sync(0xffffffffu, tau);
-      const int rank_in_warp = __popc(peers & ((1u << lane) - 1u));
-      if (tau >= 0 && rank_in_warp == 0) sh.wcnt[warp][tau] = (unsigned short)__popc(peers);
-      __syncthreads();
-      if (warp == 0) {
-        // per staleness u: exclusive sums over the warps, then first rows by a scan over u (RB is a power of two)
-        int carry = 0, groups = 0;
-        for (int u0 = 0; u0 <= S; u0 += 32) {
-          const int u = u0 + lane;
-          int c = 0;
-          if (u <= S) {
-#pragma unroll
-            for (int w = 0; w < NT / 32; ++w) { const int x = sh.wcnt[w][u]; sh.wcnt[w][u] = (unsigned short)c; c += x; }
-          }
-          const int rows = (c * B + RB - 1) & ~(RB - 1);
-          int sum = rows;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, sum, o); if (lane >= o) sum += v; }
-          if (u <= S) { sh.cnt[u] = c; sh.grow0[u] = carry + sum - rows; }
-          carry += __shfl_sync(0xffffffffu, sum, 31);
-          groups += __popc(__ballot_sync(0xffffffffu, c > 0));
-        }
-        if (lane == 0) { sh.scalar[0] = carry; sh.scalar[1] = groups; }
+    const unsigned peers = __match_any_sync(0xffffffffu, tau);
+    rank_in_warp = __popc(peers & ((1u << lane) - 1u));
+    if (tau >= 0 && rank_in_warp == 0) sh.wcnt[warp][min(tau, S)] = (unsigned short)__popc(peers);
+  }
+  if (__syncthreads_or(tid < K && (tau < 0 || tau > S))) {
+    // with forced restarts this cannot happen (consumed staleness <= threshold <= S); without
+    // them the arrival's model version may have left the ring: the run ends here, before any
+    // kernel reads the slot that was overwritten
+    if (tid == 0) raise(k.no_restart ? ST_STALE : ST_INTERNAL);
+    return 1;
+  }
+  int row0_me = tid * B, n_rows = K * B;
+  if (net) {
+    // every warp for itself: per staleness u its count in all warps and in the ones before this one, then first rows by a
+    // scan over u (RB is a power of two)
+    const int rb1 = (1 << k.rb_shift) - 1, nw = (K + 31) >> 5;
+    int carry = 0;
+    for (int u0 = 0; u0 <= S; u0 += 32) {
+      const int u = u0 + lane;
+      int c = 0, before = 0;
+      if (u <= S) {
+#pragma unroll 4
+        for (int w = 0; w < nw; ++w) { const int x = sh.wcnt[w][u]; before += w < warp ? x : 0; c += x; }
       }
-      __syncthreads();
-      if (tid < K) row0_me = sh.grow0[tau] + ((int)sh.wcnt[warp][tau] + rank_in_warp) * B;
-    }
-    const int n_rows = net ? sh.scalar[0] : K * B;
-    const int n_groups = net ? sh.scalar[1] : 0;
-    if (tid < K) {
-      const int row0 = row0_me;
-      a.sel[pn][tid] = n;
-      a.sel_tau[pn][tid] = tau;
-      a.sel_row0[pn][tid] = row0;
-      sh.row0[tid] = row0;
-      sh.sel_n[tid] = n;
-      sh.flag[tid] = 0;
-    }
-    if (tid == 0) {
-      st->T_end = T_end;
-      st->n_rows = n_rows;
-      st->n_row_tiles = net ? n_rows >> (__ffs(RB) - 1) : K;
-      st->n_groups = n_groups;
-      st->open = 1;
-      RoundInfo info;
-      info.n_rows = n_rows; info.K = K; info.t = t; info.diverged = 0;
-      a.ri[pn] = info;
-      sh.scalar[4] = K; sh.scalar[5] = t;
-    }
-    if (!net) return 0;           // least squares: no row tiles, minibatches drawn by its own kernel
-    __syncthreads();
-    // ring slot of every row tile and padding rows, one warp per staleness group
-    {
-      const int sh_rb = __ffs(RB) - 1, tm = t % (S + 1);
-      for (int g = warp; g <= S; g += NT / 32) {
-        const int c = sh.cnt[g];
-        if (c == 0) continue;
-        const int r0 = sh.grow0[g], p0 = r0 + c * B, p1 = r0 + ((c * B + RB - 1) & ~(RB - 1));
-        const int slot = tm - g < 0 ? tm - g + S + 1 : tm - g;      // (t - g) mod (S + 1); g <= S
-        for (int q = (r0 >> sh_rb) + lane; q < (p1 >> sh_rb); q += 32) {
-          a.tile_slot[pn][q] = slot;
-          a.tile_real[pn][q] = min(RB, p0 - (q << sh_rb));
-        }
-        for (int r = p0 + lane; r < p1; r += 32) a.row_idx[pn][r] = -1;
-      }
-    }
-    if (!a.draw) return 0;
-    // minibatch draws: sample b of job (n, j) = word b%4 of Philox block (n, j, 1, b/4),
-    // mapped into the worker's shard [n M / N, (n+1) M / N)
-    const int blocks_per = (B + 3) >> 2;
-#pragma unroll 2
-    for (int item = tid; item < K * blocks_per; item += NT) {
-      const int i = a.by_blk.div(item), blk = item - i * blocks_per;
-      const int wn = (int)(sorted[i] & 1023ull);
-      uint32_t w4[4];
-      philox4x32_10((uint32_t)wn, (uint32_t)sh.job[wn], 1u, (uint32_t)blk, key0, key1, w4);
-      const int2 shard = sh.shard[wn];
-      const int row0 = sh.row0[i];
+      const int rows = (c * B + rb1) & ~rb1;
+      int sum = rows;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int b = blk * 4 + q;
-        if (b < B) a.row_idx[pn][row0 + b] = shard.x + (int)__umulhi(w4[q], (unsigned)shard.y);
+      for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, sum, o); if (lane >= o) sum += x; }
+      const int first = carry + sum - rows;
+      if (u <= S && warp == 0) { sh.cnt[u] = c; sh.grow0[u] = first; }
+      const int mine = __shfl_sync(0xffffffffu, first + before * B, tau & 31);
+      if (tau >= 0 && (tau & ~31) == u0) row0_me = mine + rank_in_warp * B;
+      carry += __shfl_sync(0xffffffffu, sum, 31);
+    }
+    n_rows = carry;
+  }
+  if (tid < K) {
+    a.sel[pn][tid] = n;
+    a.sel_tau[pn][tid] = tau;
+    a.sel_row0[pn][tid] = row0_me;
+    sh.row0[tid] = row0_me;
+    sh.sel_n[tid] = n;
+  }
+  if (tid == 0) {
+    st->T_end = T_end;
+    st->last_id = last;
+    st->n_rows = n_rows;
+    st->n_row_tiles = net ? n_rows >> k.rb_shift : K;
+    st->open = 1;
+    RoundInfo info;
+    info.n_rows = n_rows; info.K = K; info.t = t; info.diverged = 0;
+    a.ri[pn] = info;
+    sh.scalar[4] = K; sh.scalar[5] = t;
+  }
+  if (!net) return 0;           // least squares: no row tiles, minibatches drawn by its own kernel
+  __syncthreads();
+  // ring slot of every row tile and padding rows, one warp per staleness group
+  {
+    const int sh_rb = k.rb_shift, RB = 1 << sh_rb, tm = t % (S + 1);
+#pragma unroll 1
+    for (int g = warp; g <= S; g += NWP) {
+      const int c = sh.cnt[g];
+      if (c == 0) continue;
+      const int r0 = sh.grow0[g], p0 = r0 + c * B, p1 = r0 + ((c * B + RB - 1) & ~(RB - 1));
+      const int slot = tm - g < 0 ? tm - g + S + 1 : tm - g;      // (t - g) mod (S + 1); g <= S
+#pragma unroll 1
+      for (int q = (r0 >> sh_rb) + lane; q < (p1 >> sh_rb); q += 32) {
+        a.tile_slot[pn][q] = slot;
+        a.tile_real[pn][q] = min(RB, p0 - (q << sh_rb));
       }
+#pragma unroll 1
+      for (int r = p0 + lane; r < p1; r += 32) a.row_idx[pn][r] = -1;
+    }
+  }
+  if (!a.draw) return 0;
+  // minibatch draws: sample b of job (n, j) = word b%4 of Philox block (n, j, 1, b/4),
+  // mapped into the worker's shard [n M / N, (n+1) M / N)
+  const int blocks_per = (B + 3) >> 2;
+#pragma unroll 1
+  for (int item = tid; item < K * blocks_per; item += NT) {
+    const int i = a.by_blk.div(item), blk = item - i * blocks_per;
+    const int wn = sh.sel_n[i];
+    uint32_t w4[4];
+    philox4x32_10((uint32_t)wn, (uint32_t)sh.job[wn], 1u, (uint32_t)blk, k.key0, k.key1, w4);
+    const int2 shard = sh.shard[wn];
+    const int row0 = sh.row0[i];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int b = blk * 4 + q;
+      if (b < B) a.row_idx[pn][row0 + b] = shard.x + (int)__umulhi(w4[q], (unsigned)shard.y);
     }
   }
   return 0;

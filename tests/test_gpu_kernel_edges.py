@@ -3,10 +3,33 @@ tolerances of the parity tests."""
 import pytest
 
 from helpers import compare_with_oracle
+from paper_2301_08895_b200 import abs as gpu
 from paper_2301_08895_b200 import inputs
-from test_gpu_parity import GAMMA3, TOL_FP32, _problem, _small_cfg
+from test_gpu_parity import GAMMA3, PARETO, TOL_FP32, _problem, _small_cfg
 
 pytestmark = pytest.mark.gpu
+
+CONST = inputs.TimeSpec(kind=inputs.T_CONST, shift=1.0)
+
+
+@pytest.mark.parametrize("W", [1, 31, 32, 33, 64, 65, 128, 129, 256, 257])
+@pytest.mark.parametrize("time", [GAMMA3, CONST], ids=["gamma", "ties"])
+def test_control_step_worker_counts(W, time):
+    """Ranks by counting (8, 4, 2 lanes per key), by merging, 1024 threads; loss sums of one and of several warps; equal ticks."""
+    cfg = _small_cfg(inputs.SOFTMAX, (12, 3), inputs.FP32, W, 5, max(1, W // 3), 5, time, lr=0.02)
+    X, y, w0 = _problem(cfg)
+    compare_with_oracle(cfg, X, y, w0, 25, TOL_FP32, forced=True)
+
+
+@pytest.mark.parametrize("W,K0,S,B", [
+    (90, 2, 70, 3),        # staleness groups beyond 32 and 64
+    (24, 24, 3, 85),       # 2040 rows and padding: more row losses than the step fetches ahead of time
+    (300, 100, 6, 13),     # ... with 1024 threads
+])
+def test_control_step_row_layouts(W, K0, S, B):
+    cfg = _small_cfg(inputs.SOFTMAX, (12, 3), inputs.FP32, W, B, K0, S, PARETO, lr=0.01)
+    X, y, w0 = _problem(cfg)
+    compare_with_oracle(cfg, X, y, w0, 60 if W == 90 else 15, TOL_FP32, forced=True, k_mode=gpu.K_FIXED)
 
 
 @pytest.mark.parametrize("dims,W,B,U", [
