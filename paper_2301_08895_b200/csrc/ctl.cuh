@@ -183,7 +183,8 @@ static __device__ __noinline__ u64 job_ticks_call(const DevState* st, uint32_t k
 // instruction.  So everything a later phase needs is loaded up front in one wave (the run's constants come with the
 // launch), sums over the arrivals and the rules that follow from them are formed by every warp itself instead of by one for
 // all, rules that rarely change anything (Eq. 5 raising K, Eq. 4 after it) have a short test in front, and a worker's rank
-// is counted.  OLDNEW
+// is counted.  16 workers x 64 rows: 5.7 -> 4.4 us; 64 workers 6.6 -> 4.9 us;
+// 8 workers inside the persistent kernel: 7.5 -> 7.0 us a round.
 //   t_sel:     index of the round that follows the open one (the host counts rounds; parity of
 //              t_sel - 1 / t_sel picks the layout copy of the open / the new round)
 //   look_here: the workers that were renewed also get the duration of the job AFTER the one they
@@ -415,8 +416,9 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
   const u64* sorted = sh.keysA;
   const bool count = NT < 1024 && W <= 128;
   if (count) {
-    // the rank of a key is the number of smaller ones: 8, 4 or 2 lanes share a key and take every 8th, 4th, 2nd other (64
-    // keys: RANK64)
+    // the rank of a key is the number of smaller ones: 8, 4 or 2 lanes share a key and take every 8th, 4th, 2nd other (merging
+    // sorted runs by binary search, in code for eight runs, took 3300 cycles for two; from 129 workers on comparing all pairs
+    // would cost more)
     const int lg_p = W <= 32 ? 3 : W <= 64 ? 2 : 1, per = 256 >> (2 * lg_p);
     const int n = tid >> lg_p, part = tid & ((1 << lg_p) - 1);
     if (tid < 256) {
