@@ -774,6 +774,8 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
       q.X = (const __nv_bfloat16*)ctx->X; q.y = a.y; q.ring = (const __nv_bfloat16*)a.ring; q.slot_stride = a.slot_stride;
       q.loss_part = ctx->at<float>(L.row_loss); q.G = a.G; q.d = a.d; q.stages = ctx->lsq_stages;
       q.groups = (m.batch + lsqp::GROUP - 1) / lsqp::GROUP;
+      q.by_groups = FastDiv(q.groups);
+      q.W = ctx->W; q.B = m.batch; q.S = ctx->S; q.sa = m.sa_penalty; q.key0 = ctx->ctl.k.key0; q.key1 = ctx->ctl.k.key1;
       const size_t sm = lsqp::smem_bytes(a.d, ctx->lsq_stages);
       launch_ex(ctx, ABS_KC_LSQ, lsqp::lsq_pipe_kernel, dim3(ctx->lsq_grid), dim3(lsqp::THREADS), sm, q);
     } else if (ctx->lsq_v2) {
@@ -1067,7 +1069,7 @@ void enqueue_update(abs_ctx* ctx, int par) {
     q.master = ctx->at<float>(L.master); q.ring = ctx->at<void>(L.ring); q.G = ctx->at<float>(L.G);
     q.d_pad = L.d_pad; q.d = ctx->m.dims[0]; q.P = ctx->lsq_grid; q.lr = ctx->m.lr;
     q.loss_part = ctx->lsq_pipe ? ctx->at<float>(L.row_loss) : nullptr;
-    q.loss = ctx->ctl.loss; q.groups = (ctx->m.batch + lsqp::GROUP - 1) / lsqp::GROUP;
+    q.loss = ctx->ctl.loss; q.groups = (ctx->m.batch + lsqp::TROWS - 1) / lsqp::TROWS;
     const int blocks = std::max((q.d + 31) / 32, (ctx->W + 31) / 32);
     launch_ex(ctx, ABS_KC_UPDATE, lsq_update_kernel<T>, dim3(blocks), dim3(256), 0, q);
     return;
@@ -1399,7 +1401,7 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
     // the pipeline kernel leaves per-group loss sums: the control step finishes the uploaded losses
     // itself (it runs next to the Eq. 3 kernel, which finishes them too, for its own divergence check)
     ctx->ctl.loss_part = ctx->at<float>(L.row_loss);
-    ctx->ctl.loss_groups = (model->batch + lsqp::GROUP - 1) / lsqp::GROUP;
+    ctx->ctl.loss_groups = (model->batch + lsqp::TROWS - 1) / lsqp::TROWS;
   }
   rc = setup_tc(ctx);
   if (rc != ABS_OK) return bail(rc);

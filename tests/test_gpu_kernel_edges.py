@@ -5,7 +5,7 @@ import pytest
 from helpers import compare_with_oracle
 from paper_2301_08895_b200 import abs as gpu
 from paper_2301_08895_b200 import inputs
-from test_gpu_parity import GAMMA3, PARETO, TOL_FP32, _problem, _small_cfg
+from test_gpu_parity import GAMMA3, PARETO, TOL_BF16, TOL_FP32, _problem, _small_cfg
 
 pytestmark = pytest.mark.gpu
 
@@ -41,3 +41,11 @@ def test_local_steps_rows_per_owner(dims, W, B, U):
     cfg = _small_cfg(inputs.SOFTMAX, dims, inputs.FP32, W, B, 3, 5, GAMMA3, lr=0.02)
     X, y, w0 = _problem(cfg)
     compare_with_oracle(cfg, X, y, w0, 6, TOL_FP32, forced=True, local_steps=U)
+
+
+@pytest.mark.parametrize("d,B", [(8, 9), (2040, 13), (2048, 4), (2056, 5), (4096, 1), (4096, 3), (4088, 16)])
+def test_least_squares_pipeline_teams(d, B):
+    """Rows for one team only, one column slice per thread, items more than the first four of a CTA."""
+    cfg = _small_cfg(inputs.LSQ, (d, 1), inputs.BF16, 300, B, 150, 6, GAMMA3, lr=0.02 / d)
+    X, y, w0 = _problem(cfg)
+    compare_with_oracle(cfg, X, y, w0, 6, TOL_BF16, forced=True, loss_tol=5e-2)
