@@ -840,13 +840,14 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     a.delta_in = (l == 0) ? nullptr : ctx->at<void>(L.delta[l]);
     a.row_loss = L.local_net ? ctx->at<float>(L.row_loss) : ctx->ctl.row_loss; a.G = ctx->at<float>(L.G); a.P = L.P;
     a.rpb = L.narrow_rpb;
+    a.sa = m.sa_penalty ? (L.local_net ? 2 : 1) : 0; a.S = ctx->S;
     return a;
   };
   auto conv_mma_args = [&]() {
     cmma::Args c;
     memset(&c, 0, sizeof c);
     c.st = st; c.ri = ri; c.tile_slot = ctx->ctl.tile_slot[par]; c.row_idx = ctx->ctl.row_idx[par];
-    c.ring = ctx->at<void>(L.ring); c.slot_stride = L.d_pad; c.k = L.ck;
+    c.ring = ctx->at<void>(L.ring); c.slot_stride = L.d_pad; c.k = L.ck; c.rb_shift = ctx->ctl.k.rb_shift;
     conv_blocks(L, c.b);
     c.X = (const __nv_bfloat16*)ctx->X;
     c.pool1 = ctx->at<__nv_bfloat16>(L.pool1); c.arg1 = ctx->at<unsigned char>(L.arg1);
@@ -884,6 +885,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
       DrawArgs q;
       q.st = st; q.ri = ri; q.sel = ctx->ctl.sel[par]; q.sel_row0 = ctx->ctl.sel_row0[par]; q.job = ctx->ctl.job; q.shard = ctx->ctl.shard;
       q.row_idx = ctx->ctl.row_idx[par]; q.by_B = FastDiv(m.batch); q.tile_real = ctx->ctl.tile_real[par]; q.RB = L.RB;
+      q.W = ctx->W; q.B = m.batch; q.key0 = ctx->ctl.k.key0; q.key1 = ctx->ctl.k.key1;
       launch_on(ctx, ctx->overlap ? ctx->side : s, ABS_KC_GATHER, draw_gather_kernel, dim3(ctx->sm_count * 8), dim3(256), 0, q,
                 (const __nv_bfloat16*)ctx->X, ctx->at<__nv_bfloat16>(par ? L.act0b : L.act[0]), m.dims[0]);
     } else if (gathered)
@@ -899,6 +901,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     a.X = L.cnn ? ctx->at<void>(par ? L.act0b : L.act[0]) : ctx->X;
     a.gather = L.cnn ? 0 : 1;
     a.job = ctx->ctl.job; a.next_dur = ctx->ctl.next_dur; a.dur_job = ctx->ctl.dur_job; a.W = ctx->W;
+    a.sa = m.sa_penalty; a.S = ctx->S;
     a.n_layers = nl; a.want_d0 = L.cnn ? 1 : 0; a.row_loss = ctx->ctl.row_loss;
     for (int l = 0; l <= nl; ++l) {
       a.dims[l] = m.dims[l];
@@ -1107,6 +1110,7 @@ void enqueue_update(abs_ctx* ctx, int par) {
   UpdateArgs u;
   u.st = ctx->at<DevState>(L.st); u.ri = ri; u.master = ctx->at<float>(L.master); u.ring = ctx->at<void>(L.ring);
   u.G = ctx->at<float>(L.G); u.d_pad = L.d_pad; u.P = L.P; u.lr = ctx->m.lr;
+  u.B = ctx->m.batch; u.S = ctx->S; u.sa = ctx->m.sa_penalty ? (L.local_net ? 2 : 1) : 0;
   u.sel_tau = ctx->ctl.sel_tau[par];
   // for the latency-bound models (always one stream) the Eq. 3 kernel also prepares the next job
   // durations (its first warps); tensor-core networks keep a small kernel of their own for that

@@ -158,6 +158,10 @@ __device__ __forceinline__ float sa_weight(int tau) { return tau > 1 ? __fdiv_rn
 __device__ __forceinline__ float sa_slot_weight(const DevState* st, int t, int slot) {
   return st->sa_penalty == 1 ? sa_weight((t - slot) % (st->S + 1)) : 1.f;
 }
+// ... with the constants handed to the kernel (a load of them in front of the kernel's other loads costs a trip to memory)
+__device__ __forceinline__ float sa_slot_weight(int sa, int S, int t, int slot) {
+  return sa == 1 ? sa_weight((t - slot) % (S + 1)) : 1.f;
+}
 
 __host__ __device__ inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 __host__ __device__ inline size_t round_up_sz(size_t a, size_t b) { return (a + b - 1) / b * b; }

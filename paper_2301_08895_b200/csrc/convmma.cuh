@@ -43,7 +43,7 @@ struct Args {
   const int* row_idx;
   const void* ring; size_t slot_stride;
   const bf16* frag; size_t frag_stride;  // [S+1][frag_stride] weights as column operands (see FragMap)
-  int k;
+  int k, rb_shift;                       // rows per tile_slot entry = 1 << rb_shift
   Block b[2];
   const bf16* X;                         // dataset images
   bf16* pool1; unsigned char* arg1;      // [rows][Ph1][Pw1][C1] pooled maps of the first block, position of each maximum
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(NT) conv_fwd_mma_kernel(const __grid_constant_
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char cs[];
   const int r0 = (int)blockIdx.x * FR;
-  const int status = a.st->status, n_rows = a.ri->n_rows, RB = a.st->RB;
+  const int status = a.st->status, n_rows = a.ri->n_rows, slot = a.tile_slot[r0 >> a.rb_shift];
   int s[FR];
   bool any = false;
 #pragma unroll
@@ -330,7 +330,6 @@ __global__ void __launch_bounds__(NT) conv_fwd_mma_kernel(const __grid_constant_
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = K ? K : a.k;
   const FwdLayout& f = a.fl;
   const Block &x = a.b[0], &y = a.b[1];
-  const int slot = a.tile_slot[r0 / RB];
   const bf16* ring = (const bf16*)a.ring + (size_t)slot * a.slot_stride;
   const int n_in = x.Hi * x.Wi * x.Ci, P1 = even(x.Wi * x.Ci), P2 = even(y.Wi * y.Ci);
   const int n1 = x.Ph * x.Pw * x.Co, n2 = y.Ph * y.Pw * y.Co;
@@ -418,7 +417,7 @@ __global__ void __launch_bounds__(NT, 3) conv_bwd_mma_kernel(const __grid_consta
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char cs[];
   const int r0 = (int)blockIdx.x * FR;
-  const int status = a.st->status, n_rows = a.ri->n_rows, RB = a.st->RB;
+  const int status = a.st->status, n_rows = a.ri->n_rows, slot = a.tile_slot[r0 >> a.rb_shift];
   int s[FR];
 #pragma unroll
   for (int j = 0; j < FR; ++j) s[j] = a.row_idx[r0 + j];
@@ -427,7 +426,6 @@ __global__ void __launch_bounds__(NT, 3) conv_bwd_mma_kernel(const __grid_consta
   const int g = lane >> 2, t = lane & 3;
   const BwdLayout& f = a.bl;
   const Block &x = a.b[0], &y = a.b[1];
-  const int slot = a.tile_slot[r0 / RB];
   bf16* im = reinterpret_cast<bf16*>(cs + f.im);
   bf16* in2 = reinterpret_cast<bf16*>(cs + f.in2);
   uint32_t* dz1 = reinterpret_cast<uint32_t*>(cs + f.dz1);

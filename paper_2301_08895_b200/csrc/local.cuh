@@ -338,12 +338,13 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
   constexpr int NT = CL_NT, GE = group_elems<T>(), C4 = CP / 4;
   DevState* st = a.st;
   RoundInfo* ri = a.ri;
-  if (st->status != ST_OK) return;
   const int Q = geo.Q, F = geo.F, RQ = geo.RQ, pitch = geo.pitch, PZ = geo.PZ, PG = geo.PG;
-  const int i = (int)blockIdx.x / Q;
-  if (i >= ri->K) return;                            // same decision in every CTA of the cluster
+  const int i = (int)blockIdx.x / Q;                 // (< W: its entries exist whether or not it is selected)
+  const int status = st->status, K = ri->K, t_round = ri->t, B = st->B, S = st->S, wn = a.sel[i], tau = a.sel_tau[i];
+  const uint32_t key0 = st->key0, key1 = st->key1;
+  if (status != ST_OK || i >= K) return;             // same decision in every CTA of the cluster
   const int rank = Q > 1 ? (int)tc::cluster_rank() : 0;
-  const int B = st->B, in = a.in, C = a.C, U = a.U;
+  const int in = a.in, C = a.C, U = a.U;
   const int n_w = in * C;
   const int m0 = rank * F, nf = max(0, min(F, in - m0));     // this CTA's features
   const int b_own = rank * RQ, n_own = max(0, min(RQ, B - b_own));      // rows whose soft-max it forms
@@ -364,14 +365,13 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
   __shared__ int gave_up;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool last_warp = warp == NT / 32 - 1;
-  const int wn = a.sel[i], jb = a.job[wn];
+  const int jb = a.job[wn];
   const int2 shard = a.shard[wn];
-  const int slot = (ri->t - a.sel_tau[i]) % (st->S + 1);
+  const int slot = (t_round - tau) % (S + 1);
   const T* w0 = (const T*)a.ring + (size_t)slot * a.slot_stride;
   const T* X = (const T*)a.X + m0;
   const int nblk = (B + 3) >> 2;
   const float step = __fdiv_rn(a.lr, (float)B);
-  const uint32_t key0 = st->key0, key1 = st->key1;
 
   auto draw = [&](int u) {                           // sample indices of step u (last warp)
     int* dst = sidx + (u % 3) * Br;

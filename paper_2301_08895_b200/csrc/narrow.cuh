@@ -48,20 +48,25 @@ struct DrawArgs {
   int* row_idx;
   const int* tile_real; int RB;
   FastDiv by_B;
+  int W, B; uint32_t key0, key1;
 };
 __global__ void __launch_bounds__(256) draw_gather_kernel(DrawArgs a, const __nv_bfloat16* X, __nv_bfloat16* act0, int in) {
   grid_dependency_sync();
-  const int status = a.st->status, K = a.ri->K, B = a.st->B, n_rows = a.ri->n_rows;
-  const uint32_t key0 = a.st->key0, key1 = a.st->key1;
-  if (status != ST_OK) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int w0 = blockIdx.x * 8 + warp, nw = gridDim.x * 8;
-  for (int it = w0; it < K * B; it += nw) {
-    const int i = a.by_B.div(it), b = it - i * B;
-    const int n = a.sel[i], r = a.sel_row0[i] + b;
+  const int w0 = blockIdx.x * 8 + warp, nw = gridDim.x * 8, B = a.B;
+  // (a selected worker's entries exist whether or not it is selected this round: they come with the round's sizes)
+  int i = a.by_B.div(w0), n = 0, row0 = 0;
+  if (i < a.W) { n = a.sel[i]; row0 = a.sel_row0[i]; }
+  const int status = a.st->status, K = a.ri->K, n_rows = a.ri->n_rows;
+  if (status != ST_OK) return;
+  for (int it = w0; it < K * B;) {
+    const int b = it - i * B, r = row0 + b;
     const int2 shard = a.shard[n];
     uint32_t w4[4];
-    philox4x32_10((uint32_t)n, (uint32_t)a.job[n], 1u, (uint32_t)(b >> 2), key0, key1, w4);
+    philox4x32_10((uint32_t)n, (uint32_t)a.job[n], 1u, (uint32_t)(b >> 2), a.key0, a.key1, w4);
+    it += nw;
+    i = a.by_B.div(it);
+    if (it < K * B) { n = a.sel[i]; row0 = a.sel_row0[i]; }
     const uint32_t wd = (b & 3) == 0 ? w4[0] : (b & 3) == 1 ? w4[1] : (b & 3) == 2 ? w4[2] : w4[3];
     const int s = shard.x + (int)__umulhi(wd, (unsigned)shard.y);
     if (lane == 0) a.row_idx[r] = s;
@@ -88,6 +93,7 @@ struct NarrowArgs {
   void* delta_in;          // [rows][in] storage type (dgrad result)
   float* row_loss;         // [rows]
   float* G; int P;
+  int sa, S;               // DevState's staleness-aware step size and ring (output-layer kernel on matrix instructions)
   int rpb;                 // gradient rows per block of the row-tiled kernels below (8..64, a multiple of 8; 0 = 64)
 };
 

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
   const int g = lane >> 2, t = lane & 3;
   // one wave of loads (the grid covers the row capacity, so every address exists); warp (mt, kh) finishes the soft-max of
   // rows 16 mt + 8 kh + g
-  const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[r0 >> a.tile_shift];
+  const int status = st->status, n_rows = ri->n_rows, t_round = ri->t, slot = a.tile_slot[r0 >> a.tile_shift];
   const int my_row = 16 * (warp & 3) + 8 * (warp >> 2) + g;
   const int my_idx = a.row_idx[r0 + my_row];
   if (status != ST_OK || r0 >= n_rows) return;
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(THREADS) out_layer_mma_kernel(NarrowArgs a, fl
                  "l"(src + (size_t)rr * IN + v * 8) : "memory");
   }
   const int lab = my_idx < 0 ? -1 : a.labels[my_idx];
-  const float sa = sa_slot_weight(st, ri->t, slot);     // staleness-aware step size: weight of these rows in Eq. 3
+  const float sa = sa_slot_weight(a.sa, a.S, t_round, slot);     // staleness-aware step size: weight of these rows in Eq. 3
   const __nv_bfloat16* Wm = (const __nv_bfloat16*)a.ring + (size_t)slot * a.slot_stride + a.w_off;
   {
     // weights + bias are contiguous and start on a 128-byte boundary: whole 16-byte pieces

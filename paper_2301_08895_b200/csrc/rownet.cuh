@@ -47,6 +47,7 @@ struct RowsArgs {
   float* row_loss;                       // [rows]
   size_t w_off[ABS_MAX_LAYERS];          // element offset of W[in][out]; the bias follows it as row `in`
   int n_layers, dims[ABS_MAX_LAYERS + 1];
+  int sa, S;                             // DevState's staleness-aware step size and ring
   int want_d0;                           // also the delta of the layer-0 input (CNN features, masked by feature > 0)
   // Weights in shared memory.  resident: every layer is copied once and stays (stage l = layer l, the backward pass
   // reads it again); otherwise chunks of rpc[l] rows stream through `stages` stages, forward and again backward.
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = (int)blockIdx.x * R;
   // one wave of loads (the grid covers the row capacity, so every address exists)
-  const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[blockIdx.x];
+  const int status = st->status, n_rows = ri->n_rows, t_round = ri->t, slot = a.tile_slot[blockIdx.x];
   const int my_idx = a.row_idx[r0 + lane % R];       // sample index of row lane % R
   if (status != ST_OK) return;
   // the fetching warps of the first CTAs also prepare job durations, off the critical path
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(THREADS, 1) rows_fma_kernel(const __grid_const
       for (int rr = warp; rr < R; rr += NW) {
         float* zr = z + (rr / 4) * C * 4 + (rr & 3);
         const float2 d = row_softmax<float>(a, lane < C ? zr[lane * 4] : 0.f, lane + 32 < C ? zr[(lane + 32) * 4] : 0.f, r0 + rr, lab[rr],
-                                            sa_slot_weight(st, ri->t, slot), lane);
+                                            sa_slot_weight(a.sa, a.S, t_round, slot), lane);
         float* gd = (float*)a.delta[L] + (size_t)(r0 + rr) * C;
         if (lane < C) { zr[lane * 4] = d.x; gd[lane] = d.x; }
         if (lane + 32 < C) { zr[(lane + 32) * 4] = d.y; gd[lane + 32] = d.y; }
@@ -613,7 +614,7 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const __grid_c
   const int r0 = (int)blockIdx.x * R;
   const int my_row = warp / WPR;                     // two warps (of 16) or one fetch a row
   // one wave of loads (the grid covers the row capacity, so every address exists)
-  const int status = st->status, n_rows = ri->n_rows, slot = a.tile_slot[blockIdx.x];
+  const int status = st->status, n_rows = ri->n_rows, t_round = ri->t, slot = a.tile_slot[blockIdx.x];
   const int my_idx = a.row_idx[r0 + my_row], lab_idx = tid < R ? a.row_idx[r0 + tid] : -1;
   if (status != ST_OK) return;
   const int look = (int)blockIdx.x * 32 < a.W ? (int)blockIdx.x * 32 + lane : a.W;
@@ -726,7 +727,7 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) rows_mma_kernel(const __grid_c
       for (int rr = warp; rr < R; rr += NWM) {
         const float* z = logits + rr * (C + 1);
         const float2 d = row_softmax<T>(a, lane < C ? z[lane] : 0.f, lane + 32 < C ? z[lane + 32] : 0.f, r0 + rr, lab[rr],
-                                        sa_slot_weight(st, ri->t, slot), lane);
+                                        sa_slot_weight(a.sa, a.S, t_round, slot), lane);
         T* gd = (T*)a.delta[L] + (size_t)(r0 + rr) * C;
         if (lane < C) { dl[rr * mma_pitch(C) + lane] = __float2bfloat16_rn(d.x); gd[lane] = __float2bfloat16_rn(d.x); }
         if (lane + 32 < C) { dl[rr * mma_pitch(C) + lane + 32] = __float2bfloat16_rn(d.y); gd[lane + 32] = __float2bfloat16_rn(d.y); }

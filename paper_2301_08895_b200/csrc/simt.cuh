@@ -337,6 +337,7 @@ struct UpdateArgs {
   const int* sel_tau;     // [K^t] staleness of each selected worker's upload (read when the staleness-aware
                           // step size is applied to whole uploads: DevState::sa_penalty == 2, P == 0)
   float lr;
+  int B, S, sa;           // constants of the run (sa: DevState's staleness-aware step size)
   // Parts of the gradient that are still per-chunk partial sums (the output layer's block left by the fused
   // output kernels; bias gradients left as column sums per 32 rows by the back-propagation GEMM): blocks
   // [n_main_blocks, gridDim.x) add the chunks of 32 parameters each in a fixed order and apply Eq. 3 to those
@@ -363,15 +364,15 @@ __global__ void __launch_bounds__(256, 4) update_kernel(UpdateArgs a) {
   grid_dependency_sync();
   const DevState* st = a.st;
   const RoundInfo* ri = a.ri;
-  if (st->status != ST_OK) return;
+  const int status = st->status, diverged = ri->diverged, K = ri->K, t = ri->t, n_rows = ri->n_rows;       // (one trip to memory)
+  if (status != ST_OK) return;
   // duration look-ahead for the workers whose job index moved (first warp of the first ceil(N/32) blocks)
   if (LOOK && threadIdx.x < 32 && (int)blockIdx.x * 32 < st->W)
     refresh_next_durations(st, a.job, a.next_dur, a.dur_job, (int)blockIdx.x * 32 + (int)threadIdx.x);
-  if (ri->diverged) return;
-  const int K = ri->K;
+  if (diverged) return;
   const int P = a.P > 0 ? a.P : K;
-  const float step = __fdiv_rn(a.lr, (float)(K * st->B));
-  const int slot = (ri->t + 1) % (st->S + 1);
+  const float step = __fdiv_rn(a.lr, (float)(K * a.B));
+  const int slot = (t + 1) % (a.S + 1);
   T* dst = (T*)a.ring + (size_t)slot * a.d_pad;
   if ((int)blockIdx.x >= a.n_main_blocks) {
     // lane w adds chunks w, w + 8, ... in order, then the 8 lanes are added in order
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(256, 4) update_kernel(UpdateArgs a) {
     for (int q = 1; q < UpdateArgs::MAX_REGIONS; ++q)
       if (q < a.n_regions && rb >= a.region[q].first_block) ri_ = q;
     const UpdateArgs::Region& R = a.region[ri_];
-    const int n_chunks = ri->n_rows / R.chunk_rows;
+    const int n_chunks = n_rows / R.chunk_rows;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int j = (rb - R.first_block) * 32 + lane;
     float acc = 0.f;
@@ -434,7 +435,7 @@ __global__ void __launch_bounds__(256, 4) update_kernel(UpdateArgs a) {
   };
   // few partials (the split counts of the weight-gradient GEMMs): two vectors per thread and
   // iteration, all loads of both issued before the first use (same sums, same order per element)
-  const bool weigh = a.P == 0 && st->sa_penalty == 2;
+  const bool weigh = a.P == 0 && a.sa == 2;
   if (P <= 4 && !weigh) {
     for (; i + stride < n4; i += 2 * stride) {
       const size_t j = i + stride;

@@ -286,8 +286,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
 
   // from here on the kernel reads what its predecessors wrote (device state, layouts, operands)
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const bool running = st->status == ST_OK;
-  const int n_rows = running ? ri->n_rows : 0;
+  // (one trip to memory: with the round's sizes comes the version of this unit's first tile, where that is tile `unit`; all
+  // rows of a 128-row tile have one version)
+  const int status = st->status, rows_now = ri->n_rows;
+  const bool slot_ahead = p0.mode != WGRAD && p1.mode < 0;
+  const int n_ct0 = (p0.N_total + BN - 1) / BN;
+  const int first_slot = slot_ahead ? p0.tile_slot[unit / n_ct0 * CG] : 0;
+  const bool running = status == ST_OK;
+  const int n_rows = running ? rows_now : 0;
   const int n_row_tiles = n_rows / TM_ROWS;
   auto make_prob = [&](const Params& q) -> Prob {
     Prob r;
@@ -341,7 +347,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   // a CTA (pair) without work, or a run that has ended, goes straight to the teardown (same
   // decision in both CTAs of a pair)
   const bool has_work = running && tile_at(0) >= 0;
-  const int RB = st->RB;
 
   auto tile_coord = [&](int gtile) -> TileCoord {
     TileCoord c;
@@ -369,7 +374,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       c.bias_tile = 0;
       c.a_row = rt * TM_ROWS + rank * BM;
       c.b_col = (tile - rt * P.n_ct) * BN;
-      c.slot = q.tile_slot[(rt * TM_ROWS) / RB];
+      c.slot = slot_ahead && tile == unit ? first_slot : q.tile_slot[rt * CG];
       c.k_begin = 0;
       c.n_kb = (q.K_total + BK - 1) / BK;
     }
