@@ -294,32 +294,6 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
-// stores to shared memory of a CTA of the cluster, counted on that CTA's mbarrier (addresses: mapa)
-__device__ __forceinline__ void st_async4(uint32_t addr, float4 v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
-               ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_async1(uint32_t addr, float v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
-}
-// the bytes other CTAs stored have arrived (acquire at cluster scope); bounded like tc::mbar_wait
-__device__ __forceinline__ uint32_t test_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-               : "=r"(ok) : "r"(tc::smem_u32(bar)), "r"(parity) : "memory");
-  return ok;
-}
-__device__ __noinline__ void wait_cluster_slow(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
-  const unsigned long long t0 = tc::global_ns();
-  for (uint32_t i = 1; i < (1u << 28); ++i) {
-    if (test_cluster(bar, parity)) return;
-    if ((i & 63u) == 0u && (*gave_up || tc::global_ns() - t0 > tc::WAIT_LIMIT_NS)) break;
-  }
-  *gave_up = 1;
-}
-__device__ __forceinline__ void wait_cluster(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
-  if (!test_cluster(bar, parity)) wait_cluster_slow(bar, parity, gave_up);
-}
 __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
 // one 16-byte group of stored values as binary32
@@ -448,7 +422,7 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
   // ---- logits, loss, deltas of this CTA's rows: four lanes per row, four classes each
   auto softmax = [&](int par, uint32_t parity) {
     if (warp * 8 >= n_own) return;
-    if (Q > 1) wait_cluster(&bar_z, parity, &gave_up);
+    if (Q > 1) tc::wait_cluster(&bar_z, parity, &gave_up);
 #pragma unroll 1
     for (int b0 = 0; b0 + warp * 8 < n_own; b0 += NT / 4) {
       const int b = b0 + (tid >> 2), l = tid & 3;    // row b_own + b
@@ -502,8 +476,8 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
         if (Q > 1) {
 #pragma unroll
           for (int q = 0; q < 8; ++q)
-            if (q < Q) st_async4(tc::map_to_cta(dl_a + off, (uint32_t)q), dv, tc::map_to_cta(bar_d_a, (uint32_t)q));
-          if (l == 0) st_async1(tc::map_to_cta(tc::smem_u32(rl + b_own + b), 0u), loss, tc::map_to_cta(bar_d_a, 0u));
+            if (q < Q) tc::st_async4(tc::map_to_cta(dl_a + off, (uint32_t)q), dv, tc::map_to_cta(bar_d_a, (uint32_t)q));
+          if (l == 0) tc::st_async1(tc::map_to_cta(tc::smem_u32(rl + b_own + b), 0u), loss, tc::map_to_cta(bar_d_a, 0u));
         } else {
           *reinterpret_cast<float4*>(dl + (size_t)b * CP + 4 * l) = dv;
           if (l == 0) rl[b] = loss;
@@ -572,7 +546,7 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
         continue;
       }
       const int owner = by_rq.div(b);                // element e of the step is element e - owner RQ C4 of its owner's
-      st_async4(tc::map_to_cta(zin_a + (uint32_t)(e - owner * RQ * C4) * 16u, (uint32_t)owner), z, tc::map_to_cta(bar_z_a, (uint32_t)owner));
+      tc::st_async4(tc::map_to_cta(zin_a + (uint32_t)(e - owner * RQ * C4) * 16u, (uint32_t)owner), z, tc::map_to_cta(bar_z_a, (uint32_t)owner));
     }
     // the next rows are fetched while the exchange is on its way (behind the soft-max by the warps that form it)
     if (Q == 1) __syncthreads();
@@ -581,7 +555,7 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
     softmax(u & 1, parity);
     if (ahead && early) fetch(u + 1);
     if (last_warp && u + 2 < U) draw(u + 2);
-    if (Q > 1) wait_cluster(&bar_d, parity, &gave_up);
+    if (Q > 1) tc::wait_cluster(&bar_d, parity, &gave_up);
     else __syncthreads();
     // ---- gradient of this slice: item = (column group, every PG-th row)
     for (int it = tid; it < groups * PG; it += NT) {

@@ -776,7 +776,7 @@ constexpr int GP = GT + 4;               // shared-memory pitch
 constexpr int MP = GT + 8;               // ... bf16 (five 16-byte units: ldmatrix reads without bank conflicts)
 
 struct StepArgs {
-  const DevState* st;
+  DevState* st;
   const RoundInfo* ri;
   const int* row_idx;
   const void* X; int gather;
@@ -799,7 +799,8 @@ struct StepArgs {
 // Four groups of 64 threads take 16 rows of a 64-row step each (fp32: 4 x 4 sums per thread, two 16-byte shared-memory
 // reads for eight packed FMAs, two steps' rows in registers on the way; bf16: matrix instructions with the products added
 // in fp32: the FMA form was bound by shared-memory reads; 201-133-10, 4096 rows: 60.7 -> 52.8 us a round, CNN 76.9 -> 75.5).  Groups are added in order, each CTA of a cluster
-// hands its sums to the owner of their share, which adds them in order and applies Eq. 3.
+// hands its sums to the owner of their share (remote stores counted on the owner's barrier: a cluster barrier's release waits
+// for all of a CTA's stores: 784-10 fp32, 1024 rows 13.74 -> 13.31 us a round, 59-10 10.39 -> 10.01), which adds them in order and applies Eq. 3.
 // Bound by the chain of dependent latencies (indices, rows, exchange), so: the tile is found before the wait for the
 // kernels in front, indices come with the round's sizes in one wave of loads, the weights a CTA updates are fetched
 // before its sums exist.  784 x 10 fp32, 1024 rows: 6.4 -> 4 us
@@ -811,8 +812,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 3) grad_step_kernel(
   __shared__ __align__(16) T tiles[4][GK][P];        // two stages of inputs, two of deltas
   T (*As)[GK][P] = tiles, (*Ds)[GK][P] = tiles + 2;
   float (*red)[GT * GT] = reinterpret_cast<float (*)[GT * GT]>(tiles);     // sums of the four groups, at the end
-  __shared__ float box[GT * GT];                     // sums of this CTA's share: [CTA of the cluster][share]
+  __shared__ __align__(16) float box[GT * GT];       // sums of this CTA's share: [CTA of the cluster][share]
+  __shared__ uint64_t box_bar;                       // ... have arrived
+  __shared__ int gave_up;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) {
+    tc::mbar_init(&box_bar, 1);
+    gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    tc::mbar_expect_tx(&box_bar, GT * GT * 4);
+  }
   const int n_tiles = a.first_tile[a.n_layers];
   const int Q = a.Q, rank = (int)blockIdx.x & (Q - 1), tile = min((int)blockIdx.x >> a.q_shift, n_tiles - 1);
   int l = 0;
@@ -825,7 +834,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 3) grad_step_kernel(
   const T* D = (const T*)a.delta[l + 1];
   const int m = m0 + lane, n = n0 + lane;
   grid_dependency_sync();
-  const DevState* st = a.st;
+  DevState* st = a.st;
   const RoundInfo* ri = a.ri;
   // row 8 i + warp of a step is loaded by this warp; lane i < 8 holds its sample index
   auto load_idx = [&](int s) -> int {
@@ -956,18 +965,27 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 3) grad_step_kernel(
   }
   __syncthreads();
   if (Q > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  {
+    const int e = 4 * tid;                           // (a share is 128 elements or more)
+    float4 v[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int e = tid + 256 * i;
-    const float v = (red[0][e] + red[1][e]) + (red[2][e] + red[3][e]);
+    for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const float4*>(&red[k][e]);
+    const float4 s = make_float4((v[0].x + v[1].x) + (v[2].x + v[3].x), (v[0].y + v[1].y) + (v[2].y + v[3].y),
+                                 (v[0].z + v[1].z) + (v[2].z + v[3].z), (v[0].w + v[1].w) + (v[2].w + v[3].w));
     if (Q > 1) {
-      const int owner = e >> (10 - a.q_shift);       // (GT x GT = 2^10)
-      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(tc::map_to_cta(tc::smem_u32(box + rank * share + (e & (share - 1))), (uint32_t)owner)), "f"(v) : "memory");
+      const uint32_t owner = (uint32_t)(e >> (10 - a.q_shift));       // (GT x GT = 2^10)
+      tc::st_async4(tc::map_to_cta(tc::smem_u32(box + rank * share + (e & (share - 1))), owner), s, tc::map_to_cta(tc::smem_u32(&box_bar), owner));
+      tc::wait_cluster(&box_bar, 0u, &gave_up);
+      if (gave_up) {                                 // (ends the run)
+        st->timeout_where = 500;
+        st->status = ST_TIMEOUT;
+        return;
+      }
     } else {
-      box[e] = v;                                    // read back by the same thread
+      *reinterpret_cast<float4*>(box + e) = s;
+      __syncthreads();
     }
   }
-  if (Q > 1) tc::cluster_sync_all();
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     if (o[i] == (size_t)-1) continue;

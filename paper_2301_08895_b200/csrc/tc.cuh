@@ -156,6 +156,32 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// stores to shared memory of a CTA of the cluster, counted on that CTA's mbarrier (addresses: mapa)
+__device__ __forceinline__ void st_async4(uint32_t addr, float4 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async1(uint32_t addr, float v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
+}
+// the bytes other CTAs stored have arrived (acquire at cluster scope); bounded like mbar_wait
+__device__ __forceinline__ uint32_t test_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+  return ok;
+}
+static __device__ __noinline__ void wait_cluster_slow(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+  const unsigned long long t0 = global_ns();
+  for (uint32_t i = 1; i < (1u << 28); ++i) {
+    if (test_cluster(bar, parity)) return;
+    if ((i & 63u) == 0u && (*gave_up || global_ns() - t0 > WAIT_LIMIT_NS)) break;
+  }
+  *gave_up = 1;
+}
+__device__ __forceinline__ void wait_cluster(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+  if (!test_cluster(bar, parity)) wait_cluster_slow(bar, parity, gave_up);
+}
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
