@@ -257,11 +257,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                const Params p0,
                const __grid_constant__ CUtensorMap map_a1, const __grid_constant__ CUtensorMap map_b1,
                const __grid_constant__ CUtensorMap map_out1, const Params p1) {
-  // The kernel in front of this one may still be running (programmatic stream serialization): the
-  // kernel behind this one may be scheduled as early, and everything that does not read the
-  // predecessors' results -- barriers, the tensor-memory allocation, descriptor prefetch -- is done
-  // before the wait for them.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The kernel in front of this one may still be running (programmatic stream serialization): everything that does not
+  // read the predecessors' results -- barriers, the tensor-memory allocation, descriptor prefetch -- is done before the
+  // wait for them.  The kernel behind this one may become resident from that wait on.
   using C = Cfg<BN, CG>;
   constexpr int TM_ROWS = BM * CG;              // rows of one tile
   extern __shared__ uint8_t smem_raw[];
@@ -310,6 +308,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   const uint32_t acc_empty0_addr = (CG == 2) ? map_to_cta(smem_u32(&acc_empty[0]), 0) : smem_u32(&acc_empty[0]);
   const uint32_t tmem_base = *tmem_slot;
 
+  // The kernel behind this one may become resident when every CTA of this one holds its SM and its tensor memory.  As the
+  // kernel's first statement this let the Eq. 3 kernel's waiting blocks take the SM slots in front of the side stream's gather,
+  // and the next forward pass waited for both (3072-1024-512-10, 16 workers x 64 rows: the gather started 79 us into a round
+  // instead of 67; us a round 96.5 -> 92.2, 32 workers 121 -> 118, 128 workers 188 -> 186; 784-256-10, ten local steps 500 ->
+  // 487; 1024-1024-1024-10, 24 workers 83.1 -> 84.3: there the gather now runs beside the weight gradient).  Behind the wait
+  // below it is too late: 784-256-10, 32 workers 37.3 -> 41.1.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // from here on the kernel reads what its predecessors wrote (device state, layouts, operands)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // (one trip to memory: with the round's sizes comes the version of this unit's first tile, where that is tile `unit`; all
