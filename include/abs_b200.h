@@ -302,9 +302,9 @@ int abs_profile_timeline(abs_ctx* ctx, int cap, int* cls, float* start_ms, float
 /* Test aid for the failure path of the device-side waits (the paper has no counterpart).  Every wait
  * inside the library's kernels (on an mbarrier or a completion counter) gives up after a time limit,
  * raises the context's device status and lets the kernel return normally.  This call launches a
- * one-warp kernel that waits, with the library's own wait routine and a limit of limit_us
- * microseconds (1 .. 1000000), on a barrier that nothing ever signals, then synchronises.  It is
- * expected to return ABS_ETIMEOUT (abs_last_error names site 900); the context is then in the same
+ * cluster of two CTAs and a one-warp kernel that wait, with the library's own wait routines and a limit of limit_us
+ * microseconds (1 .. 1000000), on barriers that nothing ever signals, then synchronises.  It is
+ * expected to return ABS_ETIMEOUT (abs_last_error names site 900 when both gave up); the context is then in the same
  * sticky state as after a real expiry: no further rounds, while abs_get_params, abs_get_trace and
  * abs_destroy keep working.  Nothing faults, traps or hangs. */
 int abs_selftest_wait_timeout(abs_ctx* ctx, int limit_us);

@@ -1141,6 +1141,7 @@ void enqueue_update(abs_ctx* ctx, int par) {
 int read_status(abs_ctx* ctx, DevState* host) {
   CU(cudaMemcpyAsync(host, ctx->at<DevState>(ctx->L.st), sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
+  if (host->timeout_where != 0) host->status = ST_TIMEOUT;       // (of the last round: no control step has seen it)
   return ABS_OK;
 }
 
@@ -1932,6 +1933,9 @@ int abs_selftest_wait_timeout(abs_ctx* ctx, int limit_us) {
   if (!ctx) return fail(ABS_EINVAL, "ctx is null");
   if (ctx->sticky != ABS_OK) return fail(ctx->sticky, "context is in a failed state (%d)", ctx->sticky);
   if (limit_us < 1 || limit_us > 1000000) return fail(ABS_EINVAL, "limit_us %d outside [1, 1000000]", limit_us);
+  ctx->next_cluster = 2;
+  launch_ex(ctx, ABS_KC_CTL, tc::wait_cluster_selftest_kernel, dim3(2), dim3(64), 0, ctx->at<DevState>(ctx->L.st), 1000ull * (unsigned long long)limit_us);
+  if (ctx->launch_error != cudaSuccess) return cuda_fail(ctx, ctx->launch_error, "kernel launch");
   tc::wait_selftest_kernel<<<1, 32, 0, ctx->stream>>>(ctx->at<DevState>(ctx->L.st), 1000ull * (unsigned long long)limit_us);
   ctx->launches += 1;
   CU(cudaGetLastError());

@@ -68,7 +68,7 @@ struct DevState {
   int last_id;                    // worker of the open round's last arrival
   i64 sel_total, rst_total;       // flat trace fill
   u64 comm;                       // communication-round counter (Sec. V-B)
-  int timeout_where;
+  int timeout_where;              // site of a bounded wait that expired (0: none); ends the run also while status is still ST_OK
 };
 
 // What the gradient kernels of one round need to know about it.  Two copies alternate by round

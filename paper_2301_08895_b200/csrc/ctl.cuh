@@ -226,7 +226,7 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     if (a.draw) my_shard = a.shard[tid];
     if (do_finish && !net && a.loss_part == nullptr) my_loss = a.loss[tid];
   }
-  const int status0 = st->status, open0 = st->open, diverged0 = a.ri[po].diverged;
+  const int status0 = st->status, expired0 = st->timeout_where, open0 = st->open, diverged0 = a.ri[po].diverged;
   const u64 T_end0 = st->T_end;
   const float L0_prev = st->L0;
   const i64 sel_off = st->sel_total, rst_off = st->rst_total;
@@ -242,6 +242,10 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     my_loss = __fdiv_rn(s, (float)B);
   }
   if (status0 != ST_OK) return 1;
+  if (expired0 != 0) {                                // (by a kernel that may not change the status while it runs)
+    if (tid == 0) raise(ST_TIMEOUT);
+    return 1;
+  }
   const bool fin = do_finish && open0;
 
   int restart = 0, renewed = 0;                       // this thread's worker started a new job in the finish step

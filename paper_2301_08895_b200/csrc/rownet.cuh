@@ -976,9 +976,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 3) grad_step_kernel(
       const uint32_t owner = (uint32_t)(e >> (10 - a.q_shift));       // (GT x GT = 2^10)
       tc::st_async4(tc::map_to_cta(tc::smem_u32(box + rank * share + (e & (share - 1))), owner), s, tc::map_to_cta(tc::smem_u32(&box_bar), owner));
       tc::wait_cluster(&box_bar, 0u, &gave_up);
-      if (gave_up) {                                 // (ends the run)
-        st->timeout_where = 500;
-        st->status = ST_TIMEOUT;
+      if (__syncthreads_or(gave_up)) {               // ends the run; all threads alike, so that no share is half applied
+        tc::leave_cluster();
+        // not st->status: a cluster that starts later must find the same status in all of its CTAs, or one of them leaves and
+        // the others store to it.  The next control step and the host take the run for ended by this word.
+        if (tid == 0) st->timeout_where = 500;
         return;
       }
     } else {

@@ -171,16 +171,23 @@ __device__ __forceinline__ uint32_t test_cluster(uint64_t* bar, uint32_t parity)
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok;
 }
-static __device__ __noinline__ void wait_cluster_slow(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+static __device__ __noinline__ void wait_cluster_slow(uint64_t* bar, uint32_t parity, volatile int* gave_up, unsigned long long limit_ns) {
   const unsigned long long t0 = global_ns();
   for (uint32_t i = 1; i < (1u << 28); ++i) {
     if (test_cluster(bar, parity)) return;
-    if ((i & 63u) == 0u && (*gave_up || global_ns() - t0 > WAIT_LIMIT_NS)) break;
+    if ((i & 63u) == 0u && (*gave_up || global_ns() - t0 > limit_ns)) break;
   }
   *gave_up = 1;
 }
-__device__ __forceinline__ void wait_cluster(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
-  if (!test_cluster(bar, parity)) wait_cluster_slow(bar, parity, gave_up);
+__device__ __forceinline__ void wait_cluster(uint64_t* bar, uint32_t parity, volatile int* gave_up, unsigned long long limit_ns = WAIT_LIMIT_NS) {
+  if (!test_cluster(bar, parity)) wait_cluster_slow(bar, parity, gave_up, limit_ns);
+}
+// The end of a CTA whose wait_cluster ran out: all its threads come here.  Another CTA of the cluster may be late and still store to
+// this one, so it stays until every thread of the cluster has come here too or has left, and then until what they sent has landed.
+__device__ __forceinline__ void leave_cluster() {
+  cluster_sync_all();
+  const unsigned long long t0 = global_ns();
+  while (global_ns() - t0 < 200000ull) {}
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -826,10 +833,29 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   }
 }
 
-// Self-test of the bounded wait: one warp initialises a barrier that expects one arrival, nobody
+// Self-test of the bounded waits.  A cluster of two CTAs: both expect bytes that nobody stores, their waits must give up, and the
+// first reports it as grad_step_kernel does (site only).  Then one warp initialises a barrier that expects one arrival, nobody
 // ever arrives, and lane 0 waits on it with the given limit.  The wait must give up, and the
-// kernel then reports it the way the round-loop kernels do (status word + site), and returns.
-constexpr int TIMEOUT_SITE_SELFTEST = 900;
+// kernel then reports it the way the other round-loop kernels do (status word + site), and returns.
+constexpr int TIMEOUT_SITE_SELFTEST = 900, TIMEOUT_SITE_SELFTEST_CLUSTER = 901;
+__global__ void wait_cluster_selftest_kernel(DevState* st, unsigned long long limit_ns) {
+  grid_dependency_sync();
+  __shared__ uint64_t bar;
+  __shared__ int gave_up;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_expect_tx(&bar, 16);
+  }
+  __syncthreads();
+  cluster_sync_all();
+  wait_cluster(&bar, 0u, &gave_up, limit_ns);
+  if (__syncthreads_or(gave_up)) {
+    leave_cluster();
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->timeout_where = TIMEOUT_SITE_SELFTEST_CLUSTER;
+  }
+}
 __global__ void wait_selftest_kernel(DevState* st, unsigned long long limit_ns) {
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
@@ -839,7 +865,7 @@ __global__ void wait_selftest_kernel(DevState* st, unsigned long long limit_ns) 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (threadIdx.x == 0 && !mbar_wait(&bar, 0u, &abort_flag, limit_ns)) {
+  if (threadIdx.x == 0 && !mbar_wait(&bar, 0u, &abort_flag, limit_ns) && st->timeout_where == TIMEOUT_SITE_SELFTEST_CLUSTER) {
     st->timeout_where = TIMEOUT_SITE_SELFTEST;
     st->status = ST_TIMEOUT;
   }

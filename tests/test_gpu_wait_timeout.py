@@ -60,3 +60,35 @@ def test_selftest_rejects_bad_limits():
         assert e.value.code == gpu.EINVAL
     ctx.run_rounds(2)                                  # an argument error is not sticky
     ctx.close()
+
+
+def test_expiry_known_by_its_site_ends_the_run_at_the_next_control_step():
+    """A kernel whose clusters must all see one status leaves only the site of an expired wait (here written by hand into the
+    device state); the next control step ends the run on it, and the host reports it where no control step follows."""
+    import torch
+    cfg = inputs.config(2).scaled(n_samples=4096)
+    X, y, _ = inputs.make_data(cfg)
+    w0 = inputs.make_w0(cfg)
+    Xd, yd = to_device(cfg, X, y)
+    probe = gpu.context_from_config(cfg, Xd, yd, w0, max_rounds=20)
+    with pytest.raises(gpu.AbsError):
+        probe.selftest_wait_timeout(1000)
+    words = probe.workspace[:1024].view(torch.int32)   # the device state is the first piece of the workspace
+    at = (words == 900).nonzero().flatten().tolist()
+    assert len(at) == 1
+    probe.close()
+    for more in (3, 0):
+        ctx = gpu.context_from_config(cfg, Xd, yd, w0, max_rounds=20)
+        ctx.run_rounds(5)
+        params = ctx.get_params()
+        ctx.workspace[:1024].view(torch.int32)[at[0]] = 500
+        torch.cuda.synchronize()
+        ctx.enqueue_rounds(more)
+        done, rc = ctx.rounds_done()
+        assert (done, rc) == (5, gpu.ETIMEOUT)
+        assert "site 500" in gpu.last_error()
+        assert np.array_equal(ctx.get_params(), params)
+        with pytest.raises(gpu.AbsError) as e:
+            ctx.run_rounds(1)
+        assert e.value.code == gpu.ETIMEOUT
+        ctx.close()
