@@ -608,6 +608,10 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
       }
     }
     __syncthreads();
+    // A wait of this step ran out: the run ends (below).  No further step, whose bytes would be announced on a barrier that still
+    // waits for this step's; the peers' waits then run out as well.  (All waits lie behind the step's first barrier and before
+    // this one, so all threads read the same.)
+    if (gave_up) break;
     if (geo.nbuf == 1 && u + 1 < U) fetch(u + 1);    // the gradient has read the only row buffer
     // ---- the local step
     for (int e = tid; e < n_g; e += NT) {
@@ -627,8 +631,14 @@ __global__ void __launch_bounds__(CL_NT, cluster_ctas_per_sm(group_elems<T>(), C
                         round_store(w.z, (const T*)nullptr), round_store(w.w, (const T*)nullptr));
     }
   }
-  if (Q > 1) tc::cluster_sync_all();                 // (a wait that ran out: no peer stores to a CTA that has left)
-  else __syncthreads();
+  if (gave_up) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    tc::leave_cluster();                             // (no peer stores to a CTA that has left)
+  } else if (Q > 1) {
+    tc::cluster_sync_all();
+  } else {
+    __syncthreads();
+  }
   float* out = a.G + (size_t)i * a.slot_stride;
   const float sa = st->sa_penalty ? sa_weight(a.sel_tau[i]) : 1.f;   // staleness-aware step size: weight of the upload in Eq. 3
   for (int e = tid; e < nf * C; e += NT) {
