@@ -250,6 +250,10 @@ bool tiles_win(const abs_model_desc* m, const Layout& L, long long rows) {
   return !L.cnn && back > 700000 && rows < 512;      // (the CNN's convolutions lose their matrix-instruction kernels with the row kernels)
 }
 
+// Staleness-aware step size: 1 applied to the delta rows / residuals by the gradient kernels; 2, with local steps on a network,
+// whose local copies need the plain gradient sums, by Eq. 3 to the uploads.
+int sa_mode(const abs_model_desc& m, const Layout& L) { return m.sa_penalty ? (L.local_net ? 2 : 1) : 0; }
+
 // Gradient rows the buffers hold when version groups are padded to L->RB rows.
 void row_capacity(const abs_model_desc* m, int W, int S, Layout* L) {
   const int groups = (W < S + 1) ? W : S + 1;
@@ -775,7 +779,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
       q.loss_part = ctx->at<float>(L.row_loss); q.G = a.G; q.d = a.d; q.stages = ctx->lsq_stages;
       q.groups = (m.batch + lsqp::GROUP - 1) / lsqp::GROUP;
       q.by_groups = FastDiv(q.groups);
-      q.W = ctx->W; q.B = m.batch; q.S = ctx->S; q.sa = m.sa_penalty; q.key0 = ctx->ctl.k.key0; q.key1 = ctx->ctl.k.key1;
+      q.W = ctx->W; q.B = m.batch; q.S = ctx->S; q.sa = sa_mode(m, L); q.key0 = ctx->ctl.k.key0; q.key1 = ctx->ctl.k.key1;
       const size_t sm = lsqp::smem_bytes(a.d, ctx->lsq_stages);
       launch_ex(ctx, ABS_KC_LSQ, lsqp::lsq_pipe_kernel, dim3(ctx->lsq_grid), dim3(lsqp::THREADS), sm, q);
     } else if (ctx->lsq_v2) {
@@ -840,7 +844,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     a.delta_in = (l == 0) ? nullptr : ctx->at<void>(L.delta[l]);
     a.row_loss = L.local_net ? ctx->at<float>(L.row_loss) : ctx->ctl.row_loss; a.G = ctx->at<float>(L.G); a.P = L.P;
     a.rpb = L.narrow_rpb;
-    a.sa = m.sa_penalty ? (L.local_net ? 2 : 1) : 0; a.S = ctx->S;
+    a.sa = sa_mode(m, L); a.S = ctx->S;
     return a;
   };
   auto conv_mma_args = [&]() {
@@ -901,7 +905,7 @@ void enqueue_gradient(abs_ctx* ctx, int par, int phase) {
     a.X = L.cnn ? ctx->at<void>(par ? L.act0b : L.act[0]) : ctx->X;
     a.gather = L.cnn ? 0 : 1;
     a.job = ctx->ctl.job; a.next_dur = ctx->ctl.next_dur; a.dur_job = ctx->ctl.dur_job; a.W = ctx->W;
-    a.sa = m.sa_penalty; a.S = ctx->S;
+    a.sa = sa_mode(m, L); a.S = ctx->S;
     a.n_layers = nl; a.want_d0 = L.cnn ? 1 : 0; a.row_loss = ctx->ctl.row_loss;
     for (int l = 0; l <= nl; ++l) {
       a.dims[l] = m.dims[l];
@@ -1110,7 +1114,7 @@ void enqueue_update(abs_ctx* ctx, int par) {
   UpdateArgs u;
   u.st = ctx->at<DevState>(L.st); u.ri = ri; u.master = ctx->at<float>(L.master); u.ring = ctx->at<void>(L.ring);
   u.G = ctx->at<float>(L.G); u.d_pad = L.d_pad; u.P = L.P; u.lr = ctx->m.lr;
-  u.B = ctx->m.batch; u.S = ctx->S; u.sa = ctx->m.sa_penalty ? (L.local_net ? 2 : 1) : 0;
+  u.B = ctx->m.batch; u.S = ctx->S; u.sa = sa_mode(ctx->m, L);
   u.sel_tau = ctx->ctl.sel_tau[par];
   // for the latency-bound models (always one stream) the Eq. 3 kernel also prepares the next job
   // durations (its first warps); tensor-core networks keep a small kernel of their own for that
@@ -1278,10 +1282,7 @@ int abs_init(abs_ctx** out, const abs_model_desc* model, int W, int K0, int stal
   h.W = W; h.K0 = K0; h.S = S_ring; h.B = model->batch; h.RB = L.RB;
   h.theta_cap = staleness_bound; h.literal_eq6 = literal;
   h.no_restart = model->restart_rule == ABS_RESTART_NONE ? 1 : 0;
-  // staleness-aware step size: applied to the delta rows / residuals by the gradient kernels, except
-  // with local steps on a network, whose local copies need the plain gradient sums (there Eq. 3
-  // weights the uploads)
-  h.sa_penalty = model->sa_penalty ? (L.local_net ? 2 : 1) : 0;
+  h.sa_penalty = sa_mode(*model, L);
   h.k_mode = model->k_mode; h.bound_mode = model->bound_mode; h.max_rounds = model->max_rounds;
   h.n_samples = model->n_samples;
   h.key0 = (uint32_t)(seed & 0xffffffffull); h.key1 = (uint32_t)(seed >> 32);

@@ -155,13 +155,11 @@ __device__ __forceinline__ float sa_weight(int tau) { return tau > 1 ? __fdiv_rn
 // Weight of the gradient rows of a tile that reads ring slot `slot` in round t: a consumed gradient
 // is at most S rounds old, so its staleness is (t - slot) mod (S + 1) (slot = version mod (S + 1)
 // and version <= t, so t - slot is never negative).
-__device__ __forceinline__ float sa_slot_weight(const DevState* st, int t, int slot) {
-  return st->sa_penalty == 1 ? sa_weight((t - slot) % (st->S + 1)) : 1.f;
-}
-// ... with the constants handed to the kernel (a load of them in front of the kernel's other loads costs a trip to memory)
+// sa, S: DevState's, handed to the kernel where a load of them in front of its other loads would cost a trip to memory.
 __device__ __forceinline__ float sa_slot_weight(int sa, int S, int t, int slot) {
   return sa == 1 ? sa_weight((t - slot) % (S + 1)) : 1.f;
 }
+__device__ __forceinline__ float sa_slot_weight(const DevState* st, int t, int slot) { return sa_slot_weight(st->sa_penalty, st->S, t, slot); }
 
 __host__ __device__ inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 __host__ __device__ inline size_t round_up_sz(size_t a, size_t b) { return (a + b - 1) / b * b; }

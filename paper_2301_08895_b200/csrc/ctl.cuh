@@ -88,15 +88,15 @@ __device__ __forceinline__ void refresh_next_durations(const DevState* st, const
 }
 
 // ---------------------------------------------------------------------------------------------
-// Sort of up to 1024 distinct 64-bit keys, one per thread, by ranking: inside a warp every key counts the smaller keys
-// of its warp (31 shuffles, no dependent chain), which leaves sorted runs of 32.  Up to eight runs are merged at once:
-// a key's place is the number of smaller keys in every other run, found by binary searches that run side by side (256
+// Sort of n = 256 (NT < 1024), 512 or 1024 distinct 64-bit keys, one per thread, by ranking: inside a warp every key counts
+// the smaller keys of its warp (31 shuffles, no dependent chain), which leaves sorted runs of 32.  Eight runs are merged at
+// once: a key's place is the number of smaller keys in every other run, found by binary searches that run side by side (256
 // keys: 1.5k cycles instead of 3.1k with pairwise merges); more runs are merged pairwise, where one search per key and
 // level is less shared-memory traffic.  Returns the buffer (A or B) that holds the sorted keys.
 template <int NT>
-__device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n_pow2) {
+__device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n) {
   const int tid = threadIdx.x, lane = tid & 31;
-  const bool active = tid < n_pow2;            // whole warps: n_pow2 is a multiple of 32
+  const bool active = tid < n;                 // whole warps
   if (active) {
     int rank = 0;
 #pragma unroll
@@ -104,11 +104,10 @@ __device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n_p
     A[(tid - lane) + rank] = key;
   }
   __syncthreads();
-  if (n_pow2 == 32) return A;
-  if (NT <= 512 && n_pow2 <= 256) {
+  if (NT < 1024) {
     if (active) {
       const u64 k = A[tid];
-      const int own = tid >> 5, runs = n_pow2 >> 5;
+      const int own = tid >> 5;
       int lo[8];
 #pragma unroll
       for (int r = 0; r < 8; ++r) lo[r] = 0;
@@ -116,11 +115,11 @@ __device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n_p
       for (int step = 16; step > 0; step >>= 1)
 #pragma unroll
         for (int r = 0; r < 8; ++r)
-          if (r < runs) lo[r] += A[r * 32 + lo[r] + step - 1] < k ? step : 0;     // at most 31 of a run after the last step
+          lo[r] += A[r * 32 + lo[r] + step - 1] < k ? step : 0;     // at most 31 of a run after the last step
       int rank = 0;
 #pragma unroll
       for (int r = 0; r < 8; ++r)
-        if (r < runs) rank += r == own ? lane : lo[r] + (A[r * 32 + lo[r]] < k ? 1 : 0);
+        rank += r == own ? lane : lo[r] + (A[r * 32 + lo[r]] < k ? 1 : 0);
       B[rank] = k;
     }
     __syncthreads();
@@ -128,7 +127,7 @@ __device__ __forceinline__ u64* rank_merge_sort(u64 key, u64* A, u64* B, int n_p
   }
   u64* src = A;
   u64* dst = B;
-  for (int L = 32; L < n_pow2; L <<= 1) {
+  for (int L = 32; L < n; L <<= 1) {
     if (active) {
       const u64 k = src[tid];
       const int pair_base = tid & ~(2 * L - 1);
@@ -437,9 +436,7 @@ __device__ __forceinline__ int ctl_round(const CtlArgs& a, CtlShared& sh, int do
     }
     __syncthreads();
   } else {
-    int n_pow2 = 32;
-    while (n_pow2 < W) n_pow2 <<= 1;
-    sorted = rank_merge_sort<NT>(sh.keysA[tid], sh.keysA, sh.keysB, n_pow2);
+    sorted = rank_merge_sort<NT>(sh.keysA[tid], sh.keysA, sh.keysB, NT < 1024 ? 256 : W <= 512 ? 512 : 1024);
   }
   int n = -1, tau = -1;
   u64 T_end = 0ull;

@@ -38,6 +38,7 @@ constexpr int CONSUMERS = TEAMS * TEAM;
 constexpr int THREADS = CONSUMERS + 64;  // + producer warp + a warp that prepares job durations
 constexpr int BATCH = 32 / GROUP;        // items whose rows the producer's lanes hold
 constexpr int MAX_STAGES = 6;
+constexpr int SA_LEN = 8;                // weights of the stages, padded: what follows starts on a 16-byte boundary
 constexpr int RS = 12;                   // floats between rows of the partial-dot table [TROWS][RS]: 16-byte reads of the rows'
                                          // halves by 8 lanes fall into different banks
 constexpr int RED = 2 * TEAMS * TROWS * RS;      // ... of both teams, twice
@@ -62,7 +63,7 @@ struct Args {
 
 inline size_t stage_bytes(int d) { return (size_t)(GROUP + 1) * d * 2; }
 inline size_t smem_bytes(int d, int stages) {
-  return std::max((size_t)stages * stage_bytes(d), (size_t)TEAM * 64) + (size_t)MAX_STAGES * (GROUP + 2) * 4 + RED * 4 +
+  return std::max((size_t)stages * stage_bytes(d), (size_t)TEAM * 64) + (size_t)(MAX_STAGES * GROUP + SA_LEN + RED) * 4 +
          2 * MAX_STAGES * 8 + 64;
 }
 
@@ -112,8 +113,8 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(const __grid_const
   const size_t stg = (size_t)(GROUP + 1) * row_bytes;
   unsigned char* stage0 = lsm;                                             // (and the teams' exchange at the end)
   float* m_y = reinterpret_cast<float*>(lsm + max((size_t)STAGES * stg, (size_t)TEAM * 64));     // [MAX_STAGES][GROUP] targets
-  float* m_sa = m_y + MAX_STAGES * GROUP;                                  // [MAX_STAGES][2] weight of the worker's gradient in Eq. 3
-  float* red = m_sa + 2 * MAX_STAGES;                                           // [2][TEAMS][TROWS][RS] partial dots, [row][warp]
+  float* m_sa = m_y + MAX_STAGES * GROUP;                                  // [MAX_STAGES] weight of the worker's gradient in Eq. 3
+  float* red = m_sa + SA_LEN;                                              // [2][TEAMS][TROWS][RS] partial dots, [row][warp]
   uint64_t* full = reinterpret_cast<uint64_t*>(red + RED);                 // [STAGES]
   uint64_t* empty = full + MAX_STAGES;                                     // [STAGES]
   volatile int* abort = reinterpret_cast<volatile int*>(empty + MAX_STAGES);
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(const __grid_const
         if ((lane >> 3) == e) {                      // the lanes that hold the item's rows; the first also the weights
           unsigned char* sb = stage0 + (size_t)stage * stg;
           if (r == 0) {
-            m_sa[2 * stage] = a.sa ? sa_weight(cur.tau) : 1.f;       // staleness-aware step size
+            m_sa[stage] = a.sa ? sa_weight(cur.tau) : 1.f;       // staleness-aware step size
             tc::mbar_expect_tx(&full[stage], (uint32_t)(rows + 1) * row_bytes);
             bulk_row(sb + (size_t)GROUP * row_bytes, a.ring + (size_t)slot * a.slot_stride, row_bytes, &full[stage]);
           }
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(THREADS, 1) lsq_pipe_kernel(const __grid_const
         }
       }
       // the rows are in registers now: hand the stage back to the producer
-      const float yv = m_y[stage * GROUP + r0 + (lane & 3)], sa = m_sa[2 * stage];
+      const float yv = m_y[stage * GROUP + r0 + (lane & 3)], sa = m_sa[stage];
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&empty[stage]);
       if (++stage == STAGES) { stage = 0; phase ^= 1u; }
