@@ -216,11 +216,13 @@ __global__ void __launch_bounds__(NT_MAX) local_sgd_kernel(Args a) {
 //     both as remote stores that complete on the receiver's mbarrier (st.async; launched as a cluster only, Q > 1): no
 //     cluster barrier inside a step,
 //   - the copies of the next rows and the draws of the step after that are issued while the exchange is on its way.
-// A step is bound by its chain of phases (partial dots, exchange, soft-max, exchange, gradient, reduction), each a few
-// hundred to 1500 cycles of dependent shared-memory reads.  With a cluster barrier and remote loads (2400 cycles: its release
-// waits for all stores), bulk copies of the row slices by one warp that also took part in the soft-max (64 copies: 6900
-// cycles) a step of 784 -> 10, 16 workers x 64 rows took 14000 cycles, now 9000 (a round of ten steps 91.7 -> 73.1 us; 20 to 64
-// workers 74 us and 143 us; 2 to 16 classes, 87 to 687 features 1.12 to 1.43 times as fast).
+// A step is bound by its chain of phases, each of dependent shared-memory reads: 784 -> 10, 16 workers x 64 rows, cycles at 1.96
+// GHz: partial logits 1930, sum and send 720, soft-max with the wait for the logits 1810, copies of the next rows 1190, wait for
+// the deltas 160, gradient 1750, local step 1390, barriers 310: 9300.  With a cluster barrier and remote loads (2400 cycles: its
+// release waits for all stores) and bulk copies of the row slices by one warp that also took part in the soft-max (64 copies:
+// 6900 cycles) a step took 14000 (a round of ten steps 91.7 -> 73.1 us; 20 to 64 workers 74 us and 143 us; 2 to 16 classes, 87
+// to 687 features 1.12 to 1.43 times as fast).  Of the kernel's 66 us the start-up (job, draws, model slice, first rows, cluster
+// start) is 5 and the upload 1.4; the steps are 46 us in 14 of the 16 clusters, 53 and 59 in the two whose CTAs share SMs.
 // Both buffers of the exchange are used again in the next step.  A CTA sends step u + 1's logits after it has all deltas of
 // step u, so every owner has read its logits of step u; an owner sends step u + 1's deltas after every CTA has sent its
 // logits of step u + 1, that is after the gradient of step u.
@@ -253,9 +255,9 @@ inline size_t cluster_smem(const Geo& g, int esz, int B, int CP) {
 // the clusters of n workers take more than one wave: for models below 2048 parameters (its CTAs are 256 threads there, and
 // several share an SM) and for large ones whose clusters of two take two partial waves.  us a round, one-CTA / cluster,
 // U = 10, all workers selected: 64 -> 10 bf16, 1024 workers, 4 rows 176 / 282, 8 rows 204 / 292, 12 rows 274 / 293; 200
-// workers, 8 rows 84 / 85, 12 rows 117 / 86; 64 -> 1 fp32, 512 workers, 4 rows 64 / 78, 8 rows 76 / 82, 12 rows 91 / 84;
-// 784 -> 10 bf16, 100 workers, 4 rows 117 / 147, 8 rows 129 / 143, 16 rows 165 / 159; 784 -> 10 fp32, 145 workers, 64 rows
-// 363 / 343.
+// workers, 6 rows 79 / 89, 8 rows 83 / 86, 10 rows 116 / 90; 64 -> 1 fp32, 512 workers, 4 rows 64 / 78, 8 rows 76 / 82, 12 rows
+// 91 / 84; 784 -> 10 bf16, 100 workers, 8 rows 131 / 146, 10 rows 144 / 156, 12 rows 148 / 156, 14 rows 165 / 166, 16 rows 167 /
+// 162; 148 workers, 8 rows 136 / 152, 12 rows 152 / 163; 784 -> 10 fp32, 145 workers, 64 rows 363 / 343.
 inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) {
   const int CP = round_up(C, 4), ge = 16 / esz;
   const int wave = PLAN_SMS * cluster_ctas_per_sm(ge, CP);
@@ -279,7 +281,7 @@ inline Geo cluster_plan(int in, int C, int n_par, int B, int W, int n, int esz) 
   Geo none = geo(1, 1);
   none.Q = 0;
   if (n_par < 2048 && (B <= 8 ? n * first > wave : B <= 12 && wave == PLAN_SMS && n * first > 2 * wave)) return none;
-  if (n_par > 6000 && B <= 8 && first == 2 && n * first > wave) return none;
+  if (n_par > 6000 && B <= 12 && first == 2 && n * first > wave) return none;
   for (int nbuf = 2; nbuf >= 1; --nbuf)
     for (int Q = first; Q <= 8; Q *= 2) {
       const Geo g = geo(Q, nbuf);

@@ -46,6 +46,14 @@ def test_local_steps_rows_per_owner(dims, W, B, U):
     compare_with_oracle(cfg, X, y, w0, 6, TOL_FP32, forced=True, local_steps=U)
 
 
+@pytest.mark.parametrize("B", [12, 13])
+def test_local_steps_few_rows_of_a_large_model(B):
+    """One CTA per worker up to 12 rows, clusters above."""
+    cfg = _small_cfg(inputs.SOFTMAX, (784, 10), inputs.BF16, 100, B, 100, 5, GAMMA3, lr=0.005)
+    X, y, w0 = _problem(cfg)
+    compare_with_oracle(cfg, X, y, w0, 4, TOL_BF16, forced=True, loss_tol=5e-2, local_steps=3)
+
+
 # Least-squares runs from a w0 of the size of the generating weights, so that x.w weighs as much as y in every residual.
 # Binary32 sums leave losses and path at 1e-6.  From round 1 on a stored weight (of size 1) may lie on the other side of a bf16
 # rounding, 2^-8 away; n of those change a residual of size sqrt(2 d) by about sqrt(n) 2^-8, a loss by 2 sqrt(n) 2^-8 / sqrt(2 d):
