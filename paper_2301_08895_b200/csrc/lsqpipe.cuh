@@ -10,10 +10,10 @@
 // r_b = x_b . w_v - y_b) and then the gradient contribution sum_b r_b x_b into accumulators that
 // persist over all items of the CTA.  Every sample row is read from HBM exactly once and from
 // shared memory exactly once.  Inside an item a team runs one chain (wait, reads, dots, exchange, residuals, gradient);
-// the teams wait for nothing of each other but the stages, so one's arithmetic fills the other's latencies.  With one team of
-// 512 threads an item took 2900 cycles whatever the copies did (its 72 KB arrive in 3100 at the copy
-// bandwidth of the whole chip); now 2700, which is 7.0 TB/s of rows.  The inner loops are packed FMAs on operands kept in
-// 64-bit registers.  A round of a few items per CTA is its start-up, so nothing is staged for all of a CTA's items first (5600
+// the teams wait for nothing of each other but the stages, so one's arithmetic fills the other's latencies.  An item's 64 KB
+// of rows per SM take 2880 cycles at the chip's copy rate (6552 GB/s; 1.947 GHz; a copy also writes); its 8 KB model vector comes
+// from L2.  An item takes 2770 cycles, 6.8 TB/s of rows, where a CTA has 28 (mean over all CTAs), 2890 where it has 3 or 4; with
+// one team of 512 threads 2900 to 3000.  The inner loops are packed FMAs on operands kept in 64-bit registers.  A round of a few items per CTA is its start-up, so nothing is staged for all of a CTA's items first (5600
 // cycles for 4 items, 10600 for 28: the targets' loads queued behind the first items' copies): the producer's lanes draw four
 // items' samples at a time, fetch what the draws of the next four need meanwhile, and a row's target arrives with its item,
 // by an asynchronous copy counted on the same barrier.  Eq. 3 only
